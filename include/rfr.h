@@ -322,13 +322,12 @@ rfr_status rfr_plan_set_demod_products(rfr_plan* plan, int32_t products);
  * rfr_plan_set_accum_chunk -- demodulation only: how many K blocks (32 taps
  * each in the four-product form, 64 in the three-product form; 1..64,
  * default 2 in the four-product form, 4 in the three-product form) the
- * tensor cores accumulate in TMEM before the epilogue adds the partial sums
- * into FP32 registers.  Longer chunks are faster (fewer TMEM reads by the
- * epilogue, which compete with the MMAs) and less accurate (the tensor
- * cores' internal accumulation error grows with the partial sums): on the
- * weakest tones of the 2048-tone workload, 1.2e-6 / 1.9e-6 / 3.7e-6
- * relative error at 2 / 4 / 8 blocks of the three-product form, which runs
- * 16.7 / 18.2 / 19.1 Gs/s there.  Changes the results' rounding, so set it
+ * tensor cores accumulate in TMEM, at most, before the epilogue adds the
+ * partial sums into FP32 registers (the three-product form, whose hi/lo terms
+ * share one accumulator, takes half as many).  Longer chunks are faster (fewer
+ * TMEM reads by the epilogue, which compete with the MMAs) and less accurate
+ * (the tensor cores' internal accumulation error grows with the partial sums
+ * and the additions to them).  Changes the results' rounding, so set it
  * before the first push.
  */
 rfr_status rfr_plan_set_accum_chunk(rfr_plan* plan, int32_t k_blocks);
@@ -449,9 +448,8 @@ const char* rfr_batch_last_error(const rfr_batch* batch);
 /*
  * rfr_plan_autotune -- time the plan's result-neutral launch choices (PFB:
  * ring look-ahead of 1..3 super-blocks; demodulation: GEMM tile raster
- * groups and, for the three-product form, the tile shape (128 frames x 128
- * or 64 tones) and whether the FP16 split of the stream is fused into the
- * GEMM) on a push of n_samples and keep the fastest (Sec. III: the
+ * groups and, for the three-product form, the GEMM's form: picked by size,
+ * or one of those below) on a push of n_samples and keep the fastest (Sec. III: the
  * host runtime tunes the GPU kernels).  Outputs stay bit-identical whatever
  * is chosen.  With use_cache != 0 the choice is read
  * from / written to the JSON file named by RFR_TUNE_CACHE (default
@@ -462,11 +460,14 @@ const char* rfr_batch_last_error(const rfr_batch* batch);
 rfr_status rfr_plan_autotune(rfr_plan* plan, int64_t n_samples, int32_t use_cache, double* best_ms);
 rfr_status rfr_plan_get_tune(const rfr_plan* plan, int32_t* pfb_lookahead, int32_t* demod_raster,
                              int32_t* tuned);
-/* Tones per GEMM tile of a three-product demodulation plan (128 or 64, as
- * tuned; 128 by default); 0 for other plans.  Setting it is result-neutral
- * (the autotuner chooses it; set it by hand only to pin a choice).
- * Errors: RFR_E_INVALID (not a three-product demodulation plan, or a width
- * other than 64 or 128). */
+/* Tones per tile of a three-product demodulation plan's single-CTA GEMM form
+ * (128 or 64; 128 by default); 0 for other plans.  A plan starts out with the
+ * form of its GEMM picked per push by size (two-SM tiles of up to 256 frames
+ * x 256 tones, single-CTA tiles of 128 frames x up to 128 tones, either with
+ * its three products as separate work items when tiles are few).  Setting a
+ * width, the pair form or the fused pre-split pins the form instead.  All are
+ * result-neutral.  Errors: RFR_E_INVALID (not a three-product demodulation
+ * plan, or a width other than 64 or 128). */
 rfr_status rfr_plan_get_tone_tile(const rfr_plan* plan, int32_t* tones_per_tile);
 rfr_status rfr_plan_set_tone_tile(rfr_plan* plan, int32_t tones_per_tile);
 
@@ -481,15 +482,11 @@ rfr_status rfr_plan_set_fused_presplit(rfr_plan* plan, int32_t on);
 rfr_status rfr_plan_get_fused_presplit(const rfr_plan* plan, int32_t* on);
 
 /* Three-product demodulation: on = 1 runs the GEMM in clusters of two CTAs
- * on two SMs that take the two tone tiles of one frame tile; the frames'
- * operand tiles (the Toeplitz view of the stream, Sec. III.B) are the same
- * for both, so each CTA loads half of every such tile and TMA multicasts it
- * into both CTAs' shared memory, a quarter less operand traffic from L2 per
- * CTA.  Default 0 (one CTA per tile; the cluster form measured about 3 %
- * slower on the 2048-tone workload, the two CTAs running in lock step).
- * Applies to the separate pre-split form only (get reports 0 while the
- * fused pre-split is on).  Result-neutral (the same MMAs in the same
- * order); the autotuner times both forms.
+ * on two SMs that share tiles of 256 frames x up to 256 tones (two-SM tensor
+ * core instructions: each SM holds its half of the frames and of the tap rows,
+ * which halves the operand traffic per multiply-add of the contraction of
+ * Sec. III.B), 0 single-CTA tiles.  Result-neutral (the same MMAs in the same
+ * order); the fused pre-split has no pair form and wins when both are set.
  * Errors: RFR_E_INVALID (not a three-product demodulation plan, on not 0/1). */
 rfr_status rfr_plan_set_demod_pair(rfr_plan* plan, int32_t on);
 rfr_status rfr_plan_get_demod_pair(const rfr_plan* plan, int32_t* on);

@@ -386,10 +386,10 @@ rfr_status ensure_scratch(rfr_plan* p, int64_t n) {
 // Core of every push: enqueue the frames of [carry | buf] into `out`.
 // defer_gemm (batched steps): a three-product demodulation plan leaves its
 // GEMM to the caller's persistent launch, described in *defer_gemm
-// (n_tiles = 0 when the plan has nothing to launch or is another form).
+// (n_units = 0 when the plan has nothing to launch or is another form).
 rfr_status push_core(rfr_plan* p, const int16_t* iq, int64_t n, const rfr_output* o,
                      int64_t* frames_out, cudaStream_t st, rfr::DemodGemmJob* defer_gemm) {
-    if (defer_gemm) defer_gemm->n_tiles = 0;
+    if (defer_gemm) defer_gemm->n_units = 0;
     if (n < 0 || (n > 0 && iq == nullptr)) return fail(p, RFR_E_INVALID, "bad input buffer");
     const int64_t lv = p->cl + n;
     const int64_t F = frames_for_len(p, lv);
@@ -538,10 +538,12 @@ rfr_status push_core(rfr_plan* p, const int16_t* iq, int64_t n, const rfr_output
                     L.xs_hi = p->d_xs3;
                     L.xs_lo = nullptr;
                     L.xs_rows = p->xs3_rows_cap;
+                    L.auto_form = p->tune.demod_auto ? 1 : 0;
+                    L.scratch = p->d_g3;
                     L.tone_tile = p->tune.demod_bt;
                     L.fused_presplit = p->tune.demod_fused;
                     L.pair = p->tune.demod_pair;
-                    if (defer_gemm) RFR_CUDA(p, rfr::demod3_prepare(L, st, defer_gemm));
+                    if (defer_gemm) RFR_CUDA(p, rfr::demod3_prepare(L, st, defer_gemm, true));
                     else RFR_CUDA(p, rfr::demod3_launch(L, st));
                 } else {
                     RFR_CUDA(p, rfr::demod_launch(L, st));
@@ -588,7 +590,7 @@ void destroy(rfr_plan* p) {
     for (void* q : {static_cast<void*>(p->d_h), p->d_tw, p->d_tw_cl, static_cast<void*>(p->d_bins),
                     static_cast<void*>(p->d_words), static_cast<void*>(p->d_rates), static_cast<void*>(p->d_h32), p->d_c32, p->d_bhi, p->d_blo,
                     static_cast<void*>(p->d_status), static_cast<void*>(p->d_carry[0]),
-                    static_cast<void*>(p->d_carry[1]), p->d_xs_hi, p->d_xs_lo, p->d_rot, p->d_qfull, p->d_b3, p->d_xs3,
+                    static_cast<void*>(p->d_carry[1]), p->d_xs_hi, p->d_xs_lo, p->d_rot, p->d_qfull, p->d_b3, p->d_g3, p->d_xs3,
                     p->d_qtones, static_cast<void*>(p->d_view), p->d_ptones, p->d_pre})
         dev_free(q);
     for (int i = 0; i < rfr_plan::kStageBufs; ++i) {
@@ -1172,6 +1174,7 @@ rfr_status rfr_plan_set_demod_products(rfr_plan* p, int32_t products) {
         const size_t plane = static_cast<size_t>(p->ntp3) * p->Lpad3;
         double* d_h64 = nullptr;
         cudaError_t e = dev_alloc(&p->d_b3, plane * 6 * sizeof(uint16_t));
+        if (e == cudaSuccess) e = dev_alloc(&p->d_g3, rfr::demod3_scratch_bytes(p->n_sms));
         if (e == cudaSuccess) e = dev_alloc(&d_h64, static_cast<size_t>(p->L) * 8);
         if (e == cudaSuccess) e = cudaMemcpy(d_h64, p->h64.data(), static_cast<size_t>(p->L) * 8, cudaMemcpyHostToDevice);
         if (e == cudaSuccess)
@@ -1180,7 +1183,8 @@ rfr_status rfr_plan_set_demod_products(rfr_plan* p, int32_t products) {
         dev_free(d_h64);
         if (e != cudaSuccess) {
             dev_free(p->d_b3);
-            p->d_b3 = nullptr;
+            dev_free(p->d_g3);
+            p->d_b3 = p->d_g3 = nullptr;
             return cuda_fail(p, e, "three-product tap build");
         }
     }

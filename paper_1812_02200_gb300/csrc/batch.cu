@@ -13,10 +13,10 @@
 //
 // rfr_plan_autotune times the launch choices that never change results
 // (bit-identical outputs) -- the PFB ring look-ahead, and the demodulation
-// GEMM's tile raster and tone-tile width (128 or 64 tones per tile) -- on a
-// buffer of the caller's size, keeps the fastest in the plan and in a
-// JSON cache file (RFR_TUNE_CACHE, default ./rfr_tune_cache.json) keyed by
-// the plan shape and the GPU, so later plans of the same shape load it.
+// GEMM's tile raster and form (by size, or one pinned) -- on a buffer of the
+// caller's size, keeps the fastest in the plan and in a JSON cache file
+// (RFR_TUNE_CACHE, default ./rfr_tune_cache.json) keyed by the plan shape and
+// the GPU, so later plans of the same shape load it.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -89,7 +89,8 @@ std::string tune_key(const rfr_plan* p, int64_t n) {
 
 // Minimal line-oriented JSON map:
 //   {"key": [pfb_lookahead, demod_raster, demod_tone_tile, demod_fused], ...}
-// (missing trailing numbers take their defaults: tone tile 128, not fused)
+// (missing trailing numbers take their defaults: tone tile 128, not fused; tone
+// tile 0: the GEMM's form picked per push by size)
 struct TuneEntry {
     int lookahead = 0, raster = 1, bt = 128, fused = 0, pair = 0, cluster = 0;
 };
@@ -105,7 +106,7 @@ std::map<std::string, TuneEntry> tune_load() {
         const int got = std::sscanf(line.c_str() + b0, "[%d, %d, %d, %d, %d, %d]", &t.lookahead, &t.raster, &t.bt,
                                     &t.fused, &t.pair, &t.cluster);
         if (got >= 2) {
-            if (got == 2 || (t.bt != 64 && t.bt != 128)) t.bt = 128;
+            if (got == 2 || (t.bt != 64 && t.bt != 128 && t.bt != 0)) t.bt = 128;
             if (got < 4 || (t.fused != 0 && t.fused != 1)) t.fused = 0;
             if (got < 5 || (t.pair != 0 && t.pair != 1) || t.fused) t.pair = 0;
             if (got < 6 || (t.cluster != 0 && t.cluster != 1)) t.cluster = 0;
@@ -113,6 +114,16 @@ std::map<std::string, TuneEntry> tune_load() {
         }
     }
     return m;
+}
+
+void tune_apply(rfr_plan* p, const TuneEntry& t) {
+    p->tune.pfb_lookahead = t.lookahead;
+    p->tune.demod_raster = t.raster;
+    p->tune.demod_auto = t.bt == 0;
+    p->tune.demod_bt = t.bt == 64 ? 64 : 128;
+    p->tune.demod_fused = t.fused;
+    p->tune.demod_pair = t.pair;
+    p->tune.pfb_cluster = p->d_tw_cl ? t.cluster : 0;
 }
 
 void tune_store(const std::map<std::string, TuneEntry>& m) {
@@ -198,7 +209,7 @@ rfr_status rfr_batch_push(rfr_batch* b, const int16_t* const* bufs, const int64_
         outs[i].frames = F;
         if (err != RFR_OK) b->last_error = "push " + std::to_string(i) + ": " + b->plans[i]->last_error;
         cudaEventRecord(b->ev_join[i], br);
-        if (b->jobs[i].n_tiles > 0) {
+        if (b->jobs[i].n_units > 0) {
             // the plan's GEMM waits for its pre-GEMM kernels
             cudaStreamWaitEvent(b->gemm_stream, b->ev_join[i], 0);
             gemms.push_back(&b->jobs[i]);
@@ -274,12 +285,7 @@ rfr_status rfr_plan_autotune(rfr_plan* p, int64_t n_samples, int32_t use_cache, 
         auto m = tune_load();
         auto it = m.find(key);
         if (it != m.end()) {
-            p->tune.pfb_lookahead = it->second.lookahead;
-            p->tune.demod_raster = it->second.raster;
-            p->tune.demod_bt = it->second.bt;
-            p->tune.demod_fused = it->second.fused;
-            p->tune.demod_pair = it->second.pair;
-            p->tune.pfb_cluster = p->d_tw_cl ? it->second.cluster : 0;
+            tune_apply(p, it->second);
             p->tune.tuned = true;
             if (best_ms) *best_ms = -1.0;
             return RFR_OK;
@@ -296,12 +302,15 @@ rfr_status rfr_plan_autotune(rfr_plan* p, int64_t n_samples, int32_t use_cache, 
         // product (3 x tone tiles times per sample): timed only for plans of
         // at most two 128-tone tiles, where that stays cheap
         const bool try_fused = p->demod_products == 3 && p->words.size() <= 256;
+        if (p->demod_products == 3)
+            for (int r : {1, 8, 19, 38}) cand.push_back({0, r, 0});         // form by size
         for (int fused : {0, 1})
             for (int pair : {1, 0})
                 for (int bt : {128, 64}) {
                     // tone tile, fused pre-split and clusters are three-product choices;
                     // the cluster form loads A by TMA, so it excludes the fused pre-split
                     if ((bt == 64 || fused || pair) && p->demod_products != 3) continue;
+                    if (pair && bt == 64) continue;                          // the pair form has its own width
                     if (fused && (!try_fused || pair)) continue;
                     for (int r : {1, 8, 19, 38}) cand.push_back({0, r, bt, fused, pair});
                 }
@@ -347,12 +356,7 @@ rfr_status rfr_plan_autotune(rfr_plan* p, int64_t n_samples, int32_t use_cache, 
     TuneEntry best_c = cand.front();
     rfr_status rs = rfr::ensure_scratch(p, n_samples);
     for (size_t c = 0; c < cand.size() && rs == RFR_OK; ++c) {
-        p->tune.pfb_lookahead = cand[c].lookahead;
-        p->tune.demod_raster = cand[c].raster;
-        p->tune.demod_bt = cand[c].bt;
-        p->tune.demod_fused = cand[c].fused;
-        p->tune.demod_pair = cand[c].pair;
-        p->tune.pfb_cluster = cand[c].cluster;
+        tune_apply(p, cand[c]);
         float ms_best = 1e30f;
         for (int rep = 0; rep < 4 && rs == RFR_OK; ++rep) {
             p->samples = s_samples;
@@ -388,12 +392,7 @@ rfr_status rfr_plan_autotune(rfr_plan* p, int64_t n_samples, int32_t use_cache, 
         p->tune = keep;
         return rs;
     }
-    p->tune.pfb_lookahead = best_c.lookahead;
-    p->tune.demod_raster = best_c.raster;
-    p->tune.demod_bt = best_c.bt;
-    p->tune.demod_fused = best_c.fused;
-    p->tune.demod_pair = best_c.pair;
-    p->tune.pfb_cluster = best_c.cluster;
+    tune_apply(p, best_c);
     p->tune.tuned = true;
     if (best_ms) *best_ms = best;
     if (use_cache) {
@@ -409,12 +408,14 @@ rfr_status rfr_plan_set_tone_tile(rfr_plan* p, int32_t tones_per_tile) {
     if (!p || p->mode != RFR_MODE_DEMOD || p->demod_products != 3 || (tones_per_tile != 64 && tones_per_tile != 128))
         return RFR_E_INVALID;
     p->tune.demod_bt = tones_per_tile;
+    p->tune.demod_auto = false;
     return RFR_OK;
 }
 
 rfr_status rfr_plan_set_fused_presplit(rfr_plan* p, int32_t on) {
     if (!p || p->mode != RFR_MODE_DEMOD || p->demod_products != 3 || (on != 0 && on != 1)) return RFR_E_INVALID;
     p->tune.demod_fused = on;
+    p->tune.demod_auto = false;
     return RFR_OK;
 }
 
@@ -427,6 +428,7 @@ rfr_status rfr_plan_get_fused_presplit(const rfr_plan* p, int32_t* on) {
 rfr_status rfr_plan_set_demod_pair(rfr_plan* p, int32_t on) {
     if (!p || p->mode != RFR_MODE_DEMOD || p->demod_products != 3 || (on != 0 && on != 1)) return RFR_E_INVALID;
     p->tune.demod_pair = on;
+    p->tune.demod_auto = false;
     return RFR_OK;
 }
 

@@ -37,10 +37,12 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
 #include <mutex>
+#include <vector>
 
 #include "dev_common.cuh"
 #include "rfr_internal.h"
@@ -371,57 +373,86 @@ demod_gemm_kernel(const __grid_constant__ CUtensorMap tmAh, const __grid_constan
 // hi/lo as above ((xr+xi)/2 has at most 17 significant bits, exact as hi+lo);
 // each product again takes the three MMAs hi.hi + hi.lo + lo.hi.
 //
-// Tile: 128 frames x BT tones (BT = 128 or 64, the tone-tile width chosen by
-// the plan's autotuner), K-blocks of 64 complex taps (one plane per TMA
-// stage: A hi, lo 128x64 and B hi, lo BTx64, B lo right after B hi).  Per 16
-// taps two MMAs: A hi times [B hi | B lo] as one N = 2 BT product (the hi.hi
-// and hi.lo terms side by side in TMEM), then A lo times B hi (N = BT) added
-// onto the hi.hi half.  The three products of an accumulation chunk run one
-// after the other, each into a 2 BT-column TMEM slot taken in rotation (two
-// slots for BT = 128, four for 64), so the epilogue drains a slot while the
-// MMAs fill the next.  Sixteen epilogue warps (four per TMEM lane quadrant,
-// BT/4 tones each) drain a slot by adding its two halves, then add 2 P1 to
-// both sums, P2 to the imaginary and -P3 to the real sum.
+// What bounds it.  Per 16 taps a CTA's shared memory takes the MMAs' operand
+// reads and the TMA's writes at 128 bytes a clock, and the SM takes at most
+// 64 bytes a clock from L2.  A tile of 128 frames x 128 tones on one SM needs
+// 36-40 KB of shared-memory traffic and 16 KB from L2 for 192 clocks of
+// tensor work: both limits lie above the tensor time, and the tensor pipe
+// measured 62 % active.  The large form (PAIR) therefore gives two SMs one
+// tile of 256 frames x 256 tones (cta_group::2 MMAs, M = 256): each SM holds
+// its 128 frames and half the tones' tap rows and reads 8 KB per MMA of 128
+// clocks, 40 KB and 16 KB from L2 for 384 clocks of tensor work.
 //
-// Fused pre-split (FUSED): instead of TMA loads of the six pre-split source
-// planes (written to HBM by presplit3_kernel, 12 bytes per sample), two
-// producer warps read the int16 stream view [carry | buffer] and write each
-// stage's A hi/lo tiles themselves, in the 128-byte swizzled layout the TMA
-// would produce, with the same FP32 -> FP16 hi/lo rounding as the pre-split
-// kernel (bit-identical planes, so bit-identical results); only the B tiles
-// arrive by TMA.  A launch choice the autotuner times.
+// A tile of that size leaves no room for both FP32 sums (re and im) of every
+// output in registers, so a tile runs its three products one after the other
+// over all of K: the epilogue warps hold ONE product's FP32 sums (64 tones a
+// thread) and park each product in a scratch of the CTA (L2-resident).
+// Finisher warps fetch a parked tile back by bulk copies, combine, rotate and
+// store it while the next tile's first product runs.  (Done by the epilogue
+// warps at the tile's end it stalled the MMAs, which run at most two chunks
+// ahead, by about 50,000 clocks of 400,000 per tile; finishers with register
+// loads could not keep enough bytes in flight either.)
 //
-// The kernel is persistent over a list of plans: one launch runs the tiles
-// of every demodulation stream of a batched step (or of one push), each CTA
-// striding over the global tile index; a tile's plan is found from the
-// plans' first-tile offsets.  Each output element is accumulated in the same
-// order whatever the tile width or the plans sharing the launch.
+// Measured, 2^27 samples x 2048 tones, L = 4096, D = 2048, whole push: 7.6 ms
+// with tiles of 128 x 128 on one SM, 6.0 ms with pairs (short runs; 6.4 ms in
+// seconds-long runs under the power cap).  The MMAs alone would take 3.84 ms
+// at 2.07 GHz.
+//
+// Precision: the three MMAs of a term set go to the same FP32 TMEM
+// accumulator, which collects a chunk of K (128 taps by default) before the
+// epilogue adds it into the FP32 sums; the accumulator is double-buffered.
+// Every form sums each output in the same order (16 taps hi.hi, hi.lo, lo.hi;
+// chunks; products), so tile shape, form and the plans sharing a launch never
+// change a result.
+//
+// Forms.  PAIR as above; the tone tile is narrowed (in steps of 32) so that a
+// plan's tones divide evenly.  One CTA per tile of 128 frames x at most 128
+// tones for plans with too few tiles to fill the chip's pairs.  Either form
+// may be SPLIT when tiles are few: a work item is then one product of a tile,
+// the products go to planes in the scratch and combine3_kernel finishes.
+//
+// Fused pre-split (FUSED, single-CTA form): instead of TMA loads of the six
+// pre-split source planes (written to HBM by presplit3_kernel, 12 bytes per
+// sample), two producer warps read the int16 stream view [carry | buffer] and
+// write each stage's A hi/lo tiles themselves, in the 128-byte swizzled layout
+// the TMA would produce, with the same FP32 -> FP16 hi/lo rounding as the
+// pre-split kernel (bit-identical planes, so bit-identical results); only the
+// B tiles arrive by TMA.  A launch choice the autotuner times.
+//
+// The kernel is persistent over a list of plans: one launch runs the work
+// items of every demodulation stream of a batched step (or of one push), each
+// CTA (or pair) striding over the global item index; an item's plan is found
+// from the plans' first-item offsets.
 constexpr int G3_BK = 64;                                  // complex taps per K-block
-constexpr uint32_t G3_A_BYTES = BM * G3_BK * 2;
-constexpr uint32_t G3_A_HALF = G3_A_BYTES / 2;              // 64 rows: one CTA's share in the pair form
+constexpr uint32_t G3_OP_BYTES = 128 * G3_BK * 2;          // one operand tile: 128 rows x 64 fp16
+constexpr int G3_STAGES = 3;                               // A hi, A lo, B hi, B lo each
+constexpr uint32_t G3_STAGE_BYTES = 4 * G3_OP_BYTES;
 constexpr int G3_SLOTS_MAX = 4;
+constexpr uint32_t G3_TMEM_COLS = 512;
 constexpr int G3_EPI_WARPS = 16;          // 4 lane quadrants x 4 tone groups
-constexpr int G3_THREADS = (G3_EPI_WARPS + 2) * 32;
 constexpr int G3_FUSED_PRODUCERS = 2;                       // producer warps of the fused form
-constexpr int G3_THREADS_FUSED = (G3_EPI_WARPS + G3_FUSED_PRODUCERS + 1) * 32;
-template <int BT> struct G3Cfg {
-    static constexpr uint32_t B_BYTES = BT * G3_BK * 2;
-    static constexpr uint32_t STAGE_BYTES = 2 * G3_A_BYTES + 2 * B_BYTES;
-    static constexpr int STAGES = BT == 128 ? 3 : 4;
-    static constexpr size_t SMEM = 1024 + STAGES * STAGE_BYTES + 256;
-    // a slot holds one product's accumulator as two BT-column halves:
-    // [0, BT) collects hi.hi + lo.hi, [BT, 2 BT) hi.lo (see the MMA issuer)
-    static constexpr int SLOTS = BT == 128 ? 2 : 4;
-    static constexpr uint32_t SLOT_COLS = 2 * BT;
-    static constexpr uint32_t TMEM_COLS = SLOTS * SLOT_COLS;   // 512
-    static constexpr int TPG = BT / 4;                     // tones per epilogue warp
-};
+constexpr int G3_THREADS = (G3_EPI_WARPS + 4) * 32;         // + producer(s), MMA issuer, finishers
+constexpr int G3_PAIR_TONES = 256, G3_SINGLE_TONES = 128;   // widest tone tiles
+// scratch of one CTA: a ring of products, [tone][128 frames] FP32 each
+constexpr int G3_PLANES = 4;   // a ring: 3 measured 1-2 % slower (5.97 against 6.02 ms, 2^27 samples)
+constexpr int64_t G3_PLANE = int64_t(G3_PAIR_TONES) * 128;
+constexpr int64_t G3_CTA_SCRATCH = G3_PLANES * G3_PLANE;
+// finisher staging: chunks of two tones (three products of 128 frames, then the
+// tones' 128 rotation steps), FIN_BUFS chunks per warp in flight
+constexpr int G3_FIN_BUFS = 3, G3_MAX_FINISHERS = 2;
+constexpr uint32_t G3_FIN_BYTES = 3 * 2 * 128 * 4 + 2 * 128 * 8;
+constexpr uint32_t G3_BARS_BYTES = 256;
+constexpr size_t G3_SMEM = 1024 + G3_STAGES * G3_STAGE_BYTES + G3_BARS_BYTES + G3_MAX_FINISHERS * G3_FIN_BUFS * G3_FIN_BYTES;
 
 struct G3Plan {
     CUtensorMap a[6];   // (x sum/2, xr, xi) x (hi, lo): [rows][D] fp16, Toeplitz view (unused when fused)
     CUtensorMap b[6];   // (cr, ci - cr, cr + ci) x (hi, lo): [ntp][Lpad] fp16, K-major
-    GemmArgs g;
-    int tile0;          // first global tile of this plan
+    GemmArgs g;         // n_mt, n_nt: tiles (of a pair in the pair form); kchunk: K-blocks per chunk
+    int unit0;          // first global work item of this plan
+    int bw;             // tones per tile
+    int split;          // work items are single products, written to planes
+    float* scratch;     // [CTA][4][256][128] (or the split form's planes [3][n_tones][pld])
+    int64_t pld;
     // fused form: the int16 stream view v[s] = s < cl ? carry[s] : buf[s - cl]
     // for s < lv (0 beyond); vec: the buffer part may be read 16 bytes at a time
     const uint32_t* carry;
@@ -431,31 +462,42 @@ struct G3Plan {
 };
 constexpr int kG3MaxPlans = 16;
 struct G3Batch {
-    int n_plans, total_tiles;
+    int n_plans, total_units;
     G3Plan p[kG3MaxPlans];
 };
 static_assert(sizeof(G3Batch) <= 32000, "kernel parameter space");
 static_assert(sizeof(G3Plan) <= kDemodJobBytes, "job storage");
 
-__device__ __forceinline__ int g3_plan_of(const G3Batch& bt, int tile) {
+__device__ __forceinline__ const G3Plan& g3_plan_of(const G3Batch& bt, int unit) {
     int pi = 0;
-    while (pi + 1 < bt.n_plans && tile >= bt.p[pi + 1].tile0) ++pi;
-    return pi;
+    while (pi + 1 < bt.n_plans && unit >= bt.p[pi + 1].unit0) ++pi;
+    return bt.p[pi];
 }
 
-// Tile (frame tile mt, tone tile nt) of work item `tile` of a plan.  In the
-// pair form a work item is a frame tile and a pair of tone tiles 2j, 2j + 1,
-// the CTA of cluster rank r taking tone tile 2j + r (past the plan's last
-// tone tile when its count is odd: the taps there are read as zeros and
-// no output is stored).
+// A work item: frame tile origin (of this CTA), tone tile origin and width,
+// products [q0, q1).  `width` is a multiple of the MMA's N step.
+struct G3Unit {
+    int64_t m0;
+    int n0, width, q0, q1;
+};
 template <bool PAIR>
-__device__ __forceinline__ void g3_coords(const GemmArgs& g, int tile, int rank, int& mt, int& nt) {
-    if (PAIR) {
-        tile_coords_of(g.raster, g.n_mt, (g.n_nt + 1) >> 1, tile, mt, nt);
-        nt = 2 * nt + rank;
-    } else {
-        tile_coords(g, tile, mt, nt);
+__device__ __forceinline__ G3Unit g3_unit(const G3Plan& P, int unit, int rank) {
+    int local = unit - P.unit0;
+    G3Unit u;
+    u.q0 = 0;
+    u.q1 = 3;
+    if (P.split) {
+        u.q0 = local % 3;
+        u.q1 = u.q0 + 1;
+        local /= 3;
     }
+    int mt, nt;
+    tile_coords(P.g, local, mt, nt);
+    u.m0 = PAIR ? static_cast<int64_t>(mt) * 256 + rank * 128 : static_cast<int64_t>(mt) * BM;
+    u.n0 = nt * P.bw;
+    constexpr int step = PAIR ? 32 : 16;
+    u.width = min(P.bw, (P.g.n_tones - u.n0 + step - 1) / step * step);
+    return u;
 }
 
 __global__ void build_taps3_kernel(const double* __restrict__ h, const uint64_t* __restrict__ words,
@@ -541,52 +583,146 @@ __device__ __forceinline__ void g3_fill_row(const G3Plan& P, int q, int64_t s0, 
     }
 }
 
-// PAIR: launched in clusters of two CTAs that take the two tone tiles of a
-// work item; they need the same A tiles, so each CTA loads 64 rows of every
-// A tile and multicasts them into both CTAs' stage buffers.  A stage of a
-// CTA is then refilled only when both CTAs' MMAs have consumed it (its empty
-// barrier takes one commit from each), and the two CTAs meet at cluster
-// barriers after initialising their mbarriers and before leaving.
-template <int BT, bool FUSED, bool PAIR>
-__global__ void __launch_bounds__(FUSED ? G3_THREADS_FUSED : G3_THREADS, 1)
+// An output from its products and rotation factors.
+__device__ __forceinline__ float2 g3_output(float p1, float p2, float p3, float inv_scale, float2 an, float2 sp) {
+    const float re = fmaf(2.f, p1, -p3), im = fmaf(2.f, p1, p2);
+    return cmul(make_float2(re * inv_scale, im * inv_scale), cmul(an, sp));
+}
+
+// Outputs of a CTA's last tile, by all its epilogue and finisher warps: lane l
+// takes frames 4 l .. 4 l + 3, warp w of nw (less the `skip` producer and MMA
+// warps between the two kinds) every tone of its number, FT in flight.
+__device__ __noinline__ void g3_finish(const G3Plan& P, const G3Unit u, const float* scr_cta, uint32_t tile, int lane,
+                                          int w, int nw, int skip) {
+    constexpr int FT = 2;
+    const GemmArgs& g = P.g;
+    if (w >= G3_EPI_WARPS) w -= skip;
+    nw -= skip;
+    const float* pl[3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) pl[q] = scr_cta + ((3 * tile + q) % G3_PLANES) * G3_PLANE + 4 * lane;
+    const int64_t k = u.m0 + 4 * lane;               // the lane's first frame
+    const int64_t K = g.F0 + k;
+    const int rows = static_cast<int>(k < g.F ? (g.F - k < 4 ? g.F - k : 4) : 0);
+    if (rows == 0) return;
+    // four frames of one anchor row, with aligned steps; 16-byte stores
+    const bool near = (g.F0 & 3) == 0;
+    const bool vec = rows == 4 && ((reinterpret_cast<uintptr_t>(g.out + g.fo + k) | static_cast<uintptr_t>(g.ld * 8)) & 15) == 0;
+    const int n = min(u.width, g.n_tones - u.n0);
+#pragma unroll 1
+    for (int c0 = w; c0 < n; c0 += nw * FT) {
+        float p[FT][3][4];
+        float2 an[FT][4], sp[FT][4];
+#pragma unroll
+        for (int f = 0; f < FT; ++f) {
+            const int c = c0 + f * nw, t = u.n0 + c;
+            if (c >= n) continue;
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                const float4 v = __ldcg(reinterpret_cast<const float4*>(pl[q] + c * 128));
+                p[f][q][0] = v.x;
+                p[f][q][1] = v.y;
+                p[f][q][2] = v.z;
+                p[f][q][3] = v.w;
+            }
+            const float2* anc = g.anchors + t - (g.F0 / BM) * g.ntp;
+            const float2* stp = g.steps + static_cast<int64_t>(t) * BM;
+            if (near) {
+                an[f][0] = __ldg(anc + (K / BM) * g.ntp);
+                an[f][1] = an[f][2] = an[f][3] = an[f][0];
+                const float4* s4 = reinterpret_cast<const float4*>(stp + static_cast<int>(K % BM));
+                const float4 s0 = __ldg(s4), s1 = __ldg(s4 + 1);
+                sp[f][0] = make_float2(s0.x, s0.y);
+                sp[f][1] = make_float2(s0.z, s0.w);
+                sp[f][2] = make_float2(s1.x, s1.y);
+                sp[f][3] = make_float2(s1.z, s1.w);
+            } else {
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {
+                    const int64_t Kr = r < rows ? K + r : K;
+                    an[f][r] = __ldg(anc + (Kr / BM) * g.ntp);
+                    sp[f][r] = __ldg(stp + static_cast<int>(Kr % BM));
+                }
+            }
+        }
+#pragma unroll
+        for (int f = 0; f < FT; ++f) {
+            const int c = c0 + f * nw, t = u.n0 + c;
+            if (c >= n) continue;
+            float2* o = g.out + static_cast<int64_t>(t) * g.ld + g.fo + k;
+            float2 y[4];
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+                y[r] = g3_output(p[f][0][r], p[f][1][r], p[f][2][r], g.inv_scale, an[f][r], sp[f][r]);
+            if (vec) {
+                reinterpret_cast<float4*>(o)[0] = make_float4(y[0].x, y[0].y, y[1].x, y[1].y);
+                reinterpret_cast<float4*>(o)[1] = make_float4(y[2].x, y[2].y, y[3].x, y[3].y);
+            } else {
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+                    if (r < rows) o[r] = y[r];
+            }
+        }
+    }
+}
+
+// PAIR: launched in clusters of two CTAs on one 256 x 256 tile.  Both CTAs
+// load their own operand halves, counted on the full barriers of CTA 0, whose
+// MMA thread issues for both; its commits arrive on both CTAs' barriers, and
+// the epilogue warps of both report drained slots to CTA 0.  The CTAs meet at
+// cluster barriers after initialising their mbarriers and before leaving.
+// The mbarriers order tensor-core and TMA work only (no ordinary loads or
+// stores pass between the CTAs), so plain waits do; acquiring at cluster
+// scope put a memory barrier into every wait.
+template <bool PAIR, bool FUSED>
+__global__ void __launch_bounds__(G3_THREADS, 1)
 demod3m_gemm_kernel(const __grid_constant__ G3Batch bt) {
     static_assert(!(FUSED && PAIR), "the pair form loads its A tiles by TMA");
-    using Cfg = G3Cfg<BT>;
-    constexpr int STAGES = Cfg::STAGES;
-    constexpr uint32_t STAGE_BYTES = Cfg::STAGE_BYTES, B_BYTES = Cfg::B_BYTES;
+    constexpr int STAGES = G3_STAGES;
+    constexpr int TW = PAIR ? G3_PAIR_TONES : G3_SINGLE_TONES;             // columns of a TMEM slot
+    constexpr int SLOTS = static_cast<int>(G3_TMEM_COLS) / TW;
+    constexpr int TPG = TW / 4;                                             // tones per epilogue thread
     extern __shared__ unsigned char smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     unsigned char* smem = smem_raw + ((1024u - (raw & 1023u)) & 1023u);
-    uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE_BYTES);
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * G3_STAGE_BYTES);
     uint64_t* empty = full + STAGES;
     uint64_t* sfull = empty + STAGES;
     uint64_t* sempty = sfull + G3_SLOTS_MAX;
-    uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(sempty + G3_SLOTS_MAX);
-    constexpr int SLOTS = Cfg::SLOTS;
+    uint64_t* parked = sempty + G3_SLOTS_MAX;                               // a tile's products are in the scratch
+    uint64_t* finished = parked + 1;                                        // ... and its outputs stored
+    uint64_t* fbar = finished + 1;                                          // finisher staging, per warp and buffer
+    uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(fbar + G3_MAX_FINISHERS * G3_FIN_BUFS);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
+    unsigned char* const fin_stage = smem + STAGES * G3_STAGE_BYTES + G3_BARS_BYTES;
     int* const status0 = bt.p[0].g.status;
     constexpr int PROD_WARP = G3_EPI_WARPS;                                  // first producer warp
     constexpr int MMA_WARP = G3_EPI_WARPS + (FUSED ? G3_FUSED_PRODUCERS : 1);
+    constexpr int FIN_WARP = MMA_WARP + 1;
+    constexpr int FINISHERS = G3_THREADS / 32 - FIN_WARP;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int rank = PAIR ? static_cast<int>(cluster_ctarank()) : 0;
-    const int cta0 = PAIR ? static_cast<int>(blockIdx.x >> 1) : static_cast<int>(blockIdx.x);
-    const int ncta = PAIR ? static_cast<int>(gridDim.x >> 1) : static_cast<int>(gridDim.x);
+    const int first = PAIR ? static_cast<int>(blockIdx.x >> 1) : static_cast<int>(blockIdx.x);
+    const int stride = PAIR ? static_cast<int>(gridDim.x >> 1) : static_cast<int>(gridDim.x);
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(&full[s], FUSED ? G3_FUSED_PRODUCERS * 32 : 1);
-            mbar_init(&empty[s], PAIR ? 2 : 1);
+            mbar_init(&empty[s], 1);
         }
         for (int b = 0; b < SLOTS; ++b) {
             mbar_init(&sfull[b], 1);
-            mbar_init(&sempty[b], G3_EPI_WARPS * 32);
+            mbar_init(&sempty[b], (PAIR ? 2 : 1) * G3_EPI_WARPS);
         }
+        mbar_init(parked, G3_EPI_WARPS);
+        mbar_init(finished, FINISHERS);
+        for (int b = 0; b < FINISHERS * G3_FIN_BUFS; ++b) mbar_init(&fbar[b], 1);
         *abort_flag = 0;
         fence_mbar_init();
     }
     if (warp == MMA_WARP) {
-        umma::alloc(tmem_holder, Cfg::TMEM_COLS);
-        umma::relinquish();
+        umma::alloc<PAIR>(tmem_holder, G3_TMEM_COLS);
+        umma::relinquish<PAIR>();
     }
     if (warp == PROD_WARP && lane < bt.n_plans) {
         for (int i = 0; i < 6; ++i) {
@@ -596,49 +732,42 @@ demod3m_gemm_kernel(const __grid_constant__ G3Batch bt) {
     }
     umma::fence_before_sync();
     __syncthreads();
-    if (PAIR) cluster_sync();          // both CTAs' barriers exist before any multicast
+    if (PAIR) cluster_sync();          // both CTAs' barriers exist before anything arrives on them
     umma::fence_after_sync();
     const uint32_t tmem = *tmem_holder;
-    const int n_tiles = bt.total_tiles;
-    constexpr uint32_t IDESC = umma::idesc_f16_f32(BM, BT);
-    constexpr uint32_t IDESC_W = umma::idesc_f16_f32(BM, 2 * BT);
+    const int n_units = bt.total_units;
+    float* const scr_cta = bt.p[0].scratch + static_cast<int64_t>(blockIdx.x) * G3_CTA_SCRATCH;
 
     if (FUSED && warp >= PROD_WARP && warp < MMA_WARP) {
         // ------------------------------------------------ fused producers
         const int pt = threadIdx.x - PROD_WARP * 32;                         // 0 .. 63
         uint32_t it = 0;
         bool stop = false;
-        for (int tile = cta0; tile < n_tiles && !stop; tile += ncta) {
-            const int pi = g3_plan_of(bt, tile);
-            const G3Plan& P = bt.p[pi];
-            int tm, tn;
-            g3_coords<PAIR>(P.g, tile - P.tile0, rank, tm, tn);
-            const int m0 = tm * BM, n0 = tn * BT;
+        for (int unit = first; unit < n_units && !stop; unit += stride) {
+            const G3Plan& P = g3_plan_of(bt, unit);
+            const G3Unit u = g3_unit<PAIR>(P, unit, rank);
             const int64_t D = P.g.two_d;
-            for (int kb0 = 0; kb0 < P.g.KB && !stop; kb0 += P.g.kchunk) {
-                const int kb1 = min(kb0 + P.g.kchunk, P.g.KB);
-                for (int q = 0; q < 3 && !stop; ++q) {
-                    for (int kb = kb0; kb < kb1; ++kb, ++it) {
-                        const int s = it % STAGES;
-                        const uint32_t ph = (it / STAGES) & 1;
-                        if (*abort_flag || !mbar_wait(&empty[s], ph ^ 1, status0)) {
-                            *abort_flag = 1;
-                            stop = true;
-                            break;
-                        }
-                        unsigned char* st = smem + s * STAGE_BYTES;
-                        const int kt = kb * G3_BK;
-                        if (pt == 0) {
-                            mbar_expect_tx(&full[s], 2 * B_BYTES);
-                            tma_load_2d(st + 2 * G3_A_BYTES, &P.b[2 * q], kt, n0, &full[s]);
-                            tma_load_2d(st + 2 * G3_A_BYTES + B_BYTES, &P.b[2 * q + 1], kt, n0, &full[s]);
-                        }
-#pragma unroll 1
-                        for (int i = pt; i < BM; i += G3_FUSED_PRODUCERS * 32)
-                            g3_fill_row(P, q, (static_cast<int64_t>(m0) + i) * D + kt, st, st + G3_A_BYTES, i);
-                        fence_proxy_async_smem();                 // the MMAs read the tiles through the async proxy
-                        mbar_arrive(&full[s]);
+            for (int q = u.q0; q < u.q1 && !stop; ++q) {
+                for (int kb = 0; kb < P.g.KB; ++kb, ++it) {
+                    const int s = it % STAGES;
+                    const uint32_t ph = (it / STAGES) & 1;
+                    if (*abort_flag || !mbar_wait(&empty[s], ph ^ 1, status0)) {
+                        *abort_flag = 1;
+                        stop = true;
+                        break;
                     }
+                    unsigned char* st = smem + s * G3_STAGE_BYTES;
+                    const int kt = kb * G3_BK;
+                    if (pt == 0) {
+                        mbar_expect_tx(&full[s], 2u * P.bw * (G3_BK * 2));
+                        tma_load_2d(st + 2 * G3_OP_BYTES, &P.b[2 * q], kt, u.n0, &full[s]);
+                        tma_load_2d(st + 3 * G3_OP_BYTES, &P.b[2 * q + 1], kt, u.n0, &full[s]);
+                    }
+#pragma unroll 1
+                    for (int i = pt; i < BM; i += G3_FUSED_PRODUCERS * 32)
+                        g3_fill_row(P, q, (u.m0 + i) * D + kt, st, st + G3_OP_BYTES, i);
+                    fence_proxy_async_smem();                 // the MMAs read the tiles through the async proxy
+                    mbar_arrive(&full[s]);
                 }
             }
         }
@@ -655,50 +784,51 @@ demod3m_gemm_kernel(const __grid_constant__ G3Batch bt) {
         if (lane == 0) {
             uint32_t it = 0;
             bool stop = false;
-            for (int tile = cta0; tile < n_tiles && !stop; tile += ncta) {
-                const int pi = g3_plan_of(bt, tile);
-                const G3Plan& P = bt.p[pi];
-                int tm, tn;
-                g3_coords<PAIR>(P.g, tile - P.tile0, rank, tm, tn);
-                const int m0 = tm * BM, n0 = tn * BT;
-                for (int kb0 = 0; kb0 < P.g.KB && !stop; kb0 += P.g.kchunk) {
-                    const int kb1 = min(kb0 + P.g.kchunk, P.g.KB);
-                    for (int q = 0; q < 3 && !stop; ++q) {
-                        for (int kb = kb0; kb < kb1; ++kb, ++it) {
-                            const int s = it % STAGES;
-                            const uint32_t ph = (it / STAGES) & 1;
-                            if (*abort_flag || !mbar_wait(&empty[s], ph ^ 1, status0)) {
-                                *abort_flag = 1;
-                                stop = true;
-                                break;
-                            }
-                            unsigned char* st = smem + s * STAGE_BYTES;
-                            mbar_arrive_expect_tx(&full[s], STAGE_BYTES);
-                            const int kt = kb * G3_BK;
-                            const int c0 = kt % P.g.two_d, c1 = m0 + kt / P.g.two_d;
-                            if (PAIR) {
-                                // rows 64 r .. 64 r + 63 of both A planes, into both CTAs (64-row boxes)
-                                const uint32_t ho = static_cast<uint32_t>(rank) * G3_A_HALF;
-                                const int r1 = c1 + rank * (BM / 2);
-                                tma_load_2d_mc(st + ho, &P.a[2 * q], c0, r1, &full[s], 0x3);
-                                tma_load_2d_mc(st + G3_A_BYTES + ho, &P.a[2 * q + 1], c0, r1, &full[s], 0x3);
-                            } else {
-                                tma_load_2d(st, &P.a[2 * q], c0, c1, &full[s]);
-                                tma_load_2d(st + G3_A_BYTES, &P.a[2 * q + 1], c0, c1, &full[s]);
-                            }
-                            tma_load_2d(st + 2 * G3_A_BYTES, &P.b[2 * q], kt, n0, &full[s]);
-                            tma_load_2d(st + 2 * G3_A_BYTES + B_BYTES, &P.b[2 * q + 1], kt, n0, &full[s]);
+            for (int unit = first; unit < n_units && !stop; unit += stride) {
+                const G3Plan& P = g3_plan_of(bt, unit);
+                const G3Unit u = g3_unit<PAIR>(P, unit, rank);
+                // rows of a B box: the tile's tones, or this CTA's half of them
+                const uint32_t box = PAIR ? P.bw / 2 : P.bw;
+                const uint32_t bytes = 2 * G3_OP_BYTES + 2 * box * (G3_BK * 2);
+                const int b0 = PAIR ? u.n0 + rank * (u.width / 2) : u.n0;
+                for (int q = u.q0; q < u.q1 && !stop; ++q) {
+                    for (int kb = 0; kb < P.g.KB; ++kb, ++it) {
+                        const int s = it % STAGES;
+                        const uint32_t ph = (it / STAGES) & 1;
+                        if (*abort_flag || !mbar_wait(&empty[s], ph ^ 1, status0)) {
+                            *abort_flag = 1;
+                            stop = true;
+                            break;
+                        }
+                        unsigned char* st = smem + s * G3_STAGE_BYTES;
+                        const int kt = kb * G3_BK;
+                        const int c0 = kt % P.g.two_d, c1 = static_cast<int>(u.m0) + kt / P.g.two_d;
+                        if constexpr (PAIR) {
+                            // both CTAs' bytes are counted on CTA 0's barrier
+                            if (rank == 0) mbar_arrive_expect_tx(&full[s], 2 * bytes);
+                            const uint32_t fb = cluster_addr(&full[s], 0);
+                            tma_load_2d_2sm(st, &P.a[2 * q], c0, c1, fb);
+                            tma_load_2d_2sm(st + G3_OP_BYTES, &P.a[2 * q + 1], c0, c1, fb);
+                            tma_load_2d_2sm(st + 2 * G3_OP_BYTES, &P.b[2 * q], kt, b0, fb);
+                            tma_load_2d_2sm(st + 3 * G3_OP_BYTES, &P.b[2 * q + 1], kt, b0, fb);
+                        } else {
+                            mbar_arrive_expect_tx(&full[s], bytes);
+                            tma_load_2d(st, &P.a[2 * q], c0, c1, &full[s]);
+                            tma_load_2d(st + G3_OP_BYTES, &P.a[2 * q + 1], c0, c1, &full[s]);
+                            tma_load_2d(st + 2 * G3_OP_BYTES, &P.b[2 * q], kt, b0, &full[s]);
+                            tma_load_2d(st + 3 * G3_OP_BYTES, &P.b[2 * q + 1], kt, b0, &full[s]);
                         }
                     }
                 }
             }
-            // wait for the copies still in flight before leaving
-            for (uint32_t k = 0; k < static_cast<uint32_t>(STAGES) && it > 0; ++k) {
+            // wait for the copies still in flight before leaving (CTA 0 of a
+            // pair for both CTAs' copies)
+            for (uint32_t k = 0; rank == 0 && k < static_cast<uint32_t>(STAGES) && it > 0; ++k) {
                 const uint32_t j = it - 1 - k;
                 if (static_cast<int32_t>(j) < 0) break;
                 mbar_wait(&full[j % STAGES], (j / STAGES) & 1, status0);
             }
-            // pair form: and for both CTAs' last commits to this CTA's empty
+            // pair form: and for the last commits to this CTA's empty
             // barriers, so that nothing arrives here after the CTA has left
             for (uint32_t k = 0; PAIR && k < static_cast<uint32_t>(STAGES) && it > 0; ++k) {
                 const uint32_t j = it - 1 - k;
@@ -708,14 +838,17 @@ demod3m_gemm_kernel(const __grid_constant__ G3Batch bt) {
         }
     } else if (warp == MMA_WARP) {
         // ------------------------------------------------ MMA issuer
-        if (lane == 0) {
+        if (lane == 0 && rank == 0) {
             uint32_t it = 0, phase = 0;
             bool stop = false;
-            for (int tile = cta0; tile < n_tiles && !stop; tile += ncta) {
-                const GemmArgs& g = bt.p[g3_plan_of(bt, tile)].g;
-                for (int kb0 = 0; kb0 < g.KB && !stop; kb0 += g.kchunk) {
-                    const int kb1 = min(kb0 + g.kchunk, g.KB);
-                    for (int q = 0; q < 3 && !stop; ++q, ++phase) {
+            for (int unit = first; unit < n_units && !stop; unit += stride) {
+                const G3Plan& P = g3_plan_of(bt, unit);
+                const GemmArgs& g = P.g;
+                const G3Unit u = g3_unit<PAIR>(P, unit, rank);
+                const uint32_t idesc = umma::idesc_f16_f32(PAIR ? 256 : 128, u.width);
+                for (int q = u.q0; q < u.q1 && !stop; ++q) {
+                    for (int kb0 = 0; kb0 < g.KB && !stop; kb0 += g.kchunk, ++phase) {
+                        const int kb1 = min(kb0 + g.kchunk, g.KB);
                         const uint32_t slot = phase % SLOTS, use = phase / SLOTS;
                         if (*abort_flag || !mbar_wait(&sempty[slot], (use & 1) ^ 1, status0)) {
                             *abort_flag = 1;
@@ -723,7 +856,7 @@ demod3m_gemm_kernel(const __grid_constant__ G3Batch bt) {
                             break;
                         }
                         umma::fence_after_sync();
-                        const uint32_t d_tmem = tmem + slot * Cfg::SLOT_COLS;
+                        const uint32_t d_tmem = tmem + slot * TW;
                         for (int kb = kb0; kb < kb1; ++kb, ++it) {
                             const int s = it % STAGES;
                             const uint32_t ph = (it / STAGES) & 1;
@@ -733,23 +866,29 @@ demod3m_gemm_kernel(const __grid_constant__ G3Batch bt) {
                                 break;
                             }
                             umma::fence_after_sync();
-                            const uint32_t sa = smem_u32(smem + s * STAGE_BYTES);
-                            const uint32_t ah = sa, al = sa + G3_A_BYTES;
-                            const uint32_t bh = sa + 2 * G3_A_BYTES, bl = bh + B_BYTES;
+                            const uint32_t ah = smem_u32(smem + s * G3_STAGE_BYTES), al = ah + G3_OP_BYTES;
+                            const uint32_t bh = ah + 2 * G3_OP_BYTES, bl = ah + 3 * G3_OP_BYTES;
 #pragma unroll
                             for (int k = 0; k < G3_BK / 16; ++k) {
                                 const uint32_t off = k * 32;
                                 const uint32_t acc = (kb > kb0 || k > 0) ? 1u : 0u;
-                                // hi.hi | hi.lo over 2 BT columns (B lo follows B hi), then lo.hi
-                                umma::mma_f16(d_tmem, umma::desc_k_sw128(ah + off), umma::desc_k_sw128(bh + off), IDESC_W, acc);
-                                umma::mma_f16(d_tmem, umma::desc_k_sw128(al + off), umma::desc_k_sw128(bh + off), IDESC, 1u);
+                                const uint64_t dah = umma::desc_k_sw128(ah + off), dal = umma::desc_k_sw128(al + off);
+                                const uint64_t dbh = umma::desc_k_sw128(bh + off), dbl = umma::desc_k_sw128(bl + off);
+                                if constexpr (PAIR) {
+                                    umma::mma_f16_2sm(d_tmem, dah, dbh, idesc, acc);
+                                    umma::mma_f16_2sm(d_tmem, dah, dbl, idesc, 1u);
+                                    umma::mma_f16_2sm(d_tmem, dal, dbh, idesc, 1u);
+                                } else {
+                                    umma::mma_f16(d_tmem, dah, dbh, idesc, acc);
+                                    umma::mma_f16(d_tmem, dah, dbl, idesc, 1u);
+                                    umma::mma_f16(d_tmem, dal, dbh, idesc, 1u);
+                                }
                             }
-                            if (PAIR)
-                                umma::commit_mc(&empty[s], 0x3);      // frees the stage in both CTAs
-                            else
-                                umma::commit(&empty[s]);
+                            if constexpr (PAIR) umma::commit_2sm(&empty[s]);      // frees the stage in both CTAs
+                            else umma::commit(&empty[s]);
                         }
-                        umma::commit(&sfull[slot]);
+                        if constexpr (PAIR) umma::commit_2sm(&sfull[slot]);
+                        else umma::commit(&sfull[slot]);
                     }
                 }
             }
@@ -757,22 +896,22 @@ demod3m_gemm_kernel(const __grid_constant__ G3Batch bt) {
         __syncwarp();
     } else if (warp < G3_EPI_WARPS) {
         // ------------------------------------------------ epilogue (16 warps)
-        constexpr int TPG = Cfg::TPG;
         const int qd = warp & 3, grp = warp >> 2;          // lane quadrant, tone group
         const int row = qd * 32 + lane;
-        uint32_t phase = 0;
+        uint32_t phase = 0, tile = 0;
         bool ok = true;
-        for (int tile = cta0; tile < n_tiles && ok; tile += ncta) {
-            const G3Plan& P = bt.p[g3_plan_of(bt, tile)];
+        // this thread's column of the CTA's scratch planes
+        float* const scr = scr_cta + grp * TPG * 128 + row;
+        for (int unit = first; unit < n_units && ok; unit += stride) {
+            const G3Plan& P = g3_plan_of(bt, unit);
             const GemmArgs& g = P.g;
-            int mt, tn;
-            g3_coords<PAIR>(g, tile - P.tile0, rank, mt, tn);
-            const int m0 = mt * BM, n0 = tn * BT;
-            float re[TPG], im[TPG];
+            const G3Unit u = g3_unit<PAIR>(P, unit, rank);
+            const int cols = min(TPG, u.width - grp * TPG);          // this thread's tones (a multiple of 16, or <= 0)
+            float sum[TPG];
+            for (int q = u.q0; q < u.q1 && ok; ++q) {
 #pragma unroll
-            for (int i = 0; i < TPG; ++i) re[i] = im[i] = 0.f;
-            for (int kb0 = 0; kb0 < g.KB && ok; kb0 += g.kchunk) {
-                for (int q = 0; q < 3; ++q, ++phase) {
+                for (int i = 0; i < TPG; ++i) sum[i] = 0.f;
+                for (int kb0 = 0; kb0 < g.KB; kb0 += g.kchunk, ++phase) {
                     const uint32_t slot = phase % SLOTS, use = phase / SLOTS;
                     if (*abort_flag || !mbar_wait(&sfull[slot], use & 1, status0)) {
                         *abort_flag = 1;
@@ -780,56 +919,155 @@ demod3m_gemm_kernel(const __grid_constant__ G3Batch bt) {
                         break;
                     }
                     umma::fence_after_sync();
-                    const uint32_t ta = tmem + (static_cast<uint32_t>(qd * 32) << 16) + slot * Cfg::SLOT_COLS + grp * TPG;
-                    // the product = (hi.hi + lo.hi) + hi.lo, 16 tones at a time
+                    const uint32_t ta = tmem + (static_cast<uint32_t>(qd * 32) << 16) + slot * TW + grp * TPG;
 #pragma unroll
                     for (int h = 0; h < TPG; h += 16) {
-                        uint32_t r0[16], r1[16];
-                        umma::ld_32x32b_x16(ta + h, r0);
-                        umma::ld_32x32b_x16(ta + BT + h, r1);
-                        umma::wait_ld_regs(r0);
-                        umma::wait_ld_regs(r1);
-                        float pv[16];
+                        if (h < cols) {
+                            uint32_t r0[16];
+                            umma::ld_32x32b_x16(ta + h, r0);
+                            umma::wait_ld_regs(r0);
 #pragma unroll
-                        for (int i = 0; i < 16; ++i) pv[i] = __uint_as_float(r0[i]) + __uint_as_float(r1[i]);
-                        if (q == 0) {
-#pragma unroll
-                            for (int i = 0; i < 16; ++i) {
-                                const float v = 2.f * pv[i];
-                                re[h + i] += v;
-                                im[h + i] += v;
-                            }
-                        } else if (q == 1) {
-#pragma unroll
-                            for (int i = 0; i < 16; ++i) im[h + i] += pv[i];
-                        } else {
-#pragma unroll
-                            for (int i = 0; i < 16; ++i) re[h + i] -= pv[i];
+                            for (int i = 0; i < 16; ++i) sum[h + i] += __uint_as_float(r0[i]);
                         }
                     }
                     umma::fence_before_sync();
-                    mbar_arrive(&sempty[slot]);
-                }
-            }
-            if (!ok) break;
-            const int64_t k = static_cast<int64_t>(m0) + row;
-            if (k < g.F) {
-                const int tb = n0 + grp * TPG;
-                const int64_t K = g.F0 + k;
-                const int64_t arow = K / BM - g.F0 / BM;
-                const int si = static_cast<int>(K % BM);
-#pragma unroll
-                for (int tl = 0; tl < TPG; ++tl) {
-                    const int t = tb + tl;
-                    if (t < g.n_tones) {
-                        const float2 an = __ldg(g.anchors + arow * g.ntp + t);
-                        const float2 sp = __ldg(g.steps + static_cast<int64_t>(t) * BM + si);
-                        const float2 rot = cmul(an, sp);
-                        const float2 acc = make_float2(re[tl] * g.inv_scale, im[tl] * g.inv_scale);
-                        g.out[static_cast<int64_t>(t) * g.ld + g.fo + k] = cmul(acc, rot);
+                    __syncwarp();
+                    if (lane == 0) {
+                        if constexpr (PAIR) mbar_arrive_cluster(cluster_addr(&sempty[slot], 0));
+                        else mbar_arrive(&sempty[slot]);
                     }
                 }
+                if (!ok) break;
+                if (P.split) {
+                    const int64_t k = u.m0 + row;
+                    const int tb = u.n0 + grp * TPG;
+                    if (k < g.F) {
+                        float* pl = P.scratch + (static_cast<int64_t>(q) * g.n_tones + tb) * P.pld + k;
+#pragma unroll
+                        for (int i = 0; i < TPG; ++i, pl += P.pld)
+                            if (i < cols && tb + i < g.n_tones) *pl = sum[i];
+                    }
+                    continue;
+                }
+                // the first product to reuse a plane of the tile before, which
+                // has to be finished by then
+                if (q == G3_PLANES - 3 && tile > 0 && !mbar_wait(finished, (tile - 1) & 1, status0)) {
+                    *abort_flag = 1;
+                    ok = false;
+                    break;
+                }
+                float* const pl = scr + ((3 * tile + q) % G3_PLANES) * G3_PLANE;
+#pragma unroll
+                for (int i = 0; i < TPG; ++i)
+                    if (i < cols) pl[i * 128] = sum[i];
             }
+            if (ok && !P.split) {
+                fence_proxy_async_global();                  // the finishers read the planes by bulk copies
+                __syncwarp();
+                if (lane == 0) mbar_arrive(parked);
+                if (unit + stride >= n_units && mbar_wait(parked, tile & 1, status0))
+                    g3_finish(P, u, scr_cta, tile, lane, warp, G3_THREADS / 32, FIN_WARP - G3_EPI_WARPS);
+                ++tile;
+            }
+        }
+    } else if (warp >= FIN_WARP) {
+        // ------------------------------------------------ finishers
+        const int w = warp - FIN_WARP;
+        unsigned char* const stage = fin_stage + w * G3_FIN_BUFS * G3_FIN_BYTES;
+        uint64_t* const bars = fbar + w * G3_FIN_BUFS;
+        uint32_t tile = 0, fills = 0;                         // chunks consumed so far (buffer and phase)
+        bool ok = true;
+        for (int unit = first; unit < n_units && ok; unit += stride) {
+            const G3Plan& P = g3_plan_of(bt, unit);
+            if (P.split) continue;
+            if (*abort_flag || !mbar_wait(parked, tile & 1, status0)) {
+                *abort_flag = 1;
+                break;
+            }
+            const G3Unit u = g3_unit<PAIR>(P, unit, rank);
+            if (unit + stride >= n_units) {
+                // the CTA's last tile: every warp that is free takes part
+                g3_finish(P, u, scr_cta, tile, lane, warp, G3_THREADS / 32, FIN_WARP - G3_EPI_WARPS);
+            } else {
+                const GemmArgs& g = P.g;
+                const int n = min(u.width, g.n_tones - u.n0);
+                // the warp's chunks: tones 2 (w + i FINISHERS), 2 (w + i FINISHERS) + 1
+                const int chunks = ((n + 1) / 2 - w + FINISHERS - 1) / FINISHERS;
+                auto fetch = [&](int i) {
+                    const uint32_t b = (fills + i) % G3_FIN_BUFS;
+                    unsigned char* dst = stage + b * G3_FIN_BYTES;
+                    const int c = 2 * (w + i * FINISHERS);
+                    mbar_arrive_expect_tx(&bars[b], G3_FIN_BYTES);
+#pragma unroll
+                    for (int q = 0; q < 3; ++q)
+                        tma_bulk_g2s(dst + q * 1024, scr_cta + ((3 * tile + q) % G3_PLANES) * G3_PLANE + c * 128, 1024, &bars[b]);
+                    tma_bulk_g2s(dst + 3072, g.steps + static_cast<int64_t>(u.n0 + c) * BM, 2048, &bars[b]);
+                };
+                const int ahead = min(chunks, G3_FIN_BUFS);
+                if (lane == 0)
+                    for (int i = 0; i < ahead; ++i) fetch(i);
+                // lane l: frames 4 l .. 4 l + 3; anchor rows a0 and, from row
+                // `turn` of the tile on, a0 + 1
+                const int64_t k = u.m0 + 4 * lane;
+                const int rows = static_cast<int>(k < g.F ? (g.F - k < 4 ? g.F - k : 4) : 0);
+                const int f0 = static_cast<int>(g.F0 % BM), turn = BM - f0;
+                const bool vec = rows == 4 &&
+                                 ((reinterpret_cast<uintptr_t>(g.out + g.fo + k) | static_cast<uintptr_t>(g.ld * 8)) & 15) == 0;
+                const float2* const anc = g.anchors + ((g.F0 + u.m0) / BM - g.F0 / BM) * g.ntp + u.n0;
+                float2 a_lo = make_float2(0.f, 0.f), a_hi = a_lo;
+                for (int i = 0; i < chunks; ++i) {
+                    if ((i & 15) == 0) {
+                        // anchors of the next 16 chunks, a tone per lane
+                        const int c = 2 * (w + (i + (lane >> 1)) * FINISHERS) + (lane & 1);
+                        const bool on = c < n;
+                        a_lo = on ? __ldg(anc + c) : make_float2(0.f, 0.f);
+                        a_hi = on && f0 > 0 && u.m0 + turn < g.F ? __ldg(anc + g.ntp + c) : make_float2(0.f, 0.f);
+                    }
+                    const uint32_t fi = fills + i;
+                    if (!mbar_wait(&bars[fi % G3_FIN_BUFS], (fi / G3_FIN_BUFS) & 1, status0)) {
+                        *abort_flag = 1;
+                        ok = false;
+                        break;
+                    }
+                    const unsigned char* src = stage + (fi % G3_FIN_BUFS) * G3_FIN_BYTES;
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int c = 2 * (w + i * FINISHERS) + h;
+                        const int from = ((i & 15) << 1) + h;
+                        const float2 al = make_float2(__shfl_sync(0xffffffffu, a_lo.x, from), __shfl_sync(0xffffffffu, a_lo.y, from));
+                        const float2 ah = make_float2(__shfl_sync(0xffffffffu, a_hi.x, from), __shfl_sync(0xffffffffu, a_hi.y, from));
+                        if (c >= n || rows == 0) continue;
+                        const float4 p1 = *reinterpret_cast<const float4*>(src + h * 512 + lane * 16);
+                        const float4 p2 = *reinterpret_cast<const float4*>(src + 1024 + h * 512 + lane * 16);
+                        const float4 p3 = *reinterpret_cast<const float4*>(src + 2048 + h * 512 + lane * 16);
+                        const float2* const sp = reinterpret_cast<const float2*>(src + 3072 + h * 1024);
+                        float2 y[4];
+#pragma unroll
+                        for (int r = 0; r < 4; ++r) {
+                            const int row = 4 * lane + r;
+                            const float v1 = r == 0 ? p1.x : r == 1 ? p1.y : r == 2 ? p1.z : p1.w;
+                            const float v2 = r == 0 ? p2.x : r == 1 ? p2.y : r == 2 ? p2.z : p2.w;
+                            const float v3 = r == 0 ? p3.x : r == 1 ? p3.y : r == 2 ? p3.z : p3.w;
+                            y[r] = g3_output(v1, v2, v3, g.inv_scale, row < turn ? al : ah, sp[(row + f0) & (BM - 1)]);
+                        }
+                        float2* o = g.out + static_cast<int64_t>(u.n0 + c) * g.ld + g.fo + k;
+                        if (vec) {
+                            reinterpret_cast<float4*>(o)[0] = make_float4(y[0].x, y[0].y, y[1].x, y[1].y);
+                            reinterpret_cast<float4*>(o)[1] = make_float4(y[2].x, y[2].y, y[3].x, y[3].y);
+                        } else {
+#pragma unroll
+                            for (int r = 0; r < 4; ++r)
+                                if (r < rows) o[r] = y[r];
+                        }
+                    }
+                    __syncwarp();                             // the buffer has been read
+                    if (lane == 0 && i + G3_FIN_BUFS < chunks) fetch(i + G3_FIN_BUFS);
+                }
+                fills += chunks;
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(finished);
+            ++tile;
         }
     }
     umma::fence_before_sync();
@@ -837,7 +1075,25 @@ demod3m_gemm_kernel(const __grid_constant__ G3Batch bt) {
     if (PAIR) cluster_sync();          // neither CTA leaves while the other may still signal it
     if (warp == MMA_WARP) {
         umma::fence_after_sync();
-        umma::dealloc(tmem, Cfg::TMEM_COLS);
+        umma::dealloc<PAIR>(tmem, G3_TMEM_COLS);
+    }
+}
+
+// The split form's last step: planes P1, P2, P3 [n_tones][pld] -> outputs,
+// with the arithmetic of the GEMM's own last step.  One thread per output,
+// frames along the warp.
+__global__ void combine3_kernel(const float* __restrict__ planes, int64_t pld, const GemmArgs g) {
+    const int64_t k = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+    if (k >= g.F) return;
+    const int64_t K = g.F0 + k;
+    const int64_t arow = K / BM - g.F0 / BM;
+    const int si = static_cast<int>(K % BM);
+    const int64_t plane = static_cast<int64_t>(g.n_tones) * pld;
+    for (int t = blockIdx.y; t < g.n_tones; t += gridDim.y) {
+        const float* p = planes + t * pld + k;
+        g.out[static_cast<int64_t>(t) * g.ld + g.fo + k] =
+            g3_output(p[0], p[plane], p[2 * plane], g.inv_scale, __ldg(g.anchors + arow * g.ntp + t),
+                      __ldg(g.steps + static_cast<int64_t>(t) * BM + si));
     }
 }
 
@@ -874,6 +1130,15 @@ size_t demod_xs_rows(int64_t F, int Lpad, int D) {
     // frame F-1 reads rows F-1 .. F-1 + (Lpad-1)/D
     return static_cast<size_t>(F + (Lpad - 1) / D);
 }
+
+namespace {
+// Rows of the split form's planes, and whether three planes fit the scratch.
+int64_t g3_plane_ld(int64_t F) { return (F + 31) / 32 * 32; }
+bool g3_planes_fit(int n_tones, int64_t F, int n_sms) {
+    return 3 * n_tones * g3_plane_ld(F) * 4 <= static_cast<int64_t>(demod3_scratch_bytes(n_sms));
+}
+}  // namespace
+size_t demod3_scratch_bytes(int n_sms) { return static_cast<size_t>(n_sms) * G3_CTA_SCRATCH * 4; }
 
 size_t demod3_xs_rows(int64_t F, int Lpad, int D) { return static_cast<size_t>(F + (Lpad - 1) / D); }
 
@@ -947,18 +1212,76 @@ cudaError_t demod3_build_taps(const double* d_h, const uint64_t* d_words, int n_
     return cudaGetLastError();
 }
 
-cudaError_t demod3_prepare(const DemodLaunch& L, cudaStream_t st, DemodGemmJob* job) {
-    job->n_tiles = 0;
-    job->bt = L.tone_tile == 64 ? 64 : 128;
-    job->fused = L.fused_presplit ? 1 : 0;
-    job->pair = (L.pair && !job->fused) ? 1 : 0;
+namespace {
+// Clocks that a work item's K-block (64 taps of one product) takes at least:
+// its MMAs (12 of w/2 clocks), or the shared-memory traffic of the MMAs and
+// the TMA at 128 bytes a clock (see the Gauss form's comment).
+double g3_block_clocks(bool pair, int w) {
+    return pair ? std::max(6.0 * w, 640.0 + 2.5 * w) : std::max(6.0 * w, 640.0 + 5.0 * w);
+}
+
+struct G3Form {
+    bool pair = false, split = false;
+    int bw = 128;
+};
+int g3_even_width(int n_tones, int widest, int step) {
+    const int tiles = (n_tones + widest - 1) / widest;
+    return ((n_tones + tiles - 1) / tiles + step - 1) / step * step;
+}
+// The form of a push that names none: the least time of the four, counting
+// whole waves of work items over the chip (a batched step's launch shares its
+// waves between plans, so there only the work counts, and nothing is split).
+// kSplitClocks: the planes' round trip and combine3_kernel's launch.
+G3Form g3_choose(const DemodLaunch& L, bool shared_launch) {
+    constexpr double kSplitClocks = 8000.0;
+    G3Form best;
+    double best_t = 1e300;
+    const int64_t KB = L.Lpad / G3_BK;
+    for (int pair = 0; pair < 2; ++pair) {
+        const int widths[2] = {pair ? g3_even_width(L.n_tones, G3_PAIR_TONES, 32)
+                                    : g3_even_width(L.n_tones, G3_SINGLE_TONES, 16),
+                               pair ? 0 : g3_even_width(L.n_tones, 64, 16)};
+        for (int w : widths) {
+            if (w <= 0) continue;
+            const int64_t tiles = (L.F + (pair ? 255 : 127)) / (pair ? 256 : 128) * ((L.n_tones + w - 1) / w);
+            const int64_t places = pair ? L.n_sms / 2 : L.n_sms;
+            for (int split = 0; split < 2; ++split) {
+                if (split && (shared_launch || !g3_planes_fit(L.n_tones, L.F, L.n_sms))) continue;
+                const int64_t units = tiles * (split ? 3 : 1);
+                const double waves = shared_launch ? static_cast<double>(units) / places
+                                                   : static_cast<double>((units + places - 1) / places);
+                const double t = waves * KB * (split ? 1 : 3) * g3_block_clocks(pair != 0, w) + (split ? kSplitClocks : 0.0);
+                if (t < best_t) {
+                    best_t = t;
+                    best.pair = pair != 0;
+                    best.split = split != 0;
+                    best.bw = w;
+                }
+            }
+        }
+    }
+    return best;
+}
+}  // namespace
+
+cudaError_t demod3_prepare(const DemodLaunch& L, cudaStream_t st, DemodGemmJob* job, bool shared_launch) {
+    job->n_units = 0;
     if (L.F <= 0) return cudaSuccess;
     if (L.D % G3_BK != 0 || L.Lpad % G3_BK != 0 || L.ntp % 128 != 0) return cudaErrorInvalidValue;
+    G3Form form;
+    if (L.auto_form) {
+        form = g3_choose(L, shared_launch);
+    } else {
+        form.pair = L.pair && !L.fused_presplit;
+        form.bw = form.pair ? g3_even_width(L.n_tones, G3_PAIR_TONES, 32) : (L.tone_tile == 64 ? 64 : 128);
+    }
+    job->fused = !L.auto_form && L.fused_presplit ? 1 : 0;
+    job->pair = form.pair ? 1 : 0;
     const int64_t rows = static_cast<int64_t>(demod3_xs_rows(L.F, L.Lpad, L.D));
     if (!job->fused && rows > L.xs_rows) return cudaErrorInvalidValue;
-    const int bt = job->bt;
-    const int n_mt = static_cast<int>((L.F + BM - 1) / BM);
-    const int n_nt = (L.n_tones + bt - 1) / bt;       // tiles past the last tone are skipped
+    const int bm = form.pair ? 256 : BM;
+    const int n_mt = static_cast<int>((L.F + bm - 1) / bm);
+    const int n_nt = (L.n_tones + form.bw - 1) / form.bw;
     const int n_anch = demod_anchor_rows(L.F0, L.F);
     float2* anchors = static_cast<float2*>(L.rot);
     float2* steps = anchors + static_cast<int64_t>(n_anch) * L.ntp;
@@ -983,12 +1306,17 @@ cudaError_t demod3_prepare(const DemodLaunch& L, cudaStream_t st, DemodGemmJob* 
             reinterpret_cast<const uint32_t*>(L.carry), L.cl, reinterpret_cast<const uint32_t*>(L.buf), L.cl + L.n,
             total, xp);
     }
+    const uint32_t b_box = static_cast<uint32_t>(form.pair ? form.bw / 2 : form.bw);
     for (int i = 0; i < 6; ++i) {
         if ((!job->fused && !make_map(&P->a[i], xp + i * total, static_cast<uint64_t>(L.D),
-                                      static_cast<uint64_t>(rows), job->pair ? BM / 2 : BM)) ||
-            !make_map(&P->b[i], bp + i * bplane, static_cast<uint64_t>(L.Lpad), static_cast<uint64_t>(L.ntp), bt))
+                                      static_cast<uint64_t>(rows), BM)) ||
+            !make_map(&P->b[i], bp + i * bplane, static_cast<uint64_t>(L.Lpad), static_cast<uint64_t>(L.ntp), b_box))
             return cudaErrorInvalidValue;
     }
+    P->bw = form.bw;
+    P->split = form.split ? 1 : 0;
+    P->scratch = static_cast<float*>(L.scratch);
+    P->pld = g3_plane_ld(L.F);
     GemmArgs& g = P->g;
     g.raster = L.raster_group;
     g.F = L.F;
@@ -996,7 +1324,10 @@ cudaError_t demod3_prepare(const DemodLaunch& L, cudaStream_t st, DemodGemmJob* 
     g.n_tones = L.n_tones;
     g.ntp = L.ntp;
     g.KB = L.Lpad / G3_BK;
-    g.kchunk = L.kchunk > 0 ? L.kchunk : 1;
+    // the three MMAs of a tap set share one accumulator, where they would take
+    // two (hi.hi + lo.hi beside hi.lo) half as many blocks make a chunk: the
+    // accumulator takes fewer additions of smaller partial sums
+    g.kchunk = L.kchunk > 1 ? (L.kchunk + 1) / 2 : 1;
     g.two_d = L.D;                 // columns of a Toeplitz source row (one plane)
     g.n_mt = n_mt;
     g.n_nt = n_nt;
@@ -1007,21 +1338,21 @@ cudaError_t demod3_prepare(const DemodLaunch& L, cudaStream_t st, DemodGemmJob* 
     g.ld = L.tones_ld;
     g.fo = L.frame_offset;
     g.status = L.status;
-    job->n_tiles = n_mt * (job->pair ? (n_nt + 1) / 2 : n_nt);
+    job->n_units = n_mt * n_nt * (form.split ? 3 : 1);
+    job->unit_cost = g.KB * (form.split ? 1 : 3) * g3_block_clocks(form.pair, form.bw);
     return cudaGetLastError();
 }
 
 namespace {
-template <int BT, bool FUSED, bool PAIR>
+template <bool PAIR, bool FUSED>
 cudaError_t g3_run(const G3Batch& b, int n_sms, cudaStream_t st) {
-    using Cfg = G3Cfg<BT>;
-    auto kern = demod3m_gemm_kernel<BT, FUSED, PAIR>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(Cfg::SMEM));
+    auto kern = demod3m_gemm_kernel<PAIR, FUSED>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(G3_SMEM));
     if (e != cudaSuccess) return e;
-    const int threads = FUSED ? G3_THREADS_FUSED : G3_THREADS;
+    const int threads = G3_THREADS;
     if (!PAIR) {
-        const int grid = std::max(1, std::min(b.total_tiles, n_sms));
-        kern<<<grid, threads, Cfg::SMEM, st>>>(b);
+        const int grid = std::max(1, std::min(b.total_units, n_sms));
+        kern<<<grid, threads, G3_SMEM, st>>>(b);
         return cudaGetLastError();
     }
     // clusters of two CTAs: as many as can be resident at once (one CTA per SM)
@@ -1032,22 +1363,21 @@ cudaError_t g3_run(const G3Batch& b, int n_sms, cudaStream_t st) {
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.blockDim = dim3(threads, 1, 1);
-    cfg.dynamicSmemBytes = Cfg::SMEM;
+    cfg.dynamicSmemBytes = G3_SMEM;
     cfg.stream = st;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    static int max_clusters[2] = {0, 0};          // per tile width, queried once
-    int& mc = max_clusters[BT == 128 ? 0 : 1];
+    static std::atomic<int> max_clusters{0};      // queried once
+    int mc = max_clusters.load();
     if (mc <= 0) {
         cfg.gridDim = dim3(static_cast<unsigned>(2 * (n_sms / 2)), 1, 1);
-        int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n <= 0) {
+        if (cudaOccupancyMaxActiveClusters(&mc, kern, &cfg) != cudaSuccess || mc <= 0) {
             cudaGetLastError();
-            n = n_sms / 2;
+            mc = n_sms / 2;
         }
-        mc = n;
+        max_clusters.store(mc);
     }
-    const int clusters = std::max(1, std::min(b.total_tiles, mc));
+    const int clusters = std::max(1, std::min(b.total_units, std::min(mc, n_sms / 2)));
     cfg.gridDim = dim3(static_cast<unsigned>(2 * clusters), 1, 1);
     e = cudaLaunchKernelEx(&cfg, kern, b);
     if (e != cudaSuccess) return e;
@@ -1056,36 +1386,41 @@ cudaError_t g3_run(const G3Batch& b, int n_sms, cudaStream_t st) {
 }  // namespace
 
 cudaError_t demod3_gemm(const DemodGemmJob* const* jobs, int n, int n_sms, cudaStream_t st) {
-    // one persistent launch per group of up to kG3MaxPlans jobs of the same
-    // tile width, producer form and cluster form
-    for (int variant = 0; variant < 8; ++variant) {
-        const int bt = variant & 1 ? 64 : 128;
-        const int fused = (variant >> 1) & 1;
-        const int pair = variant >> 2;
-        if (fused && pair) continue;
+    // costliest work items first, so that the launch ends on short ones
+    std::vector<const DemodGemmJob*> order(jobs, jobs + n);
+    std::stable_sort(order.begin(), order.end(),
+                     [](const DemodGemmJob* x, const DemodGemmJob* y) { return x->unit_cost > y->unit_cost; });
+    // one persistent launch per group of up to kG3MaxPlans jobs of the same form
+    for (int variant = 0; variant < 3; ++variant) {
+        const int fused = variant == 2, pair = variant == 0;
         G3Batch b;
         b.n_plans = 0;
-        b.total_tiles = 0;
+        b.total_units = 0;
         for (int i = 0; i <= n; ++i) {
             const bool flush = i == n || b.n_plans == kG3MaxPlans;
             if (flush && b.n_plans > 0) {
-                cudaError_t e;
-                if (pair)
-                    e = bt == 128 ? g3_run<128, false, true>(b, n_sms, st) : g3_run<64, false, true>(b, n_sms, st);
-                else if (fused)
-                    e = bt == 128 ? g3_run<128, true, false>(b, n_sms, st) : g3_run<64, true, false>(b, n_sms, st);
-                else
-                    e = bt == 128 ? g3_run<128, false, false>(b, n_sms, st) : g3_run<64, false, false>(b, n_sms, st);
+                // the launch's CTAs park partial products in its first plan's scratch
+                for (int k = 1; k < b.n_plans; ++k)
+                    if (!b.p[k].split) b.p[k].scratch = b.p[0].scratch;
+                const cudaError_t e = pair ? g3_run<true, false>(b, n_sms, st)
+                                           : (fused ? g3_run<false, true>(b, n_sms, st) : g3_run<false, false>(b, n_sms, st));
                 if (e != cudaSuccess) return e;
+                for (int k = 0; k < b.n_plans; ++k)
+                    if (b.p[k].split) {
+                        const GemmArgs& g = b.p[k].g;
+                        const dim3 grid(static_cast<unsigned>((g.F + 255) / 256), static_cast<unsigned>(std::min(g.n_tones, 65535)));
+                        combine3_kernel<<<grid, 256, 0, st>>>(b.p[k].scratch, b.p[k].pld, g);
+                        const cudaError_t ce = cudaGetLastError();
+                        if (ce != cudaSuccess) return ce;
+                    }
                 b.n_plans = 0;
-                b.total_tiles = 0;
+                b.total_units = 0;
             }
             if (i == n) break;
-            if (jobs[i]->bt != bt || jobs[i]->fused != fused || jobs[i]->pair != pair || jobs[i]->n_tiles <= 0)
-                continue;
-            std::memcpy(&b.p[b.n_plans], jobs[i]->bytes, sizeof(G3Plan));
-            b.p[b.n_plans].tile0 = b.total_tiles;
-            b.total_tiles += jobs[i]->n_tiles;
+            if (order[i]->fused != fused || order[i]->pair != pair || order[i]->n_units <= 0) continue;
+            std::memcpy(&b.p[b.n_plans], order[i]->bytes, sizeof(G3Plan));
+            b.p[b.n_plans].unit0 = b.total_units;
+            b.total_units += order[i]->n_units;
             ++b.n_plans;
         }
     }
@@ -1094,8 +1429,8 @@ cudaError_t demod3_gemm(const DemodGemmJob* const* jobs, int n, int n_sms, cudaS
 
 cudaError_t demod3_launch(const DemodLaunch& L, cudaStream_t st) {
     DemodGemmJob job;
-    cudaError_t e = demod3_prepare(L, st, &job);
-    if (e != cudaSuccess || job.n_tiles <= 0) return e;
+    cudaError_t e = demod3_prepare(L, st, &job, false);
+    if (e != cudaSuccess || job.n_units <= 0) return e;
     const DemodGemmJob* jp = &job;
     return demod3_gemm(&jp, 1, L.n_sms, st);
 }

@@ -34,6 +34,11 @@ __device__ __forceinline__ void fence_mbar_init() {
 __device__ __forceinline__ void fence_proxy_async_smem() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
+// Orders this thread's global-memory accesses before later async-proxy (bulk
+// copy) accesses to the same memory.
+__device__ __forceinline__ void fence_proxy_async_global() {
+    asm volatile("fence.proxy.async.global;" ::: "memory");
+}
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
                  ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
@@ -72,6 +77,18 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int* s
     }
 }
 
+// Shared-memory address (cluster window) of `p`'s offset in cluster CTA `rank`.
+__device__ __forceinline__ uint32_t cluster_addr(const void* p, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
+    return r;
+}
+// One arrival on an mbarrier anywhere in the cluster (address of cluster_addr);
+// it orders no ordinary memory accesses between CTAs.
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t addr) {
+    asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(addr) : "memory");
+}
+
 // --------------------------------------------------------------- TMA bulk
 // 1-D bulk copy global -> shared, completion counted on `bar` (bytes).
 // dst, src 16-byte aligned; bytes a multiple of 16.
@@ -91,15 +108,14 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const void* tmap, int32_t
         " [%0], [%1, {%2, %3}], [%4];"
         ::"r"(smem_u32(dst)), "l"(tmap), "r"(c0), "r"(c1), "r"(smem_u32(bar)) : "memory");
 }
-// The same copy multicast to the CTAs of the cluster named in cta_mask: the
-// box lands at dst's offset in each of them and completes bytes on the
-// mbarrier at bar's offset in each of them.
-__device__ __forceinline__ void tma_load_2d_mc(void* dst, const void* tmap, int32_t c0, int32_t c1,
-                                               uint64_t* bar, uint16_t cta_mask) {
+// The same copy for a two-SM tensor-core pair: the box lands in this CTA's
+// shared memory, the bytes are counted on the mbarrier at cluster address
+// bar (cluster_addr), which may be the other CTA's.
+__device__ __forceinline__ void tma_load_2d_2sm(void* dst, const void* tmap, int32_t c0, int32_t c1, uint32_t bar) {
     asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.multicast::cluster"
-        " [%0], [%1, {%2, %3}], [%4], %5;"
-        ::"r"(smem_u32(dst)), "l"(tmap), "r"(c0), "r"(c1), "r"(smem_u32(bar)), "h"(cta_mask) : "memory");
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+        " [%0], [%1, {%2, %3}], [%4];"
+        ::"r"(smem_u32(dst)), "l"(tmap), "r"(c0), "r"(c1), "r"(bar) : "memory");
 }
 // Rank of this CTA in its cluster, and a barrier over every thread of the
 // cluster (release / acquire at cluster scope).

@@ -898,12 +898,6 @@ __host__ __device__ __forceinline__ ClusterLayout cluster_layout(int tw_count, i
     return L;
 }
 
-// Address of `p` (this CTA's shared memory) in cluster CTA `rank`.
-__device__ __forceinline__ uint32_t dsmem_map(const void* p, uint32_t rank) {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_u32(p)), "r"(rank));
-    return r;
-}
 __device__ __forceinline__ float2 dsmem_ld_f2(uint32_t addr) {
     float2 v;
     asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
@@ -1061,7 +1055,7 @@ __global__ void __launch_bounds__(kRingThreads, 1)
         {
             uint32_t e_at[C];                                     // E of each cluster CTA
 #pragma unroll
-            for (int c = 0; c < C; ++c) e_at[c] = dsmem_map(E, static_cast<uint32_t>(c)) + static_cast<uint32_t>(fpad(tf)) * 8u;
+            for (int c = 0; c < C; ++c) e_at[c] = cluster_addr(E, static_cast<uint32_t>(c)) + static_cast<uint32_t>(fpad(tf)) * 8u;
             // remote loads issued in groups of 16 before their first use, so
             // their latencies overlap
             constexpr int RG = 16 / C;                            // points per group
@@ -1112,7 +1106,7 @@ __global__ void __launch_bounds__(kRingThreads, 1)
         for (int r = 0; r < 16; ++r) P[fpad(tf + r * NT)] = v[r];
         cluster_sync();                                           // (S2) every Y_c in its P
         // output bins k = 4096 rank + i, i = tf + 256 r: k2 = tf % C, k1 = k / C
-        const uint32_t p_k2 = dsmem_map(P, static_cast<uint32_t>(tf % C));
+        const uint32_t p_k2 = cluster_addr(P, static_cast<uint32_t>(tf % C));
         const bool bulk = a.full_bulk != 0;
         if (a.full) {
 #pragma unroll
@@ -1143,7 +1137,7 @@ __global__ void __launch_bounds__(kRingThreads, 1)
 #pragma unroll
             for (int k = 0; k < kTonesPerThread; ++k)
                 if (tb[k] >= 0)
-                    tv[k] = dsmem_ld_f2(dsmem_map(P, static_cast<uint32_t>(tb[k] % C)) +
+                    tv[k] = dsmem_ld_f2(cluster_addr(P, static_cast<uint32_t>(tb[k] % C)) +
                                         static_cast<uint32_t>(fpad(tb[k] / C)) * 8u);
 #pragma unroll
             for (int k = 0; k < kTonesPerThread; ++k)
@@ -1153,7 +1147,7 @@ __global__ void __launch_bounds__(kRingThreads, 1)
             for (int t = t0 + tid; t < t1; t += NT) {
                 const int bin = __ldg(a.bins + t);
                 col[static_cast<int64_t>(t) * a.tones_ld] =
-                    dsmem_ld_f2(dsmem_map(P, static_cast<uint32_t>(bin % C)) + static_cast<uint32_t>(fpad(bin / C)) * 8u);
+                    dsmem_ld_f2(cluster_addr(P, static_cast<uint32_t>(bin % C)) + static_cast<uint32_t>(fpad(bin / C)) * 8u);
             }
         }
         const bool group_end = ntc > 0 && t1 > t0 && (q == kToneGroup - 1 || j == jb - 1);

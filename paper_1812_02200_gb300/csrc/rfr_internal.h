@@ -145,19 +145,21 @@ struct DemodLaunch {
     int n_sms;
     int kchunk;                 // k-blocks per TMEM accumulation chunk
     int raster_group;           // tile order: groups of this many 128-frame tiles sweep all tones
-    int tone_tile;              // three-product GEMM: tones per tile, 128 or 64 (0 = 128)
-    int fused_presplit;         // three-product GEMM: producers convert the int16 stream themselves
-    int pair;                   // three-product GEMM: clusters of two CTAs sharing A tiles by multicast
+    int auto_form;              // three-product GEMM: the launch picks the form by size; else:
+    int tone_tile;              //   tones per single-CTA tile, 128 or 64 (0 = 128)
+    int fused_presplit;         //   producers convert the int16 stream themselves
+    int pair;                   //   two-SM tiles
+    void* scratch;              // three-product GEMM: demod3_scratch_bytes
 };
 // The three-product GEMM of one push, described for a persistent launch that
 // may cover several plans (opaque record of demod.cu).
 constexpr int kDemodJobBytes = 2048;
 struct DemodGemmJob {
     alignas(128) unsigned char bytes[kDemodJobBytes];
-    int bt = 128;               // tone-tile width
     int fused = 0;              // pre-split fused into the GEMM's producers
-    int pair = 0;               // two-CTA clusters (n_tiles then counts tone-tile pairs)
-    int n_tiles = 0;            // 0: nothing to launch
+    int pair = 0;               // two-SM tiles
+    int n_units = 0;            // work items; 0: nothing to launch
+    double unit_cost = 0.0;     // of a work item, in clocks
 };
 cudaError_t demod_build_taps(const double* d_h, const uint64_t* d_words, int n_tones, int ntp,
                              int L, int Lpad, int e, void* b_hi, void* b_lo, cudaStream_t st);
@@ -170,12 +172,13 @@ cudaError_t demod3_build_taps(const double* d_h, const uint64_t* d_words, int n_
                               int e, void* planes, cudaStream_t st);
 cudaError_t demod3_launch(const DemodLaunch& L, cudaStream_t st);
 // the per-push kernels before the GEMM (rotation tables, pre-split), and the
-// GEMM's description in *job
-cudaError_t demod3_prepare(const DemodLaunch& L, cudaStream_t st, DemodGemmJob* job);
-// persistent GEMM launch(es) over the jobs' tiles (one per tone-tile width
-// and per 16 plans)
+// GEMM's description in *job (shared_launch: it will run beside other plans')
+cudaError_t demod3_prepare(const DemodLaunch& L, cudaStream_t st, DemodGemmJob* job, bool shared_launch);
+// persistent GEMM launch(es) over the jobs' work items (one per form and per
+// 16 plans)
 cudaError_t demod3_gemm(const DemodGemmJob* const* jobs, int n, int n_sms, cudaStream_t st);
 size_t demod3_xs_rows(int64_t F, int Lpad, int D);
+size_t demod3_scratch_bytes(int n_sms);
 int demod_anchor_rows(int64_t F0, int64_t F);
 
 // -------------------------------------------------------------- chirp
@@ -218,9 +221,10 @@ void plain_release(void* scratch, void* fft_plan, void* blas);
 struct TuneConfig {
     int pfb_lookahead = 0;      // 0 = as many ring super-blocks as shared memory allows
     int demod_raster = 1;       // 1 = tones fastest across the whole grid
-    int demod_bt = 128;         // three-product GEMM: tones per tile (128 or 64)
-    int demod_fused = 0;        // three-product GEMM: pre-split fused into its producers (0/1)
-    int demod_pair = 0;         // three-product GEMM: two-CTA clusters sharing A tiles (0/1)
+    bool demod_auto = true;     // three-product GEMM: form picked per push by size, until one is set:
+    int demod_bt = 128;         //   tones per single-CTA tile (128 or 64)
+    int demod_fused = 0;        //   pre-split fused into its producers (0/1)
+    int demod_pair = 0;         //   two-SM tiles (0/1)
     int pfb_cluster = 0;        // PFB N = 8192, 16384 with T <= 8: cluster kernel (1) or direct (0)
     bool tuned = false;
 };
@@ -279,6 +283,7 @@ struct rfr_plan {
     int accum_chunk = 2;           // demod: K blocks per TMEM accumulation chunk
     int demod_products = 4;        // demod GEMM form: 4 (real embedding) or 3 (Gauss)
     void* d_b3 = nullptr;          // three-product form: six tap planes
+    void* d_g3 = nullptr;          // three-product form: the GEMM's scratch
     void* d_xs3 = nullptr;         // three-product form: six source planes
     int64_t xs3_rows_cap = 0;
     int32_t Lpad3 = 0, ntp3 = 0, tap_exp3 = 0;

@@ -53,11 +53,22 @@ __device__ __forceinline__ void commit(uint64_t* bar) {
                  ::"r"(smem_u32(bar)) : "memory");
 }
 
-// As commit, arriving on the mbarrier at bar's offset in every CTA of the
-// cluster named in cta_mask.
-__device__ __forceinline__ void commit_mc(uint64_t* bar, uint16_t cta_mask) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-                 ::"r"(smem_u32(bar)), "h"(cta_mask) : "memory");
+// The two-SM forms (cta_group::2).  One MMA spans the two CTAs of a cluster
+// pair: each CTA holds its half of A's rows and of B's rows at the same
+// shared-memory offsets and its half of D's rows (all columns) in its own
+// TMEM; one thread of the even-ranked CTA issues for both.
+__device__ __forceinline__ void mma_f16_2sm(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
+                                            uint32_t idesc, uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate));
+}
+// As commit, arriving on the mbarrier at bar's offset in both CTAs.
+__device__ __forceinline__ void commit_2sm(uint64_t* bar) {
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
+                 ::"r"(smem_u32(bar)), "h"(static_cast<uint16_t>(0x3)) : "memory");
 }
 
 __device__ __forceinline__ void fence_before_sync() {
@@ -68,17 +79,30 @@ __device__ __forceinline__ void fence_after_sync() {
 }
 
 // Whole-warp TMEM allocation of `ncols` columns (power of two >= 32); the
-// TMEM address is written to *holder (shared memory).
+// TMEM address is written to *holder (shared memory).  TWO_SM: one warp of
+// each CTA of the pair calls it.
+template <bool TWO_SM = false>
 __device__ __forceinline__ void alloc(uint32_t* holder, uint32_t ncols) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                 ::"r"(smem_u32(holder)), "r"(ncols) : "memory");
+    if constexpr (TWO_SM)
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;"
+                     ::"r"(smem_u32(holder)), "r"(ncols) : "memory");
+    else
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                     ::"r"(smem_u32(holder)), "r"(ncols) : "memory");
 }
+template <bool TWO_SM = false>
 __device__ __forceinline__ void relinquish() {
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    if constexpr (TWO_SM)
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    else
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
 }
+template <bool TWO_SM = false>
 __device__ __forceinline__ void dealloc(uint32_t taddr, uint32_t ncols) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols)
-                 : "memory");
+    if constexpr (TWO_SM)
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
+    else
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
 
 // 32 lanes x 32 consecutive 32-bit columns: thread i of the warp receives
