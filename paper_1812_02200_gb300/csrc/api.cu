@@ -220,16 +220,6 @@ rfr_status ensure_demod_scratch(rfr_plan* p, int64_t F, int64_t F0, cudaStream_t
     return RFR_OK;
 }
 
-// Oversampled N = 4096 PFB as phase passes.  With hop H = N/R, frame
-// j = R*i + k of the push starts at view sample i*N + k*H, so the frames of
-// phase k are the critically sampled PFB of the view shifted by k*H samples
-// (one fused-kernel launch), written to full rows fo + k + R*i (row pitch
-// R*ld) and tone columns fo + k + R*i (column stride R).  The channel phase
-// of the absolute time origin is exp(-2*pi*i*c*s/N) with s = (a0 + k*H) mod N
-// a multiple of H, i.e. (-i)^(c*m) with m = s/H (R = 4) or (-1)^(c*m)
-// (R = 2): an exact swap/negation of each bin, applied by the kernel.  A
-// push that is not 16-byte aligned (or whose carry is not a multiple of 4
-// samples) first copies [carry | buffer] into one aligned scratch view.
 // Rows for the tones of every phase pass of a push of F frames: R x tones
 // rows of ceil(F / R) frames, rounded up to an even count (the tone tile's
 // TMA stores need 16-byte row pitches).  Grows outside stream capture only.
@@ -252,31 +242,18 @@ cudaError_t ensure_pass_tones(rfr_plan* p, int64_t F, cudaStream_t st) {
     return e;
 }
 
+// Oversampled N = 4096 PFB as phase passes.  With hop H = N/R, frame
+// j = R*i + k of the push starts at view sample i*N + k*H, so the frames of
+// phase k are the critically sampled PFB of the view shifted by k*H samples
+// (one fused-kernel launch), written to full rows fo + k + R*i (row pitch
+// R*ld) and tone columns fo + k + R*i (column stride R).  The channel phase
+// of the absolute time origin is exp(-2*pi*i*c*s/N) with s = (a0 + k*H) mod N
+// a multiple of H, i.e. (-i)^(c*m) with m = s/H (R = 4) or (-1)^(c*m)
+// (R = 2): an exact swap/negation of each bin, applied by the kernel.
 rfr_status phase_passes(rfr_plan* p, const rfr::PfbLaunch& L0, const rfr_output* o, int64_t lv, int64_t F,
                         cudaStream_t st) {
     const int R = p->phase_R;
     const int64_t H = p->H, N = p->N;
-    const int16_t* vcarry = L0.carry;
-    const int16_t* vbuf = L0.buf;
-    int64_t vcl = L0.cl;
-    const bool aligned = (reinterpret_cast<uintptr_t>(L0.buf) % 16 == 0) && (L0.cl % 4 == 0) &&
-                         (reinterpret_cast<uintptr_t>(L0.carry) % 16 == 0);
-    if (!aligned) {
-        if (lv > p->view_cap) {
-            const rfr_status rs = refuse_growth_in_capture(p, st);
-            if (rs != RFR_OK) return rs;
-            cudaDeviceSynchronize();
-            dev_free(p->d_view);
-            p->d_view = nullptr;
-            p->view_cap = 0;
-            RFR_CUDA(p, dev_alloc(&p->d_view, static_cast<size_t>(lv) * 4));
-            p->view_cap = lv;
-        }
-        RFR_CUDA(p, rfr::carry_update(L0.carry, L0.cl, L0.buf, L0.n, 0, lv, p->d_view, st));
-        vcarry = p->d_view;
-        vbuf = p->d_view;
-        vcl = 0;
-    }
     // each pass writes its tones as dense rows [k][tone][i] through the tone
     // tile's TMA stores; one kernel then interleaves them into [tone][frame]
     // (written at a column stride of R, each 32-byte sector of a tone row
@@ -293,14 +270,12 @@ rfr_status phase_passes(rfr_plan* p, const rfr::PfbLaunch& L0, const rfr_output*
         if (Fk <= 0) continue;
         const int64_t off = k * H;
         rfr::PfbLaunch L = L0;
-        if (off < vcl) {
-            L.carry = vcarry + 2 * off;
-            L.cl = vcl - off;
-            L.buf = vbuf;
+        if (off < L0.cl) {
+            L.carry = L0.carry + 2 * off;
+            L.cl = L0.cl - off;
         } else {
-            L.carry = vcarry;
             L.cl = 0;
-            L.buf = vbuf + 2 * (off - vcl);
+            L.buf = L0.buf + 2 * (off - L0.cl);
         }
         L.n = (lv - off) - L.cl;
         L.F = Fk;
@@ -363,7 +338,8 @@ rfr_status ensure_scratch(rfr_plan* p, int64_t n) {
     // later pushes of up to n samples never allocate (nor synchronise)
     const int64_t F = frames_for_len(p, std::max<int64_t>(p->cl, p->W - 1) + n);
     if (p->mode == RFR_MODE_PFB && p->gen && F > 0) RFR_CUDA(p, rfr::gen_plan_reserve(&p->gplan, F));
-    if (p->mode == RFR_MODE_PFB && (p->phase_R > 1 || (!p->gen && rfr::pfb_split16(p->log2n, p->Tk)))) {
+    if (p->mode == RFR_MODE_PFB && p->phase_R > 1) RFR_CUDA(p, ensure_pass_tones(p, F, nullptr));
+    if (p->mode == RFR_MODE_PFB && !p->gen && p->phase_R == 1 && rfr::pfb_split16(p->log2n, p->Tk)) {
         const int64_t lv = std::max<int64_t>(p->cl, p->W - 1) + n;
         if (lv > p->view_cap) {
             cudaDeviceSynchronize();
@@ -373,7 +349,6 @@ rfr_status ensure_scratch(rfr_plan* p, int64_t n) {
             RFR_CUDA(p, dev_alloc(&p->d_view, static_cast<size_t>(lv) * 4));
             p->view_cap = lv;
         }
-        if (p->phase_R > 1) RFR_CUDA(p, ensure_pass_tones(p, F, nullptr));
     }
     if (p->mode == RFR_MODE_PFB && !p->gen && p->phase_R == 1 && rfr::pfb_pre_rows(p->log2n, p->Tk)) {
         const rfr_status rs = ensure_pre_rows(p, F, nullptr);

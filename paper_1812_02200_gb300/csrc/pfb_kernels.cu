@@ -15,9 +15,9 @@
 //  TMEM   (N = 4096, T <= 8, 16-byte aligned pushes): the FP32 delay line in
 //         tensor memory, int16 blocks by 1-D TMA, spectrum rows by TMA bulk
 //         stores and tone groups by 2-D TMA tensor stores (see below); the
-//         symmetric-tap form (exactly symmetric taps, the plan default) pairs
-//         mirrored rows per lane pair and also runs the phase passes of
-//         oversampled plans; a seeded form continues FIR sums from pre-sum
+//         symmetric-tap form (T = 8, exactly symmetric taps, the plan default;
+//         pushes of any alignment) works on two frames at a time with two
+//         groups of warps and also runs the phase passes of oversampled plans; a seeded form continues FIR sums from pre-sum
 //         rows (N = 4096 with 9..16 taps: first-half pass + taps 8..15).
 //  RING   (N <= 4096, T <= 8 after padding): each CTA owns a contiguous run
 //         of "super-blocks" (4096 samples = G = 4096/N frames' worth of new
@@ -39,6 +39,7 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cstdio>
 #include <cstring>
 
@@ -536,320 +537,391 @@ __global__ void __launch_bounds__(kRingThreads, 1)
 // ------------------------------------------------- TMEM, symmetric taps
 // N = 4096, T = 8 with an exactly symmetric prototype, h[j] = h[8N - 1 - j]
 // (the plan builds it so).  Same stream view, TMEM delay line, sum order
-// and outputs as pfb_tmem_kernel (bit-identical results), arranged so that
-// a frame costs two CTA barriers instead of three and no twiddle traffic
-// through shared memory:
-//   - Lanes l and 31 - l of a warp own the mirrored FFT rows tf and 255 - tf
-//     (row tf = the points tf + 256 r).  A thread filters its row's points
-//     r < 8 and the mirror points (255 - tf, 15 - r), whose taps are the same
-//     values in reverse tap order, so it holds 64 tap registers instead of
+// and outputs as pfb_tmem_kernel (bit-identical results), for any alignment of
+// the push.
+//
+// What bounds it: one frame at a time on 8 warps (all that 247 registers a
+// thread leave room for) kept the issue slots 44 % busy, every pass exposing
+// the latency of its shared-memory and TMEM reads.  Two groups of 8 warps
+// therefore work on different frames: the FIR group converts the newest block,
+// filters frame j + 1 and runs its first radix-16 pass while the FFT group
+// runs the other two passes and the outputs of frame j.  The groups' shares
+// are about equal (some 400 instructions per 16 points each) and each keeps
+// only its own constants in registers (152 and 104 a thread):
+//   - FIR group.  Lanes l and 31 - l of a warp own the mirrored FFT rows tf and
+//     255 - tf (row tf = the points tf + 256 r).  A thread filters its row's
+//     points r < 8 and the mirror points (255 - tf, 15 - r), whose taps are the
+//     same values in reverse tap order, so it holds 64 tap registers instead of
 //     128; one warp shuffle per value then swaps the mirrored halves so that
-//     every thread has its whole row for the first radix-16 pass.
-//   - The 2 x 15 twiddles of passes 1 and 2 depend only on the row: they
-//     live in registers.
-//   - Three exchange buffers: pass 0 writes B0, pass 1 B1, pass 2 writes the
-//     spectrum to B2 (natural order).  The spectrum of frame j is stored (TMA
-//     bulk) and its tones gathered while pass 1 of frame j + 1 runs, so the
-//     iteration has one barrier after pass 0 and one after pass 1.
-constexpr size_t kSymXb = static_cast<size_t>(4096 + 256) * 8;
+//     every thread has its whole row for the first radix-16 pass.  No thread
+//     reads another's delay line, so the group needs no barrier of its own.
+//   - FFT group.  Warp w takes columns k = 2w, 2w + 1 of pass 1's 256 x 16 view
+//     of the frame (lane: k's low bit and the row a within 16): the 16 x 16
+//     exchange between passes 1 and 2 then stays within the warp, and goes
+//     back in place into the elements the warp alone has read.  So a frame
+//     has one barrier of the group, behind the spectrum (B2, two buffers),
+//     whose TMA row store and tone gather run into the next frame.  Pass 2's
+//     15 twiddles depend only on the thread and live in registers; pass 1's
+//     15 x 16 come from shared memory.
+//   - Between the groups two pass-0 buffers (B0) with full / empty mbarriers.
+// Every buffer is 256 rows of 16 points (128 bytes) whose 16-byte pairs are
+// permuted by XOR with the row mod 8 (the 128-byte swizzle of TMA, which undoes
+// it in the row store): no pattern of the passes meets a bank twice.
+// Staging: a block of the buffer starts anywhere in a 16-byte line, so the
+// bulk copy takes the line it starts in and one line more than 4096 samples
+// when it is not aligned (`mis` samples are skipped); every line copied holds
+// a sample of the block.  The one block across the carry's end is read by
+// plain loads.
+//
+// Measured (full + 1000 tones): 2^28 samples 988 -> 818 us against one group of
+// 8 warps (0.56 -> 0.68 of the HBM copy rate); the hop N/4 plan's four passes
+// and interleave, 2^26 samples, 1312 -> 1134 us; a 2^18-sample push 22.5 -> 16.4
+// us; 3,000,001-sample pushes, tones only, 62 -> 25 us (unaligned ones ran on the
+// ring kernel).  Now the FP32 pipe is 51 % busy, the issue slots 59 % and the
+// shared-memory pipe 59 %.  Register splits of 144 / 112 and 160 / 96 measured
+// 870 and 830 us; one warp refilling the stage always 839; gathering the tones
+// behind the next frame's first loads 897.
+constexpr int kSymThreads = 512;
+constexpr int kSymStage = 3;                       // staging slots
+constexpr int kSymSlotWords = 4096 + 4;
+constexpr int kSymFirRegs = 152, kSymFftRegs = 104, kSymLaunchRegs = 128;
+static_assert(256 * (kSymFirRegs + kSymFftRegs) <= kSymThreads * kSymLaunchRegs, "register split");
+constexpr size_t kSymXb = static_cast<size_t>(4096) * 8;
+__host__ __device__ __forceinline__ int sym_swizzle(int i) { return i ^ (((i >> 4) & 7) << 1); }
 struct SymLayout {
-    size_t b0, b1, b2, bins, tile, bars, total;
+    size_t b2, stage, tw, tile, bars, total;
 };
 __host__ __device__ __forceinline__ SymLayout sym_layout(int nb) {
-    SymLayout L{};
-    L.b0 = static_cast<size_t>(kTmemStage) * 4096 * 4;
-    L.b1 = L.b0 + kSymXb;
-    L.b2 = L.b1 + kSymXb;
-    size_t o = L.b2 + static_cast<size_t>(4096) * 8;
-    L.bins = o;
-    o = (o + static_cast<size_t>(nb) * 4 + 1023) / 1024 * 1024;
+    SymLayout L{};                                                 // two pass-0 buffers at 0
+    L.b2 = 2 * kSymXb;                                             // two spectra
+    L.stage = L.b2 + 2 * kSymXb;
+    L.tw = L.stage + static_cast<size_t>(kSymStage) * kSymSlotWords * 4;   // pass 1's twiddles
+    size_t o = (L.tw + 240 * 8 + 127) / 128 * 128;
     L.tile = o;
     o += static_cast<size_t>((nb + kToneBox - 1) / kToneBox * kToneBox) * kToneGroup * 8;
     L.bars = o;
-    L.total = o + kTmemStage * 8 + 16;
+    L.total = o + (2 * kSymStage + 5) * 8 + 16;
     return L;
 }
 
 template <bool PHASE>
-__global__ void __launch_bounds__(kRingThreads, 1)
-    pfb_tmem_sym_kernel(const PfbArgs a, const __grid_constant__ CUtensorMap tm_tones) {
-    constexpr int N = 4096, NT = 256, T = 8;
+__global__ void __launch_bounds__(kSymThreads, 1)
+    pfb_tmem_sym_kernel(const PfbArgs a, const __grid_constant__ CUtensorMap tm_tones,
+                        const __grid_constant__ CUtensorMap tm_full) {
+    constexpr int N = 4096, NT = 256, T = 8, S = kSymStage;
     // PHASE: a phase pass of an oversampled plan (tone columns a.tone_cs
     // apart, bins turned by (-i)^(c * a.rot)); otherwise adjacent columns, no turn
     const int64_t tcs = PHASE ? a.tone_cs : 1;
     extern __shared__ __align__(1024) unsigned char smem[];
     const int nb_smem = a.nb_smem;
     const SymLayout lay = sym_layout(nb_smem);
-    uint32_t* stage = reinterpret_cast<uint32_t*>(smem);
-    float2* const B0 = reinterpret_cast<float2*>(smem + lay.b0);
-    float2* const B1 = reinterpret_cast<float2*>(smem + lay.b1);
+    float2* const B0 = reinterpret_cast<float2*>(smem);
     float2* const B2 = reinterpret_cast<float2*>(smem + lay.b2);
-    int32_t* sbins = reinterpret_cast<int32_t*>(smem + lay.bins);
-    float2* tile = reinterpret_cast<float2*>(smem + lay.tile);   // tone t, group frame q at t*kToneGroup + q
-    uint64_t* bars = reinterpret_cast<uint64_t*>(smem + lay.bars);
-    uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bars + kTmemStage);
-    volatile int* s_ok = reinterpret_cast<volatile int*>(tmem_holder + 1);
+    uint32_t* const stage = reinterpret_cast<uint32_t*>(smem + lay.stage);
+    float2* const tw1 = reinterpret_cast<float2*>(smem + lay.tw);
+    float2* const tile = reinterpret_cast<float2*>(smem + lay.tile);   // tone t, group frame q at t*kToneGroup + q
+    uint64_t* const sfull = reinterpret_cast<uint64_t*>(smem + lay.bars);
+    uint64_t* const sempty = sfull + S;
+    uint64_t* const b0full = sempty + S;
+    uint64_t* const b0empty = b0full + 2;
+    uint64_t* const tfull = b0empty + 2;                               // tone tile complete
+    uint32_t* const tmem_holder = reinterpret_cast<uint32_t*>(tfull + 1);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int tf = lane < 16 ? 16 * warp + lane : 224 - 16 * warp + lane;   // partner lane 31 - l: 255 - tf
     const int64_t shift = a.frame_offset & (kToneGroup - 1);
     const int64_t ja = max_i64(0, static_cast<int64_t>(blockIdx.x) * a.iters_per_cta - shift);
     const int64_t jb = min_i64(a.F, static_cast<int64_t>(blockIdx.x + 1) * a.iters_per_cta - shift);
     if (ja >= jb) return;
-    const int64_t b0 = ja, b1 = jb + T - 1;                     // blocks [b0, b1)
-    const int64_t need = (a.F + T - 1) * static_cast<int64_t>(N);
+    const int nf = static_cast<int>(jb - ja);                   // frames of this CTA; blocks ja .. ja + nf + T - 2
 
     if (warp == 0) {
         umma::alloc(tmem_holder, 512);
         umma::relinquish();
     }
     if (tid == 0) {
-        for (int s = 0; s < kTmemStage; ++s) mbar_init(&bars[s], 1);
+        for (int s = 0; s < S; ++s) {
+            mbar_init(&sfull[s], 1);
+            mbar_init(&sempty[s], 8);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&b0full[b], 8);
+            mbar_init(&b0empty[b], 8);
+        }
+        mbar_init(tfull, 8);
         fence_mbar_init();
     }
-    for (int i = tid; i < nb_smem; i += blockDim.x) sbins[i] = __ldg(a.bins + i);
-    // taps of the own points (tf, q), q < 8; the mirror point (255-tf, 15-q)
-    // takes tap t from H[T-1-t][q]
-    float H[T][8];
-#pragma unroll
-    for (int t = 0; t < T; ++t)
-#pragma unroll
-        for (int q = 0; q < 8; ++q) H[t][q] = __ldg(a.h + t * N + tf + q * NT);
-    float2 w1[15], w2[15];
-    {
-        const int k = tf & 15;
-#pragma unroll
-        for (int r = 1; r < 16; ++r) {
-            w1[r - 1] = __ldg(a.tw + (r - 1) * 16 + k);
-            w2[r - 1] = __ldg(a.tw + 240 + (r - 1) * 256 + tf);
-        }
-    }
+    for (int i = tid; i < 240; i += kSymThreads) tw1[i] = __ldg(a.tw + i);
     umma::fence_before_sync();
     __syncthreads();
     umma::fence_after_sync();
-    const uint32_t tbase = *tmem_holder + (static_cast<uint32_t>(32 * (warp & 3)) << 16) +
-                           static_cast<uint32_t>(256 * (warp >> 2));
-    if (tid == 0)
-        for (int64_t b = b0; b < min_i64(b0 + kTmemStage, b1); ++b)
-            issue_sb_tma(a, b, need, stage + (b % kTmemStage) * N, &bars[b % kTmemStage]);
 
-    // int16 block b (staging slot s) -> FP32 -> the thread's TMEM columns of
-    // slot b mod 8: points (tf, q) then the mirror points (255-tf, 15-m), as
-    // planar pairs (re_q, re_q+1, im_q, im_q+1)
-    auto ingest = [&](int64_t b, int s) {
-        // the phase completed already (thread 0 saw it before the last
-        // barrier); each thread's own wait makes the copy visible to it
-        mbar_wait(&bars[s], static_cast<uint32_t>(((b - b0) / kTmemStage) & 1), a.status);
-        uint32_t xr[32];
-        const uint32_t* sg = stage + s * N;
-#pragma unroll
-        for (int q = 0; q < 16; q += 2) {
-            const int p0 = q < 8 ? tf + q * NT : 4095 - tf - (q - 8) * NT;
-            const int p1 = q < 8 ? tf + (q + 1) * NT : 4095 - tf - (q - 7) * NT;
-            const float2 f0 = iq_to_f2(sg[p0]);
-            const float2 f1 = iq_to_f2(sg[p1]);
-            xr[2 * q] = __float_as_uint(f0.x);
-            xr[2 * q + 1] = __float_as_uint(f1.x);
-            xr[2 * q + 2] = __float_as_uint(f0.y);
-            xr[2 * q + 3] = __float_as_uint(f1.y);
-        }
-        umma::st_32x32b_x32(tbase + 32u * static_cast<uint32_t>(b % kTmemSlots), xr);
-        umma::wait_st();
-    };
-    auto stage_parity = [&](int64_t b) { return static_cast<uint32_t>(((b - b0) / kTmemStage) & 1); };
-
-    // warm-up: the T - 1 blocks before the first frame's last one
-    bool ok = true;
-    for (int64_t b = b0; b < b0 + T - 1; ++b) {
-        const int s = static_cast<int>(b % kTmemStage);
-        const bool got = mbar_wait(&bars[s], stage_parity(b), a.status);
-        if (__syncthreads_or(!got)) {
-            ok = false;
-            break;
-        }
-        ingest(b, s);
-        __syncthreads();                                         // staging slot s read by all
-        if (tid == 0 && b + kTmemStage < b1)
-            issue_sb_tma(a, b + kTmemStage, need, stage + s * N, &bars[s]);
-    }
-    if (ok) {
-        if (tid == 0) *s_ok = mbar_wait(&bars[(b0 + T - 1) % kTmemStage], stage_parity(b0 + T - 1), a.status) ? 1 : 0;
-        __syncthreads();
-        ok = *s_ok != 0;
-    }
-    const bool bulk = a.full_bulk != 0;
-    int64_t jp = -1;                                             // frame whose spectrum is in B2
-    // stores and gathers the spectrum of frame jp (in B2) into the tone tile
-    auto gather = [&](int64_t j) {
-        if (bulk && tid == 0) {
-            tma_bulk_s2g(a.full + (a.frame_offset + j) * a.full_ld, B2, N * 8);
-            bulk_commit();
-        }
-        if (nb_smem > 0) {
-            const int q = static_cast<int>((a.frame_offset + j) & (kToneGroup - 1));
-            int bk[kTonesPerThread];
-#pragma unroll
-            for (int k = 0; k < kTonesPerThread; ++k) bk[k] = tid + k * NT < nb_smem ? sbins[tid + k * NT] : -1;
-            float2 tv[kTonesPerThread];
-#pragma unroll
-            for (int k = 0; k < kTonesPerThread; ++k)
-                if (bk[k] >= 0) tv[k] = B2[bk[k]];
-#pragma unroll
-            for (int k = 0; k < kTonesPerThread; ++k)
-                if (bk[k] >= 0) tile[(tid + k * NT) * kToneGroup + q] = tv[k];
-        } else if (a.n_tones > 0) {
-            float2* col = a.tones + (a.frame_offset + j) * tcs;
-            for (int t = tid; t < a.n_tones; t += NT) col[t * a.tones_ld] = B2[__ldg(a.bins + t)];
-        }
-    };
-    // group of frame j complete (last of a tone group or of the CTA's range)?
-    auto closes_group = [&](int64_t j) {
-        return nb_smem > 0 && ((((a.frame_offset + j) & (kToneGroup - 1)) == kToneGroup - 1) || j == jb - 1);
-    };
-    auto tile_by_tma = [&](int64_t j) {
-        const int q = static_cast<int>((a.frame_offset + j) & (kToneGroup - 1));
-        return a.tones_tma && q == kToneGroup - 1 && j - q >= ja;
-    };
-    // writes the tone group that frame j closed (after a barrier that
-    // follows every thread's gather)
-    auto flush_group = [&](int64_t j) {
-        const int q = static_cast<int>((a.frame_offset + j) & (kToneGroup - 1));
-        if (tile_by_tma(j)) {
-            if (tid == 0) {
-                const int32_t x0 = static_cast<int32_t>(a.frame_offset + j - q);
-                for (int r0 = 0; r0 < nb_smem; r0 += kToneBox)
-                    tma_store_2d(&tm_tones, x0, r0, tile + static_cast<size_t>(r0) * kToneGroup);
-                bulk_commit();
-            }
-        } else {
-            // frames j - q .. j of the group that this CTA produced
-            const int q0 = static_cast<int>(max_i64(0, ja - (j - q)));
-            const int nq = q + 1 - q0;
-            float2* base = a.tones + (a.frame_offset + (j - q)) * tcs;
-            for (int it = tid; it < nq * nb_smem; it += NT) {
-                const int t = it / nq, qq = q0 + (it - t * nq);
-                base[static_cast<int64_t>(t) * a.tones_ld + qq * tcs] = tile[t * kToneGroup + qq];
-            }
-        }
+    // A thread whose bounded wait gave up goes on without waiting (on whatever
+    // its buffers hold), so that no barrier misses an arrival; the status word
+    // tells the host.
+    bool dead = false;
+    auto wait = [&](uint64_t* bar, uint32_t parity) {
+        if (!dead && !mbar_wait(bar, parity, a.status)) dead = true;
     };
 
-    for (int64_t j = ja; ok && j < jb; ++j) {
-        const int64_t b = j + T - 1;                             // the block that completes frame j
-        const int s = static_cast<int>(b % kTmemStage);
-        ingest(b, s);
-        // polyphase FIR, taps in order t = 0..T-1 (slot halves: own points,
-        // then mirror points, the next load in flight during the FMAs)
-        float are[16], aim[16];
-#pragma unroll
-        for (int r = 0; r < 16; ++r) are[r] = aim[r] = 0.f;
-        uint32_t xa[16], xb[16];
-        umma::ld_32x32b_x16(tbase + 32u * static_cast<uint32_t>(j % kTmemSlots), xa);
-        umma::wait_ld_regs(xa);
-#pragma unroll
-        for (int t = 0; t < T; ++t) {
-            const uint32_t col = tbase + 32u * static_cast<uint32_t>((j + t) % kTmemSlots);
-            umma::ld_32x32b_x16(col + 16u, xb);
-#pragma unroll
-            for (int q = 0; q < 8; q += 2) {
-                ffma2(are[q], are[q + 1], H[t][q], H[t][q + 1], __uint_as_float(xa[2 * q]),
-                      __uint_as_float(xa[2 * q + 1]));
-                ffma2(aim[q], aim[q + 1], H[t][q], H[t][q + 1], __uint_as_float(xa[2 * q + 2]),
-                      __uint_as_float(xa[2 * q + 3]));
+    if (warp < 8) {
+        // ------------------------------------------------ FIR group
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kSymFirRegs));
+        const int tf = lane < 16 ? 16 * warp + lane : 224 - 16 * warp + lane;   // partner lane 31 - l: 255 - tf
+        const uint32_t tbase = *tmem_holder + (static_cast<uint32_t>(32 * (warp & 3)) << 16) +
+                               static_cast<uint32_t>(256 * (warp >> 2));
+        // samples skipped at the start of a buffer block's first 16-byte line
+        const int mis = static_cast<int>((reinterpret_cast<uintptr_t>(a.buf) / 4 - static_cast<uintptr_t>(a.cl)) & 3);
+        // blocks wholly in the carry: [0, c_lo); across its end: c_lo if c_lo < c_hi; the rest in the buffer
+        const int64_t c_lo = a.cl > 0 ? a.cl / N : 0, c_hi = a.cl > 0 ? (a.cl + N - 1) / N : 0;
+        auto issue = [&](int i) {                               // block i of the CTA into slot i mod S (one thread)
+            const int64_t b = ja + i;
+            const int s = i % S;
+            uint32_t* dst = stage + s * kSymSlotWords;
+            if (b < c_lo) {
+                mbar_arrive_expect_tx(&sfull[s], N * 4);
+                tma_bulk_g2s(dst, a.carry + b * N, N * 4, &sfull[s]);
+            } else if (b < c_hi) {
+                mbar_arrive(&sfull[s]);
+            } else {
+                const uint32_t bytes = (mis ? kSymSlotWords : N) * 4;
+                mbar_arrive_expect_tx(&sfull[s], bytes);
+                tma_bulk_g2s(dst, a.buf + (b * N - a.cl) - mis, bytes, &sfull[s]);
             }
-            umma::wait_ld_regs(xb);
-            if (t + 1 < T)
-                umma::ld_32x32b_x16(tbase + 32u * static_cast<uint32_t>((j + t + 1) % kTmemSlots), xa);
+        };
+        if (tid == 0)
+            for (int i = 0; i < min(S, nf + T - 1); ++i) issue(i);
+        // taps of the own points (tf, q), q < 8; the mirror point (255-tf, 15-q)
+        // takes tap t from H[T-1-t][q]
+        float H[T][8];
 #pragma unroll
-            for (int m = 0; m < 8; m += 2) {
-                ffma2(are[8 + m], are[9 + m], H[T - 1 - t][m], H[T - 1 - t][m + 1], __uint_as_float(xb[2 * m]),
-                      __uint_as_float(xb[2 * m + 1]));
-                ffma2(aim[8 + m], aim[9 + m], H[T - 1 - t][m], H[T - 1 - t][m + 1],
-                      __uint_as_float(xb[2 * m + 2]), __uint_as_float(xb[2 * m + 3]));
+        for (int t = 0; t < T; ++t)
+#pragma unroll
+            for (int q = 0; q < 8; ++q) H[t][q] = __ldg(a.h + t * N + tf + q * NT);
+
+#pragma unroll 1
+        for (int i = 0; i < nf + T - 1; ++i) {
+            const int s = i % S;
+            wait(&sfull[s], (i / S) & 1);
+            // int16 block i -> FP32 -> the thread's TMEM columns of slot i mod 8:
+            // points (tf, q) then the mirror points (255-tf, 15-m), as planar
+            // pairs (re_q, re_q+1, im_q, im_q+1)
+            {
+                uint32_t xr[32];
+                const int64_t b = ja + i;
+                auto convert = [&](auto&& at) {
+#pragma unroll
+                    for (int q = 0; q < 16; q += 2) {
+                        const int p0 = q < 8 ? tf + q * NT : 4095 - tf - (q - 8) * NT;
+                        const int p1 = q < 8 ? tf + (q + 1) * NT : 4095 - tf - (q - 7) * NT;
+                        const float2 f0 = iq_to_f2(at(p0));
+                        const float2 f1 = iq_to_f2(at(p1));
+                        xr[2 * q] = __float_as_uint(f0.x);
+                        xr[2 * q + 1] = __float_as_uint(f1.x);
+                        xr[2 * q + 2] = __float_as_uint(f0.y);
+                        xr[2 * q + 3] = __float_as_uint(f1.y);
+                    }
+                };
+                if (b >= c_lo && b < c_hi) {
+                    convert([&](int p) { return vload(a, b * N + p); });
+                } else {
+                    const uint32_t* sg = stage + s * kSymSlotWords + (b >= c_hi ? mis : 0);
+                    convert([&](int p) { return sg[p]; });
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&sempty[s]);          // the slot has been read
+                umma::st_32x32b_x32(tbase + 32u * static_cast<uint32_t>(i & (kTmemSlots - 1)), xr);
+                umma::wait_st();
             }
-            if (t + 1 < T) umma::wait_ld_regs(xa);
+            // refill the slot of the block before (read by all warps by now, or
+            // soon), the warps in turn: always the same one fell behind the rest
+            if (warp == (i & 7) && lane == 0 && i >= 1 && i - 1 + S < nf + T - 1) {
+                wait(&sempty[(i - 1) % S], ((i - 1) / S) & 1);
+                issue(i - 1 + S);
+            }
+            __syncwarp();
+            const int f = i - (T - 1);                           // frame completed by block i
+            if (f < 0) continue;
+            // polyphase FIR, taps in order t = 0..T-1 (slot halves: own points,
+            // then mirror points, the next load in flight during the FMAs)
+            float are[16], aim[16];
+#pragma unroll
+            for (int r = 0; r < 16; ++r) are[r] = aim[r] = 0.f;
+            uint32_t xa[16], xb[16];
+            umma::ld_32x32b_x16(tbase + 32u * static_cast<uint32_t>(f & (kTmemSlots - 1)), xa);
+            umma::wait_ld_regs(xa);
+#pragma unroll
+            for (int t = 0; t < T; ++t) {
+                const uint32_t col = tbase + 32u * static_cast<uint32_t>((f + t) & (kTmemSlots - 1));
+                umma::ld_32x32b_x16(col + 16u, xb);
+#pragma unroll
+                for (int q = 0; q < 8; q += 2) {
+                    ffma2(are[q], are[q + 1], H[t][q], H[t][q + 1], __uint_as_float(xa[2 * q]),
+                          __uint_as_float(xa[2 * q + 1]));
+                    ffma2(aim[q], aim[q + 1], H[t][q], H[t][q + 1], __uint_as_float(xa[2 * q + 2]),
+                          __uint_as_float(xa[2 * q + 3]));
+                }
+                umma::wait_ld_regs(xb);
+                if (t + 1 < T)
+                    umma::ld_32x32b_x16(tbase + 32u * static_cast<uint32_t>((f + t + 1) & (kTmemSlots - 1)), xa);
+#pragma unroll
+                for (int m = 0; m < 8; m += 2) {
+                    ffma2(are[8 + m], are[9 + m], H[T - 1 - t][m], H[T - 1 - t][m + 1], __uint_as_float(xb[2 * m]),
+                          __uint_as_float(xb[2 * m + 1]));
+                    ffma2(aim[8 + m], aim[9 + m], H[T - 1 - t][m], H[T - 1 - t][m + 1],
+                          __uint_as_float(xb[2 * m + 2]), __uint_as_float(xb[2 * m + 3]));
+                }
+                if (t + 1 < T) umma::wait_ld_regs(xa);
+            }
+            // the partner (lane 31 - l) filtered this row's points 8..15
+            float2 v[16];
+#pragma unroll
+            for (int r = 0; r < 8; ++r) v[r] = make_float2(are[r], aim[r]);
+#pragma unroll
+            for (int m = 0; m < 8; ++m)
+                v[15 - m] = make_float2(__shfl_xor_sync(0xffffffffu, are[8 + m], 31),
+                                        __shfl_xor_sync(0xffffffffu, aim[8 + m], 31));
+            dft16(v);                                            // pass 0
+            float4* const P = reinterpret_cast<float4*>(B0 + (f & 1) * N + 16 * tf);   // row tf
+            wait(&b0empty[f & 1], ((f >> 1) & 1) ^ 1);
+#pragma unroll
+            for (int r = 0; r < 16; r += 2) P[(r / 2) ^ (tf & 7)] = make_float4(v[r].x, v[r].y, v[r + 1].x, v[r + 1].y);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&b0full[f & 1]);
         }
-        // the partner (lane 31 - l) filtered this row's points 8..15
+    } else {
+        // ------------------------------------------------ FFT group
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kSymFftRegs));
+        const int tg = tid - 256;                               // thread of the group
+        const int w = warp - 8, row = lane >> 1, k = 2 * w + (lane & 1);
+        auto group_sync = [] { asm volatile("bar.sync 1, 256;" ::: "memory"); };
+        // own element of rows `row` + 16 r; the exchange's places (see below)
+        const int own = sym_swizzle(16 * row + k);
+        const int back = 256 * row + ((row & 7) * 18 ^ k);      // + XOR with 18 (a & 7) + 16 (a & 8)
+        float2 w2[15];
+#pragma unroll
+        for (int r = 1; r < 16; ++r) w2[r - 1] = __ldg(a.tw + 240 + (r - 1) * 256 + 16 * row + k);
+        const bool bulk = a.full_bulk != 0;
+        // output frame of the CTA's frame f, and its place in its tone group
+        const int64_t o0 = a.frame_offset + ja;
+        auto place = [&](int f) { return static_cast<int>((o0 + f) & (kToneGroup - 1)); };
+        // group of frame f complete (last of a tone group or of the CTA's range)?
+        auto closes_group = [&](int f) { return nb_smem > 0 && (place(f) == kToneGroup - 1 || f == nf - 1); };
+        uint32_t closed = 0;                                     // groups flushed
+        // writes the tone group that frame f closed, once every warp has gathered it
+        auto flush_group = [&](int f) {
+            const int q = place(f);
+            if (a.tones_tma && q == kToneGroup - 1 && f >= q) {
+                if (tg == 0) {
+                    wait(tfull, closed & 1);
+                    const int32_t x0 = static_cast<int32_t>(o0 + f - q);
+                    for (int r0 = 0; r0 < nb_smem; r0 += kToneBox)
+                        tma_store_2d(&tm_tones, x0, r0, tile + static_cast<size_t>(r0) * kToneGroup);
+                    bulk_commit();
+                }
+            } else {
+                // frames f - q .. f of the group that this CTA produced
+                wait(tfull, closed & 1);
+                const int q0 = max(0, q - f);
+                const int nq = q + 1 - q0;
+                float2* base = a.tones + (o0 + f - q) * tcs;
+                for (int it = tg; it < nq * nb_smem; it += NT) {
+                    const int t = it / nq, qq = q0 + (it - t * nq);
+                    base[static_cast<int64_t>(t) * a.tones_ld + qq * tcs] = tile[t * kToneGroup + qq];
+                }
+            }
+            ++closed;
+        };
+        // places of the thread's tones tg + 256 i in the spectrum buffer (0xffff: none), two to a register
+        uint32_t bk2[(kTonesPerThread + 1) / 2];
+#pragma unroll
+        for (int i = 0; i < kTonesPerThread + 1; i += 2) {
+            auto at = [&](int t) { return t < nb_smem ? static_cast<uint32_t>(sym_swizzle(__ldg(a.bins + t))) : 0xffffu; };
+            bk2[i / 2] = at(tg + i * NT) | ((i + 1 < kTonesPerThread ? at(tg + (i + 1) * NT) : 0xffffu) << 16);
+        }
         float2 v[16];
+#pragma unroll 1
+        for (int f = 0; f < nf; ++f) {
+            // pass 1: rows row + 16 r of column k
+            const int pown = (f & 1) * static_cast<int>(kSymXb) + own * 8, pback = (f & 1) * static_cast<int>(kSymXb) + back * 8;
+            auto at = [&](int byte) -> float2& { return *reinterpret_cast<float2*>(smem + byte); };   // B0 is at 0
+            wait(&b0full[f & 1], (f >> 1) & 1);
 #pragma unroll
-        for (int r = 0; r < 8; ++r) v[r] = make_float2(are[r], aim[r]);
+            for (int r = 0; r < 16; ++r) v[r] = at(pown + r * NT * 8);
 #pragma unroll
-        for (int m = 0; m < 8; ++m)
-            v[15 - m] = make_float2(__shfl_xor_sync(0xffffffffu, are[8 + m], 31),
-                                    __shfl_xor_sync(0xffffffffu, aim[8 + m], 31));
-        // pass 0 -> B0
-        dft16(v);
-#pragma unroll
-        for (int r = 0; r < 16; ++r) B0[fpad(16 * tf + r)] = v[r];
-        if (tid == 0) bulk_wait_read_all();                     // tile stores done reading the tile
-        __syncthreads();                                         // (1) B0 written, staging slot s read
-        if (tid == 0 && b + kTmemStage < b1)
-            issue_sb_tma(a, b + kTmemStage, need, stage + s * N, &bars[s]);
-        // outputs of the previous frame while pass 1 of this one runs
-        if (jp >= 0) gather(jp);
-        {
-            const int k = tf & 15;
-#pragma unroll
-            for (int r = 0; r < 16; ++r) v[r] = B0[fpad(tf + r * NT)];
-#pragma unroll
-            for (int r = 1; r < 16; ++r) v[r] = cmul(v[r], w1[r - 1]);
+            for (int r = 1; r < 16; ++r) v[r] = cmul(v[r], tw1[(r - 1) * 16 + k]);
             dft16(v);
-            const int base = (tf >> 4) * 256 + k;
+            // exchange within the warp, in place: output r of thread `row` goes to
+            // row 16 r + (row ^ (r & 7)) of column k, where thread r finds it
+            __syncwarp();
 #pragma unroll
-            for (int r = 0; r < 16; ++r) B1[fpad(base + r * 16)] = v[r];
-        }
-        const bool close_prev = jp >= 0 && closes_group(jp);
-        if (close_prev && tile_by_tma(jp)) fence_proxy_async_smem();
-        if (tid == 0) {
-            bulk_wait_read_all();                                // B2 read by its row store
-            *s_ok = (j + 1 < jb) ? (mbar_wait(&bars[(b + 1) % kTmemStage], stage_parity(b + 1), a.status) ? 1 : 0) : 1;
-        }
-        __syncthreads();                                         // (2) B1 written, gathers done
-        if (close_prev) flush_group(jp);
-        {
+            for (int r = 0; r < 16; ++r) at((pown ^ (8 * 18 * (r & 7))) + r * NT * 8) = v[r];
+            __syncwarp();
 #pragma unroll
-            for (int r = 0; r < 16; ++r) v[r] = B1[fpad(tf + r * NT)];
+            for (int r = 0; r < 16; ++r) v[r] = at(pback ^ (8 * (18 * (r & 7) + 16 * (r & 8))));
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&b0empty[f & 1]);
+            if (f > 0 && closes_group(f - 1)) flush_group(f - 1);
+            // pass 2: v[r] = bin 16 row + k + 256 r
 #pragma unroll
             for (int r = 1; r < 16; ++r) v[r] = cmul(v[r], w2[r - 1]);
-            dft16(v);                                            // v[r] = bin tf + 256 r
-        }
-        if (PHASE && a.rot) {
-            // (-i)^e, e = (c * rot) mod 4 for c = tf + 256 r: the same power for
-            // all r, and it differs between the lanes of a warp, so it is applied
-            // without branches: odd e swaps re and im, then sign bits are flipped
-            // (e = 1: (im, -re); 2: (-re, -im); 3: (-im, re)); exact
-            const int e = (tf * a.rot) & 3;
-            const bool sw = (e & 1) != 0;
-            const uint32_t m_re = (e == 2 || e == 3) ? 0x80000000u : 0u;
-            const uint32_t m_im = (e == 1 || e == 2) ? 0x80000000u : 0u;
+            dft16(v);
+            if (PHASE && a.rot) {
+                // (-i)^e, e = (c * rot) mod 4 for bin c: the same power for all r,
+                // and it differs between the lanes of a warp, so it is applied
+                // without branches: odd e swaps re and im, then sign bits are flipped
+                // (e = 1: (im, -re); 2: (-re, -im); 3: (-im, re)); exact
+                const int e = (k * a.rot) & 3;
+                const bool sw = (e & 1) != 0;
+                const uint32_t m_re = (e == 2 || e == 3) ? 0x80000000u : 0u;
+                const uint32_t m_im = (e == 1 || e == 2) ? 0x80000000u : 0u;
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                const float2 u = v[i];
-                const float re = sw ? u.y : u.x, im = sw ? u.x : u.y;
-                v[i] = make_float2(__uint_as_float(__float_as_uint(re) ^ m_re), __uint_as_float(__float_as_uint(im) ^ m_im));
+                for (int i = 0; i < 16; ++i) {
+                    const float2 u = v[i];
+                    const float re = sw ? u.y : u.x, im = sw ? u.x : u.y;
+                    v[i] = make_float2(__uint_as_float(__float_as_uint(re) ^ m_re),
+                                       __uint_as_float(__float_as_uint(im) ^ m_im));
+                }
+            }
+            float2* const Y = B2 + (f & 1) * N;
+#pragma unroll
+            for (int i = 0; i < 16; ++i) Y[own + i * NT] = v[i];
+            fence_proxy_async_smem();
+            // the other spectrum and the tile have been read by their stores
+            if (tg == 0) bulk_wait_read_all();
+            group_sync();                                        // spectrum in Y, the frame before gathered
+            if (bulk && tg == 0) {
+                tma_store_3d(&tm_full, 0, 0, static_cast<int32_t>(o0 + f), Y);
+                bulk_commit();
+            }
+            if (a.full && !bulk) {
+                float2* out = a.full + (o0 + f) * a.full_ld;
+#pragma unroll 4
+                for (int i = tg; i < N; i += NT) out[i] = Y[sym_swizzle(i)];
+            }
+            if (nb_smem > 0) {
+                const int q = place(f);
+                float2 tv[kTonesPerThread];
+#pragma unroll
+                for (int i = 0; i < kTonesPerThread; ++i) {
+                    const uint32_t at = (bk2[i / 2] >> (16 * (i & 1))) & 0xffffu;
+                    if (at != 0xffffu) tv[i] = Y[at];
+                }
+#pragma unroll
+                for (int i = 0; i < kTonesPerThread; ++i)
+                    if (((bk2[i / 2] >> (16 * (i & 1))) & 0xffffu) != 0xffffu) tile[(tg + i * NT) * kToneGroup + q] = tv[i];
+                if (closes_group(f)) {
+                    fence_proxy_async_smem();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(tfull);
+                }
+            } else if (a.n_tones > 0) {
+                float2* col = a.tones + (o0 + f) * tcs;
+                for (int t = tg; t < a.n_tones; t += NT) col[t * a.tones_ld] = Y[sym_swizzle(__ldg(a.bins + t))];
             }
         }
-        if (a.full && !bulk) {
-            float2* row = a.full + (a.frame_offset + j) * a.full_ld;
-#pragma unroll
-            for (int i = 0; i < 16; ++i) row[tf + i * NT] = v[i];
-        }
-#pragma unroll
-        for (int i = 0; i < 16; ++i) B2[tf + i * NT] = v[i];
-        fence_proxy_async_smem();
-        jp = j;
-        ok = *s_ok != 0;
+        if (closes_group(nf - 1)) flush_group(nf - 1);
+        if (tg == 0) bulk_wait_all();
     }
-    if (ok && jp >= 0) {
-        if (tid == 0) bulk_wait_read_all();                     // tile stores done reading the tile
-        __syncthreads();                                         // spectrum of the last frame in B2
-        gather(jp);
-        if (closes_group(jp)) {
-            if (tile_by_tma(jp)) fence_proxy_async_smem();
-            __syncthreads();
-            flush_group(jp);
-        }
-    }
-    if (tid == 0) bulk_wait_all();
     umma::fence_before_sync();
     __syncthreads();
     if (warp == 0) {
@@ -1445,15 +1517,32 @@ cudaError_t launch_tmem_sym(PfbArgs a, int n_sms, int max_smem, cudaStream_t st)
     const size_t smem = sym_layout(a.nb_smem).total;
     if (smem > static_cast<size_t>(max_smem)) return cudaErrorInvalidConfiguration;
     const int64_t shift = a.frame_offset & (kToneGroup - 1);
+    // one wave of CTAs; long ranges are whole tone groups (32-byte sectors of
+    // the tone rows), short ones are cut evenly (a push of 64 frames on 64 CTAs
+    // instead of 16)
     const int64_t grid = std::min<int64_t>(a.F, n_sms);
-    a.iters_per_cta = ((a.F + shift + grid - 1) / grid + kToneGroup - 1) / kToneGroup * kToneGroup;
+    a.iters_per_cta = (a.F + shift + grid - 1) / grid;
+    if (a.iters_per_cta >= 4 * kToneGroup) a.iters_per_cta = (a.iters_per_cta + kToneGroup - 1) / kToneGroup * kToneGroup;
     const int64_t grid2 = (a.F + shift + a.iters_per_cta - 1) / a.iters_per_cta;
-    a.full_bulk = (a.full != nullptr && (reinterpret_cast<uintptr_t>(a.full) % 16) == 0 &&
-                   (a.full_ld % 2) == 0) ? 1 : 0;
-    CUtensorMap tm;
+    CUtensorMap tm, tf;
     std::memset(&tm, 0, sizeof tm);
+    std::memset(&tf, 0, sizeof tf);
     a.tones_tma = 0;
     auto enc = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(tmap_encode_tiled_fn());
+    // spectrum rows as [frame][256][16] 8-byte elements, one frame a box, the
+    // kernel's buffers in the 128-byte swizzle
+    a.full_bulk = 0;
+    if (a.full && enc && (reinterpret_cast<uintptr_t>(a.full) % 16) == 0 && (a.full_ld % 2) == 0 &&
+        a.frame_offset + a.F < (int64_t(1) << 31)) {
+        cuuint64_t dims[3] = {16, 256, static_cast<cuuint64_t>(a.frame_offset + a.F)};
+        cuuint64_t strides[2] = {128, static_cast<cuuint64_t>(a.full_ld) * 8};
+        cuuint32_t box[3] = {16, 256, 1};
+        cuuint32_t estr[3] = {1, 1, 1};
+        if (enc(&tf, CU_TENSOR_MAP_DATA_TYPE_UINT64, 3, a.full, dims, strides, box, estr,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS)
+            a.full_bulk = 1;
+    }
     if (a.nb_smem > 0 && enc && a.tone_cs == 1 && (reinterpret_cast<uintptr_t>(a.tones) % 16) == 0 &&
         (a.tones_ld % 2) == 0 && a.frame_offset + a.F < (int64_t(1) << 31)) {
         cuuint64_t dims[2] = {static_cast<cuuint64_t>(a.frame_offset + a.F), static_cast<cuuint64_t>(a.n_tones)};
@@ -1469,7 +1558,18 @@ cudaError_t launch_tmem_sym(PfbArgs a, int n_sms, int max_smem, cudaStream_t st)
     auto k = phase ? pfb_tmem_sym_kernel<true> : pfb_tmem_sym_kernel<false>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k<<<static_cast<unsigned>(grid2), kRingThreads, smem, st>>>(a, tm);
+    // the kernel's register split waits forever unless the launch holds it
+    static std::atomic<int> regs[2];
+    int r = regs[phase ? 1 : 0].load();
+    if (r == 0) {
+        cudaFuncAttributes fa;
+        e = cudaFuncGetAttributes(&fa, k);
+        if (e != cudaSuccess) return e;
+        r = fa.numRegs;
+        regs[phase ? 1 : 0].store(r);
+    }
+    if ((r + 7) / 8 * 8 < kSymLaunchRegs) return cudaErrorInvalidConfiguration;
+    k<<<static_cast<unsigned>(grid2), kSymThreads, smem, st>>>(a, tm, tf);
     return cudaGetLastError();
 }
 
@@ -1636,11 +1736,11 @@ cudaError_t pfb_launch(const PfbLaunch& L, cudaStream_t st) {
     }
     if (a.tone_cs != 1 || a.rot != 0) {
         // phase passes of an oversampled plan: only the symmetric-tap kernel has them
-        if (lg != 12 || !a.use_tma || L.taps_kernel != 8 || !L.sym_taps) return cudaErrorInvalidValue;
+        if (lg != 12 || L.taps_kernel != 8 || !L.sym_taps) return cudaErrorInvalidValue;
         return launch_tmem_sym(a, L.n_sms, L.max_smem, st);
     }
+    if (lg == 12 && L.taps_kernel == 8 && L.sym_taps && L.variant == 0) return launch_tmem_sym(a, L.n_sms, L.max_smem, st);
     if (lg == 12 && a.use_tma && L.variant != 1) {
-        if (L.taps_kernel == 8 && L.sym_taps && L.variant != 2) return launch_tmem_sym(a, L.n_sms, L.max_smem, st);
         if (L.taps_kernel == 4) return launch_tmem<4>(a, L.n_sms, L.max_smem, st);
         if (L.taps_kernel == 8) return launch_tmem<8>(a, L.n_sms, L.max_smem, st);
     }

@@ -246,7 +246,7 @@ struct rfr_plan {
     bool sym_taps = false;                     // PFB kernel taps exactly symmetric (Tk == T)
     int phase_R = 1;                           // oversampled N = 4096 PFB: hop = N / phase_R, run as
                                                // phase_R critically sampled passes (see push_core)
-    int16_t* d_view = nullptr;                 // phase passes: contiguous copy of [carry | buffer]
+    int16_t* d_view = nullptr;                 // 16-tap N = 4096: contiguous copy of [carry | buffer]
     int64_t view_cap = 0;                      //   when the push is not 16-byte aligned (samples)
     void* d_ptones = nullptr;                  // phase passes: each pass's tones [pass][tone][frame]
     int64_t ptones_cap = 0;                    //   frames per pass row
