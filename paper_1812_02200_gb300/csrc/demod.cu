@@ -30,6 +30,7 @@
 //                           samples (the Toeplitz view's 2-D tensor).
 //   gemm        (per push)  TMA -> smem (128B swizzle) -> tcgen05.mma -> TMEM
 //                           -> register sums -> rotation -> [tone][frame] out.
+//   prep3       (per push)  the three-product form's rotation tables and planes
 //   *3 variants             the Gauss three-product form (see below), a plan
 //                           option (rfr_plan_set_demod_products).
 #include <cuda.h>
@@ -412,7 +413,7 @@ demod_gemm_kernel(const __grid_constant__ CUtensorMap tmAh, const __grid_constan
 // the products go to planes in the scratch and combine3_kernel finishes.
 //
 // Fused pre-split (FUSED, single-CTA form): instead of TMA loads of the six
-// pre-split source planes (written to HBM by presplit3_kernel, 12 bytes per
+// pre-split source planes (written to HBM by prep3_kernel, 12 bytes per
 // sample), two producer warps read the int16 stream view [carry | buffer] and
 // write each stage's A hi/lo tiles themselves, in the 128-byte swizzled layout
 // the TMA would produce, with the same FP32 -> FP16 hi/lo rounding as the
@@ -524,20 +525,103 @@ __global__ void build_taps3_kernel(const double* __restrict__ h, const uint64_t*
     }
 }
 
-// Sample s of [carry | buffer] -> the six planes ((xr+xi)/2, xr, xi) x (hi, lo).
-__global__ void presplit3_kernel(const uint32_t* __restrict__ carry, int64_t cl, const uint32_t* __restrict__ buf,
-                                 int64_t lv, int64_t total, __half* __restrict__ planes) {
-    for (int64_t s = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; s < total;
-         s += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        uint32_t w = 0;
-        if (s < lv) w = s < cl ? carry[s] : buf[s - cl];
-        const float2 f = iq_to_f2(w);
-        const float v[3] = {0.5f * (f.x + f.y), f.x, f.y};      // exact in FP32
+// Plane q ((xr+xi)/2, xr or xi; exact in FP32) of two samples -> packed FP16 hi and lo.
+__device__ __forceinline__ void g3_split_pair(uint32_t w0, uint32_t w1, int q, uint32_t& hi, uint32_t& lo) {
+    const float2 f0 = iq_to_f2(w0), f1 = iq_to_f2(w1);
+    const float v0 = q == 0 ? 0.5f * (f0.x + f0.y) : (q == 1 ? f0.x : f0.y);
+    const float v1 = q == 0 ? 0.5f * (f1.x + f1.y) : (q == 1 ? f1.x : f1.y);
+    const __half h0 = __float2half_rn(v0), h1 = __float2half_rn(v1);
+    const __half l0 = __float2half_rn(v0 - __half2float(h0));
+    const __half l1 = __float2half_rn(v1 - __half2float(h1));
+    hi = static_cast<uint32_t>(__half_as_ushort(h0)) | (static_cast<uint32_t>(__half_as_ushort(h1)) << 16);
+    lo = static_cast<uint32_t>(__half_as_ushort(l0)) | (static_cast<uint32_t>(__half_as_ushort(l1)) << 16);
+}
+
+// What a three-product push needs ahead of its GEMM, in one launch: the first
+// rot_blocks blocks write the rotation tables (FP64-bound), the others the six
+// source planes (memory-bound), so the two overlap.
+//   anchors, steps: as rot_kernel, in runs of 8 absolute indices from one exact
+// FP64 evaluation each, the others by FP64 products with the run's step (within
+// 8 x 2^-52 of exact, far inside the FP32 rounding; runs start at absolute
+// multiples of 8, so every push of a stream gets the same values).  FP64 issues
+// one warp instruction in 16 clocks on an SM, so a block takes `rot_items` threads'
+// worth of runs, few enough that all SMs share a small push's.
+//   planes: eight samples s of [carry | buffer] per thread -> ((xr+xi)/2, xr,
+// xi) x (hi, lo), one 16-byte store per plane.
+// Measured: 300 tones x 10^6 samples 47.0 -> 38.6 us a push (two launches, 11.4 us,
+// before); of a push of 2^27 samples x 2048 tones 555 -> 343 us (its bytes: 316).
+constexpr int kRotRun = 8;
+struct Prep3Args {
+    const uint64_t* words;
+    int n_tones, ntp, L, D, n_anch, rot_blocks, rot_items;
+    int64_t A0;                      // first anchor's absolute index
+    float2* anchors;
+    float2* steps;
+    const uint32_t* carry;
+    const uint32_t* buf;
+    int64_t cl, lv, total;           // total: samples of a plane (a multiple of 64); 0: no planes
+    __half* planes;
+};
+__global__ void __launch_bounds__(256) prep3_kernel(const Prep3Args a) {
+    if (static_cast<int>(blockIdx.x) < a.rot_blocks) {
+        const int64_t runs0 = a.A0 / kRotRun;
+        const int64_t n_runs = (a.A0 + a.n_anch - 1) / kRotRun - runs0 + 1;
+        const int64_t na = n_runs * a.ntp, total = na + static_cast<int64_t>(a.ntp) * (BM / kRotRun);
+        if (static_cast<int>(threadIdx.x) >= a.rot_items) return;
+        for (int64_t idx = static_cast<int64_t>(blockIdx.x) * a.rot_items + threadIdx.x; idx < total;
+             idx += static_cast<int64_t>(a.rot_blocks) * a.rot_items) {
+            const bool anchor = idx < na;
+            const int64_t j = anchor ? idx : idx - na;
+            const int t = static_cast<int>(j % a.ntp);
+            const int64_t run = j / a.ntp;                   // of anchors (from runs0) or of steps
+            double c = 0.0, sn = 0.0, dc = 0.0, ds = 0.0;
+            if (t < a.n_tones) {
+                const uint64_t w = a.words[t];
+                const int64_t K = (runs0 + run) * kRotRun * BM;
+                const uint64_t ph = w * static_cast<uint64_t>(anchor ? (K + 1) * a.D - a.L : run * kRotRun * a.D);
+                const uint64_t dp = w * static_cast<uint64_t>(anchor ? static_cast<int64_t>(BM) * a.D : static_cast<int64_t>(a.D));
+                sincospi(static_cast<double>(static_cast<int64_t>(ph)) * 0x1p-63, &sn, &c);
+                sincospi(static_cast<double>(static_cast<int64_t>(dp)) * 0x1p-63, &ds, &dc);
+            }
+#pragma unroll 4
+            for (int i = 0; i < kRotRun; ++i) {
+                const float2 r = make_float2(static_cast<float>(c), static_cast<float>(-sn));
+                if (anchor) {
+                    const int64_t row = (runs0 + run) * kRotRun + i - a.A0;
+                    if (row >= 0 && row < a.n_anch) a.anchors[row * a.ntp + t] = r;
+                } else {
+                    a.steps[static_cast<int64_t>(t) * BM + run * kRotRun + i] = r;
+                }
+                const double nc = fma(c, dc, -sn * ds);
+                sn = fma(c, ds, sn * dc);
+                c = nc;
+            }
+        }
+        return;
+    }
+    const int64_t nb = gridDim.x - a.rot_blocks;
+    for (int64_t g = (blockIdx.x - a.rot_blocks) * 256 + threadIdx.x; g < a.total / 8; g += nb * 256) {
+        const int64_t s0 = g * 8;
+        uint32_t w[8];
+        const uint32_t* bp = a.buf + (s0 - a.cl);
+        if (s0 >= a.cl && s0 + 8 <= a.lv && (reinterpret_cast<uintptr_t>(bp) & 15) == 0) {
+            const uint4 u0 = __ldg(reinterpret_cast<const uint4*>(bp)), u1 = __ldg(reinterpret_cast<const uint4*>(bp) + 1);
+            w[0] = u0.x; w[1] = u0.y; w[2] = u0.z; w[3] = u0.w;
+            w[4] = u1.x; w[5] = u1.y; w[6] = u1.z; w[7] = u1.w;
+        } else {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int64_t s = s0 + e;
+                w[e] = s < a.lv ? (s < a.cl ? __ldg(a.carry + s) : __ldg(a.buf + (s - a.cl))) : 0u;
+            }
+        }
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
-            const __half hv = __float2half_rn(v[q]);
-            planes[(2 * q) * total + s] = hv;
-            planes[(2 * q + 1) * total + s] = __float2half_rn(v[q] - __half2float(hv));
+            uint32_t hi[4], lo[4];
+#pragma unroll
+            for (int e = 0; e < 8; e += 2) g3_split_pair(w[e], w[e + 1], q, hi[e / 2], lo[e / 2]);
+            *reinterpret_cast<uint4*>(a.planes + (2 * q) * a.total + s0) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+            *reinterpret_cast<uint4*>(a.planes + (2 * q + 1) * a.total + s0) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
         }
     }
 }
@@ -567,16 +651,7 @@ __device__ __forceinline__ void g3_fill_row(const G3Plan& P, int q, int64_t s0, 
         }
         uint32_t hi[4], lo[4];
 #pragma unroll
-        for (int e = 0; e < 8; e += 2) {
-            const float2 f0 = iq_to_f2(w[e]), f1 = iq_to_f2(w[e + 1]);
-            const float v0 = q == 0 ? 0.5f * (f0.x + f0.y) : (q == 1 ? f0.x : f0.y);   // exact in FP32
-            const float v1 = q == 0 ? 0.5f * (f1.x + f1.y) : (q == 1 ? f1.x : f1.y);
-            const __half h0 = __float2half_rn(v0), h1 = __float2half_rn(v1);
-            const __half l0 = __float2half_rn(v0 - __half2float(h0));
-            const __half l1 = __float2half_rn(v1 - __half2float(h1));
-            hi[e / 2] = static_cast<uint32_t>(__half_as_ushort(h0)) | (static_cast<uint32_t>(__half_as_ushort(h1)) << 16);
-            lo[e / 2] = static_cast<uint32_t>(__half_as_ushort(l0)) | (static_cast<uint32_t>(__half_as_ushort(l1)) << 16);
-        }
+        for (int e = 0; e < 8; e += 2) g3_split_pair(w[e], w[e + 1], q, hi[e / 2], lo[e / 2]);
         const uint32_t off = static_cast<uint32_t>(i) * 128u + (static_cast<uint32_t>(c ^ (i & 7)) << 4);
         *reinterpret_cast<uint4*>(ahi + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
         *reinterpret_cast<uint4*>(alo + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
@@ -1285,9 +1360,6 @@ cudaError_t demod3_prepare(const DemodLaunch& L, cudaStream_t st, DemodGemmJob* 
     const int n_anch = demod_anchor_rows(L.F0, L.F);
     float2* anchors = static_cast<float2*>(L.rot);
     float2* steps = anchors + static_cast<int64_t>(n_anch) * L.ntp;
-    const int64_t nrot = static_cast<int64_t>(n_anch) * L.ntp + static_cast<int64_t>(L.ntp) * BM;
-    rot_kernel<<<grid_for(nrot, L.n_sms), 256, 0, st>>>(L.words, L.n_tones, L.ntp, L.F0 / BM, L.L, L.D, n_anch,
-                                                         anchors, steps);
     G3Plan* P = reinterpret_cast<G3Plan*>(job->bytes);
     std::memset(P, 0, sizeof(G3Plan));
     const __half* bp = static_cast<const __half*>(L.b_hi);
@@ -1301,11 +1373,29 @@ cudaError_t demod3_prepare(const DemodLaunch& L, cudaStream_t st, DemodGemmJob* 
         P->cl = L.cl;
         P->lv = L.cl + L.n;
         P->vec = (reinterpret_cast<uintptr_t>(L.buf) % 16 == 0) && ((L.cl % 4) + 4) % 4 == 0 ? 1 : 0;
-    } else {
-        presplit3_kernel<<<grid_for(total, L.n_sms), 256, 0, st>>>(
-            reinterpret_cast<const uint32_t*>(L.carry), L.cl, reinterpret_cast<const uint32_t*>(L.buf), L.cl + L.n,
-            total, xp);
     }
+    Prep3Args pa{};
+    pa.words = L.words;
+    pa.n_tones = L.n_tones;
+    pa.ntp = L.ntp;
+    pa.L = L.L;
+    pa.D = L.D;
+    pa.n_anch = n_anch;
+    pa.A0 = L.F0 / BM;
+    pa.anchors = anchors;
+    pa.steps = steps;
+    pa.carry = reinterpret_cast<const uint32_t*>(L.carry);
+    pa.buf = reinterpret_cast<const uint32_t*>(L.buf);
+    pa.cl = L.cl;
+    pa.lv = L.cl + L.n;
+    pa.total = job->fused ? 0 : total;
+    pa.planes = xp;
+    const int64_t rot_items = ((pa.A0 + n_anch - 1) / kRotRun - pa.A0 / kRotRun + 1 + BM / kRotRun) * L.ntp;
+    pa.rot_items = static_cast<int>(std::min<int64_t>(256, (rot_items / (2 * L.n_sms) + 31) / 32 * 32));
+    if (pa.rot_items < 32) pa.rot_items = 32;
+    pa.rot_blocks = static_cast<int>(std::min<int64_t>((rot_items + pa.rot_items - 1) / pa.rot_items, int64_t(L.n_sms) * 8));
+    const unsigned plane_blocks = pa.total ? grid_for(pa.total / 8, L.n_sms) : 0;
+    prep3_kernel<<<pa.rot_blocks + plane_blocks, 256, 0, st>>>(pa);
     const uint32_t b_box = static_cast<uint32_t>(form.pair ? form.bw / 2 : form.bw);
     for (int i = 0; i < 6; ++i) {
         if ((!job->fused && !make_map(&P->a[i], xp + i * total, static_cast<uint64_t>(L.D),
