@@ -242,6 +242,108 @@ __global__ void __launch_bounds__(kChirpThreads) chirp_demod_kernel(const ChirpA
     }
 }
 
+// Overlapping frames (L > D, D a multiple of 256): a sample's mixer value does
+// not depend on the frame, so each is evaluated once for the J = ceil(L / D)
+// frames that use it.  The sine and cosine bound the kernel above (about 40
+// issue slots per evaluation), so this divides its time by almost J.
+//
+// A CTA takes a run of frames on one SM, in segments whose samples fit its
+// shared memory (packed int16, converted at use).  Four workers of 256 threads
+// share a segment: a work item is a chirp over `sub` of the segment's frames,
+// walked block by block (block b: the D samples from v[b D]) with one pair of
+// sums per frame in progress: block b adds taps jD .. jD + D - 1 to frame b - j.
+// A thread's samples are those the kernel above gives it, in the same order,
+// and the reduction is the same, so the frames are bit-identical to its frames.
+// Measured, 2^24 samples, 8 chirps, L = 4096, D = 2048: 467 -> 303 us.
+constexpr int kOvWorkers = 4;
+constexpr int kOvSub = 32;                              // frames per work item at most
+struct ChirpOverlap {
+    int seg, sub;                                       // frames per segment, per work item
+    int64_t per_cta;                                    // frames per CTA
+};
+template <int J, bool FULL>                             // FULL: L == J * D
+__global__ void __launch_bounds__(kOvWorkers * kChirpThreads, 1)
+    chirp_overlap_kernel(const ChirpArgs a, const ChirpOverlap o) {
+    extern __shared__ uint32_t xs32[];                  // [(seg + J - 1) * D]
+    __shared__ double2 red[kOvWorkers][kOvSub][kChirpThreads / 32];
+    const int wk = threadIdx.x / kChirpThreads, tid = threadIdx.x % kChirpThreads;
+    const int warp = tid >> 5, lane = tid & 31;
+    auto worker_sync = [&] { asm volatile("bar.sync %0, 256;" ::"r"(1 + wk) : "memory"); };
+    const int64_t k_end = a.F < (blockIdx.x + 1) * o.per_cta ? a.F : (blockIdx.x + 1) * o.per_cta;
+    for (int64_t k0 = blockIdx.x * o.per_cta; k0 < k_end; k0 += o.seg) {
+        const int seg = static_cast<int>(k_end - k0 < o.seg ? k_end - k0 : o.seg);
+        // the segment's samples: those of its last frame end L - 1 past its start
+        const int need = (seg - 1) * a.D + a.L;
+        __syncthreads();                                // previous segment's readers are done
+        for (int n = threadIdx.x; n < need; n += kOvWorkers * kChirpThreads) {
+            const int64_t vi = k0 * a.D + n;
+            xs32[n] = vi < a.cl ? __ldg(a.carry + vi) : __ldg(a.buf + (vi - a.cl));
+        }
+        __syncthreads();
+        const int subs = (seg + o.sub - 1) / o.sub;
+        for (int item = wk; item < a.n_chirps * subs; item += kOvWorkers) {
+            const int c = item / subs, f0 = (item - c * subs) * o.sub;
+            const int nf = seg - f0 < o.sub ? seg - f0 : o.sub;
+            const uint64_t s = __ldg(a.s + c), r = __ldg(a.r + c);
+            const uint64_t m = static_cast<uint64_t>(a.a0 + (k0 + f0) * a.D + tid);
+            uint64_t p = chirp_phase(s, r, static_cast<int64_t>(m));
+            uint64_t d = s * 256ull + r * (512ull * m + 65536ull);
+            const uint64_t dd = r * 131072ull;
+            float ar[J], ai[J];                          // frame b - j
+#pragma unroll
+            for (int j = 0; j < J; ++j) ar[j] = ai[j] = 0.f;
+            for (int b = 0; b < nf + J - 1; ++b) {
+                const uint32_t* xb = xs32 + (f0 + b) * a.D;
+                const int limit = need - (f0 + b) * a.D;     // samples of the segment from this block on
+                for (int n = tid; n < a.D && (FULL || n < limit); n += kChirpThreads) {
+                    const float2 x = iq_to_f2(xb[n]);
+                    float sn, cs;
+                    sincospif(static_cast<float>(static_cast<int32_t>(p >> 32)) * 0x1p-31f, &sn, &cs);
+                    const float mr = fmaf(x.x, cs, x.y * sn), mi = fmaf(x.y, cs, -x.x * sn);
+#pragma unroll
+                    for (int j = 0; j < J; ++j) {
+                        if (FULL || j * a.D + n < a.L) {
+                            const float hn = __ldg(a.h + j * a.D + n);
+                            ar[j] = fmaf(hn, mr, ar[j]);
+                            ai[j] = fmaf(hn, mi, ai[j]);
+                        }
+                    }
+                    p += d;
+                    d += dd;
+                }
+                // frame b - (J - 1) is complete
+                const int f = b - (J - 1);
+                if (f >= 0) {
+                    float tr = ar[J - 1], ti = ai[J - 1];
+#pragma unroll
+                    for (int w = 16; w > 0; w >>= 1) {
+                        tr += __shfl_xor_sync(0xffffffffu, tr, w);
+                        ti += __shfl_xor_sync(0xffffffffu, ti, w);
+                    }
+                    if (lane == 0) red[wk][f][warp] = make_double2(tr, ti);
+                }
+#pragma unroll
+                for (int j = J - 1; j > 0; --j) {
+                    ar[j] = ar[j - 1];
+                    ai[j] = ai[j - 1];
+                }
+                ar[0] = ai[0] = 0.f;
+            }
+            worker_sync();
+            if (tid < nf) {
+                double tr = 0.0, ti = 0.0;
+                for (int w = 0; w < kChirpThreads / 32; ++w) {
+                    tr += red[wk][tid][w].x;
+                    ti += red[wk][tid][w].y;
+                }
+                a.out[static_cast<int64_t>(c) * a.ld + a.fo + k0 + f0 + tid] =
+                    make_float2(static_cast<float>(tr), static_cast<float>(ti));
+            }
+            worker_sync();
+        }
+    }
+}
+
 }  // namespace
 
 namespace {
@@ -303,6 +405,44 @@ cudaError_t chirp_demod_launch(const ChirpLaunch& L, cudaStream_t st) {
     a.out = static_cast<float2*>(L.tones);
     a.ld = L.tones_ld;
     a.fo = L.frame_offset;
+    // overlapping frames: each mixer value once for all its frames, where at
+    // least a segment of two frames fits
+    const int J = (L.L + L.D - 1) / L.D;
+    constexpr int kOvSamples = 48 * 1024;               // of a segment: 192 KB
+    const int jt = J <= 2 ? 2 : (J <= 4 ? 4 : 8);       // compiled widths; the blocks past L add nothing
+    if (J >= 2 && J <= 8 && L.D % kChirpThreads == 0 && (jt + 1) * L.D <= kOvSamples) {
+        const bool full = L.L == jt * L.D;
+        ChirpOverlap o{};
+        const int64_t grid = std::min<int64_t>(L.F, L.n_sms);
+        o.per_cta = (L.F + grid - 1) / grid;
+        const int64_t widest = kOvSamples / L.D - (jt - 1) > 0 ? kOvSamples / L.D - (jt - 1) : 1;
+        const int64_t n_seg = (o.per_cta + widest - 1) / widest;
+        o.seg = static_cast<int>((o.per_cta + n_seg - 1) / n_seg);
+        // frames per work item: the fewest rounds of block walks for the four workers
+        int64_t best = INT64_MAX;
+        for (int parts = 1; parts <= 4 || (o.seg + parts - 1) / parts > kOvSub; parts *= 2) {
+            const int sub = (o.seg + parts - 1) / parts;
+            if (sub > kOvSub) continue;
+            const int64_t items = static_cast<int64_t>(a.n_chirps) * ((o.seg + sub - 1) / sub);
+            const int64_t cost = (items + kOvWorkers - 1) / kOvWorkers * (sub + jt - 1);
+            if (cost < best) {
+                best = cost;
+                o.sub = sub;
+            }
+        }
+        const size_t bytes = static_cast<size_t>(o.seg + jt - 1) * L.D * 4;
+        auto run = [&](auto kern) {
+            const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+            if (e != cudaSuccess) return e;
+            kern<<<static_cast<unsigned>((L.F + o.per_cta - 1) / o.per_cta), kOvWorkers * kChirpThreads, bytes, st>>>(a, o);
+            return cudaGetLastError();
+        };
+        switch (jt) {
+        case 2: return full ? run(chirp_overlap_kernel<2, true>) : run(chirp_overlap_kernel<2, false>);
+        case 4: return full ? run(chirp_overlap_kernel<4, true>) : run(chirp_overlap_kernel<4, false>);
+        default: return full ? run(chirp_overlap_kernel<8, true>) : run(chirp_overlap_kernel<8, false>);
+        }
+    }
     const size_t smem = static_cast<size_t>(L.L) * sizeof(float2);
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(chirp_demod_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
