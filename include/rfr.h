@@ -133,8 +133,9 @@ typedef struct {
  *              no prime factor above 7 (N = 2^a 3^b 5^c 7^d); any other N
  *              returns RFR_E_UNSUPPORTED.  Powers of two from 16 to 16384 run
  *              the single-CTA-per-frame kernels (FIR, FFT and gather fused
- *              where the delay line fits one SM; for N = 8192, 16384 or
- *              T > 8 the FIR as a separate pre-sum pass first), every other
+ *              where one SM holds what the FIR needs; for N = 8192, 16384,
+ *              or N = 2048 and 4096 with T > 8, the FIR as a separate pre-sum
+ *              pass first), every other
  *              N the mixed-radix kernels (one pass up to 8192, a four-step
  *              two-pass form above).
  *              0: direct demodulation.
@@ -162,7 +163,7 @@ typedef struct {
  * never allocates).  Demodulation plans likewise allocate their per-push
  * scratch (the FP16 split of the stream and the rotation tables) on the first
  * push of a given size, and so do PFB plans that run their FIR as a separate
- * pre-sum pass (N = 8192; N = 16384 with T > 4; N = 256 to 4096 with T > 8:
+ * pre-sum pass (N = 8192; N = 16384 with T > 4; N = 2048 and 4096 with T > 8:
  * 8 bytes per channel and frame) or the oversampled phase passes; a
  * push that grows scratch synchronises the device and sizes it for that many
  * samples after any carry.  Inside a stream capture such a push fails with

@@ -122,10 +122,12 @@ __device__ __forceinline__ float2 tw_load(const float2* t, int i) {
 // polyphase outputs).  On exit v holds y at the indices given by
 // fft_out_index(), and nothing of the spectrum is in `buf` (the caller stores
 // it there if it needs it).  All CTA threads must call this together (it
-// contains __syncthreads); threads of masked frames still call it.
-template <int LOG2N, bool TW_SMEM>
+// contains __syncthreads); threads of masked frames still call it.  TWO: the
+// passes alternate between buf and buf2 (one barrier a pass instead of two);
+// buf is free on entry, buf2 once every thread has arrived at the first barrier.
+template <int LOG2N, bool TW_SMEM, bool TWO = false>
 __device__ __forceinline__ void fft_frame(float2 (&v)[16], float2* buf, int tf,
-                                          const float2* tw) {
+                                          const float2* tw, float2* buf2 = nullptr) {
     constexpr int N = 1 << LOG2N;
     constexpr int NT = N / 16;
     constexpr int P16 = LOG2N / 4;
@@ -151,7 +153,13 @@ __device__ __forceinline__ void fft_frame(float2 (&v)[16], float2* buf, int tf,
             dft16(v);
             const bool last = (s == P16 - 1) && (RF == 1);
             if (!last) {
-                __syncthreads();
+                if constexpr (TWO) {
+                    float2* const other = buf2;
+                    buf2 = buf;
+                    buf = other;
+                } else {
+                    __syncthreads();
+                }
                 const int base = (tf / ns) * 16 * ns + k;
 #pragma unroll
                 for (int r = 0; r < 16; ++r) buf[fpad(base + r * ns)] = v[r];

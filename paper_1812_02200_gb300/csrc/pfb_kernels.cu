@@ -19,7 +19,11 @@
 //         pushes of any alignment) works on two frames at a time with two
 //         groups of warps and also runs the phase passes of oversampled plans; a seeded form continues FIR sums from pre-sum
 //         rows (N = 4096 with 9..16 taps: first-half pass + taps 8..15).
-//  RING   (N <= 4096, T <= 8 after padding): each CTA owns a contiguous run
+//  TILE   (N = 64 .. 1024, T <= 16; N = 2048, T = 5 .. 8 or unaligned): one CTA
+//         per 4096 points, the FIR of a branch's consecutive frames in one
+//         thread (each sample converted once for all of them), any alignment.
+//  RING   (N = 16, 32, 2048 and 4096, T <= 8 after padding, where no other
+//         kernel takes the shape): each CTA owns a contiguous run
 //         of "super-blocks" (4096 samples = G = 4096/N frames' worth of new
 //         samples).  A ring of super-blocks in shared memory is filled by
 //         1-D TMA bulk copies (cp.async.bulk + mbarrier complete_tx), P
@@ -29,9 +33,9 @@
 //         sharing the FFT through distributed shared memory.
 //  DIRECT (any other N <= 16384, T <= 16): the in-CTA FFT per frame, its FIR
 //         either a separate DRAM-streaming pre-sum pass (fir_pre_kernel; N =
-//         8192, 16384 with T > 4, N = 256 .. 2048 with T > 8) or read from
-//         global memory inside the kernel (L2 serves the T-fold reuse).
-// RING and DIRECT run the in-CTA FFT of fft_dev.cuh (TMEM the same passes
+//         8192, 16384 with T > 4, N = 2048 with T > 8) or read from global
+//         memory inside the kernel (L2 serves the T-fold reuse).
+// TILE, RING and DIRECT run the in-CTA FFT of fft_dev.cuh (TMEM the same passes
 // written out for N = 4096); all write
 //   full[(frame_offset + j) * full_ld + c]      (natural bin order)
 //   tones[s * tones_ld + frame_offset + j] = y_j[bin[s]].
@@ -1314,6 +1318,94 @@ __global__ void __launch_bounds__(LOG2N >= 14 ? 1024 : (LOG2N == 13 ? 512 : 256)
     }
 }
 
+// ---------------------------------------------------------------- TILE
+// N = 64 .. 1024, T <= 16, and N = 2048 with 4 < T <= 8.  A CTA takes one tile of
+// G = 4096 / N frames (16 points a thread).  FIR: a thread owns C = max(1, N /
+// 256) branches and RF = 16 / C consecutive frames of each, loads every sample of its window from
+// global memory (consecutive branches across the warp) and converts it once for
+// all its frames; the sums go through shared memory to the FFT's layout (points
+// tf + r N/16 of a frame), and the passes alternate between two padded buffers.
+// Any alignment and carry.  Sums, passes and outputs as in the other kernels
+// (bit-identical results).
+//
+// Why: the int16 ring's FIR converted each sample once per tap (8 times at T =
+// 8), 56 of 86 instructions a point, on 8 warps an SM; here it is converted (RF +
+// T - 1) / RF times, on 24 warps an SM (two CTAs an SM measured 10-20 % slower, 512
+// threads and 8192 points 10-20 % slower at N = 1024).  More than 8 taps took a
+// pre-sum pass through memory (16 bytes a sample more).
+// Measured, 2^25 samples, full + N / 4 tones, before -> after (us):
+//   N       T = 4        T = 8        T = 16
+//   64    237 -> 115   345 -> 118   695 -> 126     (floor of the bytes: 69)
+//   256   173 -> 119   202 -> 128   214 -> 144
+//   1024  185 -> 160   225 -> 171   226 -> 205
+//   2048  202 -> 206   239 -> 222   238 -> 277
+// so N = 2048 keeps the ring at T <= 4 (aligned pushes; unaligned ones, which the
+// ring copies by threads, come here) and the pre-sum pass at T > 8: a thread
+// there owns two frames only and loads T + 1 samples for two sums.
+constexpr int kTileThreads = 256;
+template <int LOG2N, int TMAX>
+__global__ void __launch_bounds__(kTileThreads, 3) pfb_tile_kernel(const PfbArgs a) {
+    constexpr int N = 1 << LOG2N, NT = N / 16, THREADS = kTileThreads, G = THREADS / NT;
+    constexpr int C = N > THREADS ? N / THREADS : 1, RF = 16 / C, R = RF + TMAX - 1;
+    constexpr int FSTRIDE = N + N / 16;
+    extern __shared__ __align__(1024) unsigned char smem[];
+    float2* const xa = reinterpret_cast<float2*>(smem);
+    float2* const xb = xa + G * FSTRIDE;
+    const int tid = threadIdx.x;
+    const int64_t j0 = static_cast<int64_t>(blockIdx.x) * G;
+    const int T = a.T;
+    {
+        // frames g0 .. g0 + RF - 1 of the tile, branches p0 + c THREADS
+        const int p0 = tid & (N - 1 < THREADS - 1 ? N - 1 : THREADS - 1);
+        const int g0 = C == 1 ? (tid / N) * RF : 0;
+        const int64_t base = (j0 + g0) * N + p0;                 // the window's first sample
+        const int64_t lim = (a.F + T - 1) * N;                   // samples of the push's frames
+        const bool inside = base >= a.cl && base + static_cast<int64_t>(R - 1) * N + (C - 1) * THREADS < lim;
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            float h[TMAX];
+#pragma unroll
+            for (int t = 0; t < TMAX; ++t) h[t] = t < T ? __ldg(a.h + t * N + p0 + c * THREADS) : 0.f;
+            uint32_t x[R];
+            const int64_t b = base + c * THREADS;
+            if (inside) {
+                const uint32_t* src = a.buf + (b - a.cl);
+#pragma unroll
+                for (int r = 0; r < R; ++r) x[r] = __ldg(src + static_cast<int64_t>(r) * N);
+            } else {
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    const int64_t i = b + static_cast<int64_t>(r) * N;
+                    x[r] = i < lim ? vload(a, i) : 0u;
+                }
+            }
+            float2 acc[RF];
+#pragma unroll
+            for (int g = 0; g < RF; ++g) acc[g] = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const float2 v = iq_to_f2(x[r]);
+#pragma unroll
+                for (int g = 0; g < RF; ++g) {
+                    const int t = r - g;
+                    if (t >= 0 && t < TMAX) ffma2(acc[g].x, acc[g].y, h[t], h[t], v.x, v.y);
+                }
+            }
+#pragma unroll
+            for (int g = 0; g < RF; ++g) xa[(g0 + g) * FSTRIDE + fpad(p0 + c * THREADS)] = acc[g];
+        }
+    }
+    __syncthreads();
+    const int g = tid / NT, tf = tid % NT;
+    const int64_t j = j0 + g;
+    float2 v[16];
+#pragma unroll
+    for (int r = 0; r < 16; ++r) v[r] = xa[g * FSTRIDE + fpad(tf + r * NT)];
+    fft_frame<LOG2N, false, true>(v, xb + g * FSTRIDE, tf, a.tw, xa + g * FSTRIDE);
+    // the last pass read from xb (two passes) or xa (three)
+    pfb_outputs<LOG2N>(a, v, (LOG2N > 8 ? xb : xa), g, tf, j, j < a.F, G, j0);
+}
+
 // ------------------------------------------------------------ launcher
 namespace {
 
@@ -1359,7 +1451,7 @@ cudaError_t launch_direct(PfbArgs a, int n_sms, int max_smem, cudaStream_t st) {
     const int64_t n_iter = (a.F + G - 1) / G;
     int per_sm = 1;
     // pre-sum instances only for the shapes that take them (pfb_pre_rows)
-    constexpr bool kPre = (LOG2N >= 8 && LOG2N <= 11) || LOG2N == 13 || LOG2N == 14;
+    constexpr bool kPre = LOG2N == 11 || LOG2N == 13 || LOG2N == 14;
     if (a.pre && !kPre) return cudaErrorInvalidValue;
     auto k = a.pre ? pfb_direct_kernel<LOG2N, kPre> : pfb_direct_kernel<LOG2N, false>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -1368,6 +1460,23 @@ cudaError_t launch_direct(PfbArgs a, int n_sms, int max_smem, cudaStream_t st) {
     const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(n_iter, static_cast<int64_t>(n_sms) * std::max(per_sm, 1)));
     k<<<static_cast<unsigned>(grid), threads, smem, st>>>(a);
     return cudaGetLastError();
+}
+
+template <int LOG2N>
+cudaError_t launch_tile(const PfbArgs& a, cudaStream_t st) {
+    constexpr int N = 1 << LOG2N, G = kTileThreads / (N / 16);
+    constexpr size_t smem = static_cast<size_t>(2) * G * (N + N / 16) * 8;
+    const int64_t tiles = (a.F + G - 1) / G;
+    if (tiles > 0x7fffffff) return cudaErrorInvalidValue;
+    auto run = [&](auto k) {
+        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+        if (e != cudaSuccess) return e;
+        k<<<static_cast<unsigned>(tiles), kTileThreads, smem, st>>>(a);
+        return cudaGetLastError();
+    };
+    if (a.T <= 4) return run(pfb_tile_kernel<LOG2N, 4>);
+    if constexpr (LOG2N == 11) return a.T <= 8 ? run(pfb_tile_kernel<LOG2N, 8>) : cudaErrorInvalidValue;
+    else return a.T <= 8 ? run(pfb_tile_kernel<LOG2N, 8>) : run(pfb_tile_kernel<LOG2N, 16>);
 }
 
 // FIR sums of the first T (<= TMAX) taps of every frame of the stream view
@@ -1462,9 +1571,6 @@ cudaError_t launch_pre(const PfbArgs& a, int lg, int T, float2* pre, cudaStream_
     }
     // more taps: one point and eight frames per thread
     switch (lg) {
-    case 8: return launch_pre_n<16, 1, 8, 8>(a, T, pre, st);
-    case 9: return launch_pre_n<16, 1, 8, 9>(a, T, pre, st);
-    case 10: return launch_pre_n<16, 1, 8, 10>(a, T, pre, st);
     case 11: return launch_pre_n<16, 1, 8, 11>(a, T, pre, st);
     case 13: return launch_pre_n<16, 1, 8, 13>(a, T, pre, st);
     case 14: return launch_pre_n<16, 1, 8, 14>(a, T, pre, st);
@@ -1655,14 +1761,12 @@ bool pfb_split16(int log2n, int taps) { return log2n == 12 && taps == 16; }
 // Where the direct kernel takes its FIR from a pre-sum pass (measured, 2^28
 // samples, full + tones): N = 8192 at every T (T = 8: 3.14 -> 1.81 ms),
 // N = 16384 from T = 8 on (2.73 -> 1.85 ms; T = 4 1.87 -> 2.14 ms, so not
-// there), N = 256 .. 2048 with T > 8 (T = 16: N = 1024 5.39 -> 3.15 ms,
-// N = 256 with 64 tones 4.39 -> 1.61 ms).  Smaller N, or T <= 8 below
-// N = 4096, run on the shared-memory ring kernel.
+// there), N = 2048 with T > 8 (smaller N run on the tile kernel).
 bool pfb_pre_rows(int log2n, int taps) {
     if (pfb_split16(log2n, taps)) return true;
     if (log2n == 13) return true;
     if (log2n == 14) return taps > 4;
-    return log2n >= 8 && log2n <= 11 && taps > 8;
+    return log2n == 11 && taps > 8;
 }
 int pfb_kernel_taps(int log2n, int taps) {
     if (pfb_uses_ring(log2n, taps) || pfb_cluster_size(log2n, taps) > 0) return taps <= 4 ? 4 : 8;
@@ -1744,16 +1848,23 @@ cudaError_t pfb_launch(const PfbLaunch& L, cudaStream_t st) {
         if (L.taps_kernel == 4) return launch_tmem<4>(a, L.n_sms, L.max_smem, st);
         if (L.taps_kernel == 8) return launch_tmem<8>(a, L.n_sms, L.max_smem, st);
     }
+    // the tile kernel's shapes (see its figures)
+    switch (lg) {
+    case 6: return launch_tile<6>(a, st);
+    case 7: return launch_tile<7>(a, st);
+    case 8: return launch_tile<8>(a, st);
+    case 9: return launch_tile<9>(a, st);
+    case 10: return launch_tile<10>(a, st);
+    case 11:
+        if (L.taps_kernel <= 8 && (L.taps_kernel > 4 || !aligned)) return launch_tile<11>(a, st);
+        break;
+    default: break;
+    }
     if (pfb_uses_ring(lg, L.taps_kernel)) {
         switch (lg) {
         case 4: return dispatch_ring_T<4>(a, L.taps_kernel, L.n_sms, L.max_smem, L.lookahead, st);
         case 5: return dispatch_ring_T<5>(a, L.taps_kernel, L.n_sms, L.max_smem, L.lookahead, st);
-        case 6: return dispatch_ring_T<6>(a, L.taps_kernel, L.n_sms, L.max_smem, L.lookahead, st);
-        case 7: return dispatch_ring_T<7>(a, L.taps_kernel, L.n_sms, L.max_smem, L.lookahead, st);
-        case 8: return dispatch_ring_T<8>(a, L.taps_kernel, L.n_sms, L.max_smem, L.lookahead, st);
-        case 9: return dispatch_ring_T<9>(a, L.taps_kernel, L.n_sms, L.max_smem, L.lookahead, st);
-        case 10: return dispatch_ring_T<10>(a, L.taps_kernel, L.n_sms, L.max_smem, L.lookahead, st);
-        case 11: return dispatch_ring_T<11>(a, L.taps_kernel, L.n_sms, L.max_smem, L.lookahead, st);
+        case 11: return launch_ring<11, 4>(a, L.n_sms, L.max_smem, L.lookahead, st);
         case 12: return dispatch_ring_T<12>(a, L.taps_kernel, L.n_sms, L.max_smem, L.lookahead, st);
         default: return cudaErrorInvalidValue;
         }
@@ -1769,13 +1880,7 @@ cudaError_t pfb_launch(const PfbLaunch& L, cudaStream_t st) {
     switch (lg) {
     case 4: return launch_direct<4>(a, L.n_sms, L.max_smem, st);
     case 5: return launch_direct<5>(a, L.n_sms, L.max_smem, st);
-    case 6: return launch_direct<6>(a, L.n_sms, L.max_smem, st);
-    case 7: return launch_direct<7>(a, L.n_sms, L.max_smem, st);
-    case 8: return launch_direct<8>(a, L.n_sms, L.max_smem, st);
-    case 9: return launch_direct<9>(a, L.n_sms, L.max_smem, st);
-    case 10: return launch_direct<10>(a, L.n_sms, L.max_smem, st);
     case 11: return launch_direct<11>(a, L.n_sms, L.max_smem, st);
-    case 12: return launch_direct<12>(a, L.n_sms, L.max_smem, st);
     case 13: return launch_direct<13>(a, L.n_sms, L.max_smem, st);
     case 14: return launch_direct<14>(a, L.n_sms, L.max_smem, st);
     default: return cudaErrorInvalidValue;

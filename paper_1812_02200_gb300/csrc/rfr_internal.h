@@ -110,7 +110,7 @@ int pfb_cluster_size(int log2n, int taps);
 // seeded with it (aligned view, PfbLaunch::pre for the frames).
 bool pfb_split16(int log2n, int taps);
 // PFB plans whose pushes take FIR pre-sum rows (PfbLaunch::pre): the 16-tap
-// N = 4096 form and the direct kernel's shapes (N = 8192, 16384; T > 8).
+// N = 4096 form and the direct kernel's shapes (N = 8192, 16384; N = 2048 with T > 8).
 bool pfb_pre_rows(int log2n, int taps);
 cudaError_t pfb_launch(const PfbLaunch& L, cudaStream_t st);
 cudaError_t gen_pfb_launch(const PfbLaunch& L, const GenPlan& g, cudaStream_t st);
