@@ -361,7 +361,12 @@ __device__ float2* gen_fft_to(float2* buf0, float2* buf1, const GenFft& f, int g
 // the same order (so the same results), with the length, the span, the
 // group count and every stride known at compile time, so the index
 // arithmetic folds into constants and immediate offsets.
-template <int R, int TH, int N, int GL2, int NS, bool OUT, typename Sink>
+// IN: where the points come from.  0: a padded buffer (gpad); the first stage
+// may also read them as a copy left them: 1 interleaved without padding (point
+// j of transform g at j G + g), 2 one transform after the other (at g N + j).
+// Such a stage fences its reads for the next copy into the same place.
+// PADO: the stage's own output buffer is padded.
+template <int R, int TH, int N, int GL2, int NS, bool OUT, int IN = 0, bool PADO = true, typename Sink>
 __device__ __forceinline__ void fixed_stage(const float2* __restrict__ src, float2* __restrict__ dst,
                                             const float2* __restrict__ tw, Sink& sink) {
     constexpr int nb = (N / R) << GL2;
@@ -370,10 +375,16 @@ __device__ __forceinline__ void fixed_stage(const float2* __restrict__ src, floa
     for (int i = 0; i < iters; ++i) {
         const int u = static_cast<int>(threadIdx.x) + i * TH;
         if (nb % TH != 0 && u >= nb) break;
-        const int g = u & ((1 << GL2) - 1), j = u >> GL2;
+        constexpr int nR = N / R;
+        const int g = IN == 2 ? u / nR : u & ((1 << GL2) - 1), j = IN == 2 ? u % nR : u >> GL2;
         const int k = NS == 1 ? 0 : j % NS;
         float2 v[R];
-        load_strided<R>(v, src, u, nb);                      // points (j + r*nR)*G + g
+        if constexpr (IN == 0) {
+            load_strided<R>(v, src, u, nb);                  // points (j + r*nR)*G + g
+        } else {
+#pragma unroll
+            for (int r = 0; r < R; ++r) v[r] = IN == 1 ? src[u + r * nb] : src[g * N + j + r * nR];
+        }
         if constexpr (NS > 1) {
 #pragma unroll
             for (int r = 1; r < R; ++r) v[r] = cmul(v[r], __ldg(tw + (r - 1) * NS + k));
@@ -383,10 +394,14 @@ __device__ __forceinline__ void fixed_stage(const float2* __restrict__ src, floa
         if constexpr (OUT) {
 #pragma unroll
             for (int r = 0; r < R; ++r) sink(((base + r * NS) << GL2) + g, v[r]);
+        } else if constexpr (!PADO) {
+#pragma unroll
+            for (int r = 0; r < R; ++r) dst[((base + r * NS) << GL2) + g] = v[r];
         } else {
             store_strided<R>(v, dst, (base << GL2) + g, NS << GL2);
         }
     }
+    if constexpr (IN != 0 && !OUT) fence_proxy_async_smem();
     if constexpr (!OUT) __syncthreads();
 }
 
@@ -425,10 +440,8 @@ template <int TH, int PASS, typename Sink>
 __device__ __forceinline__ float2* fft_to(float2* buf0, float2* buf1, const GenFft& f, int gl2,
                                           const float2* __restrict__ tw, int fix, Sink sink) {
     const float2* t0 = tw + f.tw_off[0];
-    if constexpr (TH == 256 && PASS == 0) {
-        if (fix == 1) return FixedFft<TH, 3, 400, 1, 25, 16>::run(buf0, buf1, t0, sink);
-    } else if constexpr (TH == 256) {
-        if (fix == 2) return FixedFft<TH, 4, 250, 1, 25, 10>::run(buf0, buf1, t0, sink);
+    if constexpr (TH == 256) {
+        // N = 10^5's shapes are compiled into the passes themselves
     } else if constexpr (PASS == 0) {
         if (fix == 4) return FixedFft<TH, 1, 3125, 1, 25, 25, 5>::run(buf0, buf1, t0, sink);
     } else {
@@ -836,19 +849,58 @@ __global__ void __launch_bounds__(TH, GenCfg<TH>::kMinBlocks)
     }
     __syncthreads();
     uint32_t vphase = 0;
+    // points p1*GA + g = V[kk][p1*N2 + g0 + g]: boxes of rows of V
+    // viewed as [frames*N1][N2] (columns past N2 read as zero); one thread
+    auto fetch = [&](int64_t it) {
+        const int64_t kk = it / groups;
+        const int g0 = static_cast<int>(it - kk * groups) << a.gla;
+        mbar_arrive_expect_tx(vbar, static_cast<uint32_t>(a.vboxes * a.vbox_rows * GA * 8));
+        for (int b = 0; b < a.vboxes; ++b)
+            tma_load_2d(vst + b * a.vsstride, &tmv, g0, static_cast<int32_t>(kk * a.N1 + b * a.vbox_rows), vbar);
+    };
+    if constexpr (TH == 256) {
+        // N = 10^5 (two compiled-in stages), boxes end to end: the first stage
+        // reads the boxes as they land, and the next group's boxes are fetched
+        // into the same place while the second stage runs.  (Fetched at the
+        // group's start and copied into the padded layout first, every group
+        // waited for its load: 659 us a 2^27-sample push, now 435, at 63 % of
+        // the DRAM peak; pass B, likewise, 508 -> 425.)
+        if (a.fixa == 1 && a.vtma && a.vsstride == a.vbox_rows * GA) {
+            constexpr int R0 = 25, R1 = 16, NN = 400, GL = 3;
+            const float2* const t0 = a.tw_a + a.fa.tw_off[0];
+            if (threadIdx.x == 0 && blockIdx.x < a.F * groups) fetch(blockIdx.x);
+            for (int64_t it = blockIdx.x; it < a.F * groups; it += gridDim.x) {
+                const int64_t kk = it / groups;
+                const int g0 = static_cast<int>(it - kk * groups) << GL;
+                const int N2 = a.N2;
+                if (!mbar_wait(vbar, vphase, a.status)) return;
+                vphase ^= 1u;
+                auto none = [](int, float2) {};
+                // (no padding between the stages: butterflies' outputs start 200
+                // points apart, 8 modulo the 16 banks, and 8 transforms fill those)
+                fixed_stage<R0, TH, NN, GL, 1, false, 1, false>(vst, sm, t0, none);
+                if (threadIdx.x == 0 && it + gridDim.x < a.F * groups) fetch(it + gridDim.x);
+                float2* zf = a.z + kk * a.N;
+                auto sink = [=](int e, float2 v) {
+                    const int g = e & ((1 << GL) - 1), c1 = e >> GL, p2 = g0 + g;
+                    if (p2 < N2) {
+                        const int m = p2 * c1;
+                        const float2 w = cmul(cmul(stw[m & 255], stw[kTwDigit + ((m >> 8) & 255)]), stw[2 * kTwDigit + (m >> 16)]);
+                        zf[static_cast<int64_t>(c1) * N2 + p2] = cmul(v, w);
+                    }
+                };
+                fixed_stage<R1, TH, NN, GL, R0, true, 1>(sm, sm, t0, sink);
+                __syncthreads();
+            }
+            return;
+        }
+    }
     for (int64_t it = blockIdx.x; it < a.F * groups; it += gridDim.x) {
         const int64_t kk = it / groups;
         const int g0 = static_cast<int>(it - kk * groups) << a.gla;
         const int N2 = a.N2, gla = a.gla;
         if (a.vtma) {
-            // points p1*GA + g = V[kk][p1*N2 + g0 + g]: boxes of rows of V
-            // viewed as [frames*N1][N2] (columns past N2 read as zero)
-            if (threadIdx.x == 0) {
-                mbar_arrive_expect_tx(vbar, static_cast<uint32_t>(a.vboxes * a.vbox_rows * GA * 8));
-                for (int b = 0; b < a.vboxes; ++b)
-                    tma_load_2d(vst + b * a.vsstride, &tmv, g0,
-                                static_cast<int32_t>(kk * a.N1 + b * a.vbox_rows), vbar);
-            }
+            if (threadIdx.x == 0) fetch(it);
             if (!mbar_wait(vbar, vphase, a.status)) return;
             vphase ^= 1u;
             for (int b = 0; b < a.vboxes; ++b) {
@@ -902,6 +954,79 @@ __global__ void __launch_bounds__(TH, GenCfg<TH>::kMinBlocks) gen_pass_b_kernel(
     }
     __syncthreads();
     uint32_t zphase = 0;
+    if constexpr (TH == 256) {
+        // N = 10^5, as in pass A: the first stage reads the rows as the bulk
+        // copy left them, and the next group's copy runs behind the second
+        // stage, whose outputs reach the tone gather through its own input
+        if (a.fixb == 2 && a.zbulk) {
+            constexpr int R0 = 25, R1 = 10, NN = 250, GL = 4, nb = (NN / R1) << GL, iters = (nb + TH - 1) / TH;
+            const float2* const t0 = a.tw_b + a.fb.tw_off[0];
+            auto fetch = [&](int64_t it) {
+                const int64_t kk = it / groups;
+                const int c0 = static_cast<int>(it - kk * groups) << GL;
+                const uint32_t bytes = static_cast<uint32_t>(min(1 << GL, a.N1 - c0) * NN) * 8u;
+                mbar_arrive_expect_tx(zbar, bytes);
+                tma_bulk_g2s(zst, a.z + kk * a.N + static_cast<int64_t>(c0) * NN, bytes, zbar);
+            };
+            const bool keep = a.n_tones > 0;
+            const int N1 = a.N1;
+            if (threadIdx.x == 0 && blockIdx.x < a.F * groups) fetch(blockIdx.x);
+            for (int64_t it = blockIdx.x; it < a.F * groups; it += gridDim.x) {
+                const int64_t kk = it / groups;
+                const int c0 = static_cast<int>(it - kk * groups) << GL;
+                if (!mbar_wait(zbar, zphase, a.status)) return;
+                zphase ^= 1u;
+                auto none = [](int, float2) {};
+                // (rows past a last group's are not copied: their outputs go nowhere)
+                fixed_stage<R0, TH, NN, GL, 1, false, 2>(zst, sm, t0, none);
+                if (threadIdx.x == 0 && it + gridDim.x < a.F * groups) fetch(it + gridDim.x);
+                const int64_t k = a.k0 + kk;
+                float2* row = a.full ? a.full + (a.fo + k) * a.full_ld + c0 : nullptr;
+                // the group's tones, a thread each (their loads in flight meanwhile)
+                int i0 = 0, i1 = 0;
+                int2 te = make_int2(0, 0);
+                if (keep) {
+                    i0 = __ldg(a.goff + (c0 >> GL)) + threadIdx.x;
+                    i1 = __ldg(a.goff + (c0 >> GL) + 1);
+                    if (i0 < i1) te = __ldg(a.gtone + i0);
+                }
+                float2 v[iters][R1];
+#pragma unroll
+                for (int i = 0; i < iters; ++i) {
+                    const int u = static_cast<int>(threadIdx.x) + i * TH;
+                    if (u >= nb) break;
+                    load_strided<R1>(v[i], sm, u, nb);
+                    const int kt = (u >> GL) % R0;
+#pragma unroll
+                    for (int r = 1; r < R1; ++r) v[i][r] = cmul(v[i][r], __ldg(t0 + (r - 1) * R0 + kt));
+                    dft_any<R1>(v[i]);
+                }
+                if (keep) __syncthreads();                   // the stage's reads of sm are done
+#pragma unroll
+                for (int i = 0; i < iters; ++i) {
+                    const int u = static_cast<int>(threadIdx.x) + i * TH;
+                    if (u >= nb) break;
+                    const int g = u & ((1 << GL) - 1), j = u >> GL, kt = j % R0;
+                    const int base = (j - kt) * R1 + kt;
+#pragma unroll
+                    for (int r = 0; r < R1; ++r) {
+                        const int c2 = base + r * R0;
+                        if (row && c0 + g < N1) row[g + static_cast<int64_t>(N1) * c2] = v[i][r];
+                        if (keep) sm[gpad((c2 << GL) + g)] = v[i][r];
+                    }
+                }
+                __syncthreads();
+                if (keep) {
+                    for (int i = i0; i < i1; i += TH) {
+                        if (i != i0) te = __ldg(a.gtone + i);
+                        a.tones[te.x * a.tones_ld + a.fo + k] = sm[gpad(te.y)];
+                    }
+                    __syncthreads();
+                }
+            }
+            return;
+        }
+    }
     for (int64_t it = blockIdx.x; it < a.F * groups; it += gridDim.x) {
         const int64_t kk = it / groups;
         const int c0 = static_cast<int>(it - kk * groups) << a.glb;
