@@ -99,6 +99,12 @@ __global__ void interleave_tones_kernel(const float2* __restrict__ src, int64_t 
 }
 
 // -------------------------------------------------------------- carry copy
+// The next push's carry.  It reads what the push's other kernels read (the old
+// carry and the buffer) and writes the other carry buffer, which only the push
+// before used, so outside stream capture it is launched as a programmatic
+// dependent of the push's last kernel and runs beside it: serialised it cost a
+// small push 2-3 us of 12-25.  It completes only after that kernel has (the
+// wait at its end), so whatever follows on the stream follows both.
 __global__ void carry_update_kernel(const uint32_t* __restrict__ old_carry, int64_t cl,
                                     const uint32_t* __restrict__ buf, int64_t from, int64_t count,
                                     uint32_t* __restrict__ out) {
@@ -107,6 +113,7 @@ __global__ void carry_update_kernel(const uint32_t* __restrict__ old_carry, int6
         const int64_t idx = from + i;
         out[i] = idx < cl ? old_carry[idx] : buf[idx - cl];
     }
+    rfr::wait_for_primary();
 }
 
 // Self-test of the bounded waits: one thread waits on an mbarrier phase that
@@ -530,7 +537,8 @@ rfr_status push_core(rfr_plan* p, const int16_t* iq, int64_t n, const rfr_output
     const int64_t ncl = lv - F * p->H;
     if (ncl > 0) {
         if (ncl > p->carry_cap) return fail(p, RFR_E_INVALID, "internal: carry overflow");
-        RFR_CUDA(p, rfr::carry_update(carry, p->cl, iq, n, F * p->H, ncl, p->d_carry[p->cur ^ 1], st));
+        RFR_CUDA(p, rfr::carry_update(carry, p->cl, iq, n, F * p->H, ncl, p->d_carry[p->cur ^ 1], st,
+                                   F > 0 && (p->mode == RFR_MODE_PFB || !p->words.empty())));
         p->cur ^= 1;
     }
     p->cl = ncl;
@@ -588,15 +596,31 @@ void destroy(rfr_plan* p) {
 
 namespace rfr {
 cudaError_t carry_update(const int16_t* old_carry, int64_t cl, const int16_t* buf, int64_t n,
-                         int64_t from, int64_t count, int16_t* new_carry, cudaStream_t st) {
+                         int64_t from, int64_t count, int16_t* new_carry, cudaStream_t st, bool beside) {
     (void)n;
     if (count <= 0) return cudaSuccess;
     const int threads = 256;
     const int64_t blocks = std::min<int64_t>((count + threads - 1) / threads, 4096);
-    carry_update_kernel<<<static_cast<unsigned>(blocks), threads, 0, st>>>(
-        reinterpret_cast<const uint32_t*>(old_carry), cl, reinterpret_cast<const uint32_t*>(buf),
-        from, count, reinterpret_cast<uint32_t*>(new_carry));
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(blocks), 1, 1);
+    cfg.blockDim = dim3(threads, 1, 1);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    if (beside) {
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        const cudaError_t e = cudaStreamIsCapturing(st, &cs);
+        if (e != cudaSuccess) return e;
+        if (cs == cudaStreamCaptureStatusNone) {
+            attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            attr[0].val.programmaticStreamSerializationAllowed = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+        }
+    }
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, carry_update_kernel, reinterpret_cast<const uint32_t*>(old_carry), cl,
+                                             reinterpret_cast<const uint32_t*>(buf), from, count,
+                                             reinterpret_cast<uint32_t*>(new_carry));
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 cudaError_t interleave_tones(const void* src, int64_t src_ld, int R, int n_tones, int64_t F, void* out,

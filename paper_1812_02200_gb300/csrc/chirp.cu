@@ -192,6 +192,7 @@ __global__ void __launch_bounds__(kChirpThreads) chirp_demod_kernel(const ChirpA
     extern __shared__ float2 xs[];                      // [L]
     __shared__ double2 red[kChirpGroup][kChirpThreads / 32];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    allow_dependents();
     for (int64_t k = blockIdx.x; k < a.F; k += gridDim.x) {
         __syncthreads();                                // previous frame's readers are done
         for (int n = tid; n < a.L; n += kChirpThreads) {
@@ -268,6 +269,7 @@ __global__ void __launch_bounds__(kOvWorkers * kChirpThreads, 1)
     __shared__ double2 red[kOvWorkers][kOvSub][kChirpThreads / 32];
     const int wk = threadIdx.x / kChirpThreads, tid = threadIdx.x % kChirpThreads;
     const int warp = tid >> 5, lane = tid & 31;
+    allow_dependents();
     auto worker_sync = [&] { asm volatile("bar.sync %0, 256;" ::"r"(1 + wk) : "memory"); };
     const int64_t k_end = a.F < (blockIdx.x + 1) * o.per_cta ? a.F : (blockIdx.x + 1) * o.per_cta;
     for (int64_t k0 = blockIdx.x * o.per_cta; k0 < k_end; k0 += o.seg) {

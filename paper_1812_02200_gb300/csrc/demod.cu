@@ -811,6 +811,7 @@ demod3m_gemm_kernel(const __grid_constant__ G3Batch bt) {
     umma::fence_after_sync();
     const uint32_t tmem = *tmem_holder;
     const int n_units = bt.total_units;
+    allow_dependents();
     float* const scr_cta = bt.p[0].scratch + static_cast<int64_t>(blockIdx.x) * G3_CTA_SCRATCH;
 
     if (FUSED && warp >= PROD_WARP && warp < MMA_WARP) {
@@ -1159,6 +1160,7 @@ demod3m_gemm_kernel(const __grid_constant__ G3Batch bt) {
 // frames along the warp.
 __global__ void combine3_kernel(const float* __restrict__ planes, int64_t pld, const GemmArgs g) {
     const int64_t k = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+    allow_dependents();
     if (k >= g.F) return;
     const int64_t K = g.F0 + k;
     const int64_t arow = K / BM - g.F0 / BM;

@@ -609,6 +609,7 @@ __host__ __device__ __forceinline__ SymLayout sym_layout(int nb) {
 }
 
 template <bool PHASE>
+    allow_dependents();
 __global__ void __launch_bounds__(kSymThreads, 1)
     pfb_tmem_sym_kernel(const PfbArgs a, const __grid_constant__ CUtensorMap tm_tones,
                         const __grid_constant__ CUtensorMap tm_full) {
@@ -1331,6 +1332,7 @@ __global__ void __launch_bounds__(LOG2N >= 14 ? 1024 : (LOG2N == 13 ? 512 : 256)
 // Why: the int16 ring's FIR converted each sample once per tap (8 times at T =
 // 8), 56 of 86 instructions a point, on 8 warps an SM; here it is converted (RF +
 // T - 1) / RF times, on 24 warps an SM (two CTAs an SM measured 10-20 % slower, 512
+    allow_dependents();
 // threads and 8192 points 10-20 % slower at N = 1024).  More than 8 taps took a
 // pre-sum pass through memory (16 bytes a sample more).
 // Measured, 2^25 samples, full + N / 4 tones, before -> after (us):

@@ -227,11 +227,13 @@ struct TuneConfig {
     int demod_pair = 0;         //   two-SM tiles (0/1)
     int pfb_cluster = 0;        // PFB N = 8192, 16384 with T <= 8: cluster kernel (1) or direct (0)
     bool tuned = false;
+// beside: as a programmatic dependent of the kernel launched before it, which
+// must be one of the same push.
 };
 
 // ------------------------------------------------------------- state
 cudaError_t carry_update(const int16_t* old_carry, int64_t cl, const int16_t* buf, int64_t n,
-                         int64_t from, int64_t count, int16_t* new_carry, cudaStream_t st);
+                         int64_t from, int64_t count, int16_t* new_carry, cudaStream_t st, bool beside = false);
 // out[t * ld + R m + k] = src[(k * n_tones + t) * src_ld + m] for R m + k < F:
 // the R phase passes' tone rows interleaved into [tone][frame].
 cudaError_t interleave_tones(const void* src, int64_t src_ld, int R, int n_tones, int64_t F, void* out,
