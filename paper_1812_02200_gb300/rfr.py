@@ -147,10 +147,27 @@ def word_to_bin(word: int, n: int) -> int:
     return int(_lib.rfr_word_to_bin(int(word) & (2 ** 64 - 1), int(n)))
 
 
+_raw_stream = None
+
+
+def _find_raw_stream():
+    """The current stream's address on the current device.  The direct query
+    takes 0.4 us where building a torch.cuda.Stream object for it takes 3, a
+    quarter of a small push's host time."""
+    import torch
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None:
+        return lambda: torch.cuda.current_stream().cuda_stream
+    device = torch.cuda.current_device
+    return lambda: raw(device())
+
+
 def _stream_ptr(stream):
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        global _raw_stream
+        if _raw_stream is None:
+            _raw_stream = _find_raw_stream()
+        return _raw_stream()
     return getattr(stream, "cuda_stream", stream)
 
 
