@@ -346,17 +346,6 @@ rfr_status ensure_scratch(rfr_plan* p, int64_t n) {
     const int64_t F = frames_for_len(p, std::max<int64_t>(p->cl, p->W - 1) + n);
     if (p->mode == RFR_MODE_PFB && p->gen && F > 0) RFR_CUDA(p, rfr::gen_plan_reserve(&p->gplan, F));
     if (p->mode == RFR_MODE_PFB && p->phase_R > 1) RFR_CUDA(p, ensure_pass_tones(p, F, nullptr));
-    if (p->mode == RFR_MODE_PFB && !p->gen && p->phase_R == 1 && rfr::pfb_split16(p->log2n, p->Tk)) {
-        const int64_t lv = std::max<int64_t>(p->cl, p->W - 1) + n;
-        if (lv > p->view_cap) {
-            cudaDeviceSynchronize();
-            dev_free(p->d_view);
-            p->d_view = nullptr;
-            p->view_cap = 0;
-            RFR_CUDA(p, dev_alloc(&p->d_view, static_cast<size_t>(lv) * 4));
-            p->view_cap = lv;
-        }
-    }
     if (p->mode == RFR_MODE_PFB && !p->gen && p->phase_R == 1 && rfr::pfb_pre_rows(p->log2n, p->Tk)) {
         const rfr_status rs = ensure_pre_rows(p, F, nullptr);
         if (rs != RFR_OK) return rs;
@@ -419,36 +408,6 @@ rfr_status push_core(rfr_plan* p, const int16_t* iq, int64_t n, const rfr_output
             if (p->phase_R > 1) {
                 rfr_status rs = phase_passes(p, L, o, lv, F, st);
                 if (rs != RFR_OK) return rs;
-            } else if (!p->gen && rfr::pfb_split16(p->log2n, p->Tk)) {
-                // the two-pass 16-tap form needs a 16-byte aligned view: an
-                // unaligned push goes through a contiguous copy of it.  Scratch
-                // that has to grow is sized for a push of n samples after any
-                // carry (so that a later push of that size never grows it)
-                const int64_t lv_max = std::max<int64_t>(p->cl, p->W - 1) + n;
-                const bool aligned = (reinterpret_cast<uintptr_t>(iq) % 16 == 0) && (p->cl % 4 == 0) &&
-                                     (reinterpret_cast<uintptr_t>(carry) % 16 == 0);
-                if (!aligned) {
-                    if (lv > p->view_cap) {
-                        const rfr_status rs = refuse_growth_in_capture(p, st);
-                        if (rs != RFR_OK) return rs;
-                        cudaDeviceSynchronize();
-                        dev_free(p->d_view);
-                        p->d_view = nullptr;
-                        p->view_cap = 0;
-                        RFR_CUDA(p, dev_alloc(&p->d_view, static_cast<size_t>(lv_max) * 4));
-                        p->view_cap = lv_max;
-                    }
-                    RFR_CUDA(p, rfr::carry_update(carry, p->cl, iq, n, 0, lv, p->d_view, st));
-                    L.carry = p->d_view;
-                    L.cl = 0;
-                    L.buf = p->d_view;
-                    L.n = lv;
-                }
-                const rfr_status rs = ensure_pre_rows(p, F <= p->pre_cap ? F : frames_for_len(p, lv_max), st);
-                if (rs != RFR_OK) return rs;
-                L.pre = p->d_pre;
-                L.pre_cap = p->pre_cap;
-                RFR_CUDA(p, rfr::pfb_launch(L, st));
             } else {
                 if (!p->gen && rfr::pfb_pre_rows(p->log2n, p->Tk) && !L.cluster) {
                     // FIR pre-sum rows, sized for a push of n samples after any
@@ -574,7 +533,7 @@ void destroy(rfr_plan* p) {
                     static_cast<void*>(p->d_words), static_cast<void*>(p->d_rates), static_cast<void*>(p->d_h32), p->d_c32, p->d_bhi, p->d_blo,
                     static_cast<void*>(p->d_status), static_cast<void*>(p->d_carry[0]),
                     static_cast<void*>(p->d_carry[1]), p->d_xs_hi, p->d_xs_lo, p->d_rot, p->d_qfull, p->d_b3, p->d_g3, p->d_xs3,
-                    p->d_qtones, static_cast<void*>(p->d_view), p->d_ptones, p->d_pre})
+                    p->d_qtones, p->d_ptones, p->d_pre})
         dev_free(q);
     for (int i = 0; i < rfr_plan::kStageBufs; ++i) {
         dev_free(p->d_stage_in[i]);
@@ -730,6 +689,18 @@ rfr_status rfr_plan_create(rfr_plan** out, int32_t channels, int32_t taps, const
         for (int s = 0; s < nt; ++s) p->bins[s] = rfr::word_to_bin(p->words[s], channels);
         std::vector<float> tw = p->gen ? std::vector<float>() : make_twiddles(p->log2n);
         p->tw_count = static_cast<int>(tw.size() / 2);
+        if (!p->gen && p->log2n >= 12) {
+            // again from the third pass on, the low eight index bits 16 h + 2 w + b
+            // as 32 w + 2 h + b: consecutive for the lanes of pfb_rows_kernel
+            const int at = 240, n = p->tw_count - at;
+            tw.resize(tw.size() + 2 * static_cast<size_t>(n));
+            for (int i = 0; i < n; ++i) {
+                const int lo = i & 255, h = lo >> 4, w = (lo >> 1) & 7, b = lo & 1;
+                const size_t to = static_cast<size_t>(p->tw_count + (i & ~255) + 32 * w + 2 * h + b);
+                tw[2 * to] = tw[2 * static_cast<size_t>(at + i)];
+                tw[2 * to + 1] = tw[2 * static_cast<size_t>(at + i) + 1];
+            }
+        }
         std::vector<float> tw_cl;
         const int ccl = p->gen ? 0 : rfr::pfb_cluster_size(p->log2n, p->Tk);
         if (ccl > 0) {

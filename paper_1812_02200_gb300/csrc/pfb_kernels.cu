@@ -15,10 +15,10 @@
 //  TMEM   (N = 4096, T <= 8, 16-byte aligned pushes): the FP32 delay line in
 //         tensor memory, int16 blocks by 1-D TMA, spectrum rows by TMA bulk
 //         stores and tone groups by 2-D TMA tensor stores (see below); the
-//         symmetric-tap form (T = 8, exactly symmetric taps, the plan default;
-//         pushes of any alignment) works on two frames at a time with two
-//         groups of warps and also runs the phase passes of oversampled plans; a seeded form continues FIR sums from pre-sum
-//         rows (N = 4096 with 9..16 taps: first-half pass + taps 8..15).
+//         symmetric-tap form (T = 4 or 8, exactly symmetric taps, the plan
+//         default; pushes of any alignment) works on two frames at a time with
+//         two groups of warps and also runs the phase passes of oversampled
+//         plans.
 //  TILE   (N = 64 .. 1024, T <= 16; N = 2048, T = 5 .. 8 or unaligned): one CTA
 //         per 4096 points, the FIR of a branch's consecutive frames in one
 //         thread (each sample converted once for all of them), any alignment.
@@ -31,10 +31,12 @@
 //         taps of the thread's 16 branches live in registers.
 //  CLUSTER (N = 8192, 16384, T <= 8; a plan choice): N/4096 CTAs per frame
 //         sharing the FFT through distributed shared memory.
-//  DIRECT (any other N <= 16384, T <= 16): the in-CTA FFT per frame, its FIR
-//         either a separate DRAM-streaming pre-sum pass (fir_pre_kernel; N =
-//         8192, 16384 with T > 4, N = 2048 with T > 8) or read from global
-//         memory inside the kernel (L2 serves the T-fold reuse).
+//  ROWS   (N = 4096 with T > 8, N = 8192, 16384): the FFT of FIR sums that a
+//         DRAM-streaming pre-sum pass (fir_pre_kernel) left in memory, exchanges
+//         in place and mostly within warps.
+//  DIRECT (N = 16 and 32 with T > 8; N = 2048 with T > 8): the in-CTA FFT per
+//         frame, its FIR read from global memory inside the kernel (L2 serves
+//         the T-fold reuse) or, N = 2048, from the pre-sum pass.
 // TILE, RING and DIRECT run the in-CTA FFT of fft_dev.cuh (TMEM the same passes
 // written out for N = 4096); all write
 //   full[(frame_offset + j) * full_ld + c]      (natural bin order)
@@ -81,7 +83,7 @@ struct PfbArgs {
     int* status;
     int tone_cs;             // symmetric-tap kernel: tone columns of consecutive frames this far apart
     int rot;                 // symmetric-tap kernel: bin c multiplied by (-i)^((c * rot) mod 4)
-    const float2* pre;       // TMEM kernel <T, true>: [F][4096] FIR partial sums the frames' FIR starts from
+    const float2* pre;       // ROWS, DIRECT <.., true>: [F][N] FIR sums of the frames
     int64_t q_lo, q_hi;      // iteration range
     int64_t iters_per_cta;
     int ring_sb;             // RING: super-blocks in the ring
@@ -289,10 +291,7 @@ __host__ __device__ __forceinline__ TmemLayout tmem_layout(int tw_count, int nb)
     return L;
 }
 
-// PRE: each frame's FIR accumulators start from a.pre's row of the frame
-// (the first half of a 16-tap FIR, see fir_pre_kernel) instead of zero;
-// the next frame's row is loaded while this frame's FFT runs.
-template <int T, bool PRE>
+template <int T>
 __global__ void __launch_bounds__(kRingThreads, 1)
     pfb_tmem_kernel(const PfbArgs a, const __grid_constant__ CUtensorMap tm_tones) {
     constexpr int N = 4096, NT = 256;
@@ -347,16 +346,6 @@ __global__ void __launch_bounds__(kRingThreads, 1)
 
     bool ok = true;
     float are[16], aim[16];
-    bool pre_loaded = false;
-    auto load_pre = [&](int64_t jj) {
-        const float2* row = a.pre + jj * N + tf;
-#pragma unroll
-        for (int r = 0; r < 16; ++r) {
-            const float2 q = __ldg(row + r * NT);
-            are[r] = q.x;
-            aim[r] = q.y;
-        }
-    };
     for (int64_t b = b0; b < b1; ++b) {
         const int s = static_cast<int>(b % kTmemStage);
         if (!mbar_wait(&bars[s], static_cast<uint32_t>(((b - b0) / kTmemStage) & 1), a.status)) {
@@ -383,13 +372,8 @@ __global__ void __launch_bounds__(kRingThreads, 1)
                 issue_sb_tma(a, b + kTmemStage, need, stage + s * N, &bars[s]);
             continue;
         }
-        if constexpr (PRE) {
-            if (!pre_loaded) load_pre(j);                        // the CTA's first frame
-            pre_loaded = false;
-        } else {
 #pragma unroll
-            for (int r = 0; r < 16; ++r) are[r] = aim[r] = 0.f;
-        }
+        for (int r = 0; r < 16; ++r) are[r] = aim[r] = 0.f;
         // taps in order t = 0..T-1; each slot read as two 16-column halves,
         // the next half's load in flight while this half's FMAs issue
         uint32_t xa[16], xb[16];
@@ -421,12 +405,6 @@ __global__ void __launch_bounds__(kRingThreads, 1)
         float2 v[16];
 #pragma unroll
         for (int r = 0; r < 16; ++r) v[r] = make_float2(are[r], aim[r]);
-        if constexpr (PRE) {
-            if (j + 1 < jb) {
-                load_pre(j + 1);
-                pre_loaded = true;
-            }
-        }
         // 4096-point Stockham FFT, 3 radix-16 passes (as fft_frame<12>):
         // pass 0 -> P, pass 1 P -> Q, pass 2 Q -> registers; spectrum -> P.
         float2* const P = (j & 1) ? xb1 : xb0;
@@ -539,7 +517,7 @@ __global__ void __launch_bounds__(kRingThreads, 1)
 }
 
 // ------------------------------------------------- TMEM, symmetric taps
-// N = 4096, T = 8 with an exactly symmetric prototype, h[j] = h[8N - 1 - j]
+// N = 4096, T = 4 or 8 with an exactly symmetric prototype, h[j] = h[TN - 1 - j]
 // (the plan builds it so).  Same stream view, TMEM delay line, sum order
 // and outputs as pfb_tmem_kernel (bit-identical results), for any alignment of
 // the push.
@@ -555,8 +533,8 @@ __global__ void __launch_bounds__(kRingThreads, 1)
 //   - FIR group.  Lanes l and 31 - l of a warp own the mirrored FFT rows tf and
 //     255 - tf (row tf = the points tf + 256 r).  A thread filters its row's
 //     points r < 8 and the mirror points (255 - tf, 15 - r), whose taps are the
-//     same values in reverse tap order, so it holds 64 tap registers instead of
-//     128; one warp shuffle per value then swaps the mirrored halves so that
+//     same values in reverse tap order, so it holds 8 T tap registers instead of
+//     16 T; one warp shuffle per value then swaps the mirrored halves so that
 //     every thread has its whole row for the first radix-16 pass.  No thread
 //     reads another's delay line, so the group needs no barrier of its own.
 //   - FFT group.  Warp w takes columns k = 2w, 2w + 1 of pass 1's 256 x 16 view
@@ -608,12 +586,12 @@ __host__ __device__ __forceinline__ SymLayout sym_layout(int nb) {
     return L;
 }
 
-template <bool PHASE>
-    allow_dependents();
+template <int T, bool PHASE>
 __global__ void __launch_bounds__(kSymThreads, 1)
     pfb_tmem_sym_kernel(const PfbArgs a, const __grid_constant__ CUtensorMap tm_tones,
                         const __grid_constant__ CUtensorMap tm_full) {
-    constexpr int N = 4096, NT = 256, T = 8, S = kSymStage;
+    constexpr int N = 4096, NT = 256, S = kSymStage;
+    static_assert(T <= kTmemSlots, "delay line fits in TMEM");
     // PHASE: a phase pass of an oversampled plan (tone columns a.tone_cs
     // apart, bins turned by (-i)^(c * a.rot)); otherwise adjacent columns, no turn
     const int64_t tcs = PHASE ? a.tone_cs : 1;
@@ -633,6 +611,7 @@ __global__ void __launch_bounds__(kSymThreads, 1)
     uint32_t* const tmem_holder = reinterpret_cast<uint32_t*>(tfull + 1);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    allow_dependents();
     const int64_t shift = a.frame_offset & (kToneGroup - 1);
     const int64_t ja = max_i64(0, static_cast<int64_t>(blockIdx.x) * a.iters_per_cta - shift);
     const int64_t jb = min_i64(a.F, static_cast<int64_t>(blockIdx.x + 1) * a.iters_per_cta - shift);
@@ -1263,11 +1242,10 @@ __global__ void __launch_bounds__(kRingThreads, 1)
 
 // -------------------------------------------------------------- DIRECT
 // PRE: the frames' FIR sums come from a.pre (fir_pre_kernel) instead of
-// the in-kernel FIR.  Launched with max(N/16, 256) threads; below N = 8192
-// four CTAs per SM with the in-kernel FIR (64 registers), two with PRE.
+// the in-kernel FIR.  256 threads; four CTAs per SM with the in-kernel FIR (64
+// registers), two with PRE.
 template <int LOG2N, bool PRE>
-__global__ void __launch_bounds__(LOG2N >= 14 ? 1024 : (LOG2N == 13 ? 512 : 256),
-                                  LOG2N >= 13 ? 1 : (PRE ? 2 : 4))
+__global__ void __launch_bounds__(256, PRE ? 2 : 4)
     pfb_direct_kernel(const PfbArgs a) {
     constexpr int N = 1 << LOG2N;
     constexpr int NT = N / 16;
@@ -1293,8 +1271,7 @@ __global__ void __launch_bounds__(LOG2N >= 14 ? 1024 : (LOG2N == 13 ? 512 : 256)
 #pragma unroll
             for (int r = 0; r < 16; ++r) v[r] = __ldg(row + r * NT);
             // the next frame's rows on their way to L2 (one request per
-            // 128-byte line: 16 consecutive points; at N = 16384 it costs a
-            // few spilled registers and still measured 9 % faster)
+            // 128-byte line: 16 consecutive points)
             const int64_t jn = j + static_cast<int64_t>(gridDim.x) * G;
             if (jn < a.F && (tf & 15) == 0) {
                 const float2* nrow = a.pre + jn * N + tf;
@@ -1332,7 +1309,6 @@ __global__ void __launch_bounds__(LOG2N >= 14 ? 1024 : (LOG2N == 13 ? 512 : 256)
 // Why: the int16 ring's FIR converted each sample once per tap (8 times at T =
 // 8), 56 of 86 instructions a point, on 8 warps an SM; here it is converted (RF +
 // T - 1) / RF times, on 24 warps an SM (two CTAs an SM measured 10-20 % slower, 512
-    allow_dependents();
 // threads and 8192 points 10-20 % slower at N = 1024).  More than 8 taps took a
 // pre-sum pass through memory (16 bytes a sample more).
 // Measured, 2^25 samples, full + N / 4 tones, before -> after (us):
@@ -1356,6 +1332,7 @@ __global__ void __launch_bounds__(kTileThreads, 3) pfb_tile_kernel(const PfbArgs
     const int tid = threadIdx.x;
     const int64_t j0 = static_cast<int64_t>(blockIdx.x) * G;
     const int T = a.T;
+    allow_dependents();
     {
         // frames g0 .. g0 + RF - 1 of the tile, branches p0 + c THREADS
         const int p0 = tid & (N - 1 < THREADS - 1 ? N - 1 : THREADS - 1);
@@ -1408,6 +1385,123 @@ __global__ void __launch_bounds__(kTileThreads, 3) pfb_tile_kernel(const PfbArgs
     pfb_outputs<LOG2N>(a, v, (LOG2N > 8 ? xb : xa), g, tf, j, j < a.F, G, j0);
 }
 
+// ---------------------------------------------------------------- ROWS
+// N = 4096 RF, RF = 1, 2, 4: the FFT of frames whose FIR sums are in memory
+// (a.pre, fir_pre_kernel), N / 16 threads a frame, the whole frame in one
+// shared-memory buffer and every exchange in place.  The passes are those of
+// fft_frame<LOG2N> (16, 16, 16, RF: same butterflies and twiddles, the same bits);
+// what differs is who meets whom.  Element (row, k) of the buffer is point 16 row +
+// k.  Pass 1 reads rows RF h + l + 16 RF r (r < 16) of column k, pass 2 needs for
+// the same (l, k) the 16 x 16 transpose over (h, r): warp (l, k / 2) holds both
+// columns' 16 threads h, so that exchange stays within the warp.  The last pass
+// (RF > 1) combines l = 0 .. RF - 1: a barrier of the RF warps of a column pair.
+// Left are four barriers of the CTA a frame (three for RF = 1; the FFT through
+// fft_frame took eight), the first behind the next frame's loads.  The spectrum leaves by swizzled TMA stores
+// of 4096 bins.
+// Rows are placed so that neither eight consecutive rows (pass 0's stores) nor
+// eight rows RF apart (everything else) share a bank: rows' low bits XOR bits 3
+// (and 4), then 16-byte pairs XOR the row mod 8, TMA's 128-byte swizzle.  All maps
+// are linear over XOR, so a thread's places are one address XOR constants.
+// Measured, 2^26 samples, full + 1000 tones, T = 4 / 8 / 16, before -> after (us):
+//   N = 4096      -   /  -  / 526 ->  -  /  -  / 481   (was: the pre-sum of taps 0..7,
+//                then the TMEM kernel for taps 8..15 on top of it)
+//   N = 8192     544 / 479 / 512 -> 389 / 407 / 441
+//   N = 16384    467 / 487 / 523 -> 404 / 424 / 460   (T = 4 was FIR in the kernel)
+// (floors 138, 128, 123).  The twiddles are read in lane order from a permuted
+// table: in natural order, 16 lines a load, the same kernel took 568 at T = 8.
+template <int LOG2N>
+__global__ void __launch_bounds__(1 << (LOG2N - 4), 1 << (14 - LOG2N))
+    pfb_rows_kernel(const PfbArgs a, const __grid_constant__ CUtensorMap tm_full) {
+    constexpr int N = 1 << LOG2N, NT = N / 16, RF = N / 4096, NQ = 16 / RF;
+    extern __shared__ __align__(1024) unsigned char smem[];
+    float2* const buf = reinterpret_cast<float2*>(smem);
+    auto place_row = [](int row) { return row ^ ((row >> 3) & (RF - 1)); };
+    // element (row, 0) of a buffer; linear over XOR in row
+    auto at_row = [&](int row) { return (place_row(row) << 4) | ((place_row(row) & 7) << 1); };
+    const int tid = threadIdx.x, wid = tid >> 5, lane = tid & 31;
+    const int w = wid & 7, l = wid >> 3, h = lane >> 1, k = 2 * w + (lane & 1);
+    const int own = at_row(RF * h + l) ^ k;
+    const int nat = sym_swizzle(16 * h + k) + 256 * l;
+    const float2* const twl = a.tw + a.tw_count + 32 * w + lane;   // passes 2 and 3, in lane order
+    float4* const row0 = reinterpret_cast<float4*>(buf) + place_row(tid) * 8;
+    const int x0 = place_row(tid) & 7;
+    float2 v[16];
+    auto load = [&](int64_t j) {
+        const float2* row = a.pre + j * N + tid;
+#pragma unroll
+        for (int r = 0; r < 16; ++r) v[r] = __ldg(row + r * NT);
+    };
+    if (static_cast<int64_t>(blockIdx.x) < a.F) load(blockIdx.x);
+    for (int64_t j = blockIdx.x; j < a.F; j += gridDim.x) {
+        const int64_t jn = j + gridDim.x;
+        dft16(v);                                                // pass 0
+        if (tid == 0) bulk_wait_read_all();
+        __syncthreads();                                         // the frame before has left the buffer
+#pragma unroll
+        for (int r = 0; r < 16; r += 2) row0[(r / 2) ^ x0] = make_float4(v[r].x, v[r].y, v[r + 1].x, v[r + 1].y);
+        if (jn < a.F && (tid & 15) == 0) {
+            // the next frame's rows on their way to L2 (a request per 128-byte line)
+            const float2* nrow = a.pre + jn * N + tid;
+#pragma unroll
+            for (int r = 0; r < 16; ++r) prefetch_l2(nrow + r * NT);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < 16; ++r) v[r] = buf[own + r * NT];
+#pragma unroll
+        for (int r = 1; r < 16; ++r) v[r] = cmul(v[r], __ldg(a.tw + (r - 1) * 16 + k));
+        dft16(v);                                                // pass 1
+        __syncwarp();
+#pragma unroll
+        for (int r = 0; r < 16; ++r) buf[(own ^ at_row(RF * r)) + r * NT] = v[r];
+        __syncwarp();
+#pragma unroll
+        for (int r = 0; r < 16; ++r) v[r] = buf[(own ^ at_row(RF * r)) + h * NT];
+#pragma unroll
+        for (int r = 1; r < 16; ++r) v[r] = cmul(v[r], __ldg(twl + (r - 1) * 256));
+        dft16(v);                                                // pass 2: points 4096 l + 16 h + k + 256 r
+        __syncwarp();
+        if constexpr (RF == 1) {
+            // the spectrum's places are the thread's own
+#pragma unroll
+            for (int r = 0; r < 16; ++r) buf[nat + r * NT] = v[r];
+        } else {
+#pragma unroll
+        for (int r = 0; r < 16; ++r) buf[own + r * NT] = v[r];
+        asm volatile("bar.sync %0, %1;" ::"r"(1 + w), "n"(32 * RF) : "memory");
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+#pragma unroll
+            for (int m = 0; m < RF; ++m) v[q * RF + m] = buf[(own ^ (18 * (l ^ m))) + (l + RF * q) * NT];
+#pragma unroll
+            for (int m = 1; m < RF; ++m) v[q * RF + m] = cmul(v[q * RF + m], __ldg(twl + 3840 + (m - 1) * 4096 + 256 * (l + RF * q)));
+            dft_small<RF>(v + q * RF);                           // bins 16 h + k + 256 l + NT q + 4096 m
+        }
+        __syncthreads();                                         // every read of the exchange is done
+#pragma unroll
+        for (int q = 0; q < NQ; ++q)
+#pragma unroll
+            for (int m = 0; m < RF; ++m) buf[nat + NT * q + 4096 * m] = v[q * RF + m];
+        }
+        fence_proxy_async_smem();
+        if (jn < a.F) load(jn);
+        __syncthreads();                                         // spectrum complete
+        const int64_t o = a.frame_offset + j;
+        if (a.full_bulk) {
+            if (tid == 0) {
+#pragma unroll
+                for (int m = 0; m < RF; ++m) tma_store_3d(&tm_full, 0, 256 * m, static_cast<int32_t>(o), buf + 4096 * m);
+                bulk_commit();
+            }
+        } else if (a.full) {
+            float2* out = a.full + o * a.full_ld;
+            for (int i = tid; i < N; i += NT) out[i] = buf[sym_swizzle(i)];
+        }
+        for (int t = tid; t < a.n_tones; t += NT) a.tones[t * a.tones_ld + o] = buf[sym_swizzle(__ldg(a.bins + t))];
+    }
+    if (tid == 0) bulk_wait_all();
+}
+
 // ------------------------------------------------------------ launcher
 namespace {
 
@@ -1453,7 +1547,7 @@ cudaError_t launch_direct(PfbArgs a, int n_sms, int max_smem, cudaStream_t st) {
     const int64_t n_iter = (a.F + G - 1) / G;
     int per_sm = 1;
     // pre-sum instances only for the shapes that take them (pfb_pre_rows)
-    constexpr bool kPre = LOG2N == 11 || LOG2N == 13 || LOG2N == 14;
+    constexpr bool kPre = LOG2N == 11;
     if (a.pre && !kPre) return cudaErrorInvalidValue;
     auto k = a.pre ? pfb_direct_kernel<LOG2N, kPre> : pfb_direct_kernel<LOG2N, false>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -1484,9 +1578,8 @@ cudaError_t launch_tile(const PfbArgs& a, cudaStream_t st) {
 // FIR sums of the first T (<= TMAX) taps of every frame of the stream view
 // [carry | buffer] (N channels):
 //   pre[j][p] = sum_{t<T} h[t N + p] x[(j + t) N + p],
-// FMAs in tap order from zero, the order of the fused kernels' FIRs, which
-// continue these sums (the 16-tap N = 4096 form: taps 0..7 here, 8..15 in
-// the TMEM kernel) or take them whole (the direct kernel).  A thread takes
+// FMAs in tap order from zero, the order of the fused kernels' FIRs (the rows and
+// direct kernels take the sums from here).  A thread takes
 // P points (kPreThreads apart) of G consecutive frames and loads and
 // converts each of their G + T - 1 input blocks once; the frame
 // groups of a point range are consecutive CTAs, so the blocks two groups
@@ -1563,9 +1656,9 @@ cudaError_t launch_pre_n(const PfbArgs& a, int T, float2* pre, cudaStream_t st) 
 // points at N = 16384.
 cudaError_t launch_pre(const PfbArgs& a, int lg, int T, float2* pre, cudaStream_t st) {
     if (T < 1 || T > 16) return cudaErrorInvalidValue;
+    if (T <= 4 && lg >= 13) return lg == 13 ? launch_pre_n<4, 2, 8, 13>(a, T, pre, st) : launch_pre_n<4, 2, 8, 14>(a, T, pre, st);
     if (T <= 8) {
         switch (lg) {
-        case 12: return launch_pre_n<8, 2, 8, 12>(a, T, pre, st);
         case 13: return launch_pre_n<8, 2, 8, 13>(a, T, pre, st);
         case 14: return launch_pre_n<8, 2, 8, 14>(a, T, pre, st);
         default: return cudaErrorInvalidValue;
@@ -1574,13 +1667,14 @@ cudaError_t launch_pre(const PfbArgs& a, int lg, int T, float2* pre, cudaStream_
     // more taps: one point and eight frames per thread
     switch (lg) {
     case 11: return launch_pre_n<16, 1, 8, 11>(a, T, pre, st);
+    case 12: return launch_pre_n<16, 1, 8, 12>(a, T, pre, st);
     case 13: return launch_pre_n<16, 1, 8, 13>(a, T, pre, st);
     case 14: return launch_pre_n<16, 1, 8, 14>(a, T, pre, st);
     default: return cudaErrorInvalidValue;
     }
 }
 
-template <int T, bool PRE = false>
+template <int T>
 cudaError_t launch_tmem(PfbArgs a, int n_sms, int max_smem, cudaStream_t st) {
     a.nb_smem = (a.n_tones > 0 && a.n_tones <= kTonesPerThread * kRingThreads &&
                  tmem_layout(a.tw_count, a.n_tones).total <= static_cast<size_t>(max_smem))
@@ -1611,13 +1705,44 @@ cudaError_t launch_tmem(PfbArgs a, int n_sms, int max_smem, cudaStream_t st) {
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS)
             a.tones_tma = 1;
     }
-    auto k = pfb_tmem_kernel<T, PRE>;
+    auto k = pfb_tmem_kernel<T>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     k<<<static_cast<unsigned>(grid2), kRingThreads, smem, st>>>(a, tm);
     return cudaGetLastError();
 }
 
+// Spectrum rows as [frame][N / 16][16] 8-byte elements, boxes of 4096 bins from
+// shared memory in the 128-byte swizzle; false: rows that cannot leave by TMA.
+bool full_row_map(const PfbArgs& a, int n, CUtensorMap* m) {
+    auto enc = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(tmap_encode_tiled_fn());
+    if (!a.full || !enc || (reinterpret_cast<uintptr_t>(a.full) % 16) != 0 || (a.full_ld % 2) != 0 ||
+        a.frame_offset + a.F >= (int64_t(1) << 31))
+        return false;
+    cuuint64_t dims[3] = {16, static_cast<cuuint64_t>(n / 16), static_cast<cuuint64_t>(a.frame_offset + a.F)};
+    cuuint64_t strides[2] = {128, static_cast<cuuint64_t>(a.full_ld) * 8};
+    cuuint32_t box[3] = {16, 256, 1};
+    cuuint32_t estr[3] = {1, 1, 1};
+    return enc(m, CU_TENSOR_MAP_DATA_TYPE_UINT64, 3, a.full, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+template <int LOG2N>
+cudaError_t launch_rows(PfbArgs a, int n_sms, cudaStream_t st) {
+    constexpr int N = 1 << LOG2N;
+    CUtensorMap tf;
+    std::memset(&tf, 0, sizeof tf);
+    a.full_bulk = full_row_map(a, N, &tf) ? 1 : 0;
+    const int smem = N * 8;
+    const cudaError_t e = cudaFuncSetAttribute(pfb_rows_kernel<LOG2N>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    const int64_t grid = std::min<int64_t>(a.F, static_cast<int64_t>(n_sms) << (14 - LOG2N));
+    pfb_rows_kernel<LOG2N><<<static_cast<unsigned>(grid), N / 16, smem, st>>>(a, tf);
+    return cudaGetLastError();
+}
+
+template <int T>
 cudaError_t launch_tmem_sym(PfbArgs a, int n_sms, int max_smem, cudaStream_t st) {
     a.nb_smem = (a.n_tones > 0 && a.n_tones <= kTonesPerThread * kRingThreads &&
                  sym_layout(a.n_tones).total <= static_cast<size_t>(max_smem))
@@ -1637,20 +1762,7 @@ cudaError_t launch_tmem_sym(PfbArgs a, int n_sms, int max_smem, cudaStream_t st)
     std::memset(&tf, 0, sizeof tf);
     a.tones_tma = 0;
     auto enc = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(tmap_encode_tiled_fn());
-    // spectrum rows as [frame][256][16] 8-byte elements, one frame a box, the
-    // kernel's buffers in the 128-byte swizzle
-    a.full_bulk = 0;
-    if (a.full && enc && (reinterpret_cast<uintptr_t>(a.full) % 16) == 0 && (a.full_ld % 2) == 0 &&
-        a.frame_offset + a.F < (int64_t(1) << 31)) {
-        cuuint64_t dims[3] = {16, 256, static_cast<cuuint64_t>(a.frame_offset + a.F)};
-        cuuint64_t strides[2] = {128, static_cast<cuuint64_t>(a.full_ld) * 8};
-        cuuint32_t box[3] = {16, 256, 1};
-        cuuint32_t estr[3] = {1, 1, 1};
-        if (enc(&tf, CU_TENSOR_MAP_DATA_TYPE_UINT64, 3, a.full, dims, strides, box, estr,
-                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
-                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS)
-            a.full_bulk = 1;
-    }
+    a.full_bulk = full_row_map(a, 4096, &tf) ? 1 : 0;
     if (a.nb_smem > 0 && enc && a.tone_cs == 1 && (reinterpret_cast<uintptr_t>(a.tones) % 16) == 0 &&
         (a.tones_ld % 2) == 0 && a.frame_offset + a.F < (int64_t(1) << 31)) {
         cuuint64_t dims[2] = {static_cast<cuuint64_t>(a.frame_offset + a.F), static_cast<cuuint64_t>(a.n_tones)};
@@ -1663,7 +1775,8 @@ cudaError_t launch_tmem_sym(PfbArgs a, int n_sms, int max_smem, cudaStream_t st)
             a.tones_tma = 1;
     }
     const bool phase = a.tone_cs != 1 || a.rot != 0;
-    auto k = phase ? pfb_tmem_sym_kernel<true> : pfb_tmem_sym_kernel<false>;
+    if (phase && T != 8) return cudaErrorInvalidValue;              // phase passes are 8-tap plans'
+    auto k = phase ? pfb_tmem_sym_kernel<8, true> : pfb_tmem_sym_kernel<T, false>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     // the kernel's register split waits forever unless the launch holds it
@@ -1759,20 +1872,15 @@ cudaError_t dispatch_ring_T(PfbArgs a, int tk, int n_sms, int max_smem, int la, 
 
 bool pfb_uses_ring(int log2n, int taps) { return log2n >= 4 && log2n <= 12 && taps <= 8; }
 int pfb_cluster_size(int log2n, int taps) { return (log2n == 13 || log2n == 14) && taps <= 8 ? 1 << (log2n - 12) : 0; }
-bool pfb_split16(int log2n, int taps) { return log2n == 12 && taps == 16; }
-// Where the direct kernel takes its FIR from a pre-sum pass (measured, 2^28
-// samples, full + tones): N = 8192 at every T (T = 8: 3.14 -> 1.81 ms),
-// N = 16384 from T = 8 on (2.73 -> 1.85 ms; T = 4 1.87 -> 2.14 ms, so not
-// there), N = 2048 with T > 8 (smaller N run on the tile kernel).
+// Shapes whose FIR is a pre-sum pass: those of the rows kernel, and N = 2048 with
+// T > 8 (2^25 samples 238 us; the tile kernel 277).
 bool pfb_pre_rows(int log2n, int taps) {
-    if (pfb_split16(log2n, taps)) return true;
-    if (log2n == 13) return true;
-    if (log2n == 14) return taps > 4;
-    return log2n == 11 && taps > 8;
+    if (log2n >= 13) return true;
+    return (log2n == 11 || log2n == 12) && taps > 8;
 }
 int pfb_kernel_taps(int log2n, int taps) {
     if (pfb_uses_ring(log2n, taps) || pfb_cluster_size(log2n, taps) > 0) return taps <= 4 ? 4 : 8;
-    if (log2n == 12 && taps > 8 && taps <= 16) return 16;     // first-half pass + seeded TMEM kernel (pfb_launch)
+    if (log2n == 12 && taps > 8 && taps <= 16) return 16;     // zero-padded at the oldest end
     return taps;
 }
 
@@ -1813,39 +1921,15 @@ cudaError_t pfb_launch(const PfbLaunch& L, cudaStream_t st) {
         return L.taps_kernel == 4 ? launch_cluster<4, 4>(a, L.n_sms, L.max_smem, st)
                                   : launch_cluster<4, 8>(a, L.n_sms, L.max_smem, st);
     }
-    if (pfb_split16(lg, L.taps_kernel)) {
-        // N = 4096, T = 16 (9 .. 16 taps, zero-padded at the oldest end):
-        // the FIR of taps 0..7 over the window's first 8 blocks by
-        // fir_pre_kernel into L.pre, then the TMEM kernel over the view 8N
-        // samples on with taps 8..15, its FIR sums starting from those rows
-        // (the same FMA chain as one 16-tap FIR).  The caller passes a
-        // 16-byte aligned view and L.pre for at least F frames.
-        if (a.tone_cs != 1 || a.rot != 0 || !a.use_tma || !L.pre || L.pre_cap < a.F) return cudaErrorInvalidValue;
-        constexpr int64_t half = int64_t(8) * 4096;
-        PfbArgs a1 = a;
-        a1.T = 8;
-        cudaError_t e = launch_pre(a1, 12, 8, static_cast<float2*>(L.pre), st);
-        if (e != cudaSuccess) return e;
-        PfbArgs a2 = a1;
-        a2.h = a.h + half;
-        if (a.cl >= half) {
-            a2.carry = a.carry + half;
-            a2.cl = a.cl - half;
-        } else {
-            a2.carry = a.carry;
-            a2.cl = 0;
-            a2.buf = a.buf + (half - a.cl);
-            a2.n = a.n - (half - a.cl);
-        }
-        a2.pre = static_cast<const float2*>(L.pre);
-        return launch_tmem<8, true>(a2, L.n_sms, L.max_smem, st);
-    }
     if (a.tone_cs != 1 || a.rot != 0) {
         // phase passes of an oversampled plan: only the symmetric-tap kernel has them
         if (lg != 12 || L.taps_kernel != 8 || !L.sym_taps) return cudaErrorInvalidValue;
-        return launch_tmem_sym(a, L.n_sms, L.max_smem, st);
+        return launch_tmem_sym<8>(a, L.n_sms, L.max_smem, st);
     }
-    if (lg == 12 && L.taps_kernel == 8 && L.sym_taps && L.variant == 0) return launch_tmem_sym(a, L.n_sms, L.max_smem, st);
+    if (lg == 12 && L.sym_taps && L.variant == 0) {
+        if (L.taps_kernel == 8) return launch_tmem_sym<8>(a, L.n_sms, L.max_smem, st);
+        if (L.taps_kernel == 4) return launch_tmem_sym<4>(a, L.n_sms, L.max_smem, st);
+    }
     if (lg == 12 && a.use_tma && L.variant != 1) {
         if (L.taps_kernel == 4) return launch_tmem<4>(a, L.n_sms, L.max_smem, st);
         if (L.taps_kernel == 8) return launch_tmem<8>(a, L.n_sms, L.max_smem, st);
@@ -1883,8 +1967,9 @@ cudaError_t pfb_launch(const PfbLaunch& L, cudaStream_t st) {
     case 4: return launch_direct<4>(a, L.n_sms, L.max_smem, st);
     case 5: return launch_direct<5>(a, L.n_sms, L.max_smem, st);
     case 11: return launch_direct<11>(a, L.n_sms, L.max_smem, st);
-    case 13: return launch_direct<13>(a, L.n_sms, L.max_smem, st);
-    case 14: return launch_direct<14>(a, L.n_sms, L.max_smem, st);
+    case 12: return a.pre ? launch_rows<12>(a, L.n_sms, st) : cudaErrorInvalidValue;
+    case 13: return a.pre ? launch_rows<13>(a, L.n_sms, st) : cudaErrorInvalidValue;
+    case 14: return a.pre ? launch_rows<14>(a, L.n_sms, st) : cudaErrorInvalidValue;
     default: return cudaErrorInvalidValue;
     }
 }

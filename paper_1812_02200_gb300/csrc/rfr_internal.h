@@ -106,11 +106,8 @@ void gen_plan_free(GenPlan* g);
 int pfb_kernel_taps(int log2n, int taps);
 // CTAs per cluster of the cluster PFB kernel (N = 8192, 16384 with T <= 8), else 0.
 int pfb_cluster_size(int log2n, int taps);
-// N = 4096 with 16 kernel taps: a first-half FIR pass, then the TMEM kernel
-// seeded with it (aligned view, PfbLaunch::pre for the frames).
-bool pfb_split16(int log2n, int taps);
-// PFB plans whose pushes take FIR pre-sum rows (PfbLaunch::pre): the 16-tap
-// N = 4096 form and the direct kernel's shapes (N = 8192, 16384; N = 2048 with T > 8).
+// PFB plans whose pushes take FIR pre-sum rows (PfbLaunch::pre): N = 8192 and
+// 16384; N = 2048 and 4096 with T > 8.
 bool pfb_pre_rows(int log2n, int taps);
 cudaError_t pfb_launch(const PfbLaunch& L, cudaStream_t st);
 cudaError_t gen_pfb_launch(const PfbLaunch& L, const GenPlan& g, cudaStream_t st);
@@ -227,11 +224,11 @@ struct TuneConfig {
     int demod_pair = 0;         //   two-SM tiles (0/1)
     int pfb_cluster = 0;        // PFB N = 8192, 16384 with T <= 8: cluster kernel (1) or direct (0)
     bool tuned = false;
-// beside: as a programmatic dependent of the kernel launched before it, which
-// must be one of the same push.
 };
 
 // ------------------------------------------------------------- state
+// beside: as a programmatic dependent of the kernel launched before it, which
+// must be one of the same push.
 cudaError_t carry_update(const int16_t* old_carry, int64_t cl, const int16_t* buf, int64_t n,
                          int64_t from, int64_t count, int16_t* new_carry, cudaStream_t st, bool beside = false);
 // out[t * ld + R m + k] = src[(k * n_tones + t) * src_ld + m] for R m + k < F:
@@ -248,8 +245,6 @@ struct rfr_plan {
     bool sym_taps = false;                     // PFB kernel taps exactly symmetric (Tk == T)
     int phase_R = 1;                           // oversampled N = 4096 PFB: hop = N / phase_R, run as
                                                // phase_R critically sampled passes (see push_core)
-    int16_t* d_view = nullptr;                 // 16-tap N = 4096: contiguous copy of [carry | buffer]
-    int64_t view_cap = 0;                      //   when the push is not 16-byte aligned (samples)
     void* d_ptones = nullptr;                  // phase passes: each pass's tones [pass][tone][frame]
     int64_t ptones_cap = 0;                    //   frames per pass row
     void* d_pre = nullptr;                     // FIR pre-sum rows (rfr::pfb_pre_rows plans)

@@ -1,4 +1,4 @@
-"""The N = 4096, T = 8 filter bank (Sec. III.A) on pushes of any alignment and
+"""The N = 4096 filter banks of 8 and 4 taps (Sec. III.A) on pushes of any alignment and
 length: buffers that start 0 .. 3 samples into a 16-byte line, carries of any
 length (the block across the carry's end), frame counts around one frame per
 CTA and whole tone groups, spectrum rows of odd pitch, up to 1280 tones held on
@@ -15,7 +15,7 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 DEV = "cuda:0"
-N, T = 4096, 8
+N = 4096
 
 
 def _words(nt, seed):
@@ -37,12 +37,12 @@ def _out(F, nt, pad):
     return full, torch.zeros((nt, F + pad), dtype=torch.complex64, device=DEV)
 
 
-@pytest.mark.parametrize("hop", [4096, 2048, 1024])
+@pytest.mark.parametrize("T,hop", [(8, 4096), (4, 4096), (8, 2048), (8, 1024)])
 @pytest.mark.parametrize("off,first,frames,nt,pad", [
     (0, 4096, 1, 5, 0), (1, 1, 3, 1000, 0), (2, 4095, 151, 37, 1), (3, 4097, 152, 1280, 0), (1, 5000, 153, 1281, 0),
     (0, 8190, 610, 1025, 2), (3, 40000, 700, 1000, 0), (2, 3, 2500, 64, 3),
 ])
-def test_any_alignment_equals_aligned_push(lib, hop, off, first, frames, nt, pad):
+def test_any_alignment_equals_aligned_push(lib, T, hop, off, first, frames, nt, pad):
     n = frames * hop + 17
     words = _words(nt, 90 + nt)
     mk = lambda: lib.Plan(N, T, window="kaiser", beta=9.0, words=words, decimation=hop)

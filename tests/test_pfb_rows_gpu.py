@@ -1,0 +1,53 @@
+"""The filter banks whose FIR sums go through memory (Sec. III.A; N = 4096 with
+9 .. 16 taps, N = 8192 and 16384): pushes of one frame to several frames per CTA,
+split anywhere, buffers at any 4-byte offset, spectrum rows that leave by TMA and
+rows of odd pitch that cannot, tones only.  Every form agrees bit for bit, tone
+rows equal their spectrum columns, and both match the FP64 oracle."""
+import numpy as np
+import pytest
+
+import oracle
+import siggen
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+DEV = "cuda:0"
+
+
+@pytest.mark.parametrize("N,T,frames,first,off,pad", [
+    (4096, 9, 1, 4095, 0, 1), (4096, 16, 620, 100001, 1, 1), (4096, 12, 7, 3, 2, 3),
+    (8192, 1, 2, 8191, 3, 1), (8192, 4, 305, 5, 1, 1), (8192, 8, 310, 700000, 0, 3), (8192, 13, 5, 9000, 2, 1),
+    (16384, 3, 153, 16385, 1, 1), (16384, 8, 160, 1234567, 3, 1), (16384, 16, 3, 20000, 2, 5),
+])
+def test_rows_any_split_pitch_and_oracle(lib, N, T, frames, first, off, pad):
+    rng = np.random.default_rng(N + T + frames)
+    n = frames * N + N // 3
+    xn = rng.integers(-8192, 8192, size=(n, 2)).astype(np.int16)
+    nt = 37
+    words = siggen.bin_words(rng.integers(0, N, nt), N)
+    mk = lambda full: lib.Plan(N, T, window="hamming", words=words, full=full)
+    buf = torch.zeros((n + off, 2), dtype=torch.int16, device=DEV)
+    buf[off:] = torch.from_numpy(xn).to(DEV)
+    x = buf[off:]
+    ref = torch.zeros((frames, N), dtype=torch.complex64, device=DEV)
+    rt = torch.zeros((nt, frames), dtype=torch.complex64, device=DEV)
+    p = mk(True)
+    assert p.push_into(torch.from_numpy(xn).to(DEV), ref, rt) == frames
+    full = torch.zeros((frames + 1, N + pad), dtype=torch.complex64, device=DEV)
+    tones = torch.zeros((nt, frames + pad), dtype=torch.complex64, device=DEV)
+    q = mk(True)
+    cut = min(first, n)
+    f0 = q.push_into(x[:cut], full, tones)
+    assert f0 + (q.push_into(x[cut:], full, tones, frame_offset=f0) if cut < n else 0) == frames
+    only = torch.zeros((nt, frames), dtype=torch.complex64, device=DEV)
+    assert mk(False).push_into(x, tones=only) == frames
+    torch.cuda.synchronize()
+    assert torch.equal(full[:frames, :N], ref) and torch.equal(tones[:, :frames], rt) and torch.equal(only, rt)
+    assert not full[frames].any() and not full[:, N:].any() and not tones[:, frames:].any()
+    assert torch.equal(rt, ref[:, torch.from_numpy(p.bins().astype(np.int64)).to(DEV)].T)
+    k = min(frames, 12)
+    h64, _ = oracle.pfb_prototype(N, T, "hamming")
+    y = oracle.pfb(xn[:k * N], N, T, h64)["full"]
+    # FP32 rounding of taps, FIR and up to four passes: a few 1e-7
+    assert np.linalg.norm(ref[:k].cpu().numpy() - y) <= 1e-6 * np.linalg.norm(y)
