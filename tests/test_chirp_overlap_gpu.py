@@ -43,3 +43,29 @@ def test_overlapping_frames_equal_single_frames_and_oracle(lib, L, D, nc, frames
     got = out[:, :k].cpu().numpy()
     # FP32 mixer and sums: a few 1e-7 of the frames' norm
     assert np.linalg.norm(got - ref) <= 1e-5 * np.linalg.norm(ref)
+
+
+def test_mixer_error_bound(lib):
+    """With one tap of weight 1 and samples (8191, 0) a frame is 8191 exp(-i p(m)):
+    the mixer itself.  Bound: phase rounding pi 2^-27, the two series' rounding
+    (a few half units of 2^-24) and the product's 2^-24, 2.5e-7 in all; phases
+    anywhere, and within a few units of every quadrant's edges."""
+    D, frames = 64, 4096
+    rng = np.random.default_rng(3)
+    edges = [(q << 62) + d for q in range(4) for d in (-(1 << 33), -1, 0, 1, 1 << 32)]
+    edges += [(q << 62) + (1 << 61) + d for q in range(4) for d in (-(1 << 33), -1, 0, 1, 1 << 32)]
+    # frame k's sample is m = (k + 1) D - 1: a start word w gives phase w m
+    sw = np.array([e * pow(2 * D - 1, -1, 1 << 64) % (1 << 64) for e in edges], np.uint64)   # phase e at frame 1
+    sw = np.concatenate([sw, siggen.random_words(rng, 24)])
+    rw = np.concatenate([np.zeros(len(edges), np.uint64), rng.integers(0, 2 ** 50, 24).astype(np.uint64)])
+    x = torch.zeros((frames * D, 2), dtype=torch.int16, device=DEV)
+    x[:, 0] = 8191
+    p = lib.Plan.chirp(1, sw, rw, window="rect", decimation=D)
+    out = torch.zeros((len(sw), frames), dtype=torch.complex64, device=DEV)
+    assert p.push_into(x, tones=out) == frames
+    got = out.cpu().numpy() / 8191.0
+    m = (np.arange(frames, dtype=np.uint64) + np.uint64(1)) * np.uint64(D) - np.uint64(1)
+    with np.errstate(over="ignore"):
+        ph = sw[:, None] * m[None, :] + rw[:, None] * (m * m)[None, :]
+    ang = ph.view(np.int64).astype(np.float64) * (np.pi / 2.0 ** 63)
+    assert np.abs(got - np.exp(-1j * ang)).max() <= 2.5e-7
