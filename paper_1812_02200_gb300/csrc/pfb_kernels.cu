@@ -555,11 +555,11 @@ __global__ void __launch_bounds__(kRingThreads, 1)
 // a sample of the block.  The one block across the carry's end is read by
 // plain loads.
 //
-// Measured (full + 1000 tones): 2^28 samples 988 -> 818 us against one group of
+// Measured (full + 1000 tones): 2^28 samples 988 -> 806 us against one group of
 // 8 warps (0.56 -> 0.68 of the HBM copy rate); the hop N/4 plan's four passes
-// and interleave, 2^26 samples, 1312 -> 1134 us; a 2^18-sample push 22.5 -> 16.4
-// us; 3,000,001-sample pushes, tones only, 62 -> 25 us (unaligned ones ran on the
-// ring kernel).  Now the FP32 pipe is 51 % busy, the issue slots 59 % and the
+// and interleave, 2^26 samples, 1312 -> 1117 us; a 2^18-sample push 22.5 -> 12.3
+// us; 3,000,001-sample pushes, tones only, 62 -> 22.5 us (unaligned ones ran on the
+// ring kernel).  4 taps, 2^26 samples: 264 -> 209 us.  Now the FP32 pipe is 51 % busy, the issue slots 59 % and the
 // shared-memory pipe 59 %.  Register splits of 144 / 112 and 160 / 96 measured
 // 870 and 830 us; one warp refilling the stage always 839; gathering the tones
 // behind the next frame's first loads 897.
@@ -569,6 +569,7 @@ constexpr int kSymSlotWords = 4096 + 4;
 constexpr int kSymFirRegs = 152, kSymFftRegs = 104, kSymLaunchRegs = 128;
 static_assert(256 * (kSymFirRegs + kSymFftRegs) <= kSymThreads * kSymLaunchRegs, "register split");
 constexpr size_t kSymXb = static_cast<size_t>(4096) * 8;
+constexpr int kSymTwRow = 18;                      // pass 1's twiddles: row k, r < 16 (two rows' pairs meet no bank)
 __host__ __device__ __forceinline__ int sym_swizzle(int i) { return i ^ (((i >> 4) & 7) << 1); }
 struct SymLayout {
     size_t b2, stage, tw, tile, bars, total;
@@ -578,7 +579,7 @@ __host__ __device__ __forceinline__ SymLayout sym_layout(int nb) {
     L.b2 = 2 * kSymXb;                                             // two spectra
     L.stage = L.b2 + 2 * kSymXb;
     L.tw = L.stage + static_cast<size_t>(kSymStage) * kSymSlotWords * 4;   // pass 1's twiddles
-    size_t o = (L.tw + 240 * 8 + 127) / 128 * 128;
+    size_t o = (L.tw + 16 * kSymTwRow * 8 + 255) / 256 * 256;
     L.tile = o;
     o += static_cast<size_t>((nb + kToneBox - 1) / kToneBox * kToneBox) * kToneGroup * 8;
     L.bars = o;
@@ -602,7 +603,7 @@ __global__ void __launch_bounds__(kSymThreads, 1)
     float2* const B2 = reinterpret_cast<float2*>(smem + lay.b2);
     uint32_t* const stage = reinterpret_cast<uint32_t*>(smem + lay.stage);
     float2* const tw1 = reinterpret_cast<float2*>(smem + lay.tw);
-    float2* const tile = reinterpret_cast<float2*>(smem + lay.tile);   // tone t, group frame q at t*kToneGroup + q
+    float2* const tile = reinterpret_cast<float2*>(smem + lay.tile);   // tone t, group frame q at tile_at(t, q)
     uint64_t* const sfull = reinterpret_cast<uint64_t*>(smem + lay.bars);
     uint64_t* const sempty = sfull + S;
     uint64_t* const b0full = sempty + S;
@@ -610,6 +611,9 @@ __global__ void __launch_bounds__(kSymThreads, 1)
     uint64_t* const tfull = b0empty + 2;                               // tone tile complete
     uint32_t* const tmem_holder = reinterpret_cast<uint32_t*>(tfull + 1);
 
+    // the tone stores' 32-byte swizzle: the halves of every other four rows swapped
+    // (half the bank conflicts of the gather's column of 8-byte values)
+    auto tile_at = [](int t, int q) { return (t * kToneGroup + q) ^ (((t >> 2) & 1) << 1); };
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     allow_dependents();
     const int64_t shift = a.frame_offset & (kToneGroup - 1);
@@ -634,7 +638,7 @@ __global__ void __launch_bounds__(kSymThreads, 1)
         mbar_init(tfull, 8);
         fence_mbar_init();
     }
-    for (int i = tid; i < 240; i += kSymThreads) tw1[i] = __ldg(a.tw + i);
+    for (int i = tid; i < 240; i += kSymThreads) tw1[(i & 15) * kSymTwRow + (i >> 4) + 1] = __ldg(a.tw + i);
     umma::fence_before_sync();
     __syncthreads();
     umma::fence_after_sync();
@@ -810,7 +814,7 @@ __global__ void __launch_bounds__(kSymThreads, 1)
                 float2* base = a.tones + (o0 + f - q) * tcs;
                 for (int it = tg; it < nq * nb_smem; it += NT) {
                     const int t = it / nq, qq = q0 + (it - t * nq);
-                    base[static_cast<int64_t>(t) * a.tones_ld + qq * tcs] = tile[t * kToneGroup + qq];
+                    base[static_cast<int64_t>(t) * a.tones_ld + qq * tcs] = tile[tile_at(t, qq)];
                 }
             }
             ++closed;
@@ -831,8 +835,15 @@ __global__ void __launch_bounds__(kSymThreads, 1)
             wait(&b0full[f & 1], (f >> 1) & 1);
 #pragma unroll
             for (int r = 0; r < 16; ++r) v[r] = at(pown + r * NT * 8);
+            {
+                const float4* const t4 = reinterpret_cast<const float4*>(tw1 + k * kSymTwRow);
 #pragma unroll
-            for (int r = 1; r < 16; ++r) v[r] = cmul(v[r], tw1[(r - 1) * 16 + k]);
+                for (int i = 0; i < 8; ++i) {
+                    const float4 t = t4[i];
+                    if (i > 0) v[2 * i] = cmul(v[2 * i], make_float2(t.x, t.y));
+                    v[2 * i + 1] = cmul(v[2 * i + 1], make_float2(t.z, t.w));
+                }
+            }
             dft16(v);
             // exchange within the warp, in place: output r of thread `row` goes to
             // row 16 r + (row ^ (r & 7)) of column k, where thread r finds it
@@ -892,7 +903,7 @@ __global__ void __launch_bounds__(kSymThreads, 1)
                 }
 #pragma unroll
                 for (int i = 0; i < kTonesPerThread; ++i)
-                    if (((bk2[i / 2] >> (16 * (i & 1))) & 0xffffu) != 0xffffu) tile[(tg + i * NT) * kToneGroup + q] = tv[i];
+                    if (((bk2[i / 2] >> (16 * (i & 1))) & 0xffffu) != 0xffffu) tile[tile_at(tg + i * NT, q)] = tv[i];
                 if (closes_group(f)) {
                     fence_proxy_async_smem();
                     __syncwarp();
@@ -1770,7 +1781,7 @@ cudaError_t launch_tmem_sym(PfbArgs a, int n_sms, int max_smem, cudaStream_t st)
         cuuint32_t box[2] = {kToneGroup, kToneBox};
         cuuint32_t estr[2] = {1, 1};
         if (enc(&tm, CU_TENSOR_MAP_DATA_TYPE_UINT64, 2, a.tones, dims, strides, box, estr,
-                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_32B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
                 CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS)
             a.tones_tma = 1;
     }
