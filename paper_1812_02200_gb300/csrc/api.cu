@@ -337,10 +337,16 @@ rfr_status push_check(rfr_plan* p, const int16_t* iq, int64_t n, const rfr_outpu
 
 // The FIR pre-sum rows of F frames (PFB plans with rfr::pfb_pre_rows);
 // growing them is refused while `st` is being captured (st null: not
-// capturing).
+// capturing).  The shapes of rfr::pfb_pre_optional go on without them
+// (pre_cap < F) where they cannot grow.
 rfr_status ensure_pre_rows(rfr_plan* p, int64_t F, cudaStream_t st) {
     if (F <= p->pre_cap) return RFR_OK;
-    if (st) {
+    const bool optional = rfr::pfb_pre_optional(p->log2n, p->Tk);
+    if (st && optional) {
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        RFR_CUDA(p, cudaStreamIsCapturing(st, &cs));
+        if (cs != cudaStreamCaptureStatusNone) return RFR_OK;
+    } else if (st) {
         const rfr_status rs = refuse_growth_in_capture(p, st);
         if (rs != RFR_OK) return rs;
     }
@@ -348,7 +354,13 @@ rfr_status ensure_pre_rows(rfr_plan* p, int64_t F, cudaStream_t st) {
     dev_free(p->d_pre);
     p->d_pre = nullptr;
     p->pre_cap = 0;
-    RFR_CUDA(p, dev_alloc(&p->d_pre, static_cast<size_t>(F) * p->N * 8));
+    const cudaError_t e = dev_alloc(&p->d_pre, static_cast<size_t>(F) * p->N * 8);
+    if (optional && e == cudaErrorMemoryAllocation) {
+        cudaGetLastError();
+        p->d_pre = nullptr;
+        return RFR_OK;
+    }
+    RFR_CUDA(p, e);
     p->pre_cap = F;
     return RFR_OK;
 }
@@ -430,7 +442,7 @@ rfr_status push_core(rfr_plan* p, const int16_t* iq, int64_t n, const rfr_output
                     const int64_t lv_max = std::max<int64_t>(p->cl, p->W - 1) + n;
                     const rfr_status rs = ensure_pre_rows(p, F <= p->pre_cap ? F : frames_for_len(p, lv_max), st);
                     if (rs != RFR_OK) return rs;
-                    L.pre = p->d_pre;
+                    if (F <= p->pre_cap) L.pre = p->d_pre;
                     L.pre_cap = p->pre_cap;
                 }
                 RFR_CUDA(p, p->gen ? rfr::gen_pfb_launch(L, p->gplan, st) : rfr::pfb_launch(L, st));

@@ -1420,7 +1420,10 @@ __global__ void __launch_bounds__(kTileThreads, 3) pfb_tile_kernel(const PfbArgs
 //   N = 16384    467 / 487 / 523 -> 404 / 424 / 460   (T = 4 was FIR in the kernel)
 // (floors 138, 128, 123).  The twiddles are read in lane order from a permuted
 // table: in natural order, 16 lines a load, the same kernel took 568 at T = 8.
-template <int LOG2N>
+// FIR: the sums in this kernel, every tap and sample through L2 per frame, for the
+// pushes of N = 16384, T <= 4 that have no room for them in memory (pfb_pre_optional);
+// the same FMA chain, the same bits: 469 us where the pass ahead gives 402.
+template <int LOG2N, bool FIR>
 __global__ void __launch_bounds__(1 << (LOG2N - 4), 1 << (14 - LOG2N))
     pfb_rows_kernel(const PfbArgs a, const __grid_constant__ CUtensorMap tm_full) {
     constexpr int N = 1 << LOG2N, NT = N / 16, RF = N / 4096, NQ = 16 / RF;
@@ -1438,9 +1441,24 @@ __global__ void __launch_bounds__(1 << (LOG2N - 4), 1 << (14 - LOG2N))
     const int x0 = place_row(tid) & 7;
     float2 v[16];
     auto load = [&](int64_t j) {
-        const float2* row = a.pre + j * N + tid;
+        if constexpr (FIR) {
 #pragma unroll
-        for (int r = 0; r < 16; ++r) v[r] = __ldg(row + r * NT);
+            for (int r = 0; r < 16; ++r) v[r] = make_float2(0.f, 0.f);
+#pragma unroll 1
+            for (int t = 0; t < a.T; ++t) {
+#pragma unroll
+                for (int r = 0; r < 16; ++r) {
+                    const float hv = __ldg(a.h + t * N + tid + r * NT);
+                    const float2 x = iq_to_f2(vload(a, (j + t) * N + tid + r * NT));
+                    v[r].x = fmaf(hv, x.x, v[r].x);
+                    v[r].y = fmaf(hv, x.y, v[r].y);
+                }
+            }
+        } else {
+            const float2* row = a.pre + j * N + tid;
+#pragma unroll
+            for (int r = 0; r < 16; ++r) v[r] = __ldg(row + r * NT);
+        }
     };
     if (static_cast<int64_t>(blockIdx.x) < a.F) load(blockIdx.x);
     for (int64_t j = blockIdx.x; j < a.F; j += gridDim.x) {
@@ -1450,7 +1468,7 @@ __global__ void __launch_bounds__(1 << (LOG2N - 4), 1 << (14 - LOG2N))
         __syncthreads();                                         // the frame before has left the buffer
 #pragma unroll
         for (int r = 0; r < 16; r += 2) row0[(r / 2) ^ x0] = make_float4(v[r].x, v[r].y, v[r + 1].x, v[r + 1].y);
-        if (jn < a.F && (tid & 15) == 0) {
+        if (!FIR && jn < a.F && (tid & 15) == 0) {
             // the next frame's rows on their way to L2 (a request per 128-byte line)
             const float2* nrow = a.pre + jn * N + tid;
 #pragma unroll
@@ -1739,17 +1757,17 @@ bool full_row_map(const PfbArgs& a, int n, CUtensorMap* m) {
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int LOG2N>
+template <int LOG2N, bool FIR = false>
 cudaError_t launch_rows(PfbArgs a, int n_sms, cudaStream_t st) {
     constexpr int N = 1 << LOG2N;
     CUtensorMap tf;
     std::memset(&tf, 0, sizeof tf);
     a.full_bulk = full_row_map(a, N, &tf) ? 1 : 0;
     const int smem = N * 8;
-    const cudaError_t e = cudaFuncSetAttribute(pfb_rows_kernel<LOG2N>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    const cudaError_t e = cudaFuncSetAttribute(pfb_rows_kernel<LOG2N, FIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     const int64_t grid = std::min<int64_t>(a.F, static_cast<int64_t>(n_sms) << (14 - LOG2N));
-    pfb_rows_kernel<LOG2N><<<static_cast<unsigned>(grid), N / 16, smem, st>>>(a, tf);
+    pfb_rows_kernel<LOG2N, FIR><<<static_cast<unsigned>(grid), N / 16, smem, st>>>(a, tf);
     return cudaGetLastError();
 }
 
@@ -1889,6 +1907,9 @@ bool pfb_pre_rows(int log2n, int taps) {
     if (log2n >= 13) return true;
     return (log2n == 11 || log2n == 12) && taps > 8;
 }
+// Of these, the ones that also run without room for the sums (a push inside a
+// stream capture that the plan has not grown for, or a full device).
+bool pfb_pre_optional(int log2n, int taps) { return log2n == 14 && taps <= 4; }
 int pfb_kernel_taps(int log2n, int taps) {
     if (pfb_uses_ring(log2n, taps) || pfb_cluster_size(log2n, taps) > 0) return taps <= 4 ? 4 : 8;
     if (log2n == 12 && taps > 8 && taps <= 16) return 16;     // zero-padded at the oldest end
@@ -1980,7 +2001,9 @@ cudaError_t pfb_launch(const PfbLaunch& L, cudaStream_t st) {
     case 11: return launch_direct<11>(a, L.n_sms, L.max_smem, st);
     case 12: return a.pre ? launch_rows<12>(a, L.n_sms, st) : cudaErrorInvalidValue;
     case 13: return a.pre ? launch_rows<13>(a, L.n_sms, st) : cudaErrorInvalidValue;
-    case 14: return a.pre ? launch_rows<14>(a, L.n_sms, st) : cudaErrorInvalidValue;
+    case 14:
+        if (a.pre) return launch_rows<14>(a, L.n_sms, st);
+        return pfb_pre_optional(lg, L.taps_kernel) ? launch_rows<14, true>(a, L.n_sms, st) : cudaErrorInvalidValue;
     default: return cudaErrorInvalidValue;
     }
 }

@@ -109,6 +109,7 @@ int pfb_cluster_size(int log2n, int taps);
 // PFB plans whose pushes take FIR pre-sum rows (PfbLaunch::pre): N = 8192 and
 // 16384; N = 2048 and 4096 with T > 8.
 bool pfb_pre_rows(int log2n, int taps);
+bool pfb_pre_optional(int log2n, int taps);
 cudaError_t pfb_launch(const PfbLaunch& L, cudaStream_t st);
 cudaError_t gen_pfb_launch(const PfbLaunch& L, const GenPlan& g, cudaStream_t st);
 

@@ -51,3 +51,30 @@ def test_rows_any_split_pitch_and_oracle(lib, N, T, frames, first, off, pad):
     y = oracle.pfb(xn[:k * N], N, T, h64)["full"]
     # FP32 rounding of taps, FIR and up to four passes: a few 1e-7
     assert np.linalg.norm(ref[:k].cpu().numpy() - y) <= 1e-6 * np.linalg.norm(y)
+
+
+@pytest.mark.parametrize("T,frames,cut", [(1, 1, 16384), (3, 155, 16387), (4, 307, 100001)])
+def test_captured_push_of_a_plan_without_rows(lib, T, frames, cut):
+    """N = 16384, T <= 4: a push captured before the plan has room for its FIR sums
+    (after none, or after a smaller push) runs the FIR in the FFT kernel; the replay's
+    frames equal a direct push's bit for bit, and the state goes on from there."""
+    N, nt = 16384, 37
+    rng = np.random.default_rng(T)
+    xn = rng.integers(-8192, 8192, size=(cut + frames * N, 2)).astype(np.int16)
+    x = torch.from_numpy(xn).to(DEV)
+    words = siggen.bin_words(rng.integers(0, N, nt), N)
+    F = x.shape[0] // N
+    out = lambda: (torch.zeros((F, N), dtype=torch.complex64, device=DEV),
+                   torch.zeros((nt, F), dtype=torch.complex64, device=DEV))
+    want, got = out(), out()
+    assert lib.Plan(N, T, window="hamming", words=words).push_into(x, *want) == F
+    p = lib.Plan(N, T, window="hamming", words=words)
+    f0 = p.push_into(x[:cut], *got) if T > 1 else 0
+    rest = x[cut:] if T > 1 else x
+    torch.cuda.synchronize()
+    s, g = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        assert f0 + p.push_into(rest, *got, frame_offset=f0, stream=s) == F
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
