@@ -78,7 +78,8 @@ struct PfbArgs {
     int64_t frame_offset;
     int use_tma;
     int tones_tma;           // TMEM variant: whole tone groups leave by 2-D TMA stores
-    int nb_smem;             // TMEM variant: tones staged in smem (0 or n_tones)
+    int nb_smem;             // TMEM variants: tones staged in smem (0 or n_tones); rows: tones kept there
+    int tone_vec;            // rows: tone rows take 16-byte stores at even frames
     int full_bulk;           // TMEM variant: full rows written by one TMA bulk store each
     int* status;
     int tone_cs;             // symmetric-tap kernel: tone columns of consecutive frames this far apart
@@ -1414,12 +1415,19 @@ __global__ void __launch_bounds__(kTileThreads, 3) pfb_tile_kernel(const PfbArgs
 // (and 4), then 16-byte pairs XOR the row mod 8, TMA's 128-byte swizzle.  All maps
 // are linear over XOR, so a thread's places are one address XOR constants.
 // Measured, 2^26 samples, full + 1000 tones, T = 4 / 8 / 16, before -> after (us):
-//   N = 4096      -   /  -  / 526 ->  -  /  -  / 481   (was: the pre-sum of taps 0..7,
+//   N = 4096      -   /  -  / 522 ->  -  /  -  / 443   (was: the pre-sum of taps 0..7,
 //                then the TMEM kernel for taps 8..15 on top of it)
 //   N = 8192     544 / 479 / 512 -> 389 / 407 / 441
 //   N = 16384    467 / 487 / 523 -> 404 / 424 / 460   (T = 4 was FIR in the kernel)
 // (floors 138, 128, 123).  The twiddles are read in lane order from a permuted
 // table: in natural order, 16 lines a load, the same kernel took 568 at T = 8.
+// Tones: at N = 4096 a CTA takes groups of four output frames and writes a tone's
+// values in 32-byte sectors, from shared memory beside the frame buffer (as many tones
+// as fit there with four CTAs an SM, 1024; the others a value at a time).  Frame by
+// frame with 8-byte stores, 2^26 / 27 / 28 samples took 502 / 1108 / 2358 us at T = 16,
+// now 443 / 856 / 1695 (the tones were 0.94 ms of the last).  Contiguous ranges of frames
+// a CTA: 461 / 895 / 1758.  Pushes of less than two groups a CTA stay frame by frame
+// for balance; so do the larger N, whose tones are fewer a sample (in ranges 8 % slower).
 // FIR: the sums in this kernel, every tap and sample through L2 per frame, for the
 // pushes of N = 16384, T <= 4 that have no room for them in memory (pfb_pre_optional);
 // the same FMA chain, the same bits: 469 us where the pass ahead gives 402.
@@ -1460,9 +1468,18 @@ __global__ void __launch_bounds__(1 << (LOG2N - 4), 1 << (14 - LOG2N))
             for (int r = 0; r < 16; ++r) v[r] = __ldg(row + r * NT);
         }
     };
-    if (static_cast<int64_t>(blockIdx.x) < a.F) load(blockIdx.x);
-    for (int64_t j = blockIdx.x; j < a.F; j += gridDim.x) {
-        const int64_t jn = j + gridDim.x;
+    float2* const kept = buf + N;                                // tones of the group's frames so far, [3][a.nb_smem]
+    const bool grouped = RF == 1 && a.nb_smem > 0;
+    const int sh = static_cast<int>(a.frame_offset & 3);
+    // the frame after j: the next of its group, then the CTA's next group (or frame)
+    auto next = [&](int64_t j) {
+        if (!grouped) return j + gridDim.x;
+        return ((j + 1 + sh) & 3) ? j + 1 : j + 1 + 4 * static_cast<int64_t>(gridDim.x - 1);
+    };
+    const int64_t j0 = grouped ? max(static_cast<int64_t>(0), 4 * static_cast<int64_t>(blockIdx.x) - sh) : blockIdx.x;
+    if (j0 < a.F) load(j0);
+    for (int64_t j = j0; j < a.F;) {
+        const int64_t jn = next(j);
         dft16(v);                                                // pass 0
         if (tid == 0) bulk_wait_read_all();
         __syncthreads();                                         // the frame before has left the buffer
@@ -1526,7 +1543,26 @@ __global__ void __launch_bounds__(1 << (LOG2N - 4), 1 << (14 - LOG2N))
             float2* out = a.full + o * a.full_ld;
             for (int i = tid; i < N; i += NT) out[i] = buf[sym_swizzle(i)];
         }
-        for (int t = tid; t < a.n_tones; t += NT) a.tones[t * a.tones_ld + o] = buf[sym_swizzle(__ldg(a.bins + t))];
+        // tones: kept (by the thread that read them) until their 4-frame group is
+        // complete or the push ends
+        const int ph = static_cast<int>(o & 3);
+        for (int t = tid; t < a.n_tones; t += NT) {
+            const float2 y = buf[sym_swizzle(__ldg(a.bins + t))];
+            float2* const out = a.tones + t * a.tones_ld + o;
+            if (!grouped || t >= a.nb_smem) {
+                *out = y;
+            } else if (ph < 3 && j + 1 < a.F) {
+                kept[ph * a.nb_smem + t] = y;
+            } else if (ph == 3 && j >= 3 && a.tone_vec) {
+                const float2 y0 = kept[t], y1 = kept[a.nb_smem + t], y2 = kept[2 * a.nb_smem + t];
+                reinterpret_cast<float4*>(out - 3)[0] = make_float4(y0.x, y0.y, y1.x, y1.y);
+                reinterpret_cast<float4*>(out - 3)[1] = make_float4(y2.x, y2.y, y.x, y.y);
+            } else {
+                for (int k = static_cast<int>(max(static_cast<int64_t>(0), ph - j)); k < ph; ++k) out[k - ph] = kept[k * a.nb_smem + t];
+                *out = y;
+            }
+        }
+        j = jn;
     }
     if (tid == 0) bulk_wait_all();
 }
@@ -1758,14 +1794,22 @@ bool full_row_map(const PfbArgs& a, int n, CUtensorMap* m) {
 }
 
 template <int LOG2N, bool FIR = false>
-cudaError_t launch_rows(PfbArgs a, int n_sms, cudaStream_t st) {
+cudaError_t launch_rows(PfbArgs a, int n_sms, int max_smem, cudaStream_t st) {
     constexpr int N = 1 << LOG2N;
     CUtensorMap tf;
     std::memset(&tf, 0, sizeof tf);
     a.full_bulk = full_row_map(a, N, &tf) ? 1 : 0;
-    const int smem = N * 8;
+    // the tones kept in shared memory (pushes of two groups a CTA or more): what the
+    // CTAs of an SM have left of it (1 KB a CTA is the system's), within a CTA's limit
+    constexpr int kSmShared = 228 * 1024, kCtas = 1 << (14 - LOG2N);
+    const int room = std::min(kSmShared / kCtas - 1024, max_smem) - N * 8;
+    a.nb_smem = LOG2N == 12 && a.F >= int64_t{8} * kCtas * n_sms ? std::max(0, std::min(a.n_tones, room / 24)) : 0;
+    a.tone_vec = reinterpret_cast<uintptr_t>(a.tones) % 16 == 0 && a.tones_ld % 2 == 0 ? 1 : 0;
+    const int smem = N * 8 + 24 * a.nb_smem;
     const cudaError_t e = cudaFuncSetAttribute(pfb_rows_kernel<LOG2N, FIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
+    // (N = 8192 and 16384 are 10 % slower with the smaller L1)
+    if (LOG2N == 12) cudaFuncSetAttribute(pfb_rows_kernel<LOG2N, FIR>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     const int64_t grid = std::min<int64_t>(a.F, static_cast<int64_t>(n_sms) << (14 - LOG2N));
     pfb_rows_kernel<LOG2N, FIR><<<static_cast<unsigned>(grid), N / 16, smem, st>>>(a, tf);
     return cudaGetLastError();
@@ -1999,11 +2043,11 @@ cudaError_t pfb_launch(const PfbLaunch& L, cudaStream_t st) {
     case 4: return launch_direct<4>(a, L.n_sms, L.max_smem, st);
     case 5: return launch_direct<5>(a, L.n_sms, L.max_smem, st);
     case 11: return launch_direct<11>(a, L.n_sms, L.max_smem, st);
-    case 12: return a.pre ? launch_rows<12>(a, L.n_sms, st) : cudaErrorInvalidValue;
-    case 13: return a.pre ? launch_rows<13>(a, L.n_sms, st) : cudaErrorInvalidValue;
+    case 12: return a.pre ? launch_rows<12>(a, L.n_sms, L.max_smem, st) : cudaErrorInvalidValue;
+    case 13: return a.pre ? launch_rows<13>(a, L.n_sms, L.max_smem, st) : cudaErrorInvalidValue;
     case 14:
-        if (a.pre) return launch_rows<14>(a, L.n_sms, st);
-        return pfb_pre_optional(lg, L.taps_kernel) ? launch_rows<14, true>(a, L.n_sms, st) : cudaErrorInvalidValue;
+        if (a.pre) return launch_rows<14>(a, L.n_sms, L.max_smem, st);
+        return pfb_pre_optional(lg, L.taps_kernel) ? launch_rows<14, true>(a, L.n_sms, L.max_smem, st) : cudaErrorInvalidValue;
     default: return cudaErrorInvalidValue;
     }
 }

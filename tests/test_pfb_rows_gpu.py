@@ -78,3 +78,27 @@ def test_captured_push_of_a_plan_without_rows(lib, T, frames, cut):
     g.replay()
     torch.cuda.synchronize()
     assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+
+
+@pytest.mark.parametrize("N,T,frames,nt,off,pad,fo", [
+    (4096, 9, 2500, 1500, 0, 0, 0), (4096, 16, 1219, 1100, 0, 2, 3), (4096, 11, 1300, 40, 1, 3, 1),
+    (8192, 8, 1000, 2500, 0, 1, 2), (8192, 5, 911, 77, 1, 1, 3), (16384, 8, 470, 4300, 0, 2, 1), (16384, 4, 457, 5, 1, 2, 0),
+])
+def test_rows_tones_in_groups(lib, N, T, frames, nt, off, pad, fo):
+    """Tone rows written four frames at a time: ranges that begin and end inside a
+    group, more tones than the kernel keeps on chip, any frame offset, row pitch and
+    8-byte offset of the rows.  Every value equals its spectrum bin; nothing else is
+    written."""
+    rng = np.random.default_rng(nt)
+    x = torch.from_numpy(rng.integers(-8192, 8192, size=(frames * N, 2)).astype(np.int16)).to(DEV)
+    words = siggen.bin_words(rng.integers(0, N, nt), N)
+    p = lib.Plan(N, T, window="hamming", words=words)
+    full = torch.zeros((fo + frames, N), dtype=torch.complex64, device=DEV)
+    ld = fo + frames + pad
+    base = torch.zeros(nt * ld + off, dtype=torch.complex64, device=DEV)
+    tones = base[off:].view(nt, ld)
+    assert p.push_into(x, full, tones, frame_offset=fo) == frames
+    torch.cuda.synchronize()
+    bins = torch.from_numpy(p.bins().astype(np.int64)).to(DEV)
+    assert torch.equal(tones[:, fo:fo + frames], full[fo:, bins].T)
+    assert not tones[:, :fo].any() and not tones[:, fo + frames:].any() and not base[:off].any()
