@@ -1429,8 +1429,8 @@ __global__ void __launch_bounds__(kTileThreads, 3) pfb_tile_kernel(const PfbArgs
 // a CTA: 461 / 895 / 1758.  Pushes of less than two groups a CTA stay frame by frame
 // for balance; so do the larger N, whose tones are fewer a sample (in ranges 8 % slower).
 // FIR: the sums in this kernel, every tap and sample through L2 per frame, for the
-// pushes of N = 16384, T <= 4 that have no room for them in memory (pfb_pre_optional);
-// the same FMA chain, the same bits: 469 us where the pass ahead gives 402.
+// pushes of N = 16384, T <= 4 that are small (pfb_pre_skip) or have no room for them in
+// memory (pfb_pre_optional); the same FMA chain, the same bits.
 template <int LOG2N, bool FIR>
 __global__ void __launch_bounds__(1 << (LOG2N - 4), 1 << (14 - LOG2N))
     pfb_rows_kernel(const PfbArgs a, const __grid_constant__ CUtensorMap tm_full) {
@@ -1954,6 +1954,14 @@ bool pfb_pre_rows(int log2n, int taps) {
 // Of these, the ones that also run without room for the sums (a push inside a
 // stream capture that the plan has not grown for, or a full device).
 bool pfb_pre_optional(int log2n, int taps) { return log2n == 14 && taps <= 4; }
+// Of these, the pushes that are faster with the FIR in the FFT kernel: two frames an
+// SM, seven when only tones leave.  Measured, T = 4, FIR in the kernel / ahead (us):
+// 2^21 samples 18.6 / 21.8 (tones only 18.5 / 22.6), 2^22 32.9 / 36.8 (30.7 / 32.9),
+// 2^23 72.6 / 68.0 (55.5 / 59.3), 2^24 128 / 115 (92.4 / 102.7), 2^25 248 / 216
+// (222 / 193).
+bool pfb_pre_skip(int log2n, int taps, int64_t F, bool full, int n_sms) {
+    return pfb_pre_optional(log2n, taps) && F <= static_cast<int64_t>(n_sms) * (full ? 2 : 7);
+}
 int pfb_kernel_taps(int log2n, int taps) {
     if (pfb_uses_ring(log2n, taps) || pfb_cluster_size(log2n, taps) > 0) return taps <= 4 ? 4 : 8;
     if (log2n == 12 && taps > 8 && taps <= 16) return 16;     // zero-padded at the oldest end

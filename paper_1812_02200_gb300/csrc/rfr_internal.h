@@ -110,6 +110,7 @@ int pfb_cluster_size(int log2n, int taps);
 // 16384; N = 2048 and 4096 with T > 8.
 bool pfb_pre_rows(int log2n, int taps);
 bool pfb_pre_optional(int log2n, int taps);
+bool pfb_pre_skip(int log2n, int taps, int64_t F, bool full, int n_sms);
 cudaError_t pfb_launch(const PfbLaunch& L, cudaStream_t st);
 cudaError_t gen_pfb_launch(const PfbLaunch& L, const GenPlan& g, cudaStream_t st);
 

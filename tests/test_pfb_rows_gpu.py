@@ -18,7 +18,8 @@ DEV = "cuda:0"
 @pytest.mark.parametrize("N,T,frames,first,off,pad", [
     (4096, 9, 1, 4095, 0, 1), (4096, 16, 620, 100001, 1, 1), (4096, 12, 7, 3, 2, 3),
     (8192, 1, 2, 8191, 3, 1), (8192, 4, 305, 5, 1, 1), (8192, 8, 310, 700000, 0, 3), (8192, 13, 5, 9000, 2, 1),
-    (16384, 3, 153, 16385, 1, 1), (16384, 8, 160, 1234567, 3, 1), (16384, 16, 3, 20000, 2, 5),
+    (16384, 3, 153, 16385, 1, 1), (16384, 4, 330, 5000000, 1, 3),
+    (16384, 8, 160, 1234567, 3, 1), (16384, 16, 3, 20000, 2, 5),
 ])
 def test_rows_any_split_pitch_and_oracle(lib, N, T, frames, first, off, pad):
     rng = np.random.default_rng(N + T + frames)
