@@ -410,10 +410,9 @@ def run_demod(args, dev, stream, rank):
                         "note": "algorithmic flops = 8*L*tones/D per sample; the default Gauss "
                                 "form issues 3 real products per complex MAC, each as 3 split-FP16 "
                                 "MMAs (2.25x the algorithmic flops on the tensor pipe); push time "
-                                "includes the rotation, pre-split and carry kernels",
+                                "includes the rotation and pre-split kernel and the carry kernel",
                         "peak_kind": f"{peak_kind} dense bf16 (fp16 has the same nominal rate)"}}
-    # -- the other cluster form of the same GEMM (two-CTA clusters sharing
-    # the frame tiles by multicast, or one CTA per tile), same tile and raster
+    # -- the other form of the same GEMM (tiles on two SMs, or on one)
     tn = plan.tune()
     pp = rfr.Plan(0, DEMOD_L, window="blackman", cutoff=DEMOD_FC, words=c["words"], decimation=DEMOD_D)
     pp.set_tone_tile(tn["tone_tile"] or 128)
@@ -429,7 +428,7 @@ def run_demod(args, dev, stream, rank):
     res["single_cta" if tn["pair"] else "pair_clusters"] = {
         "value": samples / (msp * 1e-3) / 1e6, "unit": UNIT, "ms_per_step": msp,
         "note": "the same GEMM with one CTA per tile" if tn["pair"] else
-                "the same GEMM in two-CTA clusters sharing each frame tile by TMA multicast"}
+                "the same GEMM pinned to two-SM tiles of 256 frames x 256 tones"}
     pp.close()
     # -- the same three-product GEMM with the FP16 split fused into its
     # producer warps (no pre-split kernel; each A tile converted once per tone

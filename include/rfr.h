@@ -312,8 +312,9 @@ rfr_status rfr_state_import(rfr_plan* plan, const void* host, size_t bytes);
  *   Re = 2 P1 - P3, Im = 2 P1 + P2
  * (three real products; the same definition, Sec. III.B, rounded
  * differently), which needs D % 64 == 0 (RFR_E_UNSUPPORTED otherwise) and
- * builds its tap planes on the first switch (allocates, synchronises the
- * device).  Either switch resets the accumulation chunk to the form's
+ * builds its tap planes and its scratch for finished products (512 KB an SM,
+ * 78 MB) on the first switch, at creation where it is the default (allocates,
+ * synchronises the device).  Either switch resets the accumulation chunk to the form's
  * default (64 taps in the four-product form, 256 in the three-product
  * form).  Set it before the first push of a stream.
  */
