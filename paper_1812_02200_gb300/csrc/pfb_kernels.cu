@@ -1425,7 +1425,8 @@ __global__ void __launch_bounds__(kTileThreads, 3) pfb_tile_kernel(const PfbArgs
 // values in 32-byte sectors, from shared memory beside the frame buffer (as many tones
 // as fit there with four CTAs an SM, 1024; the others a value at a time).  Frame by
 // frame with 8-byte stores, 2^26 / 27 / 28 samples took 502 / 1108 / 2358 us at T = 16,
-// now 443 / 856 / 1695 (the tones were 0.94 ms of the last).  Contiguous ranges of frames
+// now 443 / 856 / 1695 (the tones were 0.94 ms of the last).  (Neighbouring tone
+// bins; random ones, whose gather meets bank conflicts: 2390 -> 1906 at 2^28.)  Contiguous ranges of frames
 // a CTA: 461 / 895 / 1758.  Pushes of less than two groups a CTA stay frame by frame
 // for balance; so do the larger N, whose tones are fewer a sample (in ranges 8 % slower).
 // FIR: the sums in this kernel, every tap and sample through L2 per frame, for the
