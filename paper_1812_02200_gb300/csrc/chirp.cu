@@ -448,11 +448,12 @@ cudaError_t chirp_demod_launch(const ChirpLaunch& L, cudaStream_t st) {
         const int64_t widest = kOvSamples / L.D - (jt - 1) > 0 ? kOvSamples / L.D - (jt - 1) : 1;
         const int64_t n_seg = (o.per_cta + widest - 1) / widest;
         o.seg = static_cast<int>((o.per_cta + n_seg - 1) / n_seg);
-        // frames per work item: the fewest rounds of block walks for the four workers
+        // frames per work item, at most kOvSub (so from ceil(seg / kOvSub) items a chirp
+        // on): the fewest rounds of block walks for the four workers
         int64_t best = INT64_MAX;
-        for (int parts = 1; parts <= 4 || (o.seg + parts - 1) / parts > kOvSub; parts *= 2) {
+        const int least = (o.seg + kOvSub - 1) / kOvSub;
+        for (int parts = least; parts <= 4 * least; parts *= 2) {
             const int sub = (o.seg + parts - 1) / parts;
-            if (sub > kOvSub) continue;
             const int64_t items = static_cast<int64_t>(a.n_chirps) * ((o.seg + sub - 1) / sub);
             const int64_t cost = (items + kOvWorkers - 1) / kOvWorkers * (sub + jt - 1);
             if (cost < best) {
