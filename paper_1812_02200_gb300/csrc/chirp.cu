@@ -463,7 +463,7 @@ cudaError_t chirp_demod_launch(const ChirpLaunch& L, cudaStream_t st) {
         }
         const size_t bytes = static_cast<size_t>(o.seg + jt - 1) * L.D * 4;
         auto run = [&](auto kern) {
-            const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+            const cudaError_t e = allow_smem(kern, kOvSamples * 4);
             if (e != cudaSuccess) return e;
             kern<<<static_cast<unsigned>((L.F + o.per_cta - 1) / o.per_cta), kOvWorkers * kChirpThreads, bytes, st>>>(a, o);
             return cudaGetLastError();
@@ -475,11 +475,9 @@ cudaError_t chirp_demod_launch(const ChirpLaunch& L, cudaStream_t st) {
         }
     }
     const size_t smem = static_cast<size_t>(L.L) * sizeof(float2);
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(chirp_demod_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             static_cast<int>(smem));
-        if (e != cudaSuccess) return e;
-    }
+    constexpr int kMostTaps = 16384;                    // of a plan
+    const cudaError_t e = allow_smem(chirp_demod_kernel, kMostTaps * static_cast<int>(sizeof(float2)));
+    if (e != cudaSuccess) return e;
     const int per_sm = std::max(1, std::min(8, static_cast<int>((220u * 1024u) / (smem + 5u * 1024u))));
     const int64_t blocks = std::min<int64_t>(L.F, static_cast<int64_t>(L.n_sms) * per_sm);
     chirp_demod_kernel<<<static_cast<unsigned>(blocks), kChirpThreads, smem, st>>>(a);

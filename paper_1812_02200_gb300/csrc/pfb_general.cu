@@ -1278,10 +1278,10 @@ namespace {
 size_t smem_bytes(int elems) { return static_cast<size_t>(2 * (elems + elems / 16 + 1)) * sizeof(float2); }
 
 template <int TH, typename K, typename... Args>
-cudaError_t launch_gen(K kernel, int64_t items, int elems, int n_sms, cudaStream_t st, size_t extra_smem,
+cudaError_t launch_gen(K kernel, int64_t items, int elems, int n_sms, int max_smem, cudaStream_t st, size_t extra_smem,
                        const Args&... args) {
     const size_t smem = smem_bytes(elems) + extra_smem;
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    cudaError_t e = allow_smem(kernel, max_smem);
     if (e != cudaSuccess) return e;
     int occ = 1;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, TH, smem) != cudaSuccess || occ < 1)
@@ -1298,7 +1298,7 @@ cudaError_t gen_run(GenArgs a, const PfbLaunch& L, const GenPlan& g, cudaStream_
     if (g.N1 == 1) {
         a.F = L.F;
         a.k0 = 0;
-        return launch_gen<TH>(gen_single_kernel<TH>, (L.F + (1 << g.gls) - 1) >> g.gls, g.N << g.gls, L.n_sms, st,
+        return launch_gen<TH>(gen_single_kernel<TH>, (L.F + (1 << g.gls) - 1) >> g.gls, g.N << g.gls, L.n_sms, L.max_smem, st,
                               (size_t(1) << g.gls) * sizeof(int), a);
     }
     if (g.z_frames < 1 || !g.d_z) return cudaErrorInvalidValue;   // gen_plan_reserve first
@@ -1347,10 +1347,10 @@ cudaError_t gen_run(GenArgs a, const PfbLaunch& L, const GenPlan& g, cudaStream_
             }
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
         }
-        e = launch_gen<TH>(gen_pass_a_kernel<TH>, a.F * groups_a, g.N1 * ga, L.n_sms, st,
+        e = launch_gen<TH>(gen_pass_a_kernel<TH>, a.F * groups_a, g.N1 * ga, L.n_sms, L.max_smem, st,
                            3 * kTwDigit * sizeof(float2) + 16, a, tmv);
         if (e != cudaSuccess) return e;
-        e = launch_gen<TH>(gen_pass_b_kernel<TH>, a.F * groups_b, g.N2 * gb, L.n_sms, st, 16, a);
+        e = launch_gen<TH>(gen_pass_b_kernel<TH>, a.F * groups_b, g.N2 * gb, L.n_sms, L.max_smem, st, 16, a);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

@@ -1596,7 +1596,7 @@ cudaError_t launch_ring(PfbArgs a, int n_sms, int max_smem, int lookahead, cudaS
     a.iters_per_cta = (iters + grid - 1) / grid;
     const int64_t grid2 = (iters + a.iters_per_cta - 1) / a.iters_per_cta;
     auto k = pfb_ring_kernel<LOG2N, T>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k, max_smem);
     if (e != cudaSuccess) return e;
     k<<<static_cast<unsigned>(grid2), kRingThreads, smem, st>>>(a);
     return cudaGetLastError();
@@ -1616,7 +1616,7 @@ cudaError_t launch_direct(PfbArgs a, int n_sms, int max_smem, cudaStream_t st) {
     constexpr bool kPre = LOG2N == 11;
     if (a.pre && !kPre) return cudaErrorInvalidValue;
     auto k = a.pre ? pfb_direct_kernel<LOG2N, kPre> : pfb_direct_kernel<LOG2N, false>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k, max_smem);
     if (e != cudaSuccess) return e;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, smem);
     const int64_t grid = std::max<int64_t>(1, std::min<int64_t>(n_iter, static_cast<int64_t>(n_sms) * std::max(per_sm, 1)));
@@ -1631,7 +1631,7 @@ cudaError_t launch_tile(const PfbArgs& a, cudaStream_t st) {
     const int64_t tiles = (a.F + G - 1) / G;
     if (tiles > 0x7fffffff) return cudaErrorInvalidValue;
     auto run = [&](auto k) {
-        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+        const cudaError_t e = allow_smem(k, static_cast<int>(smem));
         if (e != cudaSuccess) return e;
         k<<<static_cast<unsigned>(tiles), kTileThreads, smem, st>>>(a);
         return cudaGetLastError();
@@ -1772,7 +1772,7 @@ cudaError_t launch_tmem(PfbArgs a, int n_sms, int max_smem, cudaStream_t st) {
             a.tones_tma = 1;
     }
     auto k = pfb_tmem_kernel<T>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k, max_smem);
     if (e != cudaSuccess) return e;
     k<<<static_cast<unsigned>(grid2), kRingThreads, smem, st>>>(a, tm);
     return cudaGetLastError();
@@ -1807,7 +1807,7 @@ cudaError_t launch_rows(PfbArgs a, int n_sms, int max_smem, cudaStream_t st) {
     a.nb_smem = LOG2N == 12 && a.F >= int64_t{8} * kCtas * n_sms ? std::max(0, std::min(a.n_tones, room / 24)) : 0;
     a.tone_vec = reinterpret_cast<uintptr_t>(a.tones) % 16 == 0 && a.tones_ld % 2 == 0 ? 1 : 0;
     const int smem = N * 8 + 24 * a.nb_smem;
-    const cudaError_t e = cudaFuncSetAttribute(pfb_rows_kernel<LOG2N, FIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    const cudaError_t e = allow_smem(pfb_rows_kernel<LOG2N, FIR>, max_smem);
     if (e != cudaSuccess) return e;
     // (N = 8192 and 16384 are 10 % slower with the smaller L1)
     if (LOG2N == 12) cudaFuncSetAttribute(pfb_rows_kernel<LOG2N, FIR>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
@@ -1851,7 +1851,7 @@ cudaError_t launch_tmem_sym(PfbArgs a, int n_sms, int max_smem, cudaStream_t st)
     const bool phase = a.tone_cs != 1 || a.rot != 0;
     if (phase && T != 8) return cudaErrorInvalidValue;              // phase passes are 8-tap plans'
     auto k = phase ? pfb_tmem_sym_kernel<8, true> : pfb_tmem_sym_kernel<T, false>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k, max_smem);
     if (e != cudaSuccess) return e;
     // the kernel's register split waits forever unless the launch holds it
     static std::atomic<int> regs[2];
@@ -1881,7 +1881,7 @@ cudaError_t launch_cluster(PfbArgs a, int n_sms, int max_smem, cudaStream_t st) 
     const size_t smem = cluster_layout(a.tw_count, ntc).total;
     if (smem > static_cast<size_t>(max_smem)) return cudaErrorInvalidConfiguration;
     auto k = pfb_cluster_kernel<C, T>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    cudaError_t e = allow_smem(k, max_smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[1];

@@ -14,6 +14,15 @@
 
 namespace rfr {
 
+// Raises a kernel's limit of dynamic shared memory a CTA.  The limit is the
+// process's, one for all host threads: every launch of a kernel gives the same
+// `most`, whatever it uses itself, so that a push in one thread never lowers it
+// between this call and the launch of another's.
+template <typename K>
+cudaError_t allow_smem(K kernel, int most) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+}
+
 // ------------------------------------------------------------ host tables
 // Window and prototype builders (FP64), written from the definitions in
 // Sec. III.A/B; see plan_host.cpp.
