@@ -455,7 +455,8 @@ const char* rfr_batch_last_error(const rfr_batch* batch);
  * host runtime tunes the GPU kernels).  Outputs stay bit-identical whatever
  * is chosen.  With use_cache != 0 the choice is read
  * from / written to the JSON file named by RFR_TUNE_CACHE (default
- * ./rfr_tune_cache.json), keyed by plan shape, push size and GPU.  The
+ * ./rfr_tune_cache.json), keyed by plan shape, a demodulation's product form
+ * and accumulation chunk, push size and GPU.  The
  * stream state is left unchanged.  *best_ms (may be NULL) receives the time
  * of the chosen configuration (-1 when it came from the cache).
  */

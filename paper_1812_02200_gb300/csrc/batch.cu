@@ -75,20 +75,26 @@ std::string tune_path() {
     return p && *p ? std::string(p) : std::string("rfr_tune_cache.json");
 }
 
+// What a choice was timed for: the plan's shape, a demodulation's product form
+// and accumulation chunk, the push size and the GPU.  "v2": entries written
+// before tone tile 0 existed have no such prefix and are not found (their tone
+// tile would pin a form of the GEMM that was the only one then).
 std::string tune_key(const rfr_plan* p, int64_t n) {
     cudaDeviceProp prop{};
     cudaGetDeviceProperties(&prop, p->device);
     int lg = 0;
     while ((int64_t(1) << (lg + 1)) <= n) ++lg;
     std::ostringstream k;
-    k << (p->mode == RFR_MODE_PFB ? "pfb" : "demod") << ":N" << p->N << ":T" << p->T << ":L" << p->L
-      << ":D" << p->D << ":tones" << p->words.size() << ":flags" << p->out_flags << ":n2^" << lg
+    k << "v2:" << (p->mode == RFR_MODE_PFB ? "pfb" : p->mode == RFR_MODE_CHIRP ? "chirp" : "demod") << ":N" << p->N << ":T" << p->T << ":L" << p->L
+      << ":D" << p->D << ":tones" << p->words.size() << ":flags" << p->out_flags;
+    if (p->mode == RFR_MODE_DEMOD) k << ":products" << p->demod_products << ":chunk" << p->accum_chunk;
+    k << ":n2^" << lg
       << ":sm" << prop.major << prop.minor << "x" << prop.multiProcessorCount;
     return k.str();
 }
 
 // Minimal line-oriented JSON map:
-//   {"key": [pfb_lookahead, demod_raster, demod_tone_tile, demod_fused], ...}
+//   {"key": [pfb_lookahead, demod_raster, demod_tone_tile, demod_fused, demod_pair, pfb_cluster], ...}
 // (missing trailing numbers take their defaults: tone tile 128, not fused; tone
 // tile 0: the GEMM's form picked per push by size)
 struct TuneEntry {
@@ -119,10 +125,13 @@ std::map<std::string, TuneEntry> tune_load() {
 void tune_apply(rfr_plan* p, const TuneEntry& t) {
     p->tune.pfb_lookahead = t.lookahead;
     p->tune.demod_raster = t.raster;
-    p->tune.demod_auto = t.bt == 0;
-    p->tune.demod_bt = t.bt == 64 ? 64 : 128;
-    p->tune.demod_fused = t.fused;
-    p->tune.demod_pair = t.pair;
+    if (p->demod_products == 3) {
+        // (a choice timed on another form says nothing of this one's GEMM)
+        p->tune.demod_auto = t.bt == 0;
+        p->tune.demod_bt = t.bt == 64 ? 64 : 128;
+        p->tune.demod_fused = t.fused;
+        p->tune.demod_pair = t.pair;
+    }
     p->tune.pfb_cluster = p->d_tw_cl ? t.cluster : 0;
 }
 
