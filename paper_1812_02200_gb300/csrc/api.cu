@@ -436,8 +436,17 @@ rfr_status push_core(rfr_plan* p, const int16_t* iq, int64_t n, const rfr_output
                 rfr_status rs = phase_passes(p, L, o, lv, F, st);
                 if (rs != RFR_OK) return rs;
             } else {
-                if (!p->gen && rfr::pfb_pre_rows(p->log2n, p->Tk) && !L.cluster &&
-                    !rfr::pfb_pre_skip(p->log2n, p->Tk, F, L.full != nullptr, p->n_sms)) {
+                bool pre = !p->gen && rfr::pfb_pre_rows(p->log2n, p->Tk) && !L.cluster &&
+                           !rfr::pfb_pre_skip(p->log2n, p->Tk, F, L.full != nullptr, p->n_sms);
+                if (pre && rfr::pfb_pre_optional(p->log2n, p->Tk) && !defer_gemm) {
+                    // a caller's graph of a shape that can do without the rows does not
+                    // hold on to them: a larger push later replaces them (a batched
+                    // step's graph is captured anew for every step)
+                    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+                    RFR_CUDA(p, cudaStreamIsCapturing(st, &cs));
+                    pre = cs == cudaStreamCaptureStatusNone;
+                }
+                if (pre) {
                     // FIR pre-sum rows, sized for a push of n samples after any
                     // carry when they grow
                     const int64_t lv_max = std::max<int64_t>(p->cl, p->W - 1) + n;
