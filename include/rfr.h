@@ -361,6 +361,15 @@ rfr_status rfr_plan_seek(rfr_plan* plan, int64_t start_sample, const int16_t* hi
 rfr_status rfr_plan_inject_device_status(rfr_plan* plan, int32_t status);
 
 /*
+ * rfr_plan_inject_alloc_failures -- failure injection on the host: the next
+ * `count` times that a push (or rfr_batch_push) allocates FIR rows for the plan
+ * fail as on a full device.  *left (may be NULL) receives how many of the failures
+ * asked for before were not used; count 0 ends the injection.
+ * Errors: RFR_E_INVALID.
+ */
+rfr_status rfr_plan_inject_alloc_failures(rfr_plan* plan, int32_t count, int32_t* left);
+
+/*
  * rfr_wait_selftest -- launch a kernel whose bounded device-side wait can
  * never be satisfied and check that it gives up after limit_ns (1 us .. 2 s)
  * with the library's timeout status: returns RFR_E_TIMEOUT (and the device

@@ -48,6 +48,18 @@ cudaError_t dev_alloc(T** ptr, size_t bytes) {
     return e;
 }
 
+// Scratch that a plan grows with its pushes (rfr_plan_inject_alloc_failures makes
+// these fail).
+template <typename T>
+cudaError_t scratch_alloc(rfr_plan* p, T** ptr, size_t bytes) {
+    if (p->fail_allocs > 0) {
+        --p->fail_allocs;
+        *ptr = nullptr;
+        return cudaErrorMemoryAllocation;
+    }
+    return dev_alloc(ptr, bytes);
+}
+
 void dev_free(void* p) {
     if (p) cudaFree(p);
 }
@@ -338,15 +350,34 @@ rfr_status push_check(rfr_plan* p, const int16_t* iq, int64_t n, const rfr_outpu
 // The FIR pre-sum rows of F frames (PFB plans with rfr::pfb_pre_rows);
 // growing them is refused while `st` is being captured (st null: not
 // capturing).  The shapes of rfr::pfb_pre_optional go on without them
-// (pre_cap < F) where they cannot grow.
+// (pre_cap < F) where they cannot grow: they keep the rows they have, for pushes
+// that fit, and sizes that found no room are not tried again before a reset (a
+// push that cannot grow them would otherwise stop the device each time).
 rfr_status ensure_pre_rows(rfr_plan* p, int64_t F, cudaStream_t st) {
     if (F <= p->pre_cap) return RFR_OK;
-    const bool optional = rfr::pfb_pre_optional(p->log2n, p->Tk);
-    if (st && optional) {
-        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-        RFR_CUDA(p, cudaStreamIsCapturing(st, &cs));
-        if (cs != cudaStreamCaptureStatusNone) return RFR_OK;
-    } else if (st) {
+    const size_t bytes = static_cast<size_t>(F) * p->N * 8;
+    if (rfr::pfb_pre_optional(p->log2n, p->Tk)) {
+        if (p->pre_refused > 0 && F >= p->pre_refused) return RFR_OK;
+        if (st) {
+            cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+            RFR_CUDA(p, cudaStreamIsCapturing(st, &cs));
+            if (cs != cudaStreamCaptureStatusNone) return RFR_OK;
+        }
+        void* rows = nullptr;
+        const cudaError_t e = scratch_alloc(p, &rows, bytes);
+        if (e == cudaErrorMemoryAllocation) {
+            cudaGetLastError();
+            p->pre_refused = F;
+            return RFR_OK;
+        }
+        RFR_CUDA(p, e);
+        cudaDeviceSynchronize();
+        dev_free(p->d_pre);
+        p->d_pre = rows;
+        p->pre_cap = F;
+        return RFR_OK;
+    }
+    if (st) {
         const rfr_status rs = refuse_growth_in_capture(p, st);
         if (rs != RFR_OK) return rs;
     }
@@ -354,13 +385,7 @@ rfr_status ensure_pre_rows(rfr_plan* p, int64_t F, cudaStream_t st) {
     dev_free(p->d_pre);
     p->d_pre = nullptr;
     p->pre_cap = 0;
-    const cudaError_t e = dev_alloc(&p->d_pre, static_cast<size_t>(F) * p->N * 8);
-    if (optional && e == cudaErrorMemoryAllocation) {
-        cudaGetLastError();
-        p->d_pre = nullptr;
-        return RFR_OK;
-    }
-    RFR_CUDA(p, e);
+    RFR_CUDA(p, scratch_alloc(p, &p->d_pre, bytes));
     p->pre_cap = F;
     return RFR_OK;
 }
@@ -553,6 +578,7 @@ rfr_status reset_state(rfr_plan* p) {
     p->samples = 0;
     p->frames = 0;
     p->q_frames = 0;
+    p->pre_refused = 0;
     p->cur = 0;
     p->cl = p->W - p->H;     // zero history (negative: samples skipped before frame 0)
     if (p->carry_cap > 0) {
@@ -1128,6 +1154,13 @@ rfr_status rfr_wait_selftest(int64_t limit_ns, int32_t* device_status) {
     if (e1 != cudaSuccess || e2 != cudaSuccess) return RFR_E_CUDA;
     if (device_status) *device_status = st;
     return st == DEV_TIMEOUT ? RFR_E_TIMEOUT : RFR_OK;
+}
+
+rfr_status rfr_plan_inject_alloc_failures(rfr_plan* p, int32_t count, int32_t* left) {
+    if (!p || count < 0) return RFR_E_INVALID;
+    if (left) *left = p->fail_allocs;
+    p->fail_allocs = count;
+    return RFR_OK;
 }
 
 rfr_status rfr_plan_inject_device_status(rfr_plan* p, int32_t status) {

@@ -260,6 +260,8 @@ struct rfr_plan {
     int64_t ptones_cap = 0;                    //   frames per pass row
     void* d_pre = nullptr;                     // FIR pre-sum rows (rfr::pfb_pre_rows plans)
     int64_t pre_cap = 0;                       //   [frame][N] float2, frames
+    int64_t pre_refused = 0;                   //   least frames that found no room (0: none), optional rows
+    int32_t fail_allocs = 0;                   // scratch allocations to fail (host-side injection)
     bool gen = false;                          // PFB through the any-N kernels
     rfr::GenPlan gplan;
     int32_t L = 0, D = 0, Lpad = 0;            // demod

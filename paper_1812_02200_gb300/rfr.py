@@ -115,6 +115,7 @@ _SIGS = {
     "rfr_demod_noalloc": (C.c_int, [_P, C.c_int64, _P, C.c_int32, C.c_int32, _P, C.c_int32, _P, C.c_int64, _P]),
     "rfr_demod_noalloc_status": (C.c_int, [_P, C.POINTER(C.c_int32)]),
     "rfr_plan_inject_device_status": (C.c_int, [_P, C.c_int32]),
+    "rfr_plan_inject_alloc_failures": (C.c_int, [_P, C.c_int32, C.POINTER(C.c_int32)]),
     "rfr_plan_get_tone_tile": (C.c_int, [_P, C.POINTER(C.c_int32)]),
     "rfr_plan_set_tone_tile": (C.c_int, [_P, C.c_int32]),
     "rfr_plan_set_fused_presplit": (C.c_int, [_P, C.c_int32]),
@@ -400,6 +401,13 @@ class Plan:
         """Write the plan's device status word as a timed-out kernel would
         (1), or clear it (0): host-side failure injection for tests."""
         self._check(_lib.rfr_plan_inject_device_status(self._h, int(status)), "inject_device_status")
+
+    def inject_alloc_failures(self, count: int) -> int:
+        """Makes the plan's next `count` allocations of FIR rows fail as on a full
+        device; returns how many of those asked for before were not used."""
+        left = C.c_int32()
+        self._check(_lib.rfr_plan_inject_alloc_failures(self._h, int(count), C.byref(left)), "inject_alloc_failures")
+        return left.value
 
     def autotune(self, n_samples: int, use_cache: bool = True) -> float:
         ms = C.c_double()
