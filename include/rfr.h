@@ -161,8 +161,10 @@ typedef struct {
  * first push that needs them (rfr_batch_push grows them before capturing its
  * graph; rfr_server_create sizes them for its largest buffer, so serving
  * never allocates).  Demodulation plans likewise allocate their per-push
- * scratch (the FP16 split of the stream and the rotation tables) on the first
- * push of a given size, and so do PFB plans that run their FIR as a separate
+ * scratch (the FP16 split of the stream, the rotation tables and, in the
+ * three-product form, 512 KB for each CTA that parks products: one per 128
+ * frames x 64 tones, at most one per SM, 78 MB) on the first push of a given
+ * size; a batch has the parking scratch of its one launch once.  So do PFB plans that run their FIR as a separate
  * pre-sum pass (N = 8192 and 16384; N = 2048 and 4096 with T > 8:
  * 8 bytes per channel and frame) or the oversampled phase passes; a
  * push that grows scratch synchronises the device and sizes it for that many
@@ -312,9 +314,8 @@ rfr_status rfr_state_import(rfr_plan* plan, const void* host, size_t bytes);
  *   Re = 2 P1 - P3, Im = 2 P1 + P2
  * (three real products; the same definition, Sec. III.B, rounded
  * differently), which needs D % 64 == 0 (RFR_E_UNSUPPORTED otherwise) and
- * builds its tap planes and its scratch for finished products (512 KB an SM,
- * 78 MB) on the first switch, at creation where it is the default (allocates,
- * synchronises the device).  Either switch resets the accumulation chunk to the form's
+ * builds its tap planes on the first switch, at creation where it is the
+ * default (allocates, synchronises the device).  Either switch resets the accumulation chunk to the form's
  * default (64 taps in the four-product form, 256 in the three-product
  * form).  Set it before the first push of a stream.
  */

@@ -211,7 +211,8 @@ rfr_status ensure_demod_scratch(rfr_plan* p, int64_t F, int64_t F0, cudaStream_t
         const int64_t ntp = p->demod_products == 3 ? p->ntp3 : p->ntp;
         const int64_t anchors = F0 >= 0 ? rfr::demod_anchor_rows(F0, F) : (F + rfr::kDemodBM - 2) / rfr::kDemodBM + 1;
         const int64_t rot = anchors * ntp + ntp * rfr::kDemodBM;
-        if (rows3 > p->xs3_rows_cap || rows > p->xs_rows_cap || rot > p->rot_cap) {
+        const size_t g3 = p->demod_products == 3 ? rfr::demod3_scratch_need(static_cast<int>(p->words.size()), F, p->n_sms) : 0;
+        if (rows3 > p->xs3_rows_cap || rows > p->xs_rows_cap || rot > p->rot_cap || g3 > p->g3_bytes) {
             const rfr_status rs = refuse_growth_in_capture(p, st);
             if (rs != RFR_OK) return rs;
         }
@@ -226,6 +227,16 @@ rfr_status ensure_demod_scratch(rfr_plan* p, int64_t F, int64_t F0, cudaStream_t
             p->xs3_rows_cap = 0;
             RFR_CUDA(p, dev_alloc(&p->d_xs3, static_cast<size_t>(rows3) * 6 * p->D * sizeof(uint16_t)));
             p->xs3_rows_cap = rows3;
+        }
+        // the GEMM's parked products
+        const size_t g3 = rfr::demod3_scratch_need(static_cast<int>(p->words.size()), F, p->n_sms);
+        if (g3 > p->g3_bytes) {
+            cudaDeviceSynchronize();
+            dev_free(p->d_g3);
+            p->d_g3 = nullptr;
+            p->g3_bytes = 0;
+            RFR_CUDA(p, dev_alloc(&p->d_g3, g3));
+            p->g3_bytes = g3;
         }
     }
     const int64_t rows = p->demod_products == 3 ? 0 : static_cast<int64_t>(rfr::demod_xs_rows(F, p->Lpad, p->D));
@@ -390,12 +401,16 @@ rfr_status ensure_pre_rows(rfr_plan* p, int64_t F, cudaStream_t st) {
     return RFR_OK;
 }
 
+// (a carried residue adds up to hop - 1 samples: the carry holds at most W - 1)
+int64_t frames_at_most(const rfr_plan* p, int64_t n) {
+    return frames_for_len(p, std::max<int64_t>(p->cl, p->W - 1) + n);
+}
+
 rfr_status ensure_scratch(rfr_plan* p, int64_t n) {
-    // the most frames a push of n samples can complete whatever the stream's
-    // state (a carried residue adds up to hop - 1 samples: the carry holds at
-    // most W - 1), with the rotation table sized for any first frame, so that
-    // later pushes of up to n samples never allocate (nor synchronise)
-    const int64_t F = frames_for_len(p, std::max<int64_t>(p->cl, p->W - 1) + n);
+    // for the most frames a push of n samples can complete, with the rotation
+    // table sized for any first frame, so that later pushes of up to n samples
+    // never allocate (nor synchronise)
+    const int64_t F = frames_at_most(p, n);
     if (p->mode == RFR_MODE_PFB && p->gen && F > 0) RFR_CUDA(p, rfr::gen_plan_reserve(&p->gplan, F));
     if (p->mode == RFR_MODE_PFB && p->phase_R > 1) RFR_CUDA(p, ensure_pass_tones(p, F, nullptr));
     if (p->mode == RFR_MODE_PFB && !p->gen && p->phase_R == 1 && rfr::pfb_pre_rows(p->log2n, p->Tk)) {
@@ -543,6 +558,7 @@ rfr_status push_core(rfr_plan* p, const int16_t* iq, int64_t n, const rfr_output
                     L.xs_rows = p->xs3_rows_cap;
                     L.auto_form = p->tune.demod_auto ? 1 : 0;
                     L.scratch = p->d_g3;
+                    L.scratch_bytes = p->g3_bytes;
                     L.tone_tile = p->tune.demod_bt;
                     L.fused_presplit = p->tune.demod_fused;
                     L.pair = p->tune.demod_pair;
@@ -1214,7 +1230,6 @@ rfr_status rfr_plan_set_demod_products(rfr_plan* p, int32_t products) {
         const size_t plane = static_cast<size_t>(p->ntp3) * p->Lpad3;
         double* d_h64 = nullptr;
         cudaError_t e = dev_alloc(&p->d_b3, plane * 6 * sizeof(uint16_t));
-        if (e == cudaSuccess) e = dev_alloc(&p->d_g3, rfr::demod3_scratch_bytes(p->n_sms));
         if (e == cudaSuccess) e = dev_alloc(&d_h64, static_cast<size_t>(p->L) * 8);
         if (e == cudaSuccess) e = cudaMemcpy(d_h64, p->h64.data(), static_cast<size_t>(p->L) * 8, cudaMemcpyHostToDevice);
         if (e == cudaSuccess)
@@ -1223,8 +1238,7 @@ rfr_status rfr_plan_set_demod_products(rfr_plan* p, int32_t products) {
         dev_free(d_h64);
         if (e != cudaSuccess) {
             dev_free(p->d_b3);
-            dev_free(p->d_g3);
-            p->d_b3 = p->d_g3 = nullptr;
+            p->d_b3 = nullptr;
             return cuda_fail(p, e, "three-product tap build");
         }
     }

@@ -39,6 +39,8 @@ struct rfr_batch {
     std::vector<cudaStream_t> branches;
     std::vector<cudaEvent_t> ev_join;
     std::vector<rfr::DemodGemmJob> jobs;   // deferred three-product GEMMs, one per plan
+    void* d_g3 = nullptr;                  // scratch of their launches, grown with the steps
+    size_t g3_bytes = 0;
     cudaStream_t origin = nullptr;
     cudaStream_t gemm_stream = nullptr;    // the persistent GEMM launch of the step
     cudaEvent_t ev_fork = nullptr;
@@ -64,6 +66,7 @@ void batch_destroy(rfr_batch* b) {
     if (b->ev_gemm) cudaEventDestroy(b->ev_gemm);
     if (b->origin) cudaStreamDestroy(b->origin);
     if (b->gemm_stream) cudaStreamDestroy(b->gemm_stream);
+    if (b->d_g3) cudaFree(b->d_g3);
     delete b;
 }
 
@@ -195,12 +198,27 @@ rfr_status rfr_batch_push(rfr_batch* b, const int16_t* const* bufs, const int64_
     if (!b || !bufs || !n_samples || !outs) return RFR_E_INVALID;
     const int n = static_cast<int>(b->plans.size());
     // 1. validate and grow scratch outside of any capture
+    int ctas = 0;
     for (int i = 0; i < n; ++i) {
         rfr_plan* p = b->plans[i];
         rfr_status s = rfr::push_check(p, bufs[i], n_samples[i], &outs[i]);
         if (s != RFR_OK) return batch_fail(b, s, "push " + std::to_string(i) + ": " + p->last_error);
         s = rfr::ensure_scratch(p, n_samples[i]);
         if (s != RFR_OK) return batch_fail(b, s, "scratch: " + p->last_error);
+        if (p->mode == RFR_MODE_DEMOD && p->demod_products == 3 && !p->words.empty())
+            ctas += rfr::demod3_ctas(static_cast<int>(p->words.size()), rfr::frames_at_most(p, n_samples[i]), p->n_sms);
+    }
+    const size_t g3 = rfr::demod3_scratch_bytes(std::min(ctas, b->plans[0]->n_sms));
+    if (g3 > b->g3_bytes) {
+        cudaDeviceSynchronize();
+        if (b->d_g3) cudaFree(b->d_g3);
+        b->d_g3 = nullptr;
+        b->g3_bytes = 0;
+        if (cudaMalloc(&b->d_g3, g3) != cudaSuccess) {
+            cudaGetLastError();
+            return batch_fail(b, RFR_E_NOMEM, "scratch of the batched GEMM");
+        }
+        b->g3_bytes = g3;
     }
     // 2. capture the step: fork one branch per plan, join back
     cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -228,7 +246,7 @@ rfr_status rfr_batch_push(rfr_batch* b, const int16_t* const* bufs, const int64_
     }
     if (err == RFR_OK && !gemms.empty()) {
         const cudaError_t ge = rfr::demod3_gemm(gemms.data(), static_cast<int>(gemms.size()), b->plans[0]->n_sms,
-                                                b->gemm_stream);
+                                                b->d_g3, b->g3_bytes, b->gemm_stream);
         if (ge != cudaSuccess) {
             err = RFR_E_CUDA;
             b->last_error = std::string("batched GEMM launch: ") + cudaGetErrorString(ge);

@@ -1209,13 +1209,24 @@ size_t demod_xs_rows(int64_t F, int Lpad, int D) {
 }
 
 namespace {
-// Rows of the split form's planes, and whether three planes fit the scratch.
+// Rows of the split form's planes, and whether three planes stay within what the
+// unsplit forms may need at most.
 int64_t g3_plane_ld(int64_t F) { return (F + 31) / 32 * 32; }
 bool g3_planes_fit(int n_tones, int64_t F, int n_sms) {
     return 3 * n_tones * g3_plane_ld(F) * 4 <= static_cast<int64_t>(demod3_scratch_bytes(n_sms));
 }
 }  // namespace
-size_t demod3_scratch_bytes(int n_sms) { return static_cast<size_t>(n_sms) * G3_CTA_SCRATCH * 4; }
+size_t demod3_scratch_bytes(int ctas) { return static_cast<size_t>(ctas) * G3_CTA_SCRATCH * 4; }
+// Every form's tiles hold 128 frames or more a CTA and, but for a last one, 64 tones
+// or more (a pair's odd frame tile: one CTA more).
+int demod3_ctas(int n_tones, int64_t F, int n_sms) {
+    return static_cast<int>(std::min<int64_t>(n_sms, ((F + 127) / 128 + 1) * ((n_tones + 63) / 64)));
+}
+size_t demod3_scratch_need(int n_tones, int64_t F, int n_sms) {
+    const int64_t planes = g3_planes_fit(n_tones, F, n_sms) ? 3 * n_tones * g3_plane_ld(F) * 4
+                                                            : static_cast<int64_t>(demod3_scratch_bytes(n_sms));
+    return std::max(demod3_scratch_bytes(demod3_ctas(n_tones, F, n_sms)), static_cast<size_t>(planes));
+}
 
 size_t demod3_xs_rows(int64_t F, int Lpad, int D) { return static_cast<size_t>(F + (Lpad - 1) / D); }
 
@@ -1356,6 +1367,7 @@ cudaError_t demod3_prepare(const DemodLaunch& L, cudaStream_t st, DemodGemmJob* 
     job->pair = form.pair ? 1 : 0;
     const int64_t rows = static_cast<int64_t>(demod3_xs_rows(L.F, L.Lpad, L.D));
     if (!job->fused && rows > L.xs_rows) return cudaErrorInvalidValue;
+    if (form.split && 3 * static_cast<size_t>(L.n_tones) * g3_plane_ld(L.F) * 4 > L.scratch_bytes) return cudaErrorInvalidValue;
     const int bm = form.pair ? 256 : BM;
     const int n_mt = static_cast<int>((L.F + bm - 1) / bm);
     const int n_nt = (L.n_tones + form.bw - 1) / form.bw;
@@ -1436,14 +1448,19 @@ cudaError_t demod3_prepare(const DemodLaunch& L, cudaStream_t st, DemodGemmJob* 
 }
 
 namespace {
+// room: bytes of the scratch that unsplit CTAs park their products in.
 template <bool PAIR, bool FUSED>
-cudaError_t g3_run(const G3Batch& b, int n_sms, cudaStream_t st) {
+cudaError_t g3_run(const G3Batch& b, int n_sms, size_t room, cudaStream_t st) {
+    bool parks = false;
+    for (int k = 0; k < b.n_plans; ++k) parks = parks || !b.p[k].split;
+    auto fits = [&](int grid) { return !parks || demod3_scratch_bytes(grid) <= room; };
     auto kern = demod3m_gemm_kernel<PAIR, FUSED>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(G3_SMEM));
     if (e != cudaSuccess) return e;
     const int threads = G3_THREADS;
     if (!PAIR) {
         const int grid = std::max(1, std::min(b.total_units, n_sms));
+        if (!fits(grid)) return cudaErrorInvalidValue;
         kern<<<grid, threads, G3_SMEM, st>>>(b);
         return cudaGetLastError();
     }
@@ -1470,6 +1487,7 @@ cudaError_t g3_run(const G3Batch& b, int n_sms, cudaStream_t st) {
         max_clusters.store(mc);
     }
     const int clusters = std::max(1, std::min(b.total_units, std::min(mc, n_sms / 2)));
+    if (!fits(2 * clusters)) return cudaErrorInvalidValue;
     cfg.gridDim = dim3(static_cast<unsigned>(2 * clusters), 1, 1);
     e = cudaLaunchKernelEx(&cfg, kern, b);
     if (e != cudaSuccess) return e;
@@ -1477,7 +1495,7 @@ cudaError_t g3_run(const G3Batch& b, int n_sms, cudaStream_t st) {
 }
 }  // namespace
 
-cudaError_t demod3_gemm(const DemodGemmJob* const* jobs, int n, int n_sms, cudaStream_t st) {
+cudaError_t demod3_gemm(const DemodGemmJob* const* jobs, int n, int n_sms, void* scratch, size_t room, cudaStream_t st) {
     // costliest work items first, so that the launch ends on short ones
     std::vector<const DemodGemmJob*> order(jobs, jobs + n);
     std::stable_sort(order.begin(), order.end(),
@@ -1491,11 +1509,13 @@ cudaError_t demod3_gemm(const DemodGemmJob* const* jobs, int n, int n_sms, cudaS
         for (int i = 0; i <= n; ++i) {
             const bool flush = i == n || b.n_plans == kG3MaxPlans;
             if (flush && b.n_plans > 0) {
-                // the launch's CTAs park partial products in its first plan's scratch
-                for (int k = 1; k < b.n_plans; ++k)
-                    if (!b.p[k].split) b.p[k].scratch = b.p[0].scratch;
-                const cudaError_t e = pair ? g3_run<true, false>(b, n_sms, st)
-                                           : (fused ? g3_run<false, true>(b, n_sms, st) : g3_run<false, false>(b, n_sms, st));
+                // the launch's CTAs, whatever plans' tiles they take, park products in the one
+                // scratch of the call (the kernel finds it at its first plan's)
+                for (int k = 0; k < b.n_plans; ++k)
+                    if (!b.p[k].split) b.p[k].scratch = static_cast<float*>(scratch);
+                const cudaError_t e = pair ? g3_run<true, false>(b, n_sms, room, st)
+                                           : (fused ? g3_run<false, true>(b, n_sms, room, st)
+                                                    : g3_run<false, false>(b, n_sms, room, st));
                 if (e != cudaSuccess) return e;
                 for (int k = 0; k < b.n_plans; ++k)
                     if (b.p[k].split) {
@@ -1524,7 +1544,7 @@ cudaError_t demod3_launch(const DemodLaunch& L, cudaStream_t st) {
     cudaError_t e = demod3_prepare(L, st, &job, false);
     if (e != cudaSuccess || job.n_units <= 0) return e;
     const DemodGemmJob* jp = &job;
-    return demod3_gemm(&jp, 1, L.n_sms, st);
+    return demod3_gemm(&jp, 1, L.n_sms, L.scratch, L.scratch_bytes, st);
 }
 
 }  // namespace rfr

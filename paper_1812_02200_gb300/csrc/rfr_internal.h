@@ -157,7 +157,8 @@ struct DemodLaunch {
     int tone_tile;              //   tones per single-CTA tile, 128 or 64 (0 = 128)
     int fused_presplit;         //   producers convert the int16 stream themselves
     int pair;                   //   two-SM tiles
-    void* scratch;              // three-product GEMM: demod3_scratch_bytes
+    void* scratch;              // three-product GEMM: demod3_scratch_need bytes at least
+    size_t scratch_bytes;
 };
 // The three-product GEMM of one push, described for a persistent launch that
 // may cover several plans (opaque record of demod.cu).
@@ -183,10 +184,14 @@ cudaError_t demod3_launch(const DemodLaunch& L, cudaStream_t st);
 // GEMM's description in *job (shared_launch: it will run beside other plans')
 cudaError_t demod3_prepare(const DemodLaunch& L, cudaStream_t st, DemodGemmJob* job, bool shared_launch);
 // persistent GEMM launch(es) over the jobs' work items (one per form and per
-// 16 plans)
-cudaError_t demod3_gemm(const DemodGemmJob* const* jobs, int n, int n_sms, cudaStream_t st);
+// 16 plans); scratch: room bytes for the CTAs' parked products
+cudaError_t demod3_gemm(const DemodGemmJob* const* jobs, int n, int n_sms, void* scratch, size_t room, cudaStream_t st);
 size_t demod3_xs_rows(int64_t F, int Lpad, int D);
-size_t demod3_scratch_bytes(int n_sms);
+// CTAs that a push of up to F frames launches at most (whatever its form), what they
+// park in all, and the scratch that such a push needs (never less for more frames)
+int demod3_ctas(int n_tones, int64_t F, int n_sms);
+size_t demod3_scratch_bytes(int ctas);
+size_t demod3_scratch_need(int n_tones, int64_t F, int n_sms);
 int demod_anchor_rows(int64_t F0, int64_t F);
 
 // -------------------------------------------------------------- chirp
@@ -293,7 +298,8 @@ struct rfr_plan {
     int accum_chunk = 2;           // demod: K blocks per TMEM accumulation chunk
     int demod_products = 4;        // demod GEMM form: 4 (real embedding) or 3 (Gauss)
     void* d_b3 = nullptr;          // three-product form: six tap planes
-    void* d_g3 = nullptr;          // three-product form: the GEMM's scratch
+    void* d_g3 = nullptr;          // three-product form: the GEMM's scratch, grown with the pushes
+    size_t g3_bytes = 0;
     void* d_xs3 = nullptr;         // three-product form: six source planes
     int64_t xs3_rows_cap = 0;
     int32_t Lpad3 = 0, ntp3 = 0, tap_exp3 = 0;
@@ -354,6 +360,8 @@ rfr_status push_core(rfr_plan* p, const int16_t* iq, int64_t n, const rfr_output
 // Grow the plan's per-push scratch for a push of n samples (may allocate and
 // synchronise the device; never call it during stream capture).
 rfr_status ensure_scratch(rfr_plan* p, int64_t n);
+// Most frames that a push of n samples can complete whatever the stream's state.
+int64_t frames_at_most(const rfr_plan* p, int64_t n);
 int64_t frames_for_samples(const rfr_plan* p, int64_t n);
 // Argument and capacity checks of push_core without side effects.
 rfr_status push_check(rfr_plan* p, const int16_t* iq, int64_t n, const rfr_output* o);
