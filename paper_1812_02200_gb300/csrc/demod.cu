@@ -43,6 +43,7 @@
 #include <cstdint>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 #include "dev_common.cuh"
@@ -448,7 +449,7 @@ constexpr size_t G3_SMEM = 1024 + G3_STAGES * G3_STAGE_BYTES + G3_BARS_BYTES + G
 struct G3Plan {
     CUtensorMap a[6];   // (x sum/2, xr, xi) x (hi, lo): [rows][D] fp16, Toeplitz view (unused when fused)
     CUtensorMap b[6];   // (cr, ci - cr, cr + ci) x (hi, lo): [ntp][Lpad] fp16, K-major
-    GemmArgs g;         // n_mt, n_nt: tiles (of a pair in the pair form); kchunk: K-blocks per chunk
+    GemmArgs g;         // n_mt, n_nt: tiles (of a pair in the pair form); kchunk: half K-blocks per chunk
     int unit0;          // first global work item of this plan
     int bw;             // tones per tile
     int split;          // work items are single products, written to planes
@@ -923,8 +924,11 @@ demod3m_gemm_kernel(const __grid_constant__ G3Batch bt) {
                 const G3Unit u = g3_unit<PAIR>(P, unit, rank);
                 const uint32_t idesc = umma::idesc_f16_f32(PAIR ? 256 : 128, u.width);
                 for (int q = u.q0; q < u.q1 && !stop; ++q) {
-                    for (int kb0 = 0; kb0 < g.KB && !stop; kb0 += g.kchunk, ++phase) {
-                        const int kb1 = min(kb0 + g.kchunk, g.KB);
+                    // chunks of half K-blocks (32 taps); chunks of whole blocks have their own
+                    // loop (a block's twelve MMAs in two pieces: 800 us where this takes 733,
+                    // 2^24 samples x 2048 tones)
+                    for (int h0 = 0; h0 < 2 * g.KB && !stop; h0 += g.kchunk, ++phase) {
+                        const int h1 = min(h0 + g.kchunk, 2 * g.KB);
                         const uint32_t slot = phase % SLOTS, use = phase / SLOTS;
                         if (*abort_flag || !mbar_wait(&sempty[slot], (use & 1) ^ 1, status0)) {
                             *abort_flag = 1;
@@ -933,21 +937,27 @@ demod3m_gemm_kernel(const __grid_constant__ G3Batch bt) {
                         }
                         umma::fence_after_sync();
                         const uint32_t d_tmem = tmem + slot * TW;
-                        for (int kb = kb0; kb < kb1; ++kb, ++it) {
-                            const int s = it % STAGES;
-                            const uint32_t ph = (it / STAGES) & 1;
-                            if (!mbar_wait(&full[s], ph, status0)) {
+                        auto arrived = [&] {                            // the block's operands
+                            if (!mbar_wait(&full[it % STAGES], (it / STAGES) & 1, status0)) {
                                 *abort_flag = 1;
                                 stop = true;
-                                break;
+                                return false;
                             }
                             umma::fence_after_sync();
-                            const uint32_t ah = smem_u32(smem + s * G3_STAGE_BYTES), al = ah + G3_OP_BYTES;
+                            return true;
+                        };
+                        auto release = [&] {                            // its stage, in both CTAs of a pair
+                            if constexpr (PAIR) umma::commit_2sm(&empty[it % STAGES]);
+                            else umma::commit(&empty[it % STAGES]);
+                            ++it;
+                        };
+                        auto steps = [&](auto n, uint32_t from, bool fresh) {   // n steps of 16 taps
+                            const uint32_t ah = smem_u32(smem + (it % STAGES) * G3_STAGE_BYTES) + from, al = ah + G3_OP_BYTES;
                             const uint32_t bh = ah + 2 * G3_OP_BYTES, bl = ah + 3 * G3_OP_BYTES;
 #pragma unroll
-                            for (int k = 0; k < G3_BK / 16; ++k) {
+                            for (int k = 0; k < n; ++k) {
                                 const uint32_t off = k * 32;
-                                const uint32_t acc = (kb > kb0 || k > 0) ? 1u : 0u;
+                                const uint32_t acc = (!fresh || k > 0) ? 1u : 0u;
                                 const uint64_t dah = umma::desc_k_sw128(ah + off), dal = umma::desc_k_sw128(al + off);
                                 const uint64_t dbh = umma::desc_k_sw128(bh + off), dbl = umma::desc_k_sw128(bl + off);
                                 if constexpr (PAIR) {
@@ -960,8 +970,19 @@ demod3m_gemm_kernel(const __grid_constant__ G3Batch bt) {
                                     umma::mma_f16(d_tmem, dal, dbh, idesc, 1u);
                                 }
                             }
-                            if constexpr (PAIR) umma::commit_2sm(&empty[s]);      // frees the stage in both CTAs
-                            else umma::commit(&empty[s]);
+                        };
+                        if ((g.kchunk & 1) == 0) {
+                            for (int h = h0; h < h1; h += 2) {
+                                if (!arrived()) break;
+                                steps(std::integral_constant<int, G3_BK / 16>{}, 0, h == h0);
+                                release();
+                            }
+                        } else {
+                            for (int h = h0; h < h1; ++h) {
+                                if ((h & 1) == 0 && !arrived()) break;
+                                steps(std::integral_constant<int, G3_BK / 32>{}, (h & 1) * G3_BK, h == h0);
+                                if (h & 1) release();
+                            }
                         }
                         if constexpr (PAIR) umma::commit_2sm(&sfull[slot]);
                         else umma::commit(&sfull[slot]);
@@ -987,7 +1008,7 @@ demod3m_gemm_kernel(const __grid_constant__ G3Batch bt) {
             for (int q = u.q0; q < u.q1 && ok; ++q) {
 #pragma unroll
                 for (int i = 0; i < TPG; ++i) sum[i] = 0.f;
-                for (int kb0 = 0; kb0 < g.KB; kb0 += g.kchunk, ++phase) {
+                for (int h0 = 0; h0 < 2 * g.KB; h0 += g.kchunk, ++phase) {
                     const uint32_t slot = phase % SLOTS, use = phase / SLOTS;
                     if (*abort_flag || !mbar_wait(&sfull[slot], use & 1, status0)) {
                         *abort_flag = 1;
@@ -1428,10 +1449,11 @@ cudaError_t demod3_prepare(const DemodLaunch& L, cudaStream_t st, DemodGemmJob* 
     g.n_tones = L.n_tones;
     g.ntp = L.ntp;
     g.KB = L.Lpad / G3_BK;
-    // the three MMAs of a tap set share one accumulator, where they would take
-    // two (hi.hi + lo.hi beside hi.lo) half as many blocks make a chunk: the
-    // accumulator takes fewer additions of smaller partial sums
-    g.kchunk = L.kchunk > 1 ? (L.kchunk + 1) / 2 : 1;
+    // the three MMAs of a tap set share one accumulator, where two would take them
+    // apart (hi.hi + lo.hi beside hi.lo); a chunk is half as long for that, as many
+    // half K-blocks as the plan says blocks: the accumulator takes fewer additions of
+    // smaller partial sums
+    g.kchunk = std::max(L.kchunk, 1);
     g.two_d = L.D;                 // columns of a Toeplitz source row (one plane)
     g.n_mt = n_mt;
     g.n_nt = n_nt;
