@@ -162,9 +162,8 @@ typedef struct {
  * graph; rfr_server_create sizes them for its largest buffer, so serving
  * never allocates).  Demodulation plans likewise allocate their per-push
  * scratch (the FP16 split of the stream, the rotation tables and, in the
- * three-product form, 512 KB for each CTA that parks products: one per 128
- * frames x 64 tones, at most one per SM, 78 MB) on the first push of a given
- * size; a batch has the parking scratch of its one launch once.  So do PFB plans that run their FIR as a separate
+ * three-product form, room for products, 78 MB at most) on the first push of a
+ * given size, and so do PFB plans that run their FIR as a separate
  * pre-sum pass (N = 8192 and 16384; N = 2048 and 4096 with T > 8:
  * 8 bytes per channel and frame) or the oversampled phase passes; a
  * push that grows scratch synchronises the device and sizes it for that many
@@ -476,11 +475,11 @@ rfr_status rfr_plan_get_tune(const rfr_plan* plan, int32_t* pfb_lookahead, int32
                              int32_t* tuned);
 /* Tones per tile of a three-product demodulation plan's single-CTA GEMM form
  * (128 or 64; 128 by default); 0 for other plans.  A plan starts out with the
- * form of its GEMM picked per push by size (two-SM tiles of up to 256 frames
- * x 256 tones, single-CTA tiles of 128 frames x up to 128 tones, either with
+ * form of its GEMM picked per push by size (two-SM tiles of 256 frames x up to
+ * 256 tones, single-CTA tiles of 128 frames x up to 128 tones, either with
  * its three products as separate work items when tiles are few).  Setting a
- * width, the pair form or the fused pre-split pins the form instead.  All are
- * result-neutral.  Errors: RFR_E_INVALID (not a three-product demodulation
+ * width, the pair form or the fused pre-split pins that much of the form; the
+ * rest stays picked by size.  All are result-neutral.  Errors: RFR_E_INVALID (not a three-product demodulation
  * plan, or a width other than 64 or 128). */
 rfr_status rfr_plan_get_tone_tile(const rfr_plan* plan, int32_t* tones_per_tile);
 rfr_status rfr_plan_set_tone_tile(rfr_plan* plan, int32_t tones_per_tile);

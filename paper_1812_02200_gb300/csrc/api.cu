@@ -218,24 +218,20 @@ rfr_status ensure_demod_scratch(rfr_plan* p, int64_t F, int64_t F0, cudaStream_t
         }
     }
     if (p->demod_products == 3) {
-        // six fp16 planes [rows][D] of the Gauss three-product form
+        // six fp16 planes [rows][D] of the Gauss three-product form and, behind them,
+        // the GEMM's parked products (both grow with the frames: one allocation)
         const int64_t rows3 = static_cast<int64_t>(rfr::demod3_xs_rows(F, p->Lpad3, p->D));
-        if (rows3 > p->xs3_rows_cap) {
+        const size_t g3 = rfr::demod3_scratch_need(static_cast<int>(p->words.size()), F, p->n_sms);
+        if (rows3 > p->xs3_rows_cap || g3 > p->g3_bytes) {
+            const size_t planes = (static_cast<size_t>(rows3) * 6 * p->D * sizeof(uint16_t) + 1023) / 1024 * 1024;
             cudaDeviceSynchronize();
             dev_free(p->d_xs3);
-            p->d_xs3 = nullptr;
+            p->d_xs3 = p->d_g3 = nullptr;
             p->xs3_rows_cap = 0;
-            RFR_CUDA(p, dev_alloc(&p->d_xs3, static_cast<size_t>(rows3) * 6 * p->D * sizeof(uint16_t)));
-            p->xs3_rows_cap = rows3;
-        }
-        // the GEMM's parked products
-        const size_t g3 = rfr::demod3_scratch_need(static_cast<int>(p->words.size()), F, p->n_sms);
-        if (g3 > p->g3_bytes) {
-            cudaDeviceSynchronize();
-            dev_free(p->d_g3);
-            p->d_g3 = nullptr;
             p->g3_bytes = 0;
-            RFR_CUDA(p, dev_alloc(&p->d_g3, g3));
+            RFR_CUDA(p, dev_alloc(&p->d_xs3, planes + g3));
+            p->d_g3 = static_cast<unsigned char*>(p->d_xs3) + planes;
+            p->xs3_rows_cap = rows3;
             p->g3_bytes = g3;
         }
     }
@@ -611,7 +607,7 @@ void destroy(rfr_plan* p) {
     for (void* q : {static_cast<void*>(p->d_h), p->d_tw, p->d_tw_cl, static_cast<void*>(p->d_bins),
                     static_cast<void*>(p->d_words), static_cast<void*>(p->d_rates), static_cast<void*>(p->d_h32), p->d_c32, p->d_bhi, p->d_blo,
                     static_cast<void*>(p->d_status), static_cast<void*>(p->d_carry[0]),
-                    static_cast<void*>(p->d_carry[1]), p->d_xs_hi, p->d_xs_lo, p->d_rot, p->d_qfull, p->d_b3, p->d_g3, p->d_xs3,
+                    static_cast<void*>(p->d_carry[1]), p->d_xs_hi, p->d_xs_lo, p->d_rot, p->d_qfull, p->d_b3, p->d_xs3,
                     p->d_qtones, p->d_ptones, p->d_pre})
         dev_free(q);
     for (int i = 0; i < rfr_plan::kStageBufs; ++i) {

@@ -39,7 +39,7 @@ struct rfr_batch {
     std::vector<cudaStream_t> branches;
     std::vector<cudaEvent_t> ev_join;
     std::vector<rfr::DemodGemmJob> jobs;   // deferred three-product GEMMs, one per plan
-    void* d_g3 = nullptr;                  // scratch of their launches, grown with the steps
+    void* d_g3 = nullptr;                  // scratch of their launches where no plan's is large enough
     size_t g3_bytes = 0;
     cudaStream_t origin = nullptr;
     cudaStream_t gemm_stream = nullptr;    // the persistent GEMM launch of the step
@@ -208,8 +208,16 @@ rfr_status rfr_batch_push(rfr_batch* b, const int16_t* const* bufs, const int64_
         if (p->mode == RFR_MODE_DEMOD && p->demod_products == 3 && !p->words.empty())
             ctas += rfr::demod3_ctas(static_cast<int>(p->words.size()), rfr::frames_at_most(p, n_samples[i]), p->n_sms);
     }
+    // (a plan's own scratch where one is large enough)
     const size_t g3 = rfr::demod3_scratch_bytes(std::min(ctas, b->plans[0]->n_sms));
-    if (g3 > b->g3_bytes) {
+    void* scratch = b->d_g3;
+    size_t room = b->g3_bytes;
+    for (rfr_plan* p : b->plans)
+        if (room < g3 && p->g3_bytes >= g3) {
+            scratch = p->d_g3;
+            room = p->g3_bytes;
+        }
+    if (g3 > room) {
         cudaDeviceSynchronize();
         if (b->d_g3) cudaFree(b->d_g3);
         b->d_g3 = nullptr;
@@ -218,7 +226,8 @@ rfr_status rfr_batch_push(rfr_batch* b, const int16_t* const* bufs, const int64_
             cudaGetLastError();
             return batch_fail(b, RFR_E_NOMEM, "scratch of the batched GEMM");
         }
-        b->g3_bytes = g3;
+        b->g3_bytes = room = g3;
+        scratch = b->d_g3;
     }
     // 2. capture the step: fork one branch per plan, join back
     cudaStream_t st = static_cast<cudaStream_t>(stream);
@@ -246,7 +255,7 @@ rfr_status rfr_batch_push(rfr_batch* b, const int16_t* const* bufs, const int64_
     }
     if (err == RFR_OK && !gemms.empty()) {
         const cudaError_t ge = rfr::demod3_gemm(gemms.data(), static_cast<int>(gemms.size()), b->plans[0]->n_sms,
-                                                b->d_g3, b->g3_bytes, b->gemm_stream);
+                                                scratch, room, b->gemm_stream);
         if (ge != cudaSuccess) {
             err = RFR_E_CUDA;
             b->last_error = std::string("batched GEMM launch: ") + cudaGetErrorString(ge);

@@ -380,42 +380,50 @@ demod_gemm_kernel(const __grid_constant__ CUtensorMap tmAh, const __grid_constan
 // 64 bytes a clock from L2.  A tile of 128 frames x 128 tones on one SM needs
 // 36-40 KB of shared-memory traffic and 16 KB from L2 for 192 clocks of
 // tensor work: both limits lie above the tensor time, and the tensor pipe
-// measured 62 % active.  The large form (PAIR) therefore gives two SMs one
-// tile of 256 frames x 256 tones (cta_group::2 MMAs, M = 256): each SM holds
-// its 128 frames and half the tones' tap rows and reads 8 KB per MMA of 128
-// clocks, 40 KB and 16 KB from L2 for 384 clocks of tensor work.
+// measured 62 % active.  PAIR therefore gives two SMs one tile of 256 frames
+// (cta_group::2 MMAs, M = 256): each SM holds its 128 frames and half the
+// tones' tap rows.  At 256 tones (WIDE) it reads 8 KB per MMA of 128 clocks,
+// 40 KB and 16 KB from L2 for 384 clocks of tensor work; at 128, 24 KB of reads
+// and 12 KB of writes for 192.
 //
-// A tile of that size leaves no room for both FP32 sums (re and im) of every
-// output in registers, so a tile runs its three products one after the other
-// over all of K: the epilogue warps hold ONE product's FP32 sums (64 tones a
-// thread) and park each product in a scratch of the CTA (L2-resident).
-// Finisher warps fetch a parked tile back by bulk copies, combine, rotate and
-// store it while the next tile's first product runs.  (Done by the epilogue
-// warps at the tile's end it stalled the MMAs, which run at most two chunks
-// ahead, by about 50,000 clocks of 400,000 per tile; finishers with register
-// loads could not keep enough bytes in flight either.)
+// WIDE leaves no room for both FP32 sums (re and im) of every output in
+// registers, so a tile runs its three products one after the other over all
+// of K: the epilogue warps hold ONE product's FP32 sums (64 tones a thread)
+// and park each product in a scratch of the CTA (L2-resident).  Finisher warps
+// fetch a parked tile back by bulk copies, combine, rotate and store it while
+// the next tile's first two products run.  (Done by the epilogue warps at the
+// tile's end it stalled the MMAs, which run at most two chunks ahead, by about
+// 50,000 clocks of 400,000 per tile; finishers with register loads could not
+// keep enough bytes in flight either.)  Two finisher warps take some 120,000
+// clocks a tile, more than the MMAs of filters up to 2500 taps, so short filters
+// take tiles of up to 128 tones instead: the first product's sums wait in
+// TMEM (its last 128 columns, beside three accumulators), the epilogue holds
+// im = 2 P1 + P2 and P3 of 32 tones a thread and stores the outputs itself.
 //
 // Measured, 2^27 samples x 2048 tones, L = 4096, D = 2048, whole push: 7.6 ms
 // with tiles of 128 x 128 on one SM, 6.0 ms with pairs (short runs; 6.4 ms in
 // seconds-long runs under the power cap).  The MMAs alone would take 3.84 ms
-// at 2.07 GHz.
+// at 2.07 GHz.  2^24 samples x 1000 tones, L = 1024, D = 512: 579 us with tiles
+// of 128 x 128 on one SM, 630 with wide pairs, 447 with pairs of 128 tones;
+// L = 256, D = 64: 1650, 3540 and 1280 us.
 //
 // Precision: the three MMAs of a term set go to the same FP32 TMEM
 // accumulator, which collects a chunk of K (128 taps by default) before the
-// epilogue adds it into the FP32 sums; the accumulator is double-buffered.
+// epilogue adds it into the FP32 sums; two (WIDE) or three accumulators take turns.
 // Every form sums each output in the same order (16 taps hi.hi, hi.lo, lo.hi;
 // chunks; products), so tile shape, form and the plans sharing a launch never
 // change a result.
 //
-// Forms.  PAIR as above; the tone tile is narrowed (in steps of 32) so that a
-// plan's tones divide evenly.  One CTA per tile of 128 frames x at most 128
-// tones for plans with too few tiles to fill the chip's pairs.  Either form
+// Forms.  Pairs, wide or of up to 128 tones, as above; the tone tile is narrowed
+// (in steps of 32) so that a plan's tones divide evenly.  One CTA per tile of 128
+// frames x at most 128 tones where that fills the chip's waves better.  Any form
 // may be SPLIT when tiles are few: a work item is then one product of a tile,
 // the products go to planes in the scratch and combine3_kernel finishes.
+// G3Form::clocks and g3_choose pick by size.
 //
 // Fused pre-split (FUSED, single-CTA form): instead of TMA loads of the six
 // pre-split source planes (written to HBM by prep3_kernel, 12 bytes per
-// sample), two producer warps read the int16 stream view [carry | buffer] and
+// sample), three producer warps read the int16 stream view [carry | buffer] and
 // write each stage's A hi/lo tiles themselves, in the 128-byte swizzled layout
 // the TMA would produce, with the same FP32 -> FP16 hi/lo rounding as the
 // pre-split kernel (bit-identical planes, so bit-identical results); only the
@@ -427,24 +435,34 @@ demod_gemm_kernel(const __grid_constant__ CUtensorMap tmAh, const __grid_constan
 // from the plans' first-item offsets.
 constexpr int G3_BK = 64;                                  // complex taps per K-block
 constexpr uint32_t G3_OP_BYTES = 128 * G3_BK * 2;          // one operand tile: 128 rows x 64 fp16
-constexpr int G3_STAGES = 3;                               // A hi, A lo, B hi, B lo each
-constexpr uint32_t G3_STAGE_BYTES = 4 * G3_OP_BYTES;
 constexpr int G3_SLOTS_MAX = 4;
 constexpr uint32_t G3_TMEM_COLS = 512;
 constexpr int G3_EPI_WARPS = 16;          // 4 lane quadrants x 4 tone groups
-constexpr int G3_FUSED_PRODUCERS = 2;                       // producer warps of the fused form
-constexpr int G3_THREADS = (G3_EPI_WARPS + 4) * 32;         // + producer(s), MMA issuer, finishers
-constexpr int G3_PAIR_TONES = 256, G3_SINGLE_TONES = 128;   // widest tone tiles
+constexpr int G3_FUSED_PRODUCERS = 3;                       // producer warps of the fused form
+constexpr int G3_WIDE_TONES = 256, G3_TONES = 128;          // widest tone tiles
 // scratch of one CTA: a ring of products, [tone][128 frames] FP32 each
-constexpr int G3_PLANES = 4;   // a ring: 3 measured 1-2 % slower (5.97 against 6.02 ms, 2^27 samples)
-constexpr int64_t G3_PLANE = int64_t(G3_PAIR_TONES) * 128;
+constexpr int G3_PLANES = 4;   // a ring: 3 measured 0.8 % slower (6.02 against 5.97 ms, 2^27 samples)
+constexpr int64_t G3_PLANE = int64_t(G3_WIDE_TONES) * 128;
 constexpr int64_t G3_CTA_SCRATCH = G3_PLANES * G3_PLANE;
 // finisher staging: chunks of two tones (three products of 128 frames, then the
 // tones' 128 rotation steps), FIN_BUFS chunks per warp in flight
-constexpr int G3_FIN_BUFS = 3, G3_MAX_FINISHERS = 2;
+constexpr int G3_FIN_BUFS = 3, G3_FINISHERS = 2;
 constexpr uint32_t G3_FIN_BYTES = 3 * 2 * 128 * 4 + 2 * 128 * 8;
 constexpr uint32_t G3_BARS_BYTES = 256;
-constexpr size_t G3_SMEM = 1024 + G3_STAGES * G3_STAGE_BYTES + G3_BARS_BYTES + G3_MAX_FINISHERS * G3_FIN_BUFS * G3_FIN_BYTES;
+// What the kernel's forms differ in (see the Gauss form's comment).
+template <bool PAIR, bool FUSED, bool WIDE>
+struct G3Cfg {
+    static constexpr int TW = WIDE ? G3_WIDE_TONES : G3_TONES;             // columns of a TMEM slot
+    static constexpr int SLOTS = WIDE ? 2 : 3;
+    static constexpr uint32_t PARK = 3 * G3_TONES;                         // not WIDE: the first product's columns
+    static constexpr uint32_t B_BYTES = PAIR ? TW / 2 * G3_BK * 2 : TW * G3_BK * 2;   // of a CTA's rows of B
+    static constexpr uint32_t STAGE_BYTES = 2 * G3_OP_BYTES + 2 * B_BYTES;  // A hi, A lo, B hi, B lo
+    static constexpr int STAGES = STAGE_BYTES > 48 * 1024 ? 3 : 4;
+    static constexpr int FINISHERS = WIDE ? G3_FINISHERS : 0;
+    static constexpr int MMA_WARP = G3_EPI_WARPS + (FUSED ? G3_FUSED_PRODUCERS : 1);
+    static constexpr int THREADS = (MMA_WARP + 1 + FINISHERS) * 32;
+    static constexpr size_t SMEM = 1024 + STAGES * STAGE_BYTES + G3_BARS_BYTES + FINISHERS * G3_FIN_BUFS * G3_FIN_BYTES;
+};
 
 struct G3Plan {
     CUtensorMap a[6];   // (x sum/2, xr, xi) x (hi, lo): [rows][D] fp16, Toeplitz view (unused when fused)
@@ -453,7 +471,7 @@ struct G3Plan {
     int unit0;          // first global work item of this plan
     int bw;             // tones per tile
     int split;          // work items are single products, written to planes
-    float* scratch;     // [CTA][4][256][128] (or the split form's planes [3][n_tones][pld])
+    float* scratch;     // wide form: [CTA][4][256][128]; split: planes [3][n_tones][pld]
     int64_t pld;
     // fused form: the int16 stream view v[s] = s < cl ? carry[s] : buf[s - cl]
     // for s < lv (0 beyond); vec: the buffer part may be read 16 bytes at a time
@@ -627,47 +645,44 @@ __global__ void __launch_bounds__(256) prep3_kernel(const Prep3Args a) {
     }
 }
 
-// One row (frame m) of a stage's A hi/lo tiles in the fused form: view
-// samples s0 .. s0+63 -> plane q ((xr+xi)/2, xr or xi) -> FP16 hi/lo, eight
-// samples (one 16-byte chunk) at a time, chunk c of row i stored at
-// i*128 + ((c ^ (i & 7)) << 4) (the 128-byte swizzle).
-__device__ __forceinline__ void g3_fill_row(const G3Plan& P, int q, int64_t s0, unsigned char* ahi,
-                                            unsigned char* alo, int i) {
-    const bool in_buf = P.vec && s0 >= P.cl && s0 + G3_BK <= P.lv;
-    const uint32_t* bp = P.buf + (s0 - P.cl);
-#pragma unroll 2
-    for (int c = 0; c < G3_BK / 8; ++c) {
-        uint32_t w[8];
-        if (in_buf) {
-            const uint4 u0 = __ldg(reinterpret_cast<const uint4*>(bp + c * 8));
-            const uint4 u1 = __ldg(reinterpret_cast<const uint4*>(bp + c * 8 + 4));
-            w[0] = u0.x; w[1] = u0.y; w[2] = u0.z; w[3] = u0.w;
-            w[4] = u1.x; w[5] = u1.y; w[6] = u1.z; w[7] = u1.w;
-        } else {
+// Fused pre-split: chunk c (8 samples) of row i of a stage's A hi/lo tiles of plane q,
+// the samples from s on, in the 128-byte swizzled layout of the TMA loads (16-byte
+// chunk c of row i at chunk c ^ (i & 7)).  Eight lanes take a row, so that a warp
+// reads runs of 256 bytes.
+__device__ __forceinline__ void g3_fill_chunk(const G3Plan& P, int q, int64_t s, unsigned char* ahi, unsigned char* alo,
+                                              int i, int c) {
+    uint32_t w[8];
+    const uint32_t* bp = P.buf + (s - P.cl);
+    if (P.vec && s >= P.cl && s + 8 <= P.lv && (reinterpret_cast<uintptr_t>(bp) & 15) == 0) {
+        const uint4 u0 = __ldg(reinterpret_cast<const uint4*>(bp)), u1 = __ldg(reinterpret_cast<const uint4*>(bp) + 1);
+        w[0] = u0.x; w[1] = u0.y; w[2] = u0.z; w[3] = u0.w;
+        w[4] = u1.x; w[5] = u1.y; w[6] = u1.z; w[7] = u1.w;
+    } else {
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const int64_t sv = s0 + c * 8 + e;
-                w[e] = sv < P.lv ? (sv < P.cl ? __ldg(P.carry + sv) : __ldg(P.buf + (sv - P.cl))) : 0u;
-            }
+        for (int e = 0; e < 8; ++e) {
+            const int64_t sv = s + e;
+            w[e] = sv < P.lv ? (sv < P.cl ? __ldg(P.carry + sv) : __ldg(P.buf + (sv - P.cl))) : 0u;
         }
-        uint32_t hi[4], lo[4];
-#pragma unroll
-        for (int e = 0; e < 8; e += 2) g3_split_pair(w[e], w[e + 1], q, hi[e / 2], lo[e / 2]);
-        const uint32_t off = static_cast<uint32_t>(i) * 128u + (static_cast<uint32_t>(c ^ (i & 7)) << 4);
-        *reinterpret_cast<uint4*>(ahi + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-        *reinterpret_cast<uint4*>(alo + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
     }
+    uint32_t hi[4], lo[4];
+#pragma unroll
+    for (int e = 0; e < 8; e += 2) g3_split_pair(w[e], w[e + 1], q, hi[e / 2], lo[e / 2]);
+    const uint32_t off = static_cast<uint32_t>(i) * 128u + (static_cast<uint32_t>(c ^ (i & 7)) << 4);
+    *reinterpret_cast<uint4*>(ahi + off) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+    *reinterpret_cast<uint4*>(alo + off) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
 }
 
-// An output from its products and rotation factors.
-__device__ __forceinline__ float2 g3_output(float p1, float p2, float p3, float inv_scale, float2 an, float2 sp) {
-    const float re = fmaf(2.f, p1, -p3), im = fmaf(2.f, p1, p2);
+// An output from its products (re, im) and rotation factors.
+__device__ __forceinline__ float2 g3_rotate(float re, float im, float inv_scale, float2 an, float2 sp) {
     return cmul(make_float2(re * inv_scale, im * inv_scale), cmul(an, sp));
+}
+__device__ __forceinline__ float2 g3_output(float p1, float p2, float p3, float inv_scale, float2 an, float2 sp) {
+    return g3_rotate(fmaf(2.f, p1, -p3), fmaf(2.f, p1, p2), inv_scale, an, sp);
 }
 
 // Outputs of a CTA's last tile, by all its epilogue and finisher warps: lane l
-// takes frames 4 l .. 4 l + 3, warp w of nw (less the `skip` producer and MMA
-// warps between the two kinds) every tone of its number, FT in flight.
+// takes frames l + 32 r (r < 4) of the tile, warp w of nw (less the `skip` producer
+// and MMA warps between the two kinds) every tone of its number, FT in flight.
 __device__ __noinline__ void g3_finish(const G3Plan& P, const G3Unit u, const float* scr_cta, uint32_t tile, int lane,
                                           int w, int nw, int skip) {
     constexpr int FT = 2;
@@ -676,14 +691,10 @@ __device__ __noinline__ void g3_finish(const G3Plan& P, const G3Unit u, const fl
     nw -= skip;
     const float* pl[3];
 #pragma unroll
-    for (int q = 0; q < 3; ++q) pl[q] = scr_cta + ((3 * tile + q) % G3_PLANES) * G3_PLANE + 4 * lane;
-    const int64_t k = u.m0 + 4 * lane;               // the lane's first frame
-    const int64_t K = g.F0 + k;
-    const int rows = static_cast<int>(k < g.F ? (g.F - k < 4 ? g.F - k : 4) : 0);
-    if (rows == 0) return;
-    // four frames of one anchor row, with aligned steps; 16-byte stores
-    const bool near = (g.F0 & 3) == 0;
-    const bool vec = rows == 4 && ((reinterpret_cast<uintptr_t>(g.out + g.fo + k) | static_cast<uintptr_t>(g.ld * 8)) & 15) == 0;
+    for (int q = 0; q < 3; ++q) pl[q] = scr_cta + ((3 * tile + q) % G3_PLANES) * G3_PLANE + lane;
+    const int64_t k = u.m0 + lane;                   // the lane's first frame
+    const int at = static_cast<int>(g.F0 % BM) + lane;   // its place from the tile's first anchor on
+    const float2* const anc = g.anchors + ((g.F0 + u.m0) / BM - g.F0 / BM) * g.ntp + u.n0;
     const int n = min(u.width, g.n_tones - u.n0);
 #pragma unroll 1
     for (int c0 = w; c0 < n; c0 += nw * FT) {
@@ -691,58 +702,30 @@ __device__ __noinline__ void g3_finish(const G3Plan& P, const G3Unit u, const fl
         float2 an[FT][4], sp[FT][4];
 #pragma unroll
         for (int f = 0; f < FT; ++f) {
-            const int c = c0 + f * nw, t = u.n0 + c;
+            const int c = c0 + f * nw;
             if (c >= n) continue;
 #pragma unroll
-            for (int q = 0; q < 3; ++q) {
-                const float4 v = __ldcg(reinterpret_cast<const float4*>(pl[q] + c * 128));
-                p[f][q][0] = v.x;
-                p[f][q][1] = v.y;
-                p[f][q][2] = v.z;
-                p[f][q][3] = v.w;
-            }
-            const float2* anc = g.anchors + t - (g.F0 / BM) * g.ntp;
-            const float2* stp = g.steps + static_cast<int64_t>(t) * BM;
-            if (near) {
-                an[f][0] = __ldg(anc + (K / BM) * g.ntp);
-                an[f][1] = an[f][2] = an[f][3] = an[f][0];
-                const float4* s4 = reinterpret_cast<const float4*>(stp + static_cast<int>(K % BM));
-                const float4 s0 = __ldg(s4), s1 = __ldg(s4 + 1);
-                sp[f][0] = make_float2(s0.x, s0.y);
-                sp[f][1] = make_float2(s0.z, s0.w);
-                sp[f][2] = make_float2(s1.x, s1.y);
-                sp[f][3] = make_float2(s1.z, s1.w);
-            } else {
+            for (int r = 0; r < 4; ++r) {
+                if (k + 32 * r >= g.F) continue;
 #pragma unroll
-                for (int r = 0; r < 4; ++r) {
-                    const int64_t Kr = r < rows ? K + r : K;
-                    an[f][r] = __ldg(anc + (Kr / BM) * g.ntp);
-                    sp[f][r] = __ldg(stp + static_cast<int>(Kr % BM));
-                }
+                for (int q = 0; q < 3; ++q) p[f][q][r] = __ldcg(pl[q] + c * 128 + 32 * r);
+                an[f][r] = __ldg(anc + c + (at + 32 * r >= BM ? g.ntp : 0));
+                sp[f][r] = __ldg(g.steps + static_cast<int64_t>(u.n0 + c) * BM + ((at + 32 * r) & (BM - 1)));
             }
         }
 #pragma unroll
         for (int f = 0; f < FT; ++f) {
-            const int c = c0 + f * nw, t = u.n0 + c;
+            const int c = c0 + f * nw;
             if (c >= n) continue;
-            float2* o = g.out + static_cast<int64_t>(t) * g.ld + g.fo + k;
-            float2 y[4];
+            float2* o = g.out + static_cast<int64_t>(u.n0 + c) * g.ld + g.fo + k;
 #pragma unroll
             for (int r = 0; r < 4; ++r)
-                y[r] = g3_output(p[f][0][r], p[f][1][r], p[f][2][r], g.inv_scale, an[f][r], sp[f][r]);
-            if (vec) {
-                reinterpret_cast<float4*>(o)[0] = make_float4(y[0].x, y[0].y, y[1].x, y[1].y);
-                reinterpret_cast<float4*>(o)[1] = make_float4(y[2].x, y[2].y, y[3].x, y[3].y);
-            } else {
-#pragma unroll
-                for (int r = 0; r < 4; ++r)
-                    if (r < rows) o[r] = y[r];
-            }
+                if (k + 32 * r < g.F) o[32 * r] = g3_output(p[f][0][r], p[f][1][r], p[f][2][r], g.inv_scale, an[f][r], sp[f][r]);
         }
     }
 }
 
-// PAIR: launched in clusters of two CTAs on one 256 x 256 tile.  Both CTAs
+// PAIR: launched in clusters of two CTAs on one tile of 256 frames.  Both CTAs
 // load their own operand halves, counted on the full barriers of CTA 0, whose
 // MMA thread issues for both; its commits arrive on both CTAs' barriers, and
 // the epilogue warps of both report drained slots to CTA 0.  The CTAs meet at
@@ -750,32 +733,31 @@ __device__ __noinline__ void g3_finish(const G3Plan& P, const G3Unit u, const fl
 // The mbarriers order tensor-core and TMA work only (no ordinary loads or
 // stores pass between the CTAs), so plain waits do; acquiring at cluster
 // scope put a memory barrier into every wait.
-template <bool PAIR, bool FUSED>
-__global__ void __launch_bounds__(G3_THREADS, 1)
+template <bool PAIR, bool FUSED, bool WIDE>
+__global__ void __launch_bounds__(G3Cfg<PAIR, FUSED, WIDE>::THREADS, 1)
 demod3m_gemm_kernel(const __grid_constant__ G3Batch bt) {
     static_assert(!(FUSED && PAIR), "the pair form loads its A tiles by TMA");
-    constexpr int STAGES = G3_STAGES;
-    constexpr int TW = PAIR ? G3_PAIR_TONES : G3_SINGLE_TONES;             // columns of a TMEM slot
-    constexpr int SLOTS = static_cast<int>(G3_TMEM_COLS) / TW;
-    constexpr int TPG = TW / 4;                                             // tones per epilogue thread
+    static_assert(PAIR || !WIDE, "wide tiles are a pair's");
+    using Cfg = G3Cfg<PAIR, FUSED, WIDE>;
+    constexpr int STAGES = Cfg::STAGES, TW = Cfg::TW, SLOTS = Cfg::SLOTS;
+    constexpr uint32_t STAGE_BYTES = Cfg::STAGE_BYTES, B_BYTES = Cfg::B_BYTES;
+    constexpr int TPG = TW / 4;                                             // tones per epilogue thread, at most
     extern __shared__ unsigned char smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     unsigned char* smem = smem_raw + ((1024u - (raw & 1023u)) & 1023u);
-    uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * G3_STAGE_BYTES);
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE_BYTES);
     uint64_t* empty = full + STAGES;
     uint64_t* sfull = empty + STAGES;
     uint64_t* sempty = sfull + G3_SLOTS_MAX;
     uint64_t* parked = sempty + G3_SLOTS_MAX;                               // a tile's products are in the scratch
     uint64_t* finished = parked + 1;                                        // ... and its outputs stored
     uint64_t* fbar = finished + 1;                                          // finisher staging, per warp and buffer
-    uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(fbar + G3_MAX_FINISHERS * G3_FIN_BUFS);
+    uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(fbar + G3_FINISHERS * G3_FIN_BUFS);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_holder + 1);
-    unsigned char* const fin_stage = smem + STAGES * G3_STAGE_BYTES + G3_BARS_BYTES;
+    unsigned char* const fin_stage = smem + STAGES * STAGE_BYTES + G3_BARS_BYTES;
     int* const status0 = bt.p[0].g.status;
     constexpr int PROD_WARP = G3_EPI_WARPS;                                  // first producer warp
-    constexpr int MMA_WARP = G3_EPI_WARPS + (FUSED ? G3_FUSED_PRODUCERS : 1);
-    constexpr int FIN_WARP = MMA_WARP + 1;
-    constexpr int FINISHERS = G3_THREADS / 32 - FIN_WARP;
+    constexpr int MMA_WARP = Cfg::MMA_WARP, FIN_WARP = MMA_WARP + 1, FINISHERS = Cfg::FINISHERS;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int rank = PAIR ? static_cast<int>(cluster_ctarank()) : 0;
@@ -790,9 +772,11 @@ demod3m_gemm_kernel(const __grid_constant__ G3Batch bt) {
             mbar_init(&sfull[b], 1);
             mbar_init(&sempty[b], (PAIR ? 2 : 1) * G3_EPI_WARPS);
         }
-        mbar_init(parked, G3_EPI_WARPS);
-        mbar_init(finished, FINISHERS);
-        for (int b = 0; b < FINISHERS * G3_FIN_BUFS; ++b) mbar_init(&fbar[b], 1);
+        if constexpr (WIDE) {
+            mbar_init(parked, G3_EPI_WARPS);
+            mbar_init(finished, FINISHERS);
+            for (int b = 0; b < FINISHERS * G3_FIN_BUFS; ++b) mbar_init(&fbar[b], 1);
+        }
         *abort_flag = 0;
         fence_mbar_init();
     }
@@ -813,11 +797,11 @@ demod3m_gemm_kernel(const __grid_constant__ G3Batch bt) {
     const uint32_t tmem = *tmem_holder;
     const int n_units = bt.total_units;
     allow_dependents();
-    float* const scr_cta = bt.p[0].scratch + static_cast<int64_t>(blockIdx.x) * G3_CTA_SCRATCH;
+    float* const scr_cta = WIDE ? bt.p[0].scratch + static_cast<int64_t>(blockIdx.x) * G3_CTA_SCRATCH : nullptr;
 
     if (FUSED && warp >= PROD_WARP && warp < MMA_WARP) {
         // ------------------------------------------------ fused producers
-        const int pt = threadIdx.x - PROD_WARP * 32;                         // 0 .. 63
+        const int pt = threadIdx.x - PROD_WARP * 32;                         // 0 .. 95
         uint32_t it = 0;
         bool stop = false;
         for (int unit = first; unit < n_units && !stop; unit += stride) {
@@ -833,16 +817,18 @@ demod3m_gemm_kernel(const __grid_constant__ G3Batch bt) {
                         stop = true;
                         break;
                     }
-                    unsigned char* st = smem + s * G3_STAGE_BYTES;
+                    unsigned char* st = smem + s * STAGE_BYTES;
                     const int kt = kb * G3_BK;
                     if (pt == 0) {
                         mbar_expect_tx(&full[s], 2u * P.bw * (G3_BK * 2));
                         tma_load_2d(st + 2 * G3_OP_BYTES, &P.b[2 * q], kt, u.n0, &full[s]);
-                        tma_load_2d(st + 3 * G3_OP_BYTES, &P.b[2 * q + 1], kt, u.n0, &full[s]);
+                        tma_load_2d(st + 2 * G3_OP_BYTES + B_BYTES, &P.b[2 * q + 1], kt, u.n0, &full[s]);
                     }
-#pragma unroll 1
-                    for (int i = pt; i < BM; i += G3_FUSED_PRODUCERS * 32)
-                        g3_fill_row(P, q, (u.m0 + i) * D + kt, st, st + G3_OP_BYTES, i);
+#pragma unroll 2
+                    for (int e = pt; e < BM * (G3_BK / 8); e += G3_FUSED_PRODUCERS * 32) {
+                        const int i = e / (G3_BK / 8), c = e % (G3_BK / 8);
+                        g3_fill_chunk(P, q, (u.m0 + i) * D + kt + 8 * c, st, st + G3_OP_BYTES, i, c);
+                    }
                     fence_proxy_async_smem();                 // the MMAs read the tiles through the async proxy
                     mbar_arrive(&full[s]);
                 }
@@ -877,7 +863,7 @@ demod3m_gemm_kernel(const __grid_constant__ G3Batch bt) {
                             stop = true;
                             break;
                         }
-                        unsigned char* st = smem + s * G3_STAGE_BYTES;
+                        unsigned char* st = smem + s * STAGE_BYTES;
                         const int kt = kb * G3_BK;
                         const int c0 = kt % P.g.two_d, c1 = static_cast<int>(u.m0) + kt / P.g.two_d;
                         if constexpr (PAIR) {
@@ -887,13 +873,13 @@ demod3m_gemm_kernel(const __grid_constant__ G3Batch bt) {
                             tma_load_2d_2sm(st, &P.a[2 * q], c0, c1, fb);
                             tma_load_2d_2sm(st + G3_OP_BYTES, &P.a[2 * q + 1], c0, c1, fb);
                             tma_load_2d_2sm(st + 2 * G3_OP_BYTES, &P.b[2 * q], kt, b0, fb);
-                            tma_load_2d_2sm(st + 3 * G3_OP_BYTES, &P.b[2 * q + 1], kt, b0, fb);
+                            tma_load_2d_2sm(st + 2 * G3_OP_BYTES + B_BYTES, &P.b[2 * q + 1], kt, b0, fb);
                         } else {
                             mbar_arrive_expect_tx(&full[s], bytes);
                             tma_load_2d(st, &P.a[2 * q], c0, c1, &full[s]);
                             tma_load_2d(st + G3_OP_BYTES, &P.a[2 * q + 1], c0, c1, &full[s]);
                             tma_load_2d(st + 2 * G3_OP_BYTES, &P.b[2 * q], kt, b0, &full[s]);
-                            tma_load_2d(st + 3 * G3_OP_BYTES, &P.b[2 * q + 1], kt, b0, &full[s]);
+                            tma_load_2d(st + 2 * G3_OP_BYTES + B_BYTES, &P.b[2 * q + 1], kt, b0, &full[s]);
                         }
                     }
                 }
@@ -915,63 +901,67 @@ demod3m_gemm_kernel(const __grid_constant__ G3Batch bt) {
         }
     } else if (warp == MMA_WARP) {
         // ------------------------------------------------ MMA issuer
-        if (lane == 0 && rank == 0) {
-            uint32_t it = 0, phase = 0;
-            bool stop = false;
-            for (int unit = first; unit < n_units && !stop; unit += stride) {
+        // The whole warp runs the loops and one elected thread issues, so that control
+        // flow, descriptors and addresses stay in uniform registers.  (Run by one thread
+        // alone, every MMA took about 115 clocks to issue whatever its width: 1370 a
+        // K-block, where tiles of 128 tones need 960.)
+        if (rank == 0) {
+            const bool leader = umma::elect_one();
+            const uint64_t desc0 = umma::desc_k_sw128(smem_u32(smem));
+            uint32_t phase = 0, s = 0, par = 0;             // chunk; stage and the parity of its use
+            bool go = true;
+            for (int unit = first; unit < n_units && go; unit += stride) {
                 const G3Plan& P = g3_plan_of(bt, unit);
                 const GemmArgs& g = P.g;
                 const G3Unit u = g3_unit<PAIR>(P, unit, rank);
                 const uint32_t idesc = umma::idesc_f16_f32(PAIR ? 256 : 128, u.width);
-                for (int q = u.q0; q < u.q1 && !stop; ++q) {
+                const int H = 2 * g.KB, chunk = g.kchunk;
+                for (int q = u.q0; q < u.q1 && go; ++q) {
                     // chunks of half K-blocks (32 taps); chunks of whole blocks have their own
-                    // loop (a block's twelve MMAs in two pieces: 800 us where this takes 733,
+                    // loop (a block's twelve MMAs in two pieces: 800 us where this took 733,
                     // 2^24 samples x 2048 tones)
-                    for (int h0 = 0; h0 < 2 * g.KB && !stop; h0 += g.kchunk, ++phase) {
-                        const int h1 = min(h0 + g.kchunk, 2 * g.KB);
+                    for (int h0 = 0; h0 < H && go; h0 += chunk, ++phase) {
+                        const int h1 = min(h0 + chunk, H);
                         const uint32_t slot = phase % SLOTS, use = phase / SLOTS;
-                        if (*abort_flag || !mbar_wait(&sempty[slot], (use & 1) ^ 1, status0)) {
-                            *abort_flag = 1;
-                            stop = true;
-                            break;
-                        }
+                        go = __all_sync(0xffffffffu, !*abort_flag && mbar_wait(&sempty[slot], (use & 1) ^ 1, status0));
+                        if (!go) break;
                         umma::fence_after_sync();
                         const uint32_t d_tmem = tmem + slot * TW;
                         auto arrived = [&] {                            // the block's operands
-                            if (!mbar_wait(&full[it % STAGES], (it / STAGES) & 1, status0)) {
-                                *abort_flag = 1;
-                                stop = true;
-                                return false;
-                            }
+                            go = __all_sync(0xffffffffu, mbar_wait(&full[s], par, status0));
                             umma::fence_after_sync();
-                            return true;
+                            return go;
                         };
                         auto release = [&] {                            // its stage, in both CTAs of a pair
-                            if constexpr (PAIR) umma::commit_2sm(&empty[it % STAGES]);
-                            else umma::commit(&empty[it % STAGES]);
-                            ++it;
+                            if (leader) {
+                                if constexpr (PAIR) umma::commit_2sm(&empty[s]);
+                                else umma::commit(&empty[s]);
+                            }
+                            if (++s == STAGES) {
+                                s = 0;
+                                par ^= 1u;
+                            }
                         };
                         auto steps = [&](auto n, uint32_t from, bool fresh) {   // n steps of 16 taps
-                            const uint32_t ah = smem_u32(smem + (it % STAGES) * G3_STAGE_BYTES) + from, al = ah + G3_OP_BYTES;
-                            const uint32_t bh = ah + 2 * G3_OP_BYTES, bl = ah + 3 * G3_OP_BYTES;
+                            const uint64_t ah = desc0 + ((s * STAGE_BYTES + from) >> 4);
+                            const uint64_t al = ah + (G3_OP_BYTES >> 4), bh = ah + (2 * G3_OP_BYTES >> 4), bl = bh + (B_BYTES >> 4);
+                            if (leader) {
 #pragma unroll
-                            for (int k = 0; k < n; ++k) {
-                                const uint32_t off = k * 32;
-                                const uint32_t acc = (!fresh || k > 0) ? 1u : 0u;
-                                const uint64_t dah = umma::desc_k_sw128(ah + off), dal = umma::desc_k_sw128(al + off);
-                                const uint64_t dbh = umma::desc_k_sw128(bh + off), dbl = umma::desc_k_sw128(bl + off);
-                                if constexpr (PAIR) {
-                                    umma::mma_f16_2sm(d_tmem, dah, dbh, idesc, acc);
-                                    umma::mma_f16_2sm(d_tmem, dah, dbl, idesc, 1u);
-                                    umma::mma_f16_2sm(d_tmem, dal, dbh, idesc, 1u);
-                                } else {
-                                    umma::mma_f16(d_tmem, dah, dbh, idesc, acc);
-                                    umma::mma_f16(d_tmem, dah, dbl, idesc, 1u);
-                                    umma::mma_f16(d_tmem, dal, dbh, idesc, 1u);
+                                for (int k = 0; k < n; ++k) {
+                                    const uint32_t acc = (!fresh || k > 0) ? 1u : 0u;
+                                    if constexpr (PAIR) {
+                                        umma::mma_f16_2sm(d_tmem, ah + 2 * k, bh + 2 * k, idesc, acc);
+                                        umma::mma_f16_2sm(d_tmem, ah + 2 * k, bl + 2 * k, idesc, 1u);
+                                        umma::mma_f16_2sm(d_tmem, al + 2 * k, bh + 2 * k, idesc, 1u);
+                                    } else {
+                                        umma::mma_f16(d_tmem, ah + 2 * k, bh + 2 * k, idesc, acc);
+                                        umma::mma_f16(d_tmem, ah + 2 * k, bl + 2 * k, idesc, 1u);
+                                        umma::mma_f16(d_tmem, al + 2 * k, bh + 2 * k, idesc, 1u);
+                                    }
                                 }
                             }
                         };
-                        if ((g.kchunk & 1) == 0) {
+                        if ((chunk & 1) == 0) {
                             for (int h = h0; h < h1; h += 2) {
                                 if (!arrived()) break;
                                 steps(std::integral_constant<int, G3_BK / 16>{}, 0, h == h0);
@@ -984,27 +974,33 @@ demod3m_gemm_kernel(const __grid_constant__ G3Batch bt) {
                                 if (h & 1) release();
                             }
                         }
-                        if constexpr (PAIR) umma::commit_2sm(&sfull[slot]);
-                        else umma::commit(&sfull[slot]);
+                        if (leader) {
+                            if constexpr (PAIR) umma::commit_2sm(&sfull[slot]);
+                            else umma::commit(&sfull[slot]);
+                        }
                     }
                 }
             }
+            if (!go) *abort_flag = 1;
         }
         __syncwarp();
     } else if (warp < G3_EPI_WARPS) {
         // ------------------------------------------------ epilogue (16 warps)
         const int qd = warp & 3, grp = warp >> 2;          // lane quadrant, tone group
         const int row = qd * 32 + lane;
+        const uint32_t lanes = tmem + (static_cast<uint32_t>(qd * 32) << 16);
         uint32_t phase = 0, tile = 0;
         bool ok = true;
         // this thread's column of the CTA's scratch planes
-        float* const scr = scr_cta + grp * TPG * 128 + row;
+        float* const scr = WIDE ? scr_cta + grp * TPG * 128 + row : nullptr;
         for (int unit = first; unit < n_units && ok; unit += stride) {
             const G3Plan& P = g3_plan_of(bt, unit);
             const GemmArgs& g = P.g;
             const G3Unit u = g3_unit<PAIR>(P, unit, rank);
-            const int cols = min(TPG, u.width - grp * TPG);          // this thread's tones (a multiple of 16, or <= 0)
-            float sum[TPG];
+            // this thread's tones (cols: a multiple of 16, or <= 0), from c0 on
+            const int tpg = WIDE || u.width > 64 ? TPG : 16, c0 = grp * tpg, cols = min(tpg, u.width - c0);
+            const int64_t k = u.m0 + row;                             // and its frame
+            float sum[TPG], im[WIDE ? 1 : TPG];
             for (int q = u.q0; q < u.q1 && ok; ++q) {
 #pragma unroll
                 for (int i = 0; i < TPG; ++i) sum[i] = 0.f;
@@ -1016,7 +1012,7 @@ demod3m_gemm_kernel(const __grid_constant__ G3Batch bt) {
                         break;
                     }
                     umma::fence_after_sync();
-                    const uint32_t ta = tmem + (static_cast<uint32_t>(qd * 32) << 16) + slot * TW + grp * TPG;
+                    const uint32_t ta = lanes + slot * TW + c0;
 #pragma unroll
                     for (int h = 0; h < TPG; h += 16) {
                         if (h < cols) {
@@ -1036,8 +1032,7 @@ demod3m_gemm_kernel(const __grid_constant__ G3Batch bt) {
                 }
                 if (!ok) break;
                 if (P.split) {
-                    const int64_t k = u.m0 + row;
-                    const int tb = u.n0 + grp * TPG;
+                    const int tb = u.n0 + c0;
                     if (k < g.F) {
                         float* pl = P.scratch + (static_cast<int64_t>(q) * g.n_tones + tb) * P.pld + k;
 #pragma unroll
@@ -1046,28 +1041,79 @@ demod3m_gemm_kernel(const __grid_constant__ G3Batch bt) {
                     }
                     continue;
                 }
-                // the first product to reuse a plane of the tile before, which
-                // has to be finished by then
-                if (q == G3_PLANES - 3 && tile > 0 && !mbar_wait(finished, (tile - 1) & 1, status0)) {
-                    *abort_flag = 1;
-                    ok = false;
-                    break;
-                }
-                float* const pl = scr + ((3 * tile + q) % G3_PLANES) * G3_PLANE;
+                if constexpr (WIDE) {
+                    // the first product to reuse a plane of the tile before, which
+                    // has to be finished by then
+                    if (q == G3_PLANES - 3 && tile > 0 && !mbar_wait(finished, (tile - 1) & 1, status0)) {
+                        *abort_flag = 1;
+                        ok = false;
+                        break;
+                    }
+                    float* const pl = scr + ((3 * tile + q) % G3_PLANES) * G3_PLANE;
 #pragma unroll
-                for (int i = 0; i < TPG; ++i)
-                    if (i < cols) pl[i * 128] = sum[i];
+                    for (int i = 0; i < TPG; ++i)
+                        if (i < cols) pl[i * 128] = sum[i];
+                } else if (q == 0) {
+                    // P1 waits in this thread's own TMEM columns
+                    if (cols > 0) {
+                        uint32_t w[TPG];
+#pragma unroll
+                        for (int i = 0; i < TPG; ++i) w[i] = __float_as_uint(sum[i]);
+                        umma::st_32x32b_x32(lanes + Cfg::PARK + grp * TPG, w);
+                        umma::wait_st();
+                    }
+                } else {
+                    // im = 2 P1 + P2; re = 2 P1 - P3 and the outputs, their
+                    // arithmetic that of g3_output
+#pragma unroll
+                    for (int h = 0; h < TPG; h += 16) {
+                        if (h < cols) {
+                            uint32_t p1[16];
+                            umma::ld_32x32b_x16(lanes + Cfg::PARK + grp * TPG + h, p1);
+                            umma::wait_ld_regs(p1);
+#pragma unroll
+                            for (int i = 0; i < 16; ++i) {
+                                if (q == 1) im[h + i] = fmaf(2.f, __uint_as_float(p1[i]), sum[h + i]);
+                                else sum[h + i] = fmaf(2.f, __uint_as_float(p1[i]), -sum[h + i]);
+                            }
+                        }
+                    }
+                    const int n = min(cols, g.n_tones - u.n0 - c0);
+                    if (q == 2 && k < g.F && n > 0) {
+                        const float2* const anc = g.anchors + ((g.F0 + k) / BM - g.F0 / BM) * g.ntp + u.n0 + c0;
+                        const float2* const stp = g.steps + static_cast<int64_t>(u.n0 + c0) * BM + static_cast<int>((g.F0 + k) % BM);
+                        float2* const out = g.out + static_cast<int64_t>(u.n0 + c0) * g.ld + g.fo + k;
+                        // (loads four tones at a time, unconditional: one by one their
+                        // latency adds up to more than the MMAs run ahead)
+#pragma unroll
+                        for (int h = 0; h < TPG; h += 4) {
+                            if (h >= n) break;
+                            float2 an[4], sp[4];
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                const int t = min(h + i, n - 1);
+                                an[i] = __ldg(anc + t);
+                                sp[i] = __ldg(stp + t * BM);
+                            }
+#pragma unroll
+                            for (int i = 0; i < 4; ++i)
+                                if (h + i < n) out[(h + i) * g.ld] = g3_rotate(sum[h + i], im[h + i], g.inv_scale, an[i], sp[i]);
+                        }
+                    }
+                }
             }
-            if (ok && !P.split) {
-                fence_proxy_async_global();                  // the finishers read the planes by bulk copies
-                __syncwarp();
-                if (lane == 0) mbar_arrive(parked);
-                if (unit + stride >= n_units && mbar_wait(parked, tile & 1, status0))
-                    g3_finish(P, u, scr_cta, tile, lane, warp, G3_THREADS / 32, FIN_WARP - G3_EPI_WARPS);
-                ++tile;
+            if constexpr (WIDE) {
+                if (ok && !P.split) {
+                    fence_proxy_async_global();              // the finishers read the planes by bulk copies
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(parked);
+                    if (unit + stride >= n_units && mbar_wait(parked, tile & 1, status0))
+                        g3_finish(P, u, scr_cta, tile, lane, warp, Cfg::THREADS / 32, FIN_WARP - G3_EPI_WARPS);
+                    ++tile;
+                }
             }
         }
-    } else if (warp >= FIN_WARP) {
+    } else if constexpr (WIDE) {
         // ------------------------------------------------ finishers
         const int w = warp - FIN_WARP;
         unsigned char* const stage = fin_stage + w * G3_FIN_BUFS * G3_FIN_BYTES;
@@ -1084,32 +1130,31 @@ demod3m_gemm_kernel(const __grid_constant__ G3Batch bt) {
             const G3Unit u = g3_unit<PAIR>(P, unit, rank);
             if (unit + stride >= n_units) {
                 // the CTA's last tile: every warp that is free takes part
-                g3_finish(P, u, scr_cta, tile, lane, warp, G3_THREADS / 32, FIN_WARP - G3_EPI_WARPS);
+                g3_finish(P, u, scr_cta, tile, lane, warp, Cfg::THREADS / 32, FIN_WARP - G3_EPI_WARPS);
             } else {
                 const GemmArgs& g = P.g;
                 const int n = min(u.width, g.n_tones - u.n0);
                 // the warp's chunks: tones 2 (w + i FINISHERS), 2 (w + i FINISHERS) + 1
                 const int chunks = ((n + 1) / 2 - w + FINISHERS - 1) / FINISHERS;
+                // chunk i into its buffer: lanes 0 .. 2 copy the products, lane 3 the steps
                 auto fetch = [&](int i) {
                     const uint32_t b = (fills + i) % G3_FIN_BUFS;
-                    unsigned char* dst = stage + b * G3_FIN_BYTES;
                     const int c = 2 * (w + i * FINISHERS);
-                    mbar_arrive_expect_tx(&bars[b], G3_FIN_BYTES);
-#pragma unroll
-                    for (int q = 0; q < 3; ++q)
-                        tma_bulk_g2s(dst + q * 1024, scr_cta + ((3 * tile + q) % G3_PLANES) * G3_PLANE + c * 128, 1024, &bars[b]);
-                    tma_bulk_g2s(dst + 3072, g.steps + static_cast<int64_t>(u.n0 + c) * BM, 2048, &bars[b]);
+                    if (lane == 0) mbar_arrive_expect_tx(&bars[b], G3_FIN_BYTES);
+                    __syncwarp();
+                    if (lane < 4) {
+                        const void* src = lane < 3 ? static_cast<const void*>(scr_cta + ((3 * tile + lane) % G3_PLANES) * G3_PLANE + c * 128)
+                                                   : g.steps + static_cast<int64_t>(u.n0 + c) * BM;
+                        tma_bulk_g2s(stage + b * G3_FIN_BYTES + lane * 1024, src, lane < 3 ? 1024u : 2048u, &bars[b]);
+                    }
                 };
-                const int ahead = min(chunks, G3_FIN_BUFS);
-                if (lane == 0)
-                    for (int i = 0; i < ahead; ++i) fetch(i);
-                // lane l: frames 4 l .. 4 l + 3; anchor rows a0 and, from row
-                // `turn` of the tile on, a0 + 1
-                const int64_t k = u.m0 + 4 * lane;
-                const int rows = static_cast<int>(k < g.F ? (g.F - k < 4 ? g.F - k : 4) : 0);
+                for (int i = 0; i < min(chunks, G3_FIN_BUFS); ++i) fetch(i);
+                // lane l: frames l + 32 r, so that a warp's loads and stores are runs of
+                // frames whatever the rows' alignment (four consecutive frames a lane took
+                // 480 clocks a tone in 16-byte stores and more in 8-byte ones); anchor rows
+                // a0 and, from row `turn` of the tile on, a0 + 1
+                const int64_t k = u.m0 + lane;
                 const int f0 = static_cast<int>(g.F0 % BM), turn = BM - f0;
-                const bool vec = rows == 4 &&
-                                 ((reinterpret_cast<uintptr_t>(g.out + g.fo + k) | static_cast<uintptr_t>(g.ld * 8)) & 15) == 0;
                 const float2* const anc = g.anchors + ((g.F0 + u.m0) / BM - g.F0 / BM) * g.ntp + u.n0;
                 float2 a_lo = make_float2(0.f, 0.f), a_hi = a_lo;
                 for (int i = 0; i < chunks; ++i) {
@@ -1127,38 +1172,33 @@ demod3m_gemm_kernel(const __grid_constant__ G3Batch bt) {
                         break;
                     }
                     const unsigned char* src = stage + (fi % G3_FIN_BUFS) * G3_FIN_BYTES;
+                    float p[2][3][4];
+                    float2 sp[2][4], al[2], ah[2];
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
-                        const int c = 2 * (w + i * FINISHERS) + h;
                         const int from = ((i & 15) << 1) + h;
-                        const float2 al = make_float2(__shfl_sync(0xffffffffu, a_lo.x, from), __shfl_sync(0xffffffffu, a_lo.y, from));
-                        const float2 ah = make_float2(__shfl_sync(0xffffffffu, a_hi.x, from), __shfl_sync(0xffffffffu, a_hi.y, from));
-                        if (c >= n || rows == 0) continue;
-                        const float4 p1 = *reinterpret_cast<const float4*>(src + h * 512 + lane * 16);
-                        const float4 p2 = *reinterpret_cast<const float4*>(src + 1024 + h * 512 + lane * 16);
-                        const float4 p3 = *reinterpret_cast<const float4*>(src + 2048 + h * 512 + lane * 16);
-                        const float2* const sp = reinterpret_cast<const float2*>(src + 3072 + h * 1024);
-                        float2 y[4];
+                        al[h] = make_float2(__shfl_sync(0xffffffffu, a_lo.x, from), __shfl_sync(0xffffffffu, a_lo.y, from));
+                        ah[h] = make_float2(__shfl_sync(0xffffffffu, a_hi.x, from), __shfl_sync(0xffffffffu, a_hi.y, from));
 #pragma unroll
                         for (int r = 0; r < 4; ++r) {
-                            const int row = 4 * lane + r;
-                            const float v1 = r == 0 ? p1.x : r == 1 ? p1.y : r == 2 ? p1.z : p1.w;
-                            const float v2 = r == 0 ? p2.x : r == 1 ? p2.y : r == 2 ? p2.z : p2.w;
-                            const float v3 = r == 0 ? p3.x : r == 1 ? p3.y : r == 2 ? p3.z : p3.w;
-                            y[r] = g3_output(v1, v2, v3, g.inv_scale, row < turn ? al : ah, sp[(row + f0) & (BM - 1)]);
-                        }
-                        float2* o = g.out + static_cast<int64_t>(u.n0 + c) * g.ld + g.fo + k;
-                        if (vec) {
-                            reinterpret_cast<float4*>(o)[0] = make_float4(y[0].x, y[0].y, y[1].x, y[1].y);
-                            reinterpret_cast<float4*>(o)[1] = make_float4(y[2].x, y[2].y, y[3].x, y[3].y);
-                        } else {
 #pragma unroll
-                            for (int r = 0; r < 4; ++r)
-                                if (r < rows) o[r] = y[r];
+                            for (int q = 0; q < 3; ++q)
+                                p[h][q][r] = *reinterpret_cast<const float*>(src + q * 1024 + h * 512 + r * 128 + lane * 4);
+                            sp[h][r] = *reinterpret_cast<const float2*>(src + 3072 + h * 1024 + ((lane + 32 * r + f0) & (BM - 1)) * 8);
                         }
                     }
                     __syncwarp();                             // the buffer has been read
-                    if (lane == 0 && i + G3_FIN_BUFS < chunks) fetch(i + G3_FIN_BUFS);
+                    if (i + G3_FIN_BUFS < chunks) fetch(i + G3_FIN_BUFS);
+                    const int c = 2 * (w + i * FINISHERS);
+                    float2* const o = g.out + static_cast<int64_t>(u.n0 + c) * g.ld + g.fo + k;
+#pragma unroll
+                    for (int h = 0; h < 2; ++h)
+#pragma unroll
+                        for (int r = 0; r < 4; ++r) {
+                            const float2 y = g3_output(p[h][0][r], p[h][1][r], p[h][2][r], g.inv_scale,
+                                                       lane + 32 * r < turn ? al[h] : ah[h], sp[h][r]);
+                            if (c + h < n && k + 32 * r < g.F) o[h * g.ld + 32 * r] = y;
+                        }
                 }
                 fills += chunks;
             }
@@ -1238,10 +1278,12 @@ bool g3_planes_fit(int n_tones, int64_t F, int n_sms) {
 }
 }  // namespace
 size_t demod3_scratch_bytes(int ctas) { return static_cast<size_t>(ctas) * G3_CTA_SCRATCH * 4; }
-// Every form's tiles hold 128 frames or more a CTA and, but for a last one, 64 tones
-// or more (a pair's odd frame tile: one CTA more).
+// Wide tiles: 256 frames x 256 tones at most on two CTAs (evened out, no more tiles
+// than that).
 int demod3_ctas(int n_tones, int64_t F, int n_sms) {
-    return static_cast<int>(std::min<int64_t>(n_sms, ((F + 127) / 128 + 1) * ((n_tones + 63) / 64)));
+    if (n_tones <= G3_TONES) return 0;
+    return static_cast<int>(std::min<int64_t>(
+        n_sms, 2 * ((F + 255) / 256) * ((n_tones + G3_WIDE_TONES - 1) / G3_WIDE_TONES)));
 }
 size_t demod3_scratch_need(int n_tones, int64_t F, int n_sms) {
     const int64_t planes = g3_planes_fit(n_tones, F, n_sms) ? 3 * n_tones * g3_plane_ld(F) * 4
@@ -1322,49 +1364,70 @@ cudaError_t demod3_build_taps(const double* d_h, const uint64_t* d_words, int n_
 }
 
 namespace {
-// Clocks that a work item's K-block (64 taps of one product) takes at least:
-// its MMAs (12 of w/2 clocks), or the shared-memory traffic of the MMAs and
-// the TMA at 128 bytes a clock (see the Gauss form's comment).
-double g3_block_clocks(bool pair, int w) {
-    return pair ? std::max(6.0 * w, 640.0 + 2.5 * w) : std::max(6.0 * w, 640.0 + 5.0 * w);
-}
-
+// Clocks that a work item takes.  A K-block (64 taps of one product) of a pair: its
+// MMAs, 12 of w / 2 clocks and 15 % for their gaps, or the shared-memory traffic of the
+// MMAs and the TMA at 128 bytes a clock (see the Gauss form's comment); of a single
+// CTA, fitted: 900, 1000 and 1180 clocks at w = 16, 64 and 128.  Finishing: wide tiles
+// beside the next tile's first two products, by two warps, 480 clocks a tone; others in
+// the epilogue, 75 clocks a tone of which the next tile's MMAs do not run beside.
+// Measured, 2^24 samples, D = 512, 1000 tones, L = 256 / 1024 / 2048 / 4096, in us: wide
+// 468 / 603 / 782 / 1337, pairs of 128 tones 217 / 447 / 756 / 1387, single CTAs of 128
+// 229 / 523 / 924 / 1717.
 struct G3Form {
     bool pair = false, split = false;
     int bw = 128;
+    bool wide() const { return bw > G3_TONES; }
+    double clocks(int64_t KB) const {
+        constexpr double kFinish = 480.0, kExposed = 75.0;
+        const double block = pair ? std::max(6.9 * bw, 640.0 + 2.5 * bw) : 860.0 + 2.5 * bw;
+        if (split) return KB * block;
+        if (wide()) return std::max(3 * KB * block, KB * block + kFinish * bw);
+        return 3 * KB * block + kExposed * bw;
+    }
 };
 int g3_even_width(int n_tones, int widest, int step) {
     const int tiles = (n_tones + widest - 1) / widest;
     return ((n_tones + tiles - 1) / tiles + step - 1) / step * step;
 }
-// The form of a push that names none: the least time of the four, counting
-// whole waves of work items over the chip (a batched step's launch shares its
-// waves between plans, so there only the work counts, and nothing is split).
-// kSplitClocks: the planes' round trip and combine3_kernel's launch.
+// The form of a push: the least time of those its plan allows (any, or the pinned
+// pair, tone width or fused pre-split), counting whole waves of work items over the
+// chip (a batched step's launch shares its waves between plans, so there only the
+// work counts, and nothing is split).  kSplitClocks: the planes' round trip and
+// combine3_kernel's launch.
 G3Form g3_choose(const DemodLaunch& L, bool shared_launch) {
     constexpr double kSplitClocks = 8000.0;
     G3Form best;
     double best_t = 1e300;
     const int64_t KB = L.Lpad / G3_BK;
+    const bool pinned = !L.auto_form, pinned_pair = pinned && L.pair && !L.fused_presplit;
     for (int pair = 0; pair < 2; ++pair) {
-        const int widths[2] = {pair ? g3_even_width(L.n_tones, G3_PAIR_TONES, 32)
-                                    : g3_even_width(L.n_tones, G3_SINGLE_TONES, 16),
-                               pair ? 0 : g3_even_width(L.n_tones, 64, 16)};
+        if (pinned && pair != (pinned_pair ? 1 : 0)) continue;
+        int widths[2];
+        if (pair) {
+            widths[0] = g3_even_width(L.n_tones, G3_WIDE_TONES, 32);
+            widths[1] = g3_even_width(L.n_tones, G3_TONES, 32);
+        } else if (pinned) {
+            widths[0] = widths[1] = L.tone_tile == 64 ? 64 : 128;
+        } else {
+            widths[0] = g3_even_width(L.n_tones, G3_TONES, 16);
+            widths[1] = g3_even_width(L.n_tones, 64, 16);
+        }
         for (int w : widths) {
-            if (w <= 0) continue;
             const int64_t tiles = (L.F + (pair ? 255 : 127)) / (pair ? 256 : 128) * ((L.n_tones + w - 1) / w);
             const int64_t places = pair ? L.n_sms / 2 : L.n_sms;
             for (int split = 0; split < 2; ++split) {
                 if (split && (shared_launch || !g3_planes_fit(L.n_tones, L.F, L.n_sms))) continue;
+                G3Form f;
+                f.pair = pair != 0;
+                f.split = split != 0;
+                f.bw = w;
                 const int64_t units = tiles * (split ? 3 : 1);
                 const double waves = shared_launch ? static_cast<double>(units) / places
                                                    : static_cast<double>((units + places - 1) / places);
-                const double t = waves * KB * (split ? 1 : 3) * g3_block_clocks(pair != 0, w) + (split ? kSplitClocks : 0.0);
+                const double t = waves * f.clocks(KB) + (split ? kSplitClocks : 0.0);
                 if (t < best_t) {
                     best_t = t;
-                    best.pair = pair != 0;
-                    best.split = split != 0;
-                    best.bw = w;
+                    best = f;
                 }
             }
         }
@@ -1377,17 +1440,11 @@ cudaError_t demod3_prepare(const DemodLaunch& L, cudaStream_t st, DemodGemmJob* 
     job->n_units = 0;
     if (L.F <= 0) return cudaSuccess;
     if (L.D % G3_BK != 0 || L.Lpad % G3_BK != 0 || L.ntp % 128 != 0) return cudaErrorInvalidValue;
-    G3Form form;
-    if (L.auto_form) {
-        form = g3_choose(L, shared_launch);
-    } else {
-        form.pair = L.pair && !L.fused_presplit;
-        form.bw = form.pair ? g3_even_width(L.n_tones, G3_PAIR_TONES, 32) : (L.tone_tile == 64 ? 64 : 128);
-    }
-    job->fused = !L.auto_form && L.fused_presplit ? 1 : 0;
-    job->pair = form.pair ? 1 : 0;
+    const G3Form form = g3_choose(L, shared_launch);
+    job->kind = form.wide() ? 0 : form.pair ? 1 : !L.auto_form && L.fused_presplit ? 3 : 2;
+    const bool fused = job->kind == 3;
     const int64_t rows = static_cast<int64_t>(demod3_xs_rows(L.F, L.Lpad, L.D));
-    if (!job->fused && rows > L.xs_rows) return cudaErrorInvalidValue;
+    if (!fused && rows > L.xs_rows) return cudaErrorInvalidValue;
     if (form.split && 3 * static_cast<size_t>(L.n_tones) * g3_plane_ld(L.F) * 4 > L.scratch_bytes) return cudaErrorInvalidValue;
     const int bm = form.pair ? 256 : BM;
     const int n_mt = static_cast<int>((L.F + bm - 1) / bm);
@@ -1401,7 +1458,7 @@ cudaError_t demod3_prepare(const DemodLaunch& L, cudaStream_t st, DemodGemmJob* 
     const int64_t bplane = static_cast<int64_t>(L.ntp) * L.Lpad;
     const int64_t total = rows * L.D;
     __half* xp = static_cast<__half*>(L.xs_hi);
-    if (job->fused) {
+    if (fused) {
         // the GEMM's producers read the stream view themselves
         P->carry = reinterpret_cast<const uint32_t*>(L.carry);
         P->buf = reinterpret_cast<const uint32_t*>(L.buf);
@@ -1423,7 +1480,7 @@ cudaError_t demod3_prepare(const DemodLaunch& L, cudaStream_t st, DemodGemmJob* 
     pa.buf = reinterpret_cast<const uint32_t*>(L.buf);
     pa.cl = L.cl;
     pa.lv = L.cl + L.n;
-    pa.total = job->fused ? 0 : total;
+    pa.total = fused ? 0 : total;
     pa.planes = xp;
     const int64_t rot_items = ((pa.A0 + n_anch - 1) / kRotRun - pa.A0 / kRotRun + 1 + BM / kRotRun) * L.ntp;
     pa.rot_items = static_cast<int>(std::min<int64_t>(256, (rot_items / (2 * L.n_sms) + 31) / 32 * 32));
@@ -1433,7 +1490,7 @@ cudaError_t demod3_prepare(const DemodLaunch& L, cudaStream_t st, DemodGemmJob* 
     prep3_kernel<<<pa.rot_blocks + plane_blocks, 256, 0, st>>>(pa);
     const uint32_t b_box = static_cast<uint32_t>(form.pair ? form.bw / 2 : form.bw);
     for (int i = 0; i < 6; ++i) {
-        if ((!job->fused && !make_map(&P->a[i], xp + i * total, static_cast<uint64_t>(L.D),
+        if ((!fused && !make_map(&P->a[i], xp + i * total, static_cast<uint64_t>(L.D),
                                       static_cast<uint64_t>(rows), BM)) ||
             !make_map(&P->b[i], bp + i * bplane, static_cast<uint64_t>(L.Lpad), static_cast<uint64_t>(L.ntp), b_box))
             return cudaErrorInvalidValue;
@@ -1465,25 +1522,26 @@ cudaError_t demod3_prepare(const DemodLaunch& L, cudaStream_t st, DemodGemmJob* 
     g.fo = L.frame_offset;
     g.status = L.status;
     job->n_units = n_mt * n_nt * (form.split ? 3 : 1);
-    job->unit_cost = g.KB * (form.split ? 1 : 3) * g3_block_clocks(form.pair, form.bw);
+    job->unit_cost = form.clocks(g.KB);
     return cudaGetLastError();
 }
 
 namespace {
 // room: bytes of the scratch that unsplit CTAs park their products in.
-template <bool PAIR, bool FUSED>
+template <bool PAIR, bool FUSED, bool WIDE>
 cudaError_t g3_run(const G3Batch& b, int n_sms, size_t room, cudaStream_t st) {
+    using Cfg = G3Cfg<PAIR, FUSED, WIDE>;
     bool parks = false;
-    for (int k = 0; k < b.n_plans; ++k) parks = parks || !b.p[k].split;
+    for (int k = 0; WIDE && k < b.n_plans; ++k) parks = parks || !b.p[k].split;
     auto fits = [&](int grid) { return !parks || demod3_scratch_bytes(grid) <= room; };
-    auto kern = demod3m_gemm_kernel<PAIR, FUSED>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(G3_SMEM));
+    auto kern = demod3m_gemm_kernel<PAIR, FUSED, WIDE>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(Cfg::SMEM));
     if (e != cudaSuccess) return e;
-    const int threads = G3_THREADS;
+    const int threads = Cfg::THREADS;
     if (!PAIR) {
         const int grid = std::max(1, std::min(b.total_units, n_sms));
         if (!fits(grid)) return cudaErrorInvalidValue;
-        kern<<<grid, threads, G3_SMEM, st>>>(b);
+        kern<<<grid, threads, Cfg::SMEM, st>>>(b);
         return cudaGetLastError();
     }
     // clusters of two CTAs: as many as can be resident at once (one CTA per SM)
@@ -1494,7 +1552,7 @@ cudaError_t g3_run(const G3Batch& b, int n_sms, size_t room, cudaStream_t st) {
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.blockDim = dim3(threads, 1, 1);
-    cfg.dynamicSmemBytes = G3_SMEM;
+    cfg.dynamicSmemBytes = Cfg::SMEM;
     cfg.stream = st;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
@@ -1522,9 +1580,8 @@ cudaError_t demod3_gemm(const DemodGemmJob* const* jobs, int n, int n_sms, void*
     std::vector<const DemodGemmJob*> order(jobs, jobs + n);
     std::stable_sort(order.begin(), order.end(),
                      [](const DemodGemmJob* x, const DemodGemmJob* y) { return x->unit_cost > y->unit_cost; });
-    // one persistent launch per group of up to kG3MaxPlans jobs of the same form
-    for (int variant = 0; variant < 3; ++variant) {
-        const int fused = variant == 2, pair = variant == 0;
+    // one persistent launch per group of up to kG3MaxPlans jobs of the same kind
+    for (int kind = 0; kind < 4; ++kind) {
         G3Batch b;
         b.n_plans = 0;
         b.total_units = 0;
@@ -1535,9 +1592,10 @@ cudaError_t demod3_gemm(const DemodGemmJob* const* jobs, int n, int n_sms, void*
                 // scratch of the call (the kernel finds it at its first plan's)
                 for (int k = 0; k < b.n_plans; ++k)
                     if (!b.p[k].split) b.p[k].scratch = static_cast<float*>(scratch);
-                const cudaError_t e = pair ? g3_run<true, false>(b, n_sms, room, st)
-                                           : (fused ? g3_run<false, true>(b, n_sms, room, st)
-                                                    : g3_run<false, false>(b, n_sms, room, st));
+                const cudaError_t e = kind == 0   ? g3_run<true, false, true>(b, n_sms, room, st)
+                                      : kind == 1 ? g3_run<true, false, false>(b, n_sms, room, st)
+                                      : kind == 2 ? g3_run<false, false, false>(b, n_sms, room, st)
+                                                  : g3_run<false, true, false>(b, n_sms, room, st);
                 if (e != cudaSuccess) return e;
                 for (int k = 0; k < b.n_plans; ++k)
                     if (b.p[k].split) {
@@ -1551,7 +1609,7 @@ cudaError_t demod3_gemm(const DemodGemmJob* const* jobs, int n, int n_sms, void*
                 b.total_units = 0;
             }
             if (i == n) break;
-            if (order[i]->fused != fused || order[i]->pair != pair || order[i]->n_units <= 0) continue;
+            if (order[i]->kind != kind || order[i]->n_units <= 0) continue;
             std::memcpy(&b.p[b.n_plans], order[i]->bytes, sizeof(G3Plan));
             b.p[b.n_plans].unit0 = b.total_units;
             b.total_units += order[i]->n_units;

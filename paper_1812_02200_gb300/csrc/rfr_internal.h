@@ -165,8 +165,7 @@ struct DemodLaunch {
 constexpr int kDemodJobBytes = 2048;
 struct DemodGemmJob {
     alignas(128) unsigned char bytes[kDemodJobBytes];
-    int fused = 0;              // pre-split fused into the GEMM's producers
-    int pair = 0;               // two-SM tiles
+    int kind = 0;               // the kernel's form (0 wide pair, 1 pair, 2 single CTA, 3 fused pre-split)
     int n_units = 0;            // work items; 0: nothing to launch
     double unit_cost = 0.0;     // of a work item, in clocks
 };
@@ -187,8 +186,8 @@ cudaError_t demod3_prepare(const DemodLaunch& L, cudaStream_t st, DemodGemmJob* 
 // 16 plans); scratch: room bytes for the CTAs' parked products
 cudaError_t demod3_gemm(const DemodGemmJob* const* jobs, int n, int n_sms, void* scratch, size_t room, cudaStream_t st);
 size_t demod3_xs_rows(int64_t F, int Lpad, int D);
-// CTAs that a push of up to F frames launches at most (whatever its form), what they
-// park in all, and the scratch that such a push needs (never less for more frames)
+// CTAs of a push of up to F frames that park products, at most, what they park in all,
+// and the scratch that such a push needs (never less for more frames)
 int demod3_ctas(int n_tones, int64_t F, int n_sms);
 size_t demod3_scratch_bytes(int ctas);
 size_t demod3_scratch_need(int n_tones, int64_t F, int n_sms);
@@ -298,10 +297,10 @@ struct rfr_plan {
     int accum_chunk = 2;           // demod: K blocks per TMEM accumulation chunk
     int demod_products = 4;        // demod GEMM form: 4 (real embedding) or 3 (Gauss)
     void* d_b3 = nullptr;          // three-product form: six tap planes
-    void* d_g3 = nullptr;          // three-product form: the GEMM's scratch, grown with the pushes
-    size_t g3_bytes = 0;
-    void* d_xs3 = nullptr;         // three-product form: six source planes
+    void* d_xs3 = nullptr;         // three-product form: six source planes, then the GEMM's scratch
     int64_t xs3_rows_cap = 0;
+    void* d_g3 = nullptr;          //   (in d_xs3's allocation)
+    size_t g3_bytes = 0;
     int32_t Lpad3 = 0, ntp3 = 0, tap_exp3 = 0;
     int* d_status = nullptr;
 
