@@ -290,7 +290,7 @@ struct ChirpOverlap {
     int seg, sub;                                       // frames per segment, per work item
     int64_t per_cta;                                    // frames per CTA
 };
-template <int J, bool FULL>                             // FULL: L == J * D
+template <int J, bool FULL>                             // FULL: L == J * D; J == 1: items of one frame
 __global__ void __launch_bounds__(kOvWorkers * kChirpThreads, 1)
     chirp_overlap_kernel(const ChirpArgs a, const ChirpOverlap o) {
     extern __shared__ uint32_t xs32[];                  // [(seg + J - 1) * D]
@@ -319,45 +319,64 @@ __global__ void __launch_bounds__(kOvWorkers * kChirpThreads, 1)
             uint64_t p = chirp_phase(s, r, static_cast<int64_t>(m));
             uint64_t d = s * 256ull + r * (512ull * m + 65536ull);
             const uint64_t dd = r * 131072ull;
-            float ar[J], ai[J];                          // frame b - j
+            // the sums of frame f (of the item) over the warp
+            auto reduce = [&](int f, float tr, float ti) {
 #pragma unroll
-            for (int j = 0; j < J; ++j) ar[j] = ai[j] = 0.f;
-            for (int b = 0; b < nf + J - 1; ++b) {
-                const uint32_t* xb = xs32 + (f0 + b) * a.D;
-                const int limit = need - (f0 + b) * a.D;     // samples of the segment from this block on
-                for (int n = tid; n < a.D && (FULL || n < limit); n += kChirpThreads) {
+                for (int w = 16; w > 0; w >>= 1) {
+                    tr += __shfl_xor_sync(0xffffffffu, tr, w);
+                    ti += __shfl_xor_sync(0xffffffffu, ti, w);
+                }
+                if (lane == 0) red[wk][f][warp] = make_double2(tr, ti);
+            };
+            if constexpr (J == 1) {
+                // one frame: its L samples straight through
+                const uint32_t* xb = xs32 + f0 * a.D;
+                float sr = 0.f, si = 0.f;
+#pragma unroll 2
+                for (int n = tid; n < a.L; n += kChirpThreads) {
                     const float2 x = iq_to_f2(xb[n]);
                     float sn, cs;
                     mixer(static_cast<uint32_t>(p >> 32), cs, sn);
                     const float mr = fmaf(x.x, cs, x.y * sn), mi = fmaf(x.y, cs, -x.x * sn);
-#pragma unroll
-                    for (int j = 0; j < J; ++j) {
-                        if (FULL || j * a.D + n < a.L) {
-                            const float hn = __ldg(a.h + j * a.D + n);
-                            ar[j] = fmaf(hn, mr, ar[j]);
-                            ai[j] = fmaf(hn, mi, ai[j]);
-                        }
-                    }
+                    const float hn = __ldg(a.h + n);
+                    sr = fmaf(hn, mr, sr);
+                    si = fmaf(hn, mi, si);
                     p += d;
                     d += dd;
                 }
-                // frame b - (J - 1) is complete
-                const int f = b - (J - 1);
-                if (f >= 0) {
-                    float tr = ar[J - 1], ti = ai[J - 1];
+                reduce(0, sr, si);
+            } else {
+                float ar[J], ai[J];                          // frame b - j
 #pragma unroll
-                    for (int w = 16; w > 0; w >>= 1) {
-                        tr += __shfl_xor_sync(0xffffffffu, tr, w);
-                        ti += __shfl_xor_sync(0xffffffffu, ti, w);
+                for (int j = 0; j < J; ++j) ar[j] = ai[j] = 0.f;
+                for (int b = 0; b < nf + J - 1; ++b) {
+                    const uint32_t* xb = xs32 + (f0 + b) * a.D;
+                    const int limit = (nf - 1 - b) * a.D + a.L;  // samples of the item from this block on
+                    for (int n = tid; n < a.D && (FULL || n < limit); n += kChirpThreads) {
+                        const float2 x = iq_to_f2(xb[n]);
+                        float sn, cs;
+                        mixer(static_cast<uint32_t>(p >> 32), cs, sn);
+                        const float mr = fmaf(x.x, cs, x.y * sn), mi = fmaf(x.y, cs, -x.x * sn);
+#pragma unroll
+                        for (int j = 0; j < J; ++j) {
+                            if (FULL || j * a.D + n < a.L) {
+                                const float hn = __ldg(a.h + j * a.D + n);
+                                ar[j] = fmaf(hn, mr, ar[j]);
+                                ai[j] = fmaf(hn, mi, ai[j]);
+                            }
+                        }
+                        p += d;
+                        d += dd;
                     }
-                    if (lane == 0) red[wk][f][warp] = make_double2(tr, ti);
-                }
+                    // frame b - (J - 1) is complete
+                    if (b >= J - 1) reduce(b - (J - 1), ar[J - 1], ai[J - 1]);
 #pragma unroll
-                for (int j = J - 1; j > 0; --j) {
-                    ar[j] = ar[j - 1];
-                    ai[j] = ai[j - 1];
+                    for (int j = J - 1; j > 0; --j) {
+                        ar[j] = ar[j - 1];
+                        ai[j] = ai[j - 1];
+                    }
+                    ar[0] = ai[0] = 0.f;
                 }
-                ar[0] = ai[0] = 0.f;
             }
             worker_sync();
             if (tid < nf) {
@@ -436,8 +455,10 @@ cudaError_t chirp_demod_launch(const ChirpLaunch& L, cudaStream_t st) {
     a.ld = L.tones_ld;
     a.fo = L.frame_offset;
     // overlapping frames: each mixer value once for all its frames, where at
-    // least a segment of two frames fits
+    // least a segment of two frames fits and it pays
     const int J = (L.L + L.D - 1) / L.D;
+    const size_t smem = static_cast<size_t>(L.L) * sizeof(float2);      // of the single-frame kernel
+    const int single_per_sm = std::max(1, std::min(8, static_cast<int>((220u * 1024u) / (smem + 5u * 1024u))));
     constexpr int kOvSamples = 48 * 1024;               // of a segment: 192 KB
     const int jt = J <= 2 ? 2 : (J <= 4 ? 4 : 8);       // compiled widths; the blocks past L add nothing
     if (J >= 2 && J <= 8 && L.D % kChirpThreads == 0 && (jt + 1) * L.D <= kOvSamples) {
@@ -448,38 +469,56 @@ cudaError_t chirp_demod_launch(const ChirpLaunch& L, cudaStream_t st) {
         const int64_t widest = kOvSamples / L.D - (jt - 1) > 0 ? kOvSamples / L.D - (jt - 1) : 1;
         const int64_t n_seg = (o.per_cta + widest - 1) / widest;
         o.seg = static_cast<int>((o.per_cta + n_seg - 1) / n_seg);
-        // frames per work item, at most kOvSub (so from ceil(seg / kOvSub) items a chirp
-        // on): the fewest rounds of block walks for the four workers
-        int64_t best = INT64_MAX;
-        const int least = (o.seg + kOvSub - 1) / kOvSub;
-        for (int parts = least; parts <= 4 * least; parts *= 2) {
-            const int sub = (o.seg + parts - 1) / parts;
+        // Frames per work item, at most kOvSub (so from ceil(seg / kOvSub) items a chirp
+        // on), or the kernel above: the least of these times, in issue slots, fitted to
+        // 1500 shapes of L = 307 .. 16384, D = 256 .. 4096, 1 .. 16 chirps, 20 .. 10^4
+        // frames (12 % RMS).  An item of several frames: 26 a sample and 5.6 for each
+        // frame it may belong to (8.8 where taps end inside a block), 52 a block, 95 in
+        // all; of one frame: 31 a sample, 220 in all; the kernel above: 44 and 45 a frame
+        // and chirp.  Four workers share an SM's slots, one alone gets two thirds.  (Rounds
+        // of block walks alone chose up to 1.8 times what the kernel above takes, where
+        // a CTA has one or two frames or a sample's frames are few.)
+        constexpr double kAlone = 1.5;
+        const double walk = (L.L + kChirpThreads - 1) / kChirpThreads;      // a thread's samples of a frame
+        double best = 1e300;
+        auto consider = [&](int sub) {
             const int64_t items = static_cast<int64_t>(a.n_chirps) * ((o.seg + sub - 1) / sub);
-            const int64_t cost = (items + kOvWorkers - 1) / kOvWorkers * (sub + jt - 1);
+            const double samples = (static_cast<double>(sub - 1) * L.D + L.L) / kChirpThreads;
+            const double item = sub == 1 ? 31.0 * walk + 220.0
+                                         : samples * (26.0 + (full ? 5.6 : 8.8) * jt) + 52.0 * (sub + jt - 1) + 95.0;
+            const int64_t rest = items % kOvWorkers;
+            const double cost = n_seg * item * ((items - rest) + (rest ? std::max(kAlone, static_cast<double>(rest)) : 0.0));
             if (cost < best) {
                 best = cost;
                 o.sub = sub;
             }
-        }
-        const size_t bytes = static_cast<size_t>(o.seg + jt - 1) * L.D * 4;
-        auto run = [&](auto kern) {
-            const cudaError_t e = allow_smem(kern, kOvSamples * 4);
-            if (e != cudaSuccess) return e;
-            kern<<<static_cast<unsigned>((L.F + o.per_cta - 1) / o.per_cta), kOvWorkers * kChirpThreads, bytes, st>>>(a, o);
-            return cudaGetLastError();
         };
-        switch (jt) {
-        case 2: return full ? run(chirp_overlap_kernel<2, true>) : run(chirp_overlap_kernel<2, false>);
-        case 4: return full ? run(chirp_overlap_kernel<4, true>) : run(chirp_overlap_kernel<4, false>);
-        default: return full ? run(chirp_overlap_kernel<8, true>) : run(chirp_overlap_kernel<8, false>);
+        for (int parts = (o.seg + kOvSub - 1) / kOvSub; parts < o.seg; parts = parts < 4 ? parts + 1 : parts * 3 / 2)
+            consider((o.seg + parts - 1) / parts);
+        consider(1);
+        const double per_sm = static_cast<double>(L.F) / L.n_sms;
+        const double alone = a.n_chirps * (44.0 * walk + 45.0) *
+                             std::max(per_sm, kAlone * std::ceil(static_cast<double>(L.F) / (L.n_sms * single_per_sm)));
+        if (best <= alone) {
+            const size_t bytes = static_cast<size_t>(o.seg + jt - 1) * L.D * 4;
+            auto run = [&](auto kern) {
+                const cudaError_t e = allow_smem(kern, kOvSamples * 4);
+                if (e != cudaSuccess) return e;
+                kern<<<static_cast<unsigned>((L.F + o.per_cta - 1) / o.per_cta), kOvWorkers * kChirpThreads, bytes, st>>>(a, o);
+                return cudaGetLastError();
+            };
+            if (o.sub == 1) return run(chirp_overlap_kernel<1, false>);
+            switch (jt) {
+            case 2: return full ? run(chirp_overlap_kernel<2, true>) : run(chirp_overlap_kernel<2, false>);
+            case 4: return full ? run(chirp_overlap_kernel<4, true>) : run(chirp_overlap_kernel<4, false>);
+            default: return full ? run(chirp_overlap_kernel<8, true>) : run(chirp_overlap_kernel<8, false>);
+            }
         }
     }
-    const size_t smem = static_cast<size_t>(L.L) * sizeof(float2);
     constexpr int kMostTaps = 16384;                    // of a plan
     const cudaError_t e = allow_smem(chirp_demod_kernel, kMostTaps * static_cast<int>(sizeof(float2)));
     if (e != cudaSuccess) return e;
-    const int per_sm = std::max(1, std::min(8, static_cast<int>((220u * 1024u) / (smem + 5u * 1024u))));
-    const int64_t blocks = std::min<int64_t>(L.F, static_cast<int64_t>(L.n_sms) * per_sm);
+    const int64_t blocks = std::min<int64_t>(L.F, static_cast<int64_t>(L.n_sms) * single_per_sm);
     chirp_demod_kernel<<<static_cast<unsigned>(blocks), kChirpThreads, smem, st>>>(a);
     return cudaGetLastError();
 }
