@@ -50,6 +50,7 @@
 #include <cmath>
 #include <cstdint>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "dev_common.cuh"
@@ -266,7 +267,7 @@ __device__ __forceinline__ void store_strided(const float2 (&v)[R], float2* __re
 // exact while j * Ns < 2^32 (here j, Ns < 2^13).
 template <int R, int TH>
 __device__ __forceinline__ void gen_stage(const float2* __restrict__ src, float2* __restrict__ dst, int n, int gl2,
-                                          int Ns, uint32_t ns_magic, const float2* __restrict__ tw) {
+                                          int Ns, uint32_t ns_magic, const float2* __restrict__ tw, bool fence) {
     const int nR = n / R;
     const int nb = nR << gl2;
     const int gm = (1 << gl2) - 1;
@@ -285,6 +286,7 @@ __device__ __forceinline__ void gen_stage(const float2* __restrict__ src, float2
         const int base = (j - k) * R + k;
         store_strided<R>(v, dst, (base << gl2) + g, Ns << gl2);   // points (base + r*Ns)*G + g
     }
+    if (fence) fence_proxy_async_smem();
     __syncthreads();
 }
 
@@ -314,21 +316,30 @@ __device__ __forceinline__ void gen_stage_out(const float2* __restrict__ src, in
     }
 }
 
+// No next copy to start.
+struct NoAhead {
+    __device__ __forceinline__ void operator()() const {}
+};
+
 // The whole transform with its output points delivered to `sink` by the
 // last stage; the points start in buf0.  Returns the buffer the last stage
-// did not read (free for the caller).
-template <int TH, typename Sink>
+// did not read (free for the caller); ahead() is called once every thread has done
+// with that one and the last stage is about to start: the next copy may land there
+// (fenced for it, by the caller where there is one stage only).
+template <int TH, typename Sink, typename Ahead>
 __device__ float2* gen_fft_to(float2* buf0, float2* buf1, const GenFft& f, int gl2, const float2* __restrict__ tw,
-                              Sink sink) {
+                              Sink sink, Ahead ahead) {
+    constexpr bool kAhead = !std::is_same<Ahead, NoAhead>::value;
     float2* src = buf0;
     float2* dst = buf1;
     for (int s = 0; s < f.nst; ++s) {
         const float2* t = tw + f.tw_off[s];
         const bool last = s == f.nst - 1;
+        if (last) ahead();
 #define RFR_GEN_CASE(RR)                                                                              \
     case RR:                                                                                          \
         if (last) gen_stage_out<RR, TH>(src, f.n, gl2, f.ns[s], f.ns_magic[s], t, sink);              \
-        else gen_stage<RR, TH>(src, dst, f.n, gl2, f.ns[s], f.ns_magic[s], t);                        \
+        else gen_stage<RR, TH>(src, dst, f.n, gl2, f.ns[s], f.ns_magic[s], t, kAhead && s == f.nst - 2);\
         break;
         switch (f.radix[s]) {
             RFR_GEN_CASE(16)
@@ -364,9 +375,9 @@ __device__ float2* gen_fft_to(float2* buf0, float2* buf1, const GenFft& f, int g
 // IN: where the points come from.  0: a padded buffer (gpad); the first stage
 // may also read them as a copy left them: 1 interleaved without padding (point
 // j of transform g at j G + g), 2 one transform after the other (at g N + j).
-// Such a stage fences its reads for the next copy into the same place.
+// FENCE: its reads are fenced for the next copy into the same place.
 // PADO: the stage's own output buffer is padded.
-template <int R, int TH, int N, int GL2, int NS, bool OUT, int IN = 0, bool PADO = true, typename Sink>
+template <int R, int TH, int N, int GL2, int NS, bool OUT, int IN = 0, bool PADO = true, bool FENCE = IN != 0 && !OUT, typename Sink>
 __device__ __forceinline__ void fixed_stage(const float2* __restrict__ src, float2* __restrict__ dst,
                                             const float2* __restrict__ tw, Sink& sink) {
     constexpr int nb = (N / R) << GL2;
@@ -401,21 +412,24 @@ __device__ __forceinline__ void fixed_stage(const float2* __restrict__ src, floa
             store_strided<R>(v, dst, (base << GL2) + g, NS << GL2);
         }
     }
-    if constexpr (IN != 0 && !OUT) fence_proxy_async_smem();
+    if constexpr (FENCE) fence_proxy_async_smem();
     if constexpr (!OUT) __syncthreads();
 }
 
 template <int TH, int GL2, int N, int NS, int R, int... Rest>
 struct FixedFft {
-    // stages from src; returns the buffer the last stage did not read
-    template <typename Sink>
-    __device__ __forceinline__ static float2* run(float2* src, float2* dst, const float2* __restrict__ tw, Sink& sink) {
+    // stages from src; returns the buffer the last stage did not read (ahead as in
+    // gen_fft_to)
+    template <typename Sink, typename Ahead>
+    __device__ __forceinline__ static float2* run(float2* src, float2* dst, const float2* __restrict__ tw, Sink& sink,
+                                                  Ahead& ahead) {
         if constexpr (sizeof...(Rest) == 0) {
+            ahead();
             fixed_stage<R, TH, N, GL2, NS, true>(src, dst, tw, sink);
             return dst;
         } else {
-            fixed_stage<R, TH, N, GL2, NS, false>(src, dst, tw, sink);
-            return FixedFft<TH, GL2, N, NS * R, Rest...>::run(dst, src, tw + (NS > 1 ? (R - 1) * NS : 0), sink);
+            fixed_stage<R, TH, N, GL2, NS, false, 0, true, sizeof...(Rest) == 1>(src, dst, tw, sink);
+            return FixedFft<TH, GL2, N, NS * R, Rest...>::run(dst, src, tw + (NS > 1 ? (R - 1) * NS : 0), sink, ahead);
         }
     }
 };
@@ -436,18 +450,18 @@ constexpr FixedShape kFixedShapes[] = {
 // gen_fft_to, through a compiled-in shape when `fix` names one (pass A
 // dispatches its shape, pass B its own: more shapes in one kernel made its
 // register allocation worse, with spills)
-template <int TH, int PASS, typename Sink>
+template <int TH, int PASS, typename Sink, typename Ahead>
 __device__ __forceinline__ float2* fft_to(float2* buf0, float2* buf1, const GenFft& f, int gl2,
-                                          const float2* __restrict__ tw, int fix, Sink sink) {
+                                          const float2* __restrict__ tw, int fix, Sink sink, Ahead ahead) {
     const float2* t0 = tw + f.tw_off[0];
     if constexpr (TH == 256) {
         // N = 10^5's shapes are compiled into the passes themselves
     } else if constexpr (PASS == 0) {
-        if (fix == 4) return FixedFft<TH, 1, 3125, 1, 25, 25, 5>::run(buf0, buf1, t0, sink);
+        if (fix == 4) return FixedFft<TH, 1, 3125, 1, 25, 25, 5>::run(buf0, buf1, t0, sink, ahead);
     } else {
-        if (fix == 5) return FixedFft<TH, 1, 3200, 1, 25, 16, 8>::run(buf0, buf1, t0, sink);
+        if (fix == 5) return FixedFft<TH, 1, 3200, 1, 25, 16, 8>::run(buf0, buf1, t0, sink, ahead);
     }
-    return gen_fft_to<TH>(buf0, buf1, f, gl2, tw, sink);
+    return gen_fft_to<TH>(buf0, buf1, f, gl2, tw, sink, ahead);
 }
 
 struct GenArgs {
@@ -666,7 +680,7 @@ __global__ void __launch_bounds__(TH, GenCfg<TH>::kMinBlocks) gen_single_kernel(
             const int g = e & (G - 1);
             if (rows && g < nf) rows[g * ld + (e >> gls)] = v;
             if (keep) freebuf[gpad(e)] = v;
-        });
+        }, NoAhead{});
         if (keep) {
             __syncthreads();
             for (int i = threadIdx.x; i < (a.n_tones << gls); i += TH) {
@@ -836,12 +850,13 @@ __global__ void __launch_bounds__(TH, GenCfg<TH>::kMinBlocks)
     const int GA = 1 << a.gla;
     const int groups = (a.N2 + GA - 1) >> a.gla;
     const int E = a.N1 << a.gla;
-    float2* sm1 = second_buffer(sm, E);
     // the digit tables of W_N^m, m = a*65536 + b*256 + c (N <= 2^24)
     float2* stw = sm + 2 * (gpad(E) + 1);
     for (int i = threadIdx.x; i < 3 * kTwDigit; i += TH) stw[i] = __ldg(a.tw3 + i);
-    // V's boxes land 128-byte aligned in the second buffer; mbarrier after the tables
-    float2* vst = reinterpret_cast<float2*>((reinterpret_cast<uintptr_t>(sm1) + 127) & ~uintptr_t(127));
+    // V's boxes land 128-byte aligned in one of the buffers; mbarrier after the tables
+    auto landing = [&](int off) { return sm + off + ((0u - smem_u32(sm + off)) & 127u) / 8; };
+    const int second = gpad(E) + 1;
+    float2* const vst = landing(second);
     uint64_t* vbar = reinterpret_cast<uint64_t*>(stw + 3 * kTwDigit);
     if (a.vtma && threadIdx.x == 0) {
         mbar_init(vbar, 1);
@@ -851,15 +866,15 @@ __global__ void __launch_bounds__(TH, GenCfg<TH>::kMinBlocks)
     uint32_t vphase = 0;
     // points p1*GA + g = V[kk][p1*N2 + g0 + g]: boxes of rows of V
     // viewed as [frames*N1][N2] (columns past N2 read as zero); one thread
-    auto fetch = [&](int64_t it) {
+    auto fetch = [&](int64_t it, float2* to) {
         const int64_t kk = it / groups;
         const int g0 = static_cast<int>(it - kk * groups) << a.gla;
         mbar_arrive_expect_tx(vbar, static_cast<uint32_t>(a.vboxes * a.vbox_rows * GA * 8));
         for (int b = 0; b < a.vboxes; ++b)
-            tma_load_2d(vst + b * a.vsstride, &tmv, g0, static_cast<int32_t>(kk * a.N1 + b * a.vbox_rows), vbar);
+            tma_load_2d(to + b * a.vsstride, &tmv, g0, static_cast<int32_t>(kk * a.N1 + b * a.vbox_rows), vbar);
     };
     if constexpr (TH == 256) {
-        // N = 10^5 (two compiled-in stages), boxes end to end: the first stage
+        // The compiled-in two-stage shape (N = 10^5), boxes end to end: the first stage
         // reads the boxes as they land, and the next group's boxes are fetched
         // into the same place while the second stage runs.  (Fetched at the
         // group's start and copied into the padded layout first, every group
@@ -868,7 +883,7 @@ __global__ void __launch_bounds__(TH, GenCfg<TH>::kMinBlocks)
         if (a.fixa == 1 && a.vtma && a.vsstride == a.vbox_rows * GA) {
             constexpr int R0 = 25, R1 = 16, NN = 400, GL = 3;
             const float2* const t0 = a.tw_a + a.fa.tw_off[0];
-            if (threadIdx.x == 0 && blockIdx.x < a.F * groups) fetch(blockIdx.x);
+            if (threadIdx.x == 0 && blockIdx.x < a.F * groups) fetch(blockIdx.x, vst);
             for (int64_t it = blockIdx.x; it < a.F * groups; it += gridDim.x) {
                 const int64_t kk = it / groups;
                 const int g0 = static_cast<int>(it - kk * groups) << GL;
@@ -879,7 +894,7 @@ __global__ void __launch_bounds__(TH, GenCfg<TH>::kMinBlocks)
                 // (no padding between the stages: butterflies' outputs start 200
                 // points apart, 8 modulo the 16 banks, and 8 transforms fill those)
                 fixed_stage<R0, TH, NN, GL, 1, false, 1, false>(vst, sm, t0, none);
-                if (threadIdx.x == 0 && it + gridDim.x < a.F * groups) fetch(it + gridDim.x);
+                if (threadIdx.x == 0 && it + gridDim.x < a.F * groups) fetch(it + gridDim.x, vst);
                 float2* zf = a.z + kk * a.N;
                 auto sink = [=](int e, float2 v) {
                     const int g = e & ((1 << GL) - 1), c1 = e >> GL, p2 = g0 + g;
@@ -895,19 +910,29 @@ __global__ void __launch_bounds__(TH, GenCfg<TH>::kMinBlocks)
             return;
         }
     }
+    // Any other lengths: the boxes are copied into the padded layout of the other
+    // buffer; the next group's land in the buffer that the last stage does not read,
+    // while it runs: with an odd number of stages the same one each time.  (Fetched at
+    // the group's start before; both passes, 2^26 samples, T = 4: N = 10^4 941 -> 920 us,
+    // 2 10^4 817 -> 791, 10^6 1028 -> 1018, 2 10^6 1559 -> 1417.  A first stage that reads
+    // the boxes as they landed took 910 / 786 / 1020 / 1361, but 2 to 4 % more than this
+    // for N = 5 10^4 and 78125: its registers spill.)
+    int land = second, work = 0;
+    if (a.vtma && threadIdx.x == 0 && blockIdx.x < a.F * groups) fetch(blockIdx.x, landing(land));
     for (int64_t it = blockIdx.x; it < a.F * groups; it += gridDim.x) {
         const int64_t kk = it / groups;
         const int g0 = static_cast<int>(it - kk * groups) << a.gla;
         const int N2 = a.N2, gla = a.gla;
         if (a.vtma) {
-            if (threadIdx.x == 0) fetch(it);
             if (!mbar_wait(vbar, vphase, a.status)) return;
             vphase ^= 1u;
+            const float2* const from = landing(land);
             for (int b = 0; b < a.vboxes; ++b) {
                 const int rows = min(a.vbox_rows, a.N1 - b * a.vbox_rows);
                 const int o = b * a.vbox_rows * GA;
-                for (int e = threadIdx.x; e < rows * GA; e += TH) sm[gpad(o + e)] = vst[b * a.vsstride + e];
+                for (int e = threadIdx.x; e < rows * GA; e += TH) sm[work + gpad(o + e)] = from[b * a.vsstride + e];
             }
+            fence_proxy_async_smem();
         } else {
             const int64_t base = (a.k0 + kk) * a.hop;
             const int sh = frame_shift(a, base);
@@ -919,20 +944,26 @@ __global__ void __launch_bounds__(TH, GenCfg<TH>::kMinBlocks)
                            const int q = (e >> gla) * N2 + g0 + g;          // FFT input index
                            return q >= sh ? q - sh : q - sh + N;            // window position
                        },
-                       sm);
+                       sm + work);
         }
         __syncthreads();
         // the last stage multiplies by W_N^{p2*c1} and stores Z directly
         float2* zf = a.z + kk * a.N;
-        fft_to<TH, 0>(sm, sm1, a.fa, a.gla, a.tw_a, a.fixa, [=](int e, float2 v) {
+        auto sink = [=](int e, float2 v) {
             const int g = e & (GA - 1), c1 = e >> gla, p2 = g0 + g;
             if (p2 < N2) {
                 const int m = p2 * c1;                       // < N1*N2 = N
                 const float2 w = cmul(cmul(stw[m & 255], stw[kTwDigit + ((m >> 8) & 255)]), stw[2 * kTwDigit + (m >> 16)]);
                 zf[static_cast<int64_t>(c1) * N2 + p2] = cmul(v, w);
             }
-        });
-        fence_proxy_async_smem();   // shared-memory reads done before the next box lands
+        };
+        const int next = (a.fa.nst & 1) ? land : work;
+        auto ahead = [&] {
+            if (a.vtma && threadIdx.x == 0 && it + gridDim.x < a.F * groups) fetch(it + gridDim.x, landing(next));
+        };
+        fft_to<TH, 0>(sm + work, sm + land, a.fa, a.gla, a.tw_a, a.fixa, sink, ahead);
+        work = second - next;
+        land = next;
         __syncthreads();
     }
 }
@@ -943,10 +974,11 @@ __global__ void __launch_bounds__(TH, GenCfg<TH>::kMinBlocks) gen_pass_b_kernel(
     const int GB = 1 << a.glb;
     const int groups = (a.N1 + GB - 1) >> a.glb;
     const int E = a.N2 << a.glb;
-    float2* sm1 = second_buffer(sm, E);
-    // the bulk copy lands 16-byte aligned in the second buffer (one spare
+    // the bulk copy lands 16-byte aligned in one of the buffers (one spare
     // element at its end); its mbarrier follows the two buffers
-    float2* zst = sm1 + ((reinterpret_cast<uintptr_t>(sm1) & 8) ? 1 : 0);
+    auto landing = [&](int off) { return sm + off + (smem_u32(sm + off) & 8 ? 1 : 0); };
+    const int second = gpad(E) + 1;
+    float2* const zst = landing(second);
     uint64_t* zbar = reinterpret_cast<uint64_t*>(sm + 2 * (gpad(E) + 1));
     if (a.zbulk && threadIdx.x == 0) {
         mbar_init(zbar, 1);
@@ -1027,18 +1059,27 @@ __global__ void __launch_bounds__(TH, GenCfg<TH>::kMinBlocks) gen_pass_b_kernel(
             return;
         }
     }
+    // Any other lengths: as in pass A, except that with tones the buffer that the last
+    // stage does not read holds its outputs for the gather, and the next rows land in
+    // the other one once it has been read.
+    // rows c0 .. c0+GB-1 of Z are one contiguous block of GB*N2 points
+    auto fetch = [&](int64_t it, float2* to) {
+        const int64_t kk = it / groups;
+        const int c0 = static_cast<int>(it - kk * groups) << a.glb;
+        const uint32_t bytes = static_cast<uint32_t>(min(GB, a.N1 - c0) * a.N2) * 8u;
+        mbar_arrive_expect_tx(zbar, bytes);
+        tma_bulk_g2s(to, a.z + kk * a.N + static_cast<int64_t>(c0) * a.N2, bytes, zbar);
+    };
+    const bool keep = a.n_tones > 0;
+    int land = second, work = 0;
+    if (a.zbulk && threadIdx.x == 0 && blockIdx.x < a.F * groups) fetch(blockIdx.x, landing(land));
     for (int64_t it = blockIdx.x; it < a.F * groups; it += gridDim.x) {
         const int64_t kk = it / groups;
         const int c0 = static_cast<int>(it - kk * groups) << a.glb;
-        // rows c0 .. c0+GB-1 of Z are one contiguous block of GB*N2 points
         const float2* zf = a.z + kk * a.N + static_cast<int64_t>(c0) * a.N2;
-        const int rows = min(GB, a.N1 - c0);
-        const int cnt = rows * a.N2;
+        const int cnt = min(GB, a.N1 - c0) * a.N2;
+        const float2* const from = landing(land);
         if (a.zbulk) {
-            if (threadIdx.x == 0) {
-                mbar_arrive_expect_tx(zbar, static_cast<uint32_t>(cnt) * 8u);
-                tma_bulk_g2s(zst, zf, static_cast<uint32_t>(cnt) * 8u, zbar);
-            }
             if (!mbar_wait(zbar, zphase, a.status)) return;
             zphase ^= 1u;
         }
@@ -1046,31 +1087,39 @@ __global__ void __launch_bounds__(TH, GenCfg<TH>::kMinBlocks) gen_pass_b_kernel(
         for (int f = threadIdx.x; f < E; f += TH) {
             const int g = static_cast<int>(__umulhi(static_cast<uint32_t>(f), a.n2_magic));   // f / N2
             const int p2 = f - g * a.N2;
-            sm[gpad((p2 << a.glb) + g)] = f < cnt ? (a.zbulk ? zst[f] : zf[f]) : make_float2(0.f, 0.f);
+            sm[work + gpad((p2 << a.glb) + g)] = f < cnt ? (a.zbulk ? from[f] : zf[f]) : make_float2(0.f, 0.f);
         }
+        fence_proxy_async_smem();
         __syncthreads();
         const int64_t k = a.k0 + kk;
         // the last stage stores the spectrum (runs of GB points) and, for the
         // tone gather, a copy in the free shared-memory buffer
         float2* row = a.full ? a.full + (a.fo + k) * a.full_ld : nullptr;
-        const bool keep = a.n_tones > 0;
-        float2* const freebuf = (a.fb.nst & 1) ? sm1 : sm;
+        const int freed = (a.fb.nst & 1) ? land : work;
         const int glb = a.glb, N1 = a.N1;
-        fft_to<TH, 1>(sm, sm1, a.fb, a.glb, a.tw_b, a.fixb, [=](int e, float2 v) {
+        const bool more = a.zbulk && it + gridDim.x < a.F * groups;
+        auto sink = [=](int e, float2 v) {
             const int g = e & (GB - 1), c2 = e >> glb;
             if (row && c0 + g < N1) row[c0 + g + static_cast<int64_t>(N1) * c2] = v;
-            if (keep) freebuf[gpad(e)] = v;
-        });
+            if (keep) sm[freed + gpad(e)] = v;
+        };
+        auto ahead = [&] {
+            if (!keep && more && threadIdx.x == 0) fetch(it + gridDim.x, landing(freed));
+        };
+        fft_to<TH, 1>(sm + work, sm + land, a.fb, a.glb, a.tw_b, a.fixb, sink, ahead);
+        land = keep ? second - freed : freed;            // with tones: where the last stage's points were
+        work = second - land;
         if (keep) {
+            fence_proxy_async_smem();
             __syncthreads();
+            if (more && threadIdx.x == 0) fetch(it + gridDim.x, landing(land));
             const int gi = c0 >> a.glb;
             const int i1 = __ldg(a.goff + gi + 1);
             for (int i = __ldg(a.goff + gi) + threadIdx.x; i < i1; i += TH) {
                 const int2 te = __ldg(a.gtone + i);
-                a.tones[te.x * a.tones_ld + a.fo + k] = freebuf[gpad(te.y)];
+                a.tones[te.x * a.tones_ld + a.fo + k] = sm[freed + gpad(te.y)];
             }
         }
-        fence_proxy_async_smem();   // shared-memory reads done before the next bulk copy writes
         __syncthreads();
     }
 }
