@@ -458,8 +458,9 @@ rfr_status rfr_batch_stats(const rfr_batch* batch, int64_t* steps, int64_t* grap
 const char* rfr_batch_last_error(const rfr_batch* batch);
 
 /*
- * rfr_plan_autotune -- time the plan's result-neutral launch choices (PFB:
- * ring look-ahead of 1..3 super-blocks; demodulation: GEMM tile raster
+ * rfr_plan_autotune -- time the plan's result-neutral launch choices (PFB
+ * shapes of the shared-memory ring kernel, N = 16, 32, 2048 with T <= 4 and 4096
+ * without symmetric taps: look-ahead of 1..3 super-blocks; demodulation: GEMM tile raster
  * groups and, for the three-product form, the GEMM's form: picked by size,
  * or one of those below) on a push of n_samples and keep the fastest (Sec. III: the
  * host runtime tunes the GPU kernels).  Outputs stay bit-identical whatever

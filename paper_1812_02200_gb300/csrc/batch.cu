@@ -89,7 +89,7 @@ std::string tune_key(const rfr_plan* p, int64_t n) {
     while ((int64_t(1) << (lg + 1)) <= n) ++lg;
     std::ostringstream k;
     k << "v2:" << (p->mode == RFR_MODE_PFB ? "pfb" : p->mode == RFR_MODE_CHIRP ? "chirp" : "demod") << ":N" << p->N << ":T" << p->T << ":L" << p->L
-      << ":D" << p->D << ":tones" << p->words.size() << ":flags" << p->out_flags;
+      << ":D" << p->D << ":hop" << p->H << ":tones" << p->words.size() << ":flags" << p->out_flags;
     if (p->mode == RFR_MODE_DEMOD) k << ":products" << p->demod_products << ":chunk" << p->accum_chunk;
     k << ":n2^" << lg
       << ":sm" << prop.major << prop.minor << "x" << prop.multiProcessorCount;
@@ -330,8 +330,12 @@ rfr_status rfr_plan_autotune(rfr_plan* p, int64_t n_samples, int32_t use_cache, 
     // candidates (all give bit-identical results)
     std::vector<TuneEntry> cand;
     if (p->mode == RFR_MODE_PFB) {
-        for (int la : {1, 2, 3}) cand.push_back({la, 1, 128});
-        // N = 8192, 16384 with T <= 8: the cluster kernel beside the direct one
+        // the ring kernel's look-ahead, where the shape has that kernel at all
+        if (!p->gen && p->phase_R == 1 && rfr::pfb_may_ring(p->log2n, p->Tk, p->sym_taps))
+            for (int la : {1, 2, 3}) cand.push_back({la, 1, 128});
+        else
+            cand.push_back({0, 1, 128});
+        // N = 8192, 16384 with T <= 8: the cluster kernel beside the rows kernel
         if (p->d_tw_cl) cand.push_back({0, 1, 128, 0, 0, 1});
     } else {
         // the fused pre-split converts each A tile once per tone tile and

@@ -1945,6 +1945,10 @@ cudaError_t dispatch_ring_T(PfbArgs a, int tk, int n_sms, int max_smem, int la, 
 }  // namespace
 
 bool pfb_uses_ring(int log2n, int taps) { return log2n >= 4 && log2n <= 12 && taps <= 8; }
+bool pfb_may_ring(int log2n, int taps, bool sym) {
+    if (!pfb_uses_ring(log2n, taps)) return false;
+    return log2n <= 5 || (log2n == 11 && taps == 4) || (log2n == 12 && !sym);
+}
 int pfb_cluster_size(int log2n, int taps) { return (log2n == 13 || log2n == 14) && taps <= 8 ? 1 << (log2n - 12) : 0; }
 // Shapes whose FIR is a pre-sum pass: those of the rows kernel, and N = 2048 with
 // T > 8 (2^25 samples 238 us; the tile kernel 277).
@@ -2011,11 +2015,11 @@ cudaError_t pfb_launch(const PfbLaunch& L, cudaStream_t st) {
         if (lg != 12 || L.taps_kernel != 8 || !L.sym_taps) return cudaErrorInvalidValue;
         return launch_tmem_sym<8>(a, L.n_sms, L.max_smem, st);
     }
-    if (lg == 12 && L.sym_taps && L.variant == 0) {
+    if (lg == 12 && L.sym_taps) {
         if (L.taps_kernel == 8) return launch_tmem_sym<8>(a, L.n_sms, L.max_smem, st);
         if (L.taps_kernel == 4) return launch_tmem_sym<4>(a, L.n_sms, L.max_smem, st);
     }
-    if (lg == 12 && a.use_tma && L.variant != 1) {
+    if (lg == 12 && a.use_tma) {
         if (L.taps_kernel == 4) return launch_tmem<4>(a, L.n_sms, L.max_smem, st);
         if (L.taps_kernel == 8) return launch_tmem<8>(a, L.n_sms, L.max_smem, st);
     }

@@ -54,14 +54,12 @@ struct PfbLaunch {
     int n_sms;
     int max_smem;
     int lookahead;      // ring super-blocks fetched ahead (0 = as many as fit, <= 3)
-    int variant;        // 0 = best available, 1 = shared-memory int16 ring only,
-                        // 2 = no symmetric-tap TMEM kernel
     int sym_taps;       // kernel taps exactly symmetric (h[j] == h[T*N - 1 - j])
     int tone_cs;        // tone columns of consecutive frames this far apart (0/1: adjacent)
     int rot;            // bin c multiplied by (-i)^((c * rot) mod 4) (phase passes)
     int hop;            // samples between frames (N: critically sampled)
     int64_t a0;         // absolute sample index of the virtual stream's first sample
-    int cluster;        // N = 8192, 16384 (T <= 8): the cluster kernel instead of the direct one
+    int cluster;        // N = 8192, 16384 (T <= 8): the cluster kernel instead of the rows kernel
     const void* tw_cl;  // its twiddles: the 4096-point FFT's, then W_N^(k2 p1)
     int tw_cl_count;    // entries of the 4096-point FFT part
     void* pre;          // FIR pre-sum rows [pre_cap][N] (float2) of pfb_pre_rows plans, or null
@@ -115,6 +113,9 @@ void gen_plan_free(GenPlan* g);
 int pfb_kernel_taps(int log2n, int taps);
 // CTAs per cluster of the cluster PFB kernel (N = 8192, 16384 with T <= 8), else 0.
 int pfb_cluster_size(int log2n, int taps);
+// Whether some push of the shape (pfb_kernel_taps taps) runs the ring kernel, the one
+// that PfbLaunch::lookahead is for.
+bool pfb_may_ring(int log2n, int taps, bool sym);
 // PFB plans whose pushes take FIR pre-sum rows (PfbLaunch::pre): N = 8192 and
 // 16384; N = 2048 and 4096 with T > 8.
 bool pfb_pre_rows(int log2n, int taps);
@@ -237,7 +238,7 @@ struct TuneConfig {
     int demod_bt = 128;         //   tones per single-CTA tile (128 or 64)
     int demod_fused = 0;        //   pre-split fused into its producers (0/1)
     int demod_pair = 0;         //   two-SM tiles (0/1)
-    int pfb_cluster = 0;        // PFB N = 8192, 16384 with T <= 8: cluster kernel (1) or direct (0)
+    int pfb_cluster = 0;        // PFB N = 8192, 16384 with T <= 8: cluster kernel (1) or rows kernel (0)
     bool tuned = false;
 };
 

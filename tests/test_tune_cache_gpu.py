@@ -65,3 +65,14 @@ def test_entries_of_the_older_format_are_not_found(lib, tmp_path, monkeypatch):
     assert q.autotune(FRAMES * D) == -1.0
     assert q.tune() == p.tune()
     assert old in json.loads(path.read_text())               # an older program still finds its own
+
+
+def test_look_ahead_is_timed_for_the_ring_kernel_only(lib, tmp_path, monkeypatch):
+    monkeypatch.setenv("RFR_TUNE_CACHE", str(tmp_path / "tune.json"))
+    for N, T, hop, ring in ((256, 8, 256, False), (4096, 8, 4096, False), (4096, 8, 1024, False), (8192, 16, 8192, False),
+                            (1000, 4, 1000, False), (32, 8, 32, True), (2048, 4, 2048, True), (4096, 6, 4096, True)):
+        p = lib.Plan(N, T, window="hamming", words=siggen.bin_words([1, 2], N), decimation=hop)
+        assert p.autotune(1 << 16) > 0
+        assert p.tune()["pfb_lookahead"] in ((1, 2, 3) if ring else (0,))
+        q = lib.Plan(N, T, window="hamming", words=siggen.bin_words([1, 2], N), decimation=hop)
+        assert q.autotune(1 << 16) == -1.0 and q.tune() == p.tune()
