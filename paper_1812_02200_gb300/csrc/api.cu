@@ -378,8 +378,15 @@ rfr_status ensure_pre_rows(rfr_plan* p, int64_t F, cudaStream_t st) {
             return RFR_OK;
         }
         RFR_CUDA(p, e);
-        cudaDeviceSynchronize();
-        dev_free(p->d_pre);
+        if (p->pre_held) {
+            // a caller's graph holds the smaller ones (at other shapes such a graph has to
+            // be made after the largest push; these had no scratch once)
+            p->pre_kept.push_back(p->d_pre);
+            p->pre_held = false;
+        } else {
+            cudaDeviceSynchronize();
+            dev_free(p->d_pre);
+        }
         p->d_pre = rows;
         p->pre_cap = F;
         return RFR_OK;
@@ -472,17 +479,8 @@ rfr_status push_core(rfr_plan* p, const int16_t* iq, int64_t n, const rfr_output
                 rfr_status rs = phase_passes(p, L, o, lv, F, st);
                 if (rs != RFR_OK) return rs;
             } else {
-                bool pre = !p->gen && rfr::pfb_pre_rows(p->log2n, p->Tk) && !L.cluster &&
-                           !rfr::pfb_pre_skip(p->log2n, p->Tk, F, L.full != nullptr, p->n_sms);
-                if (pre && rfr::pfb_pre_optional(p->log2n, p->Tk) && !defer_gemm) {
-                    // a caller's graph of a shape that can do without the rows does not
-                    // hold on to them: a larger push later replaces them (a batched
-                    // step's graph is captured anew for every step)
-                    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-                    RFR_CUDA(p, cudaStreamIsCapturing(st, &cs));
-                    pre = cs == cudaStreamCaptureStatusNone;
-                }
-                if (pre) {
+                if (!p->gen && rfr::pfb_pre_rows(p->log2n, p->Tk) && !L.cluster &&
+                    !rfr::pfb_pre_skip(p->log2n, p->Tk, F, L.full != nullptr, p->n_sms)) {
                     // FIR pre-sum rows, sized for a push of n samples after any
                     // carry when they grow
                     const int64_t lv_max = std::max<int64_t>(p->cl, p->W - 1) + n;
@@ -490,6 +488,13 @@ rfr_status push_core(rfr_plan* p, const int16_t* iq, int64_t n, const rfr_output
                     if (rs != RFR_OK) return rs;
                     if (F <= p->pre_cap) L.pre = p->d_pre;
                     L.pre_cap = p->pre_cap;
+                    if (L.pre && !p->pre_held && rfr::pfb_pre_optional(p->log2n, p->Tk) && !defer_gemm) {
+                        // captured into a caller's graph: these rows stay as long as the plan
+                        // (a batched step's graph is captured anew for every step)
+                        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+                        RFR_CUDA(p, cudaStreamIsCapturing(st, &cs));
+                        p->pre_held = cs != cudaStreamCaptureStatusNone;
+                    }
                 }
                 RFR_CUDA(p, p->gen ? rfr::gen_pfb_launch(L, p->gplan, st) : rfr::pfb_launch(L, st));
             }
@@ -615,6 +620,7 @@ void destroy(rfr_plan* p) {
         dev_free(p->d_stage_full[i]);
         if (p->stage_st[i]) cudaStreamDestroy(p->stage_st[i]);
     }
+    for (void* q : p->pre_kept) dev_free(q);
     for (auto& e : p->stage_ev)
         if (e) cudaEventDestroy(e);
     for (int g = 0; g < rfr_plan::kToneGroups; ++g) {

@@ -265,6 +265,8 @@ struct rfr_plan {
     int64_t ptones_cap = 0;                    //   frames per pass row
     void* d_pre = nullptr;                     // FIR pre-sum rows (rfr::pfb_pre_rows plans)
     int64_t pre_cap = 0;                       //   [frame][N] float2, frames
+    bool pre_held = false;                     //   captured into a caller's graph (optional rows)
+    std::vector<void*> pre_kept;               //   smaller rows that such graphs hold
     int64_t pre_refused = 0;                   //   least frames that found no room (0: none), optional rows
     int32_t fail_allocs = 0;                   // scratch allocations to fail (host-side injection)
     bool gen = false;                          // PFB through the any-N kernels
