@@ -843,7 +843,9 @@ __global__ void __launch_bounds__(kFirThreads) gen_fir_frames_kernel(const GenAr
     }
 }
 
-template <int TH>
+// FIX: the instance of the compiled-in two-stage shape (GenArgs::fixa 1), boxes end to
+// end; apart, because either loop's registers cost the other some.
+template <int TH, bool FIX>
 __global__ void __launch_bounds__(TH, GenCfg<TH>::kMinBlocks)
     gen_pass_a_kernel(const GenArgs a, const __grid_constant__ CUtensorMap tmv) {
     extern __shared__ float2 sm[];
@@ -856,7 +858,6 @@ __global__ void __launch_bounds__(TH, GenCfg<TH>::kMinBlocks)
     // V's boxes land 128-byte aligned in one of the buffers; mbarrier after the tables
     auto landing = [&](int off) { return sm + off + ((0u - smem_u32(sm + off)) & 127u) / 8; };
     const int second = gpad(E) + 1;
-    float2* const vst = landing(second);
     uint64_t* vbar = reinterpret_cast<uint64_t*>(stw + 3 * kTwDigit);
     if (a.vtma && threadIdx.x == 0) {
         mbar_init(vbar, 1);
@@ -873,50 +874,49 @@ __global__ void __launch_bounds__(TH, GenCfg<TH>::kMinBlocks)
         for (int b = 0; b < a.vboxes; ++b)
             tma_load_2d(to + b * a.vsstride, &tmv, g0, static_cast<int32_t>(kk * a.N1 + b * a.vbox_rows), vbar);
     };
-    if constexpr (TH == 256) {
-        // The compiled-in two-stage shape (N = 10^5), boxes end to end: the first stage
+    if constexpr (FIX) {
+        // The shape of N = 10^5, boxes end to end: the first stage
         // reads the boxes as they land, and the next group's boxes are fetched
         // into the same place while the second stage runs.  (Fetched at the
         // group's start and copied into the padded layout first, every group
         // waited for its load: 659 us a 2^27-sample push, now 435, at 63 % of
         // the DRAM peak; pass B, likewise, 508 -> 425.)
-        if (a.fixa == 1 && a.vtma && a.vsstride == a.vbox_rows * GA) {
-            constexpr int R0 = 25, R1 = 16, NN = 400, GL = 3;
-            const float2* const t0 = a.tw_a + a.fa.tw_off[0];
-            if (threadIdx.x == 0 && blockIdx.x < a.F * groups) fetch(blockIdx.x, vst);
-            for (int64_t it = blockIdx.x; it < a.F * groups; it += gridDim.x) {
-                const int64_t kk = it / groups;
-                const int g0 = static_cast<int>(it - kk * groups) << GL;
-                const int N2 = a.N2;
-                if (!mbar_wait(vbar, vphase, a.status)) return;
-                vphase ^= 1u;
-                auto none = [](int, float2) {};
-                // (no padding between the stages: butterflies' outputs start 200
-                // points apart, 8 modulo the 16 banks, and 8 transforms fill those)
-                fixed_stage<R0, TH, NN, GL, 1, false, 1, false>(vst, sm, t0, none);
-                if (threadIdx.x == 0 && it + gridDim.x < a.F * groups) fetch(it + gridDim.x, vst);
-                float2* zf = a.z + kk * a.N;
-                auto sink = [=](int e, float2 v) {
-                    const int g = e & ((1 << GL) - 1), c1 = e >> GL, p2 = g0 + g;
-                    if (p2 < N2) {
-                        const int m = p2 * c1;
-                        const float2 w = cmul(cmul(stw[m & 255], stw[kTwDigit + ((m >> 8) & 255)]), stw[2 * kTwDigit + (m >> 16)]);
-                        zf[static_cast<int64_t>(c1) * N2 + p2] = cmul(v, w);
-                    }
-                };
-                fixed_stage<R1, TH, NN, GL, R0, true, 1>(sm, sm, t0, sink);
-                __syncthreads();
-            }
-            return;
+        constexpr int R0 = 25, R1 = 16, NN = 400, GL = 3;
+        float2* const vst = landing(gpad(NN << GL) + 1);
+        const float2* const t0 = a.tw_a + a.fa.tw_off[0];
+        if (threadIdx.x == 0 && blockIdx.x < a.F * groups) fetch(blockIdx.x, vst);
+        for (int64_t it = blockIdx.x; it < a.F * groups; it += gridDim.x) {
+            const int64_t kk = it / groups;
+            const int g0 = static_cast<int>(it - kk * groups) << GL;
+            const int N2 = a.N2;
+            if (!mbar_wait(vbar, vphase, a.status)) return;
+            vphase ^= 1u;
+            auto none = [](int, float2) {};
+            // (no padding between the stages: butterflies' outputs start 200
+            // points apart, 8 modulo the 16 banks, and 8 transforms fill those)
+            fixed_stage<R0, TH, NN, GL, 1, false, 1, false>(vst, sm, t0, none);
+            if (threadIdx.x == 0 && it + gridDim.x < a.F * groups) fetch(it + gridDim.x, vst);
+            float2* zf = a.z + kk * a.N;
+            auto sink = [=](int e, float2 v) {
+                const int g = e & ((1 << GL) - 1), c1 = e >> GL, p2 = g0 + g;
+                if (p2 < N2) {
+                    const int m = p2 * c1;
+                    const float2 w = cmul(cmul(stw[m & 255], stw[kTwDigit + ((m >> 8) & 255)]), stw[2 * kTwDigit + (m >> 16)]);
+                    zf[static_cast<int64_t>(c1) * N2 + p2] = cmul(v, w);
+                }
+            };
+            fixed_stage<R1, TH, NN, GL, R0, true, 1>(sm, sm, t0, sink);
+            __syncthreads();
         }
+        return;
     }
     // Any other lengths: the boxes are copied into the padded layout of the other
     // buffer; the next group's land in the buffer that the last stage does not read,
     // while it runs: with an odd number of stages the same one each time.  (Fetched at
-    // the group's start before; both passes, 2^26 samples, T = 4: N = 10^4 941 -> 920 us,
-    // 2 10^4 817 -> 791, 10^6 1028 -> 1018, 2 10^6 1559 -> 1417.  A first stage that reads
-    // the boxes as they landed took 910 / 786 / 1020 / 1361, but 2 to 4 % more than this
-    // for N = 5 10^4 and 78125: its registers spill.)
+    // the group's start before; both passes, 2^26 samples, T = 4: N = 10^4 942 -> 911 us,
+    // 2 10^4 818 -> 781, 10^6 1030 -> 1012, 2 10^6 1566 -> 1415.  A first stage that reads
+    // the boxes as they landed gained up to 4 % more and lost 2 to 4 % for N = 5 10^4 and
+    // 78125, its registers spilling.)
     int land = second, work = 0;
     if (a.vtma && threadIdx.x == 0 && blockIdx.x < a.F * groups) fetch(blockIdx.x, landing(land));
     for (int64_t it = blockIdx.x; it < a.F * groups; it += gridDim.x) {
@@ -968,7 +968,7 @@ __global__ void __launch_bounds__(TH, GenCfg<TH>::kMinBlocks)
     }
 }
 
-template <int TH>
+template <int TH, bool FIX>                             // FIX: fixb 2 with zbulk
 __global__ void __launch_bounds__(TH, GenCfg<TH>::kMinBlocks) gen_pass_b_kernel(const GenArgs a) {
     extern __shared__ float2 sm[];
     const int GB = 1 << a.glb;
@@ -978,7 +978,6 @@ __global__ void __launch_bounds__(TH, GenCfg<TH>::kMinBlocks) gen_pass_b_kernel(
     // element at its end); its mbarrier follows the two buffers
     auto landing = [&](int off) { return sm + off + (smem_u32(sm + off) & 8 ? 1 : 0); };
     const int second = gpad(E) + 1;
-    float2* const zst = landing(second);
     uint64_t* zbar = reinterpret_cast<uint64_t*>(sm + 2 * (gpad(E) + 1));
     if (a.zbulk && threadIdx.x == 0) {
         mbar_init(zbar, 1);
@@ -986,78 +985,79 @@ __global__ void __launch_bounds__(TH, GenCfg<TH>::kMinBlocks) gen_pass_b_kernel(
     }
     __syncthreads();
     uint32_t zphase = 0;
-    if constexpr (TH == 256) {
+    if constexpr (FIX) {
         // N = 10^5, as in pass A: the first stage reads the rows as the bulk
         // copy left them, and the next group's copy runs behind the second
         // stage, whose outputs reach the tone gather through its own input
-        if (a.fixb == 2 && a.zbulk) {
-            constexpr int R0 = 25, R1 = 10, NN = 250, GL = 4, nb = (NN / R1) << GL, iters = (nb + TH - 1) / TH;
-            const float2* const t0 = a.tw_b + a.fb.tw_off[0];
-            auto fetch = [&](int64_t it) {
-                const int64_t kk = it / groups;
-                const int c0 = static_cast<int>(it - kk * groups) << GL;
-                const uint32_t bytes = static_cast<uint32_t>(min(1 << GL, a.N1 - c0) * NN) * 8u;
-                mbar_arrive_expect_tx(zbar, bytes);
-                tma_bulk_g2s(zst, a.z + kk * a.N + static_cast<int64_t>(c0) * NN, bytes, zbar);
-            };
-            const bool keep = a.n_tones > 0;
-            const int N1 = a.N1;
-            if (threadIdx.x == 0 && blockIdx.x < a.F * groups) fetch(blockIdx.x);
-            for (int64_t it = blockIdx.x; it < a.F * groups; it += gridDim.x) {
-                const int64_t kk = it / groups;
-                const int c0 = static_cast<int>(it - kk * groups) << GL;
-                if (!mbar_wait(zbar, zphase, a.status)) return;
-                zphase ^= 1u;
-                auto none = [](int, float2) {};
-                // (rows past a last group's are not copied: their outputs go nowhere)
-                fixed_stage<R0, TH, NN, GL, 1, false, 2>(zst, sm, t0, none);
-                if (threadIdx.x == 0 && it + gridDim.x < a.F * groups) fetch(it + gridDim.x);
-                const int64_t k = a.k0 + kk;
-                float2* row = a.full ? a.full + (a.fo + k) * a.full_ld + c0 : nullptr;
-                // the group's tones, a thread each (their loads in flight meanwhile)
-                int i0 = 0, i1 = 0;
-                int2 te = make_int2(0, 0);
-                if (keep) {
-                    i0 = __ldg(a.goff + (c0 >> GL)) + threadIdx.x;
-                    i1 = __ldg(a.goff + (c0 >> GL) + 1);
-                    if (i0 < i1) te = __ldg(a.gtone + i0);
-                }
-                float2 v[iters][R1];
+        constexpr int R0 = 25, R1 = 10, NN = 250, GL = 4, nb = (NN / R1) << GL, iters = (nb + TH - 1) / TH;
+        // (the second buffer's place at run time: as a constant, 1 % slower)
+        float2* const sm1 = second_buffer(sm, E);
+        float2* const zst = sm1 + ((reinterpret_cast<uintptr_t>(sm1) & 8) ? 1 : 0);
+        const float2* const t0 = a.tw_b + a.fb.tw_off[0];
+        auto fetch = [&](int64_t it) {
+            const int64_t kk = it / groups;
+            const int c0 = static_cast<int>(it - kk * groups) << GL;
+            const uint32_t bytes = static_cast<uint32_t>(min(1 << GL, a.N1 - c0) * NN) * 8u;
+            mbar_arrive_expect_tx(zbar, bytes);
+            tma_bulk_g2s(zst, a.z + kk * a.N + static_cast<int64_t>(c0) * NN, bytes, zbar);
+        };
+        const bool keep = a.n_tones > 0;
+        const int N1 = a.N1;
+        if (threadIdx.x == 0 && blockIdx.x < a.F * groups) fetch(blockIdx.x);
+        for (int64_t it = blockIdx.x; it < a.F * groups; it += gridDim.x) {
+            const int64_t kk = it / groups;
+            const int c0 = static_cast<int>(it - kk * groups) << GL;
+            if (!mbar_wait(zbar, zphase, a.status)) return;
+            zphase ^= 1u;
+            auto none = [](int, float2) {};
+            // (rows past a last group's are not copied: their outputs go nowhere)
+            fixed_stage<R0, TH, NN, GL, 1, false, 2>(zst, sm, t0, none);
+            if (threadIdx.x == 0 && it + gridDim.x < a.F * groups) fetch(it + gridDim.x);
+            const int64_t k = a.k0 + kk;
+            float2* row = a.full ? a.full + (a.fo + k) * a.full_ld + c0 : nullptr;
+            // the group's tones, a thread each (their loads in flight meanwhile)
+            int i0 = 0, i1 = 0;
+            int2 te = make_int2(0, 0);
+            if (keep) {
+                i0 = __ldg(a.goff + (c0 >> GL)) + threadIdx.x;
+                i1 = __ldg(a.goff + (c0 >> GL) + 1);
+                if (i0 < i1) te = __ldg(a.gtone + i0);
+            }
+            float2 v[iters][R1];
 #pragma unroll
-                for (int i = 0; i < iters; ++i) {
-                    const int u = static_cast<int>(threadIdx.x) + i * TH;
-                    if (u >= nb) break;
-                    load_strided<R1>(v[i], sm, u, nb);
-                    const int kt = (u >> GL) % R0;
+            for (int i = 0; i < iters; ++i) {
+                const int u = static_cast<int>(threadIdx.x) + i * TH;
+                if (u >= nb) break;
+                load_strided<R1>(v[i], sm, u, nb);
+                const int kt = (u >> GL) % R0;
 #pragma unroll
-                    for (int r = 1; r < R1; ++r) v[i][r] = cmul(v[i][r], __ldg(t0 + (r - 1) * R0 + kt));
-                    dft_any<R1>(v[i]);
-                }
-                if (keep) __syncthreads();                   // the stage's reads of sm are done
+                for (int r = 1; r < R1; ++r) v[i][r] = cmul(v[i][r], __ldg(t0 + (r - 1) * R0 + kt));
+                dft_any<R1>(v[i]);
+            }
+            if (keep) __syncthreads();                   // the stage's reads of sm are done
 #pragma unroll
-                for (int i = 0; i < iters; ++i) {
-                    const int u = static_cast<int>(threadIdx.x) + i * TH;
-                    if (u >= nb) break;
-                    const int g = u & ((1 << GL) - 1), j = u >> GL, kt = j % R0;
-                    const int base = (j - kt) * R1 + kt;
+            for (int i = 0; i < iters; ++i) {
+                const int u = static_cast<int>(threadIdx.x) + i * TH;
+                if (u >= nb) break;
+                const int g = u & ((1 << GL) - 1), j = u >> GL, kt = j % R0;
+                const int base = (j - kt) * R1 + kt;
 #pragma unroll
-                    for (int r = 0; r < R1; ++r) {
-                        const int c2 = base + r * R0;
-                        if (row && c0 + g < N1) row[g + static_cast<int64_t>(N1) * c2] = v[i][r];
-                        if (keep) sm[gpad((c2 << GL) + g)] = v[i][r];
-                    }
-                }
-                __syncthreads();
-                if (keep) {
-                    for (int i = i0; i < i1; i += TH) {
-                        if (i != i0) te = __ldg(a.gtone + i);
-                        a.tones[te.x * a.tones_ld + a.fo + k] = sm[gpad(te.y)];
-                    }
-                    __syncthreads();
+                for (int r = 0; r < R1; ++r) {
+                    const int c2 = base + r * R0;
+                    if (row && c0 + g < N1) row[g + static_cast<int64_t>(N1) * c2] = v[i][r];
+                    if (keep) sm[gpad((c2 << GL) + g)] = v[i][r];
                 }
             }
-            return;
+            __syncthreads();
+            if (keep) {
+                for (int i = i0; i < i1; i += TH) {
+                    if (i != i0) te = __ldg(a.gtone + i);
+                    a.tones[te.x * a.tones_ld + a.fo + k] = sm[gpad(te.y)];
+                }
+                __syncthreads();
+            }
         }
+        return;
     }
     // Any other lengths: as in pass A, except that with tones the buffer that the last
     // stage does not read holds its outputs for the gather, and the next rows land in
@@ -1396,10 +1396,13 @@ cudaError_t gen_run(GenArgs a, const PfbLaunch& L, const GenPlan& g, cudaStream_
             }
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
         }
-        e = launch_gen<TH>(gen_pass_a_kernel<TH>, a.F * groups_a, g.N1 * ga, L.n_sms, L.max_smem, st,
+        constexpr bool kFix = TH == 256;                         // compiled-in instances
+        const bool fa = kFix && a.fixa == 1 && a.vtma && a.vsstride == a.vbox_rows * ga;
+        const bool fb = kFix && a.fixb == 2 && a.zbulk;
+        e = launch_gen<TH>(fa ? gen_pass_a_kernel<TH, kFix> : gen_pass_a_kernel<TH, false>, a.F * groups_a, g.N1 * ga, L.n_sms, L.max_smem, st,
                            3 * kTwDigit * sizeof(float2) + 16, a, tmv);
         if (e != cudaSuccess) return e;
-        e = launch_gen<TH>(gen_pass_b_kernel<TH>, a.F * groups_b, g.N2 * gb, L.n_sms, L.max_smem, st, 16, a);
+        e = launch_gen<TH>(fb ? gen_pass_b_kernel<TH, kFix> : gen_pass_b_kernel<TH, false>, a.F * groups_b, g.N2 * gb, L.n_sms, L.max_smem, st, 16, a);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
