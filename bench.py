@@ -675,9 +675,9 @@ def run_large_n(args, dev, stream, x, words):
     two-pass form), and the workload's N = 4096, T = 8 Kaiser(9) oversampled
     4x (hop 1024, the mixed-radix one-pass form); and the batched workload's
     power-of-two shapes whose FP32 delay line does not fit one SM's tensor
-    memory (N = 16384 and 8192 with T = 8, direct kernel with its pre-sum
-    FIR pass, and cluster kernel; N = 4096 T = 16 (pre-sum pass + TMEM
-    kernel), N = 16384 T = 16 (pre-sum pass + direct kernel); Kaiser(9));
+    memory (N = 16384 and 8192 with T = 8, pre-sum FIR pass and rows kernel,
+    and cluster kernel; N = 4096 and N = 16384 with T = 16, pre-sum FIR pass
+    and rows kernel; Kaiser(9));
     each on the workload's 2^28-sample stream, full spectrum + its 1000 tones."""
     import torch
 
@@ -727,7 +727,7 @@ def run_large_n(args, dev, stream, x, words):
             cms = e0.elapsed_time(e1) / reps
             res["cluster_kernel"] = {"value": n / (cms * 1e-3) / 1e6, "unit": UNIT, "ms": cms,
                                      "form": f"clusters of {N // 4096} CTAs, filtered slices exchanged through "
-                                             "distributed shared memory (the default is the direct kernel)"}
+                                             "distributed shared memory (the default is the pre-sum pass and rows kernel)"}
             pc.close()
         if not args.no_plain and N <= 100000 and hop == N:
             # the plain FP32 form on the same stream: FP32 FIR kernel + cuFFT + gather

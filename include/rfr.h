@@ -169,7 +169,9 @@ typedef struct {
  * push that grows scratch synchronises the device and sizes it for that many
  * samples after any carry.  Inside a stream capture such a push fails with
  * RFR_E_INVALID instead, so push once at the largest size outside capture
- * first.
+ * first.  (N = 16384 with T <= 4 needs no scratch: where its rows cannot grow, in a
+ * capture or on a full device, the FIR runs in the FFT kernel, and rows that a
+ * captured push uses stay as long as the plan.)
  * Errors: RFR_E_INVALID (parameters), RFR_E_NOMEM, RFR_E_CUDA.
  */
 rfr_status rfr_plan_create(rfr_plan** plan, int32_t channels, int32_t taps,

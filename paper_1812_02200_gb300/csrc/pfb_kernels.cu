@@ -947,7 +947,7 @@ __global__ void __launch_bounds__(kSymThreads, 1)
 // no further copies) so that no peer is left waiting.  A plan choice
 // (rfr_plan_set_pfb_cluster), not the default: with one frame in flight per
 // CTA the exchanges and the two cluster barriers of every frame stay
-// exposed, and the direct kernel measured faster.
+// exposed, and the pre-sum pass with the rows kernel measured faster.
 constexpr int kClusterTonesPerCta = kTonesPerThread * kRingThreads;
 struct ClusterLayout {
     size_t xb, tw, bins, tile, bars, total;

@@ -376,8 +376,9 @@ class Plan:
         self._check(_lib.rfr_plan_seek(self._h, int(start_sample), _ptr(history), n), "seek")
 
     def set_tone_tile(self, tones_per_tile: int):
-        """Three-product demodulation: tones per GEMM tile (128 or 64);
-        result-neutral, normally chosen by autotune()."""
+        """Three-product demodulation: tones per single-CTA GEMM tile (128 or 64)
+        instead of the form picked by size; result-neutral, normally chosen by
+        autotune()."""
         self._check(_lib.rfr_plan_set_tone_tile(self._h, int(tones_per_tile)), "set_tone_tile")
 
     def set_fused_presplit(self, on: bool):
@@ -387,14 +388,15 @@ class Plan:
         self._check(_lib.rfr_plan_set_fused_presplit(self._h, 1 if on else 0), "set_fused_presplit")
 
     def set_demod_pair(self, on: bool):
-        """Three-product demodulation: the GEMM in clusters of two CTAs that
-        share each frame tile by TMA multicast (True) or one CTA per tile
-        (False, the default); result-neutral, normally chosen by autotune()."""
+        """Three-product demodulation: the GEMM on two-SM tiles of 256 frames
+        (True) or one CTA per tile of 128 (False) instead of the form picked by
+        size (the default); result-neutral, normally chosen by autotune()."""
         self._check(_lib.rfr_plan_set_demod_pair(self._h, 1 if on else 0), "set_demod_pair")
 
     def set_pfb_cluster(self, on: bool):
         """PFB N = 8192 or 16384 with T <= 8: the cluster kernel (True) or the
-        direct kernel (False, the default); set before the first push."""
+        pre-sum FIR pass and the rows kernel (False, the default); set before
+        the first push."""
         self._check(_lib.rfr_plan_set_pfb_cluster(self._h, 1 if on else 0), "set_pfb_cluster")
 
     def inject_device_status(self, status: int):
