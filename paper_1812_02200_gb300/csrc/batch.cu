@@ -42,9 +42,10 @@ struct rfr_batch {
     void* d_g3 = nullptr;                  // scratch of their launches where no plan's is large enough
     size_t g3_bytes = 0;
     cudaStream_t origin = nullptr;
-    cudaStream_t gemm_stream = nullptr;    // the persistent GEMM launch of the step
+    // the persistent GEMM launches of the step, one branch for each kind of kernel
+    cudaStream_t gemm_stream[rfr::kDemodKinds] = {};
+    cudaEvent_t ev_gemm[rfr::kDemodKinds] = {};
     cudaEvent_t ev_fork = nullptr;
-    cudaEvent_t ev_gemm = nullptr;
     cudaGraphExec_t exec = nullptr;
     int64_t steps = 0, updates = 0, instantiations = 0;
     std::string last_error;
@@ -63,9 +64,11 @@ void batch_destroy(rfr_batch* b) {
     for (auto s : b->branches) cudaStreamDestroy(s);
     for (auto e : b->ev_join) cudaEventDestroy(e);
     if (b->ev_fork) cudaEventDestroy(b->ev_fork);
-    if (b->ev_gemm) cudaEventDestroy(b->ev_gemm);
+    for (auto e : b->ev_gemm)
+        if (e) cudaEventDestroy(e);
     if (b->origin) cudaStreamDestroy(b->origin);
-    if (b->gemm_stream) cudaStreamDestroy(b->gemm_stream);
+    for (auto s : b->gemm_stream)
+        if (s) cudaStreamDestroy(s);
     if (b->d_g3) cudaFree(b->d_g3);
     delete b;
 }
@@ -174,9 +177,10 @@ rfr_status rfr_batch_create(rfr_batch** out, rfr_plan* const* plans, int32_t n) 
     b->ev_join.resize(n, nullptr);
     b->jobs.resize(n);
     bool ok = cudaStreamCreateWithFlags(&b->origin, cudaStreamNonBlocking) == cudaSuccess &&
-              cudaStreamCreateWithFlags(&b->gemm_stream, cudaStreamNonBlocking) == cudaSuccess &&
-              cudaEventCreateWithFlags(&b->ev_gemm, cudaEventDisableTiming) == cudaSuccess &&
               cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming) == cudaSuccess;
+    for (int k = 0; k < rfr::kDemodKinds; ++k)
+        ok = ok && cudaStreamCreateWithFlags(&b->gemm_stream[k], cudaStreamNonBlocking) == cudaSuccess &&
+             cudaEventCreateWithFlags(&b->ev_gemm[k], cudaEventDisableTiming) == cudaSuccess;
     for (auto& s : b->branches) ok = ok && cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) == cudaSuccess;
     for (auto& e : b->ev_join) ok = ok && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess;
     if (!ok) {
@@ -235,8 +239,8 @@ rfr_status rfr_batch_push(rfr_batch* b, const int16_t* const* bufs, const int64_
         return batch_fail(b, RFR_E_CUDA, "begin capture");
     rfr_status err = RFR_OK;
     cudaEventRecord(b->ev_fork, b->origin);
-    cudaStreamWaitEvent(b->gemm_stream, b->ev_fork, 0);
     std::vector<const rfr::DemodGemmJob*> gemms;
+    bool kinds[rfr::kDemodKinds] = {};
     for (int i = 0; i < n && err == RFR_OK; ++i) {
         cudaStream_t br = b->branches[i % b->branches.size()];
         cudaStreamWaitEvent(br, b->ev_fork, 0);
@@ -247,22 +251,28 @@ rfr_status rfr_batch_push(rfr_batch* b, const int16_t* const* bufs, const int64_
         cudaEventRecord(b->ev_join[i], br);
         if (b->jobs[i].n_units > 0) {
             // the plan's GEMM waits for its pre-GEMM kernels
-            cudaStreamWaitEvent(b->gemm_stream, b->ev_join[i], 0);
+            cudaStreamWaitEvent(b->gemm_stream[b->jobs[i].kind], b->ev_join[i], 0);
+            kinds[b->jobs[i].kind] = true;
             gemms.push_back(&b->jobs[i]);
         } else {
             cudaStreamWaitEvent(b->origin, b->ev_join[i], 0);
         }
     }
-    if (err == RFR_OK && !gemms.empty()) {
-        const cudaError_t ge = rfr::demod3_gemm(gemms.data(), static_cast<int>(gemms.size()), b->plans[0]->n_sms,
-                                                scratch, room, b->gemm_stream);
-        if (ge != cudaSuccess) {
-            err = RFR_E_CUDA;
-            b->last_error = std::string("batched GEMM launch: ") + cudaGetErrorString(ge);
+    // (each kind of kernel on a branch of its own: one's last CTAs leave room for the
+    // next's, and small steps of mixed kinds do not run one after the other)
+    for (int k = 0; k < rfr::kDemodKinds; ++k) {
+        if (!kinds[k]) continue;
+        if (err == RFR_OK) {
+            const cudaError_t ge = rfr::demod3_gemm(gemms.data(), static_cast<int>(gemms.size()), b->plans[0]->n_sms,
+                                                    scratch, room, b->gemm_stream[k], k);
+            if (ge != cudaSuccess) {
+                err = RFR_E_CUDA;
+                b->last_error = std::string("batched GEMM launch: ") + cudaGetErrorString(ge);
+            }
         }
+        cudaEventRecord(b->ev_gemm[k], b->gemm_stream[k]);
+        cudaStreamWaitEvent(b->origin, b->ev_gemm[k], 0);
     }
-    cudaEventRecord(b->ev_gemm, b->gemm_stream);
-    cudaStreamWaitEvent(b->origin, b->ev_gemm, 0);
     cudaGraph_t graph = nullptr;
     const cudaError_t ce = cudaStreamEndCapture(b->origin, &graph);
     if (err != RFR_OK) {

@@ -680,9 +680,11 @@ __device__ __forceinline__ float2 g3_output(float p1, float p2, float p3, float 
     return g3_rotate(fmaf(2.f, p1, -p3), fmaf(2.f, p1, p2), inv_scale, an, sp);
 }
 
-// Outputs of a CTA's last tile, by all its epilogue and finisher warps: lane l
-// takes frames l + 32 r (r < 4) of the tile, warp w of nw (less the `skip` producer
-// and MMA warps between the two kinds) every tone of its number, FT in flight.
+// Outputs of a CTA's last tile, by all its epilogue and finisher warps (in 16-byte
+// loads: frames l + 32 r a lane in 4-byte ones took 20 us more, 237 -> 256 for a push
+// of one wave with L = 4096): lane l
+// takes frames 4 l .. 4 l + 3, warp w of nw (less the `skip` producer and MMA
+// warps between the two kinds) every tone of its number, FT in flight.
 __device__ __noinline__ void g3_finish(const G3Plan& P, const G3Unit u, const float* scr_cta, uint32_t tile, int lane,
                                           int w, int nw, int skip) {
     constexpr int FT = 2;
@@ -691,10 +693,14 @@ __device__ __noinline__ void g3_finish(const G3Plan& P, const G3Unit u, const fl
     nw -= skip;
     const float* pl[3];
 #pragma unroll
-    for (int q = 0; q < 3; ++q) pl[q] = scr_cta + ((3 * tile + q) % G3_PLANES) * G3_PLANE + lane;
-    const int64_t k = u.m0 + lane;                   // the lane's first frame
-    const int at = static_cast<int>(g.F0 % BM) + lane;   // its place from the tile's first anchor on
-    const float2* const anc = g.anchors + ((g.F0 + u.m0) / BM - g.F0 / BM) * g.ntp + u.n0;
+    for (int q = 0; q < 3; ++q) pl[q] = scr_cta + ((3 * tile + q) % G3_PLANES) * G3_PLANE + 4 * lane;
+    const int64_t k = u.m0 + 4 * lane;               // the lane's first frame
+    const int64_t K = g.F0 + k;
+    const int rows = static_cast<int>(k < g.F ? (g.F - k < 4 ? g.F - k : 4) : 0);
+    if (rows == 0) return;
+    // four frames of one anchor row, with aligned steps; 16-byte stores
+    const bool near = (g.F0 & 3) == 0;
+    const bool vec = rows == 4 && ((reinterpret_cast<uintptr_t>(g.out + g.fo + k) | static_cast<uintptr_t>(g.ld * 8)) & 15) == 0;
     const int n = min(u.width, g.n_tones - u.n0);
 #pragma unroll 1
     for (int c0 = w; c0 < n; c0 += nw * FT) {
@@ -702,25 +708,53 @@ __device__ __noinline__ void g3_finish(const G3Plan& P, const G3Unit u, const fl
         float2 an[FT][4], sp[FT][4];
 #pragma unroll
         for (int f = 0; f < FT; ++f) {
-            const int c = c0 + f * nw;
+            const int c = c0 + f * nw, t = u.n0 + c;
             if (c >= n) continue;
 #pragma unroll
-            for (int r = 0; r < 4; ++r) {
-                if (k + 32 * r >= g.F) continue;
+            for (int q = 0; q < 3; ++q) {
+                const float4 v = __ldcg(reinterpret_cast<const float4*>(pl[q] + c * 128));
+                p[f][q][0] = v.x;
+                p[f][q][1] = v.y;
+                p[f][q][2] = v.z;
+                p[f][q][3] = v.w;
+            }
+            const float2* anc = g.anchors + t - (g.F0 / BM) * g.ntp;
+            const float2* stp = g.steps + static_cast<int64_t>(t) * BM;
+            if (near) {
+                an[f][0] = __ldg(anc + (K / BM) * g.ntp);
+                an[f][1] = an[f][2] = an[f][3] = an[f][0];
+                const float4* s4 = reinterpret_cast<const float4*>(stp + static_cast<int>(K % BM));
+                const float4 s0 = __ldg(s4), s1 = __ldg(s4 + 1);
+                sp[f][0] = make_float2(s0.x, s0.y);
+                sp[f][1] = make_float2(s0.z, s0.w);
+                sp[f][2] = make_float2(s1.x, s1.y);
+                sp[f][3] = make_float2(s1.z, s1.w);
+            } else {
 #pragma unroll
-                for (int q = 0; q < 3; ++q) p[f][q][r] = __ldcg(pl[q] + c * 128 + 32 * r);
-                an[f][r] = __ldg(anc + c + (at + 32 * r >= BM ? g.ntp : 0));
-                sp[f][r] = __ldg(g.steps + static_cast<int64_t>(u.n0 + c) * BM + ((at + 32 * r) & (BM - 1)));
+                for (int r = 0; r < 4; ++r) {
+                    const int64_t Kr = r < rows ? K + r : K;
+                    an[f][r] = __ldg(anc + (Kr / BM) * g.ntp);
+                    sp[f][r] = __ldg(stp + static_cast<int>(Kr % BM));
+                }
             }
         }
 #pragma unroll
         for (int f = 0; f < FT; ++f) {
-            const int c = c0 + f * nw;
+            const int c = c0 + f * nw, t = u.n0 + c;
             if (c >= n) continue;
-            float2* o = g.out + static_cast<int64_t>(u.n0 + c) * g.ld + g.fo + k;
+            float2* o = g.out + static_cast<int64_t>(t) * g.ld + g.fo + k;
+            float2 y[4];
 #pragma unroll
             for (int r = 0; r < 4; ++r)
-                if (k + 32 * r < g.F) o[32 * r] = g3_output(p[f][0][r], p[f][1][r], p[f][2][r], g.inv_scale, an[f][r], sp[f][r]);
+                y[r] = g3_output(p[f][0][r], p[f][1][r], p[f][2][r], g.inv_scale, an[f][r], sp[f][r]);
+            if (vec) {
+                reinterpret_cast<float4*>(o)[0] = make_float4(y[0].x, y[0].y, y[1].x, y[1].y);
+                reinterpret_cast<float4*>(o)[1] = make_float4(y[2].x, y[2].y, y[3].x, y[3].y);
+            } else {
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+                    if (r < rows) o[r] = y[r];
+            }
         }
     }
 }
@@ -904,9 +938,14 @@ demod3m_gemm_kernel(const __grid_constant__ G3Batch bt) {
         // The whole warp runs the loops and one elected thread issues, so that control
         // flow, descriptors and addresses stay in uniform registers.  (Run by one thread
         // alone, every MMA took about 115 clocks to issue whatever its width: 1370 a
-        // K-block, where tiles of 128 tones need 960.)
-        if (rank == 0) {
-            const bool leader = umma::elect_one();
+        // K-block, where tiles of 128 tones need 960.)  Wide tiles' MMAs take 128 each:
+        // there one thread runs alone.
+        if (rank == 0 && (!WIDE || lane == 0)) {
+            const bool leader = WIDE || umma::elect_one();
+            auto agreed = [](bool ok) {
+                if constexpr (WIDE) return ok;
+                else return static_cast<bool>(__all_sync(0xffffffffu, ok));
+            };
             const uint64_t desc0 = umma::desc_k_sw128(smem_u32(smem));
             uint32_t phase = 0, s = 0, par = 0;             // chunk; stage and the parity of its use
             bool go = true;
@@ -923,12 +962,12 @@ demod3m_gemm_kernel(const __grid_constant__ G3Batch bt) {
                     for (int h0 = 0; h0 < H && go; h0 += chunk, ++phase) {
                         const int h1 = min(h0 + chunk, H);
                         const uint32_t slot = phase % SLOTS, use = phase / SLOTS;
-                        go = __all_sync(0xffffffffu, !*abort_flag && mbar_wait(&sempty[slot], (use & 1) ^ 1, status0));
+                        go = agreed(!*abort_flag && mbar_wait(&sempty[slot], (use & 1) ^ 1, status0));
                         if (!go) break;
                         umma::fence_after_sync();
                         const uint32_t d_tmem = tmem + slot * TW;
                         auto arrived = [&] {                            // the block's operands
-                            go = __all_sync(0xffffffffu, mbar_wait(&full[s], par, status0));
+                            go = agreed(mbar_wait(&full[s], par, status0));
                             umma::fence_after_sync();
                             return go;
                         };
@@ -1575,13 +1614,15 @@ cudaError_t g3_run(const G3Batch& b, int n_sms, size_t room, cudaStream_t st) {
 }
 }  // namespace
 
-cudaError_t demod3_gemm(const DemodGemmJob* const* jobs, int n, int n_sms, void* scratch, size_t room, cudaStream_t st) {
+cudaError_t demod3_gemm(const DemodGemmJob* const* jobs, int n, int n_sms, void* scratch, size_t room, cudaStream_t st,
+                        int only) {
     // costliest work items first, so that the launch ends on short ones
     std::vector<const DemodGemmJob*> order(jobs, jobs + n);
     std::stable_sort(order.begin(), order.end(),
                      [](const DemodGemmJob* x, const DemodGemmJob* y) { return x->unit_cost > y->unit_cost; });
     // one persistent launch per group of up to kG3MaxPlans jobs of the same kind
-    for (int kind = 0; kind < 4; ++kind) {
+    for (int kind = 0; kind < kDemodKinds; ++kind) {
+        if (only >= 0 && kind != only) continue;
         G3Batch b;
         b.n_plans = 0;
         b.total_units = 0;

@@ -164,6 +164,7 @@ struct DemodLaunch {
 // The three-product GEMM of one push, described for a persistent launch that
 // may cover several plans (opaque record of demod.cu).
 constexpr int kDemodJobBytes = 2048;
+constexpr int kDemodKinds = 4;
 struct DemodGemmJob {
     alignas(128) unsigned char bytes[kDemodJobBytes];
     int kind = 0;               // the kernel's form (0 wide pair, 1 pair, 2 single CTA, 3 fused pre-split)
@@ -184,8 +185,10 @@ cudaError_t demod3_launch(const DemodLaunch& L, cudaStream_t st);
 // GEMM's description in *job (shared_launch: it will run beside other plans')
 cudaError_t demod3_prepare(const DemodLaunch& L, cudaStream_t st, DemodGemmJob* job, bool shared_launch);
 // persistent GEMM launch(es) over the jobs' work items (one per form and per
-// 16 plans); scratch: room bytes for the CTAs' parked products
-cudaError_t demod3_gemm(const DemodGemmJob* const* jobs, int n, int n_sms, void* scratch, size_t room, cudaStream_t st);
+// 16 plans; only: those of that kind); scratch: room bytes for the CTAs' parked
+// products (kind 0 alone has them, so that kinds may run beside each other)
+cudaError_t demod3_gemm(const DemodGemmJob* const* jobs, int n, int n_sms, void* scratch, size_t room, cudaStream_t st,
+                        int only = -1);
 size_t demod3_xs_rows(int64_t F, int Lpad, int D);
 // CTAs of a push of up to F frames that park products, at most, what they park in all,
 // and the scratch that such a push needs (never less for more frames)
